@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(128) k_adj_pairs(int n, Tape<Real> T, Grid G, 
         for (int d = 0; d < DIM; ++d) xbp[(size_t)d * n + k] = vbp[(size_t)d * n + k] = Real(0);
         sigb[k] = Real(0);
     }
-    block_partials<true>(part, partials + (size_t)blockIdx.x * kNPart);
+    block_partials(part, partials + (size_t)blockIdx.x * kNPart);
 }
 
 // ------------------------------------------------- density + drift / kick

@@ -16,9 +16,9 @@
 //                       held viscous force + g; v += dt a
 //   k_dual_drift      : x += dt/2 v
 //   k_dual_continuity : drho_i = 2 rho_i sum_j V_j (U* - U_l) dW/dr (Eq. 3
-//                       row 1, U* of Eq. 5 row 1), diagnostics partials
-//   k_dual_finalize   : reduction; the next substep size; marks the
-//                       advection step done after its last substep
+//                       row 1, U* of Eq. 5 row 1), diagnostics partials; its
+//                       last block folds them, sets the next substep size and
+//                       marks the advection step done after its last substep
 // and, once per advection step, k_dual_complete: rho += dt/2 drho of the last
 // substep.  Every substep kernel returns at once when the advection step is
 // done, so the host launches a few substeps more than it expects and waits
@@ -63,13 +63,11 @@ struct DualK {
     Real* R;                 // [DIM][n] residual
     Real* chi;               // [n] limiter
     double* du;              // DU_* state
-    double* partials;
+    GridSum B;
+    double* diag;
+    double* dt_ptr;
     uint32_t* err;
 };
-
-constexpr int kTPB64 = 256;
-constexpr int kTPB32 = 128;
-template <typename Real> constexpr int tpb() { return sizeof(Real) == 8 ? kTPB64 : kTPB32; }
 
 __device__ __forceinline__ bool dual_done(const double* du) { return du[DU_DONE] != 0.0; }
 
@@ -219,20 +217,15 @@ template <> __device__ __forceinline__ float fma_free_mul<float>(float a, float 
 
 // ------------------------------------------------------------------ begin
 
-struct DualConsts {
-    double eta, rho0, h_min, u_ref, cfl_ad, cfl_ac, c;
-};
-
 // Eq. 9-11 with h = h_min from max |v| of the fluid (the diagnostics of the
 // previous step or of sph_build_cells; the sort does not change v).
-__global__ void k_dual_begin(DualConsts D, const double* __restrict__ diag, double* __restrict__ du)
+__global__ void k_dual_begin(DtConsts D, const double* __restrict__ diag, double* __restrict__ du)
 {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     const double vmax = diag[DG_VMAX];
-    const double nu = D.eta / D.rho0;
-    const double vad = fmax(vmax, fmax(nu / D.h_min, D.u_ref));
-    const double Dt = D.cfl_ad * D.h_min / vad;
-    double dt = D.cfl_ac * D.h_min / (vmax + D.c);
+    const double vad = fmax(vmax, D.v_floor);
+    const double Dt = D.ad / vad;
+    double dt = D.ac / (vmax + D.c);
     const double rem = Dt - 0.0;
     const int last = !(dt < rem);      // also ends the step on a non-finite size
     if (last) dt = rem;
@@ -444,8 +437,50 @@ __global__ void __launch_bounds__(256) k_dual_drift(DualK<Real> A, Grid G)
     if (sizeof(Real) == 4) A.pos4[i] = make_float4(of[0], of[1], of[2], p.w);
 }
 
+// The end of a substep, from the grid's totals: advance t; pick the next
+// substep size, or finish the advection step and write the diagnostics.
+__device__ __forceinline__ void finish_substep(const double* out, const DtConsts& D, double* __restrict__ du,
+                                               double* __restrict__ diag, double* __restrict__ dt_ptr)
+{
+    if (threadIdx.x != 0) return;
+    const double vmax = out[6];
+    const double dt = du[DU_DT];
+    const double t = du[DU_T] + dt;
+    const double k = du[DU_K] + 1.0;
+    du[DU_T] = t;
+    du[DU_K] = k;
+    du[DU_HDT_PREV] = 0.5 * dt;
+    du[DU_FIRST] = 0.0;
+    if (du[DU_LAST] != 0.0) {
+        const double Dt = du[DU_DT_AD];
+        const double vad = fmax(vmax, D.v_floor);
+        diag[DG_MASS] = out[0];
+        diag[DG_MOM + 0] = out[1];
+        diag[DG_MOM + 1] = out[2];
+        diag[DG_MOM + 2] = out[3];
+        diag[DG_KE] = out[4];
+        diag[DG_NCHI] = out[5];
+        diag[DG_VMAX] = vmax;
+        diag[DG_VTMAX] = out[7];
+        diag[DG_DRMAX] = out[8];
+        diag[DG_DT] = Dt;
+        diag[DG_DTNEXT] = D.ad / vad;
+        diag[DG_STEPS] = diag[DG_STEPS] + 1.0;
+        diag[DG_SUBSTEPS] = k;
+        *dt_ptr = Dt;
+        du[DU_DONE] = 1.0;
+        return;
+    }
+    double dtn = D.ac / (vmax + D.c);
+    const double rem = du[DU_DT_AD] - t;
+    const int last = !(dtn < rem);     // also ends the step on a non-finite size
+    if (last) dtn = rem;
+    du[DU_DT] = dtn;
+    du[DU_LAST] = last;
+}
+
 template <typename Real, int DIM, typename Acc, bool UNIFORM>
-__global__ void __launch_bounds__(sizeof(Real) == 8 ? 256 : 128) k_dual_continuity(DualK<Real> A, Grid G, Consts<Real> K)
+__global__ void __launch_bounds__(sizeof(Real) == 8 ? 256 : 128) k_dual_continuity(DualK<Real> A, Grid G, Consts<Real> K, DtConsts D)
 {
     __shared__ float4 tab[kCodes];
     if (dual_done(A.du)) return;
@@ -531,63 +566,17 @@ __global__ void __launch_bounds__(sizeof(Real) == 8 ? 256 : 128) k_dual_continui
     }
     // the sums (mass, momentum, KE) only after the last substep: in the others
     // they are all zero, and their FP64 shuffles would cost every substep
-    block_partials<true>(part, A.partials + (size_t)blockIdx.x * kNPart, A.du[DU_LAST] != 0.0);
+    __shared__ double total[kNPart];
+    if (grid_partials(part, A.B, total, A.du[DU_LAST] != 0.0)) finish_substep(total, D, A.du, A.diag, A.dt_ptr);
 }
 
-// Reduce the substep's partials (in a fixed order); advance t; pick the next
-// substep size, or finish the advection step and write the diagnostics.
-__global__ void __launch_bounds__(256) k_dual_finalize(int nblocks, const double* __restrict__ partials, DualConsts D,
-                                                       double* __restrict__ du, double* __restrict__ diag,
-                                                       double* __restrict__ dt_ptr)
+// The rows of a large grid (see GridSum), and the end of the substep.
+__global__ void __launch_bounds__(256) k_fold_substep(GridSum B, int nrows, DtConsts D, double* du,
+                                                      double* __restrict__ diag, double* __restrict__ dt_ptr)
 {
     if (dual_done(du)) return;
-    double acc[kNPart];
-#pragma unroll
-    for (int k = 0; k < kNPart; ++k) acc[k] = 0.0;
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
-        const double* p = partials + (size_t)b * kNPart;
-#pragma unroll
-        for (int k = 0; k < kNPart; ++k) acc[k] = (k >= 6 && k <= 8) ? fmax(acc[k], p[k]) : acc[k] + p[k];
-    }
-    __shared__ double out[kNPart];
-    block_partials<false>(acc, out);
-    __syncthreads();
-    if (threadIdx.x != 0) return;
-    const double vmax = out[6];
-    const double dt = du[DU_DT];
-    const double t = du[DU_T] + dt;
-    const double k = du[DU_K] + 1.0;
-    du[DU_T] = t;
-    du[DU_K] = k;
-    du[DU_HDT_PREV] = 0.5 * dt;
-    du[DU_FIRST] = 0.0;
-    if (du[DU_LAST] != 0.0) {
-        const double Dt = du[DU_DT_AD];
-        const double nu = D.eta / D.rho0;
-        const double vad = fmax(vmax, fmax(nu / D.h_min, D.u_ref));
-        diag[DG_MASS] = out[0];
-        diag[DG_MOM + 0] = out[1];
-        diag[DG_MOM + 1] = out[2];
-        diag[DG_MOM + 2] = out[3];
-        diag[DG_KE] = out[4];
-        diag[DG_NCHI] = out[5];
-        diag[DG_VMAX] = vmax;
-        diag[DG_VTMAX] = out[7];
-        diag[DG_DRMAX] = out[8];
-        diag[DG_DT] = Dt;
-        diag[DG_DTNEXT] = D.cfl_ad * D.h_min / vad;
-        diag[DG_STEPS] = diag[DG_STEPS] + 1.0;
-        diag[DG_SUBSTEPS] = k;
-        *dt_ptr = Dt;
-        du[DU_DONE] = 1.0;
-        return;
-    }
-    double dtn = D.cfl_ac * D.h_min / (vmax + D.c);
-    const double rem = du[DU_DT_AD] - t;
-    const int last = !(dtn < rem);     // also ends the step on a non-finite size
-    if (last) dtn = rem;
-    du[DU_DT] = dtn;
-    du[DU_LAST] = last;
+    __shared__ double total[kNPart];
+    if (fold_grid(B, nrows, total)) finish_substep(total, D, du, diag, dt_ptr);
 }
 
 // Second half of the last substep's density update: rho += dt/2 drho.
@@ -623,53 +612,53 @@ DualK<Real> dual_k(const DualArgs& a)
     k.R = (Real*)a.R;
     k.chi = (Real*)a.chi;
     k.du = a.du;
-    k.partials = a.partials;
+    k.B = grid_sum(a.F, pair_blocks(sizeof(Real) == 8 ? 64 : 32, a.n, a.sms));
+    k.diag = a.F.diag;
+    k.dt_ptr = a.F.dt;
     k.err = a.err;
     return k;
-}
-
-DualConsts dual_consts(const sph_params& P)
-{
-    return DualConsts{P.eta, P.rho0, P.h_min, P.u_ref, P.cfl_ad, P.cfl_ac, P.c0};
 }
 
 // Pair kernel dispatch: precision, dimension, compensated sums (FP32) and
 // uniform resolution (FP32) are template arguments.
 template <template <typename, int, typename, bool> class Kern> struct Dispatch;
 
-#define SPH_DUAL_PAIR_KERNEL(name)                                                                         \
+#define SPH_DUAL_PAIR_KERNEL(name, ...)                                                                    \
     template <typename Real, int DIM, typename Acc, bool U>                                                \
     struct name##_t {                                                                                      \
-        static void run(const DualK<Real>& A, const Grid& G, const Consts<Real>& K, cudaStream_t st)     \
+        static void run(const DualK<Real>& A, const Grid& G, const Consts<Real>& K, const DtConsts& D,    \
+                        cudaStream_t st)                                                                   \
         {                                                                                                  \
             const int T = pair_threads(sizeof(Real) == 8 ? 64 : 32, A.n, G.sms);                            \
-            name<Real, DIM, Acc, U><<<nblk(A.n, T), T, 0, st>>>(A, G, K);                                    \
+            (void)D;                                                                                       \
+            name<Real, DIM, Acc, U><<<nblk(A.n, T), T, 0, st>>>(A, G, K, ##__VA_ARGS__);                     \
         }                                                                                                  \
     };
 SPH_DUAL_PAIR_KERNEL(k_dual_advect)
 SPH_DUAL_PAIR_KERNEL(k_dual_pressure)
-SPH_DUAL_PAIR_KERNEL(k_dual_continuity)
+SPH_DUAL_PAIR_KERNEL(k_dual_continuity, D)
 #undef SPH_DUAL_PAIR_KERNEL
 
 template <template <typename, int, typename, bool> class KT>
 void run_pair(int prec, int dim, const DualArgs& a, const Grid& G, const void* Kp, cudaStream_t st)
 {
+    const DtConsts D = dt_consts(*a.F.P);
     if (prec == 64) {
         const auto A = dual_k<double>(a);
         const auto& K = *(const Consts<double>*)Kp;
-        if (dim == 2) KT<double, 2, PlainD, false>::run(A, G, K, st);
-        else KT<double, 3, PlainD, false>::run(A, G, K, st);
+        if (dim == 2) KT<double, 2, PlainD, false>::run(A, G, K, D, st);
+        else KT<double, 3, PlainD, false>::run(A, G, K, D, st);
         return;
     }
     const auto A = dual_k<float>(a);
     const auto& K = *(const Consts<float>*)Kp;
     const bool u = K.uniform_h != 0, ks = K.kahan != 0;
     if (dim == 2) {
-        if (ks) u ? KT<float, 2, KSum, true>::run(A, G, K, st) : KT<float, 2, KSum, false>::run(A, G, K, st);
-        else u ? KT<float, 2, PlainF, true>::run(A, G, K, st) : KT<float, 2, PlainF, false>::run(A, G, K, st);
+        if (ks) u ? KT<float, 2, KSum, true>::run(A, G, K, D, st) : KT<float, 2, KSum, false>::run(A, G, K, D, st);
+        else u ? KT<float, 2, PlainF, true>::run(A, G, K, D, st) : KT<float, 2, PlainF, false>::run(A, G, K, D, st);
     } else {
-        if (ks) u ? KT<float, 3, KSum, true>::run(A, G, K, st) : KT<float, 3, KSum, false>::run(A, G, K, st);
-        else u ? KT<float, 3, PlainF, true>::run(A, G, K, st) : KT<float, 3, PlainF, false>::run(A, G, K, st);
+        if (ks) u ? KT<float, 3, KSum, true>::run(A, G, K, D, st) : KT<float, 3, KSum, false>::run(A, G, K, D, st);
+        else u ? KT<float, 3, PlainF, true>::run(A, G, K, D, st) : KT<float, 3, PlainF, false>::run(A, G, K, D, st);
     }
 }
 
@@ -691,11 +680,9 @@ void run_elem(int dim, const DualArgs& a, const Grid& G, int which, cudaStream_t
 
 }  // namespace
 
-int dual_pair_blocks(int prec, int n, int sms) { return pair_blocks(prec, n, sms); }
-
 cudaError_t launch_dual_begin(const sph_params& P, const double* diag, double* du, cudaStream_t st)
 {
-    k_dual_begin<<<1, 32, 0, st>>>(dual_consts(P), diag, du);
+    k_dual_begin<<<1, 32, 0, st>>>(dt_consts(P), diag, du);
     return cudaGetLastError();
 }
 
@@ -706,8 +693,7 @@ cudaError_t launch_dual_advect(int prec, int dim, const DualArgs& a, const Grid&
 }
 
 cudaError_t launch_dual_substep(int prec, int dim, const DualArgs& a, const Grid& G, const void* K,
-                                const sph_params& P, double* diag, double* dt_ptr, cudaStream_t st,
-                                int64_t* launches)
+                                cudaStream_t st, int64_t* launches)
 {
     if (prec == 64) run_elem<double>(dim, a, G, 0, st);
     else run_elem<float>(dim, a, G, 0, st);
@@ -715,11 +701,13 @@ cudaError_t launch_dual_substep(int prec, int dim, const DualArgs& a, const Grid
     if (prec == 64) run_elem<double>(dim, a, G, 1, st);
     else run_elem<float>(dim, a, G, 1, st);
     run_pair<k_dual_continuity_t>(prec, dim, a, G, K, st);
-    const int nb = dual_pair_blocks(prec, a.n, G.sms);
-    const int rows = launch_reduce_rows(nb, a.partials, a.rows, st);
-    k_dual_finalize<<<1, 256, 0, st>>>(rows ? rows : nb, rows ? a.rows : a.partials, dual_consts(P), a.du, diag,
-                                       dt_ptr);
-    *launches += rows ? 6 : 5;
+    *launches += 4;
+    const int nb = pair_blocks(prec, a.n, a.sms);
+    const GridSum B = grid_sum(a.F, nb);
+    if (B.group == 0) {
+        k_fold_substep<<<kFoldBlocks, 256, 0, st>>>(B, nb, dt_consts(*a.F.P), a.du, a.F.diag, a.F.dt);
+        ++*launches;
+    }
     return cudaGetLastError();
 }
 

@@ -11,9 +11,9 @@
 //                 viscous acceleration (Eq. 7), residual R_i = sum_j V_j
 //                 grad_i W_ij (Eq. 14); then the limiter chi_i (Eq. 15), the
 //                 displacement dr_i = xi chi_i h^2 R_i (Eq. 16), the closing
-//                 half kick, and FP64 block partials of the diagnostics.
-//   k_finalize: reduces the partials in a fixed order, computes the next
-//               step size min(dt_ad, dt_ac) (Eq. 9-11, h = h_min).
+//                 half kick, and FP64 partials of the diagnostics, folded in a
+//                 fixed order by the blocks that finish last, which also set
+//                 the next step size min(dt_ad, dt_ac) (Eq. 9-11, h = h_min).
 //
 // Readings: e_ij points from i to j (Riemann states); grad W_ij is
 // grad_i W_ij = W'(r) (x_i - x_j)/r; V_j = m_j / rho_j; rho_bar is the mean
@@ -23,6 +23,8 @@
 // FP64 form (this file): absolute FP64 positions, the nearest periodic
 // image of each pair (fixed by the stencil step of its cell), plain sums;
 // 1/rho_i once per particle.  FP32 form: k_pair32.cu.
+#include <cmath>
+
 #include "common.cuh"
 #include "launch.h"
 #include "pair_physics.cuh"
@@ -187,9 +189,10 @@ template <int DIM>
 __global__ void __launch_bounds__(256, 2) k_forces_f64(int n, StateSet<double> S, const int32_t* __restrict__ start,
                                                     Grid G, Consts<double> K, const double4_32a* __restrict__ vr,
                                                     const uint32_t* __restrict__ nbl, const int32_t* __restrict__ nbc,
-                                                    int cap, const double* __restrict__ dt_ptr, int kick_on,
+                                                    int cap, const double* dt_ptr, int kick_on,
                                                     int write_ad, double* __restrict__ Rout,
-                                                    double* __restrict__ chi_out, double* __restrict__ partials,
+                                                    double* __restrict__ chi_out, GridSum B, DtConsts D,
+                                                    double* __restrict__ diag, double* dt_next, int count_step,
                                                     const double* __restrict__ vol)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -362,7 +365,8 @@ __global__ void __launch_bounds__(256, 2) k_forces_f64(int n, StateSet<double> S
         }
         chi_out[i] = 0.0;
     }
-    block_partials<true>(part, partials + (size_t)blockIdx.x * kNPart, true, K.body_force != 0);
+    __shared__ double total[kNPart];
+    if (grid_partials(part, B, total, true, K.body_force != 0)) finish_step(total, D, diag, dt_next, count_step);
 }
 
 // ================================================ diagnostics only
@@ -370,7 +374,8 @@ __global__ void __launch_bounds__(256, 2) k_forces_f64(int n, StateSet<double> S
 // FP64 partials of the diagnostics from the stored v and dr (no pair work):
 // used when the caller supplied a and dr, so no force pass is needed.
 template <typename Real, int DIM>
-__global__ void __launch_bounds__(256) k_diag_only(int n, StateSet<Real> S, double* __restrict__ partials)
+__global__ void __launch_bounds__(256) k_diag_only(int n, StateSet<Real> S, GridSum B, DtConsts D,
+                                                   double* __restrict__ diag, double* dt_next, int count_step)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     double part[kNPart];
@@ -393,76 +398,16 @@ __global__ void __launch_bounds__(256) k_diag_only(int n, StateSet<Real> S, doub
         part[7] = v2;
         part[8] = dr2;
     }
-    block_partials<true>(part, partials + (size_t)blockIdx.x * kNPart);
+    __shared__ double total[kNPart];
+    if (grid_partials(part, B, total)) finish_step(total, D, diag, dt_next, count_step);
 }
 
-// =========================================================== finalize
-
-// First level of the diagnostics reduction: block b folds rows
-// [b * chunk, (b + 1) * chunk) of the per-block partials into row b of out,
-// in a fixed order (the result does not depend on timing).
-__global__ void __launch_bounds__(256) k_reduce_rows(int nrows, int chunk, const double* __restrict__ in,
-                                                     double* __restrict__ out)
+// The rows of a large grid (see GridSum), and the end of the step.
+__global__ void __launch_bounds__(256) k_fold_step(GridSum B, int nrows, DtConsts D, double* __restrict__ diag,
+                                                   double* dt_ptr, int count_step)
 {
-    double acc[kNPart];
-#pragma unroll
-    for (int k = 0; k < kNPart; ++k) acc[k] = 0.0;
-    const int r0 = blockIdx.x * chunk, r1 = min(nrows, r0 + chunk);
-    for (int r = r0 + threadIdx.x; r < r1; r += blockDim.x) {
-        const double* p = in + (size_t)r * kNPart;
-#pragma unroll
-        for (int k = 0; k < kNPart; ++k) acc[k] = (k >= 6 && k <= 8) ? fmax(acc[k], p[k]) : acc[k] + p[k];
-    }
-    block_partials<false>(acc, out + (size_t)blockIdx.x * kNPart);
-}
-
-struct DtConsts {
-    double eta, rho0, h_min, u_ref, cfl_ad, cfl_ac, c, fixed_dt;
-};
-
-__global__ void __launch_bounds__(256) k_finalize(int nblocks, const double* __restrict__ partials, DtConsts D,
-                                                  double* __restrict__ diag, double* __restrict__ dt_ptr,
-                                                  int count_step)
-{
-    double acc[kNPart];
-#pragma unroll
-    for (int k = 0; k < kNPart; ++k) acc[k] = 0.0;
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
-        const double* p = partials + (size_t)b * kNPart;
-#pragma unroll
-        for (int k = 0; k < kNPart; ++k) acc[k] = (k >= 6 && k <= 8) ? fmax(acc[k], p[k]) : acc[k] + p[k];
-    }
-    __shared__ double out[kNPart];
-    block_partials<false>(acc, out);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const double vmax = out[6];
-        const double dt_used = *dt_ptr;
-        // Eq. 9-11 with h = h_min
-        const double nu = D.eta / D.rho0;
-        const double vad = fmax(vmax, fmax(nu / D.h_min, D.u_ref));
-        const double dt_ad = D.cfl_ad * D.h_min / vad;
-        const double dt_ac = D.cfl_ac * D.h_min / (vmax + D.c);
-        const double dt_next = D.fixed_dt > 0.0 ? D.fixed_dt : fmin(dt_ad, dt_ac);
-        diag[DG_MASS] = out[0];
-        diag[DG_MOM + 0] = out[1];
-        diag[DG_MOM + 1] = out[2];
-        diag[DG_MOM + 2] = out[3];
-        diag[DG_KE] = out[4];
-        diag[DG_NCHI] = out[5];
-        diag[DG_VMAX] = vmax;
-        diag[DG_VTMAX] = out[7];
-        diag[DG_DRMAX] = out[8];
-        diag[DG_DT] = count_step ? dt_used : 0.0;
-        diag[DG_DTNEXT] = dt_next;
-        diag[DG_STEPS] = count_step ? diag[DG_STEPS] + 1.0 : 0.0;
-        for (int d = 0; d < 3; ++d) diag[DG_FBODY + d] = -out[9 + d];    // force on the walls
-        // simulated time and the body's impulse since sph_build_cells (the time
-        // integral of the force over the steps, each step's force times its dt)
-        for (int d = 0; d < 3; ++d) diag[DG_IMPULSE + d] = count_step ? diag[DG_IMPULSE + d] - out[9 + d] * dt_used : 0.0;
-        diag[DG_TIME] = count_step ? diag[DG_TIME] + dt_used : 0.0;
-        *dt_ptr = dt_next;
-    }
+    __shared__ double total[kNPart];
+    if (fold_grid(B, nrows, total)) finish_step(total, D, diag, dt_ptr, count_step);
 }
 
 // ============================================================ launchers
@@ -484,6 +429,22 @@ int pair_threads(int prec, int n, int sms)
 
 int pair_blocks(int prec, int n, int sms) { return nblk(n, pair_threads(prec, n, sms)); }
 
+GridSum grid_sum(const FinishArgs& F, int nblocks)
+{
+    int group = nblocks;
+    if (nblocks > kInlineBlocks) group = 0;
+    else if (nblocks > kFoldRows) group = (int)std::ceil(std::sqrt((double)nblocks));
+    return GridSum{F.partials, F.rows, F.counters, group};
+}
+
+int grid_groups() { return kMaxGroups; }
+
+DtConsts dt_consts(const sph_params& P)
+{
+    const double nu = P.eta / P.rho0;
+    return DtConsts{std::fmax(nu / P.h_min, P.u_ref), P.cfl_ad * P.h_min, P.cfl_ac * P.h_min, P.c0, P.fixed_dt};
+}
+
 cudaError_t launch_density(int prec, int dim, int n, void* S, const int32_t* start, const Grid& G, const void* K,
                            void* vr, const float4* pos4, const int32_t* cell_of, uint32_t* nbl, int32_t* nbc,
                            cudaStream_t st, double* vol, const float4* pos4c, int tiles)
@@ -504,62 +465,52 @@ cudaError_t launch_density(int prec, int dim, int n, void* S, const int32_t* sta
 
 cudaError_t launch_forces(int prec, int dim, int n, void* S, const int32_t* start, const Grid& G, const void* K,
                           const float* mf, const void* vr, const float4* pos4, const int32_t* cell_of,
-                          const uint32_t* nbl, const int32_t* nbc, const double* dt, int kick_on, int write_ad,
-                          void* Rout, void* chi, double* partials, cudaStream_t st, const double* vol)
+                          const uint32_t* nbl, const int32_t* nbc, int kick_on, int write_ad,
+                          void* Rout, void* chi, const FinishArgs& F, cudaStream_t st, const double* vol)
 {
     const int T = pair_threads(prec, n, G.sms);
     if (prec == 32)
-        return launch_forces32(dim, n, S, start, G, K, mf, vr, pos4, cell_of, nbl, nbc, dt, kick_on, write_ad, Rout,
-                               chi, partials, st);
+        return launch_forces32(dim, n, S, start, G, K, mf, vr, pos4, cell_of, nbl, nbc, kick_on, write_ad, Rout, chi,
+                               F, st);
     auto s = *(StateSet<double>*)S;
     auto k = *(const Consts<double>*)K;
     const int cap = nbl_capacity(dim);
+    const GridSum B = grid_sum(F, nblk(n, T));
+    const DtConsts D = dt_consts(*F.P);
     if (dim == 2)
-        k_forces_f64<2><<<nblk(n, T), T, 0, st>>>(n, s, start, G, k, (const double4_32a*)vr, nbl, nbc, cap, dt,
-                                                  kick_on, write_ad, (double*)Rout, (double*)chi, partials, vol);
+        k_forces_f64<2><<<nblk(n, T), T, 0, st>>>(n, s, start, G, k, (const double4_32a*)vr, nbl, nbc, cap, F.dt,
+                                                  kick_on, write_ad, (double*)Rout, (double*)chi, B, D, F.diag, F.dt,
+                                                  F.count_step, vol);
     else
-        k_forces_f64<3><<<nblk(n, T), T, 0, st>>>(n, s, start, G, k, (const double4_32a*)vr, nbl, nbc, cap, dt,
-                                                  kick_on, write_ad, (double*)Rout, (double*)chi, partials, vol);
+        k_forces_f64<3><<<nblk(n, T), T, 0, st>>>(n, s, start, G, k, (const double4_32a*)vr, nbl, nbc, cap, F.dt,
+                                                  kick_on, write_ad, (double*)Rout, (double*)chi, B, D, F.diag, F.dt,
+                                                  F.count_step, vol);
     return cudaGetLastError();
 }
 
-cudaError_t launch_diag_only(int prec, int dim, int n, void* S, double* partials, int sms, cudaStream_t st)
+cudaError_t launch_finish_step(int prec, int n, int sms, const FinishArgs& F, cudaStream_t st, int64_t* launches)
+{
+    const int nb = pair_blocks(prec, n, sms);
+    const GridSum B = grid_sum(F, nb);
+    if (B.group) return cudaSuccess;      // the pass folded its partials itself
+    k_fold_step<<<kFoldBlocks, 256, 0, st>>>(B, nb, dt_consts(*F.P), F.diag, F.dt, F.count_step);
+    ++*launches;
+    return cudaGetLastError();
+}
+
+cudaError_t launch_diag_only(int prec, int dim, int n, void* S, const FinishArgs& F, int sms, cudaStream_t st)
 {
     const int T = pair_threads(prec, n, sms);   // one partials row per block of the force pass
+    const GridSum B = grid_sum(F, nblk(n, T));
+    const DtConsts D = dt_consts(*F.P);
     if (prec == 64) {
         auto s = *(StateSet<double>*)S;
-        if (dim == 2) k_diag_only<double, 2><<<nblk(n, T), T, 0, st>>>(n, s, partials);
-        else k_diag_only<double, 3><<<nblk(n, T), T, 0, st>>>(n, s, partials);
+        if (dim == 2) k_diag_only<double, 2><<<nblk(n, T), T, 0, st>>>(n, s, B, D, F.diag, F.dt, F.count_step);
+        else k_diag_only<double, 3><<<nblk(n, T), T, 0, st>>>(n, s, B, D, F.diag, F.dt, F.count_step);
     } else {
         auto s = *(StateSet<float>*)S;
-        if (dim == 2) k_diag_only<float, 2><<<nblk(n, T), T, 0, st>>>(n, s, partials);
-        else k_diag_only<float, 3><<<nblk(n, T), T, 0, st>>>(n, s, partials);
-    }
-    return cudaGetLastError();
-}
-
-int reduce_rows_blocks() { return 256; }
-
-int launch_reduce_rows(int nblocks, const double* partials, double* rows, cudaStream_t st)
-{
-    const int G = reduce_rows_blocks();
-    if (nblocks <= 4 * G) return 0;
-    const int chunk = (nblocks + G - 1) / G;
-    k_reduce_rows<<<G, 256, 0, st>>>(nblocks, chunk, partials, rows);
-    return G;
-}
-
-cudaError_t launch_finalize(int nblocks, const double* partials, double* rows, const sph_params& P, double* diag,
-                            double* dt, int count_step, cudaStream_t st)
-{
-    DtConsts D{P.eta, P.rho0, P.h_min, P.u_ref, P.cfl_ad, P.cfl_ac, P.c0, P.fixed_dt};
-    const int G = reduce_rows_blocks();
-    if (nblocks > 4 * G) {
-        const int chunk = (nblocks + G - 1) / G;
-        k_reduce_rows<<<G, 256, 0, st>>>(nblocks, chunk, partials, rows);
-        k_finalize<<<1, 256, 0, st>>>(G, rows, D, diag, dt, count_step);
-    } else {
-        k_finalize<<<1, 256, 0, st>>>(nblocks, partials, D, diag, dt, count_step);
+        if (dim == 2) k_diag_only<float, 2><<<nblk(n, T), T, 0, st>>>(n, s, B, D, F.diag, F.dt, F.count_step);
+        else k_diag_only<float, 3><<<nblk(n, T), T, 0, st>>>(n, s, B, D, F.diag, F.dt, F.count_step);
     }
     return cudaGetLastError();
 }

@@ -1142,9 +1142,10 @@ __global__ void __launch_bounds__(kTPB32, UNIFORM ? 6 : 8) k_forces32(int n, con
                                                      StateSet<float> S, const float* __restrict__ mf,
                                                      const float4* __restrict__ vr, const uint32_t* __restrict__ nbl,
                                                      const int32_t* __restrict__ nbc, int cap,
-                                                     const double* __restrict__ dt_ptr, int kick_on, int write_ad,
+                                                     const double* dt_ptr, int kick_on, int write_ad,
                                                      float* __restrict__ Rout, float* __restrict__ chi_out,
-                                                     double* __restrict__ partials)
+                                                     GridSum B, DtConsts D, double* __restrict__ diag,
+                                                     double* dt_next, int count_step)
 {
     __shared__ float4 tab[kCodes];
     for (int t = threadIdx.x; t < kCodes; t += blockDim.x) {
@@ -1346,7 +1347,8 @@ __global__ void __launch_bounds__(kTPB32, UNIFORM ? 6 : 8) k_forces32(int n, con
         }
         chi_out[i] = 0.f;
     }
-    block_partials<true>(part, partials + (size_t)blockIdx.x * kNPart, true, K.body_force != 0);
+    __shared__ double total[kNPart];
+    if (grid_partials(part, B, total, true, K.body_force != 0)) finish_step(total, D, diag, dt_next, count_step);
 }
 
 // --------------------------------------------------------------- launchers
@@ -1406,12 +1408,14 @@ static cudaError_t density_tile_t(int mode, int n, const float4* pos4c, const in
 template <int DIM, typename Acc, bool U>
 static void forces_t(int n, const float4* pos4, const int32_t* cell_of, const int32_t* start, const Grid& G,
                      const Consts<float>& K, StateSet<float> S, const float* mf, const float4* vr,
-                     const uint32_t* nbl, const int32_t* nbc, const double* dt, int kick_on, int write_ad,
-                     float* Rout, float* chi, double* partials, cudaStream_t st)
+                     const uint32_t* nbl, const int32_t* nbc, int kick_on, int write_ad, float* Rout, float* chi,
+                     const FinishArgs& F, cudaStream_t st)
 {
     const int T = pair_threads(32, n, G.sms);
     k_forces32<DIM, Acc, U><<<nblk(n, T), T, 0, st>>>(n, pos4, cell_of, start, G, K, S, mf, vr, nbl, nbc,
-                                                      nbl_capacity(DIM), dt, kick_on, write_ad, Rout, chi, partials);
+                                                      nbl_capacity(DIM), F.dt, kick_on, write_ad, Rout, chi,
+                                                      grid_sum(F, nblk(n, T)), dt_consts(*F.P), F.diag, F.dt,
+                                                      F.count_step);
 }
 
 #define SPH_DISPATCH32(FN, ...)                                                   \
@@ -1455,13 +1459,13 @@ cudaError_t launch_density32(int dim, int n, void* Sv, const int32_t* start, con
 
 cudaError_t launch_forces32(int dim, int n, void* Sv, const int32_t* start, const Grid& G, const void* Kv,
                             const float* mf, const void* vr, const float4* pos4, const int32_t* cell_of,
-                            const uint32_t* nbl, const int32_t* nbc, const double* dt, int kick_on, int write_ad,
-                            void* Rout, void* chi, double* partials, cudaStream_t st)
+                            const uint32_t* nbl, const int32_t* nbc, int kick_on, int write_ad, void* Rout,
+                            void* chi, const FinishArgs& F, cudaStream_t st)
 {
     const StateSet<float> S = *(StateSet<float>*)Sv;
     const Consts<float>& K = *(const Consts<float>*)Kv;
-    SPH_DISPATCH32(forces_t, n, pos4, cell_of, start, G, K, S, mf, (const float4*)vr, nbl, nbc, dt, kick_on,
-                   write_ad, (float*)Rout, (float*)chi, partials, st);
+    SPH_DISPATCH32(forces_t, n, pos4, cell_of, start, G, K, S, mf, (const float4*)vr, nbl, nbc, kick_on,
+                   write_ad, (float*)Rout, (float*)chi, F, st);
     return cudaGetLastError();
 }
 

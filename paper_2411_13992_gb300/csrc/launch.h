@@ -58,6 +58,28 @@ cudaError_t launch_permute(int prec, int dim, int n, const int32_t* perm, void* 
                            const Grid& G, float4* pos4, int32_t* cell, float* mf, int uniform_h, int carry_ad,
                            cudaStream_t st, const uint32_t* varies, float4* pos4c = nullptr);
 
+// What the last block of a pass needs to fold the grid's partials and set the
+// next step size: the partials' buffers, the counters (zero between
+// launches), the diagnostics and the step size, and whether the pass ends a
+// step.
+struct FinishArgs {
+    double* partials;
+    double* rows;          // [grid_groups()][kNPart]
+    unsigned* counters;    // [1 + grid_groups()]
+    const sph_params* P;
+    double* diag;
+    double* dt;
+    int count_step;
+};
+struct GridSum;
+struct DtConsts;
+GridSum grid_sum(const FinishArgs& F, int nblocks);
+// After a pass that writes partials (forces, diag_only): the fold of a large
+// grid's rows and the end of the step; nothing for a grid that did both.
+cudaError_t launch_finish_step(int prec, int n, int sms, const FinishArgs& F, cudaStream_t st, int64_t* launches);
+int grid_groups();
+DtConsts dt_consts(const sph_params& P);
+
 // k_pair.cu (FP64 form; FP32 calls are forwarded to k_pair32.cu)
 int pair_threads(int prec, int n, int sms);
 int pair_blocks(int prec, int n, int sms);
@@ -68,8 +90,8 @@ cudaError_t launch_density(int prec, int dim, int n, void* S, const int32_t* sta
                            cudaStream_t st, double* vol = nullptr, const float4* pos4c = nullptr, int tiles = 0);
 cudaError_t launch_forces(int prec, int dim, int n, void* S, const int32_t* start, const Grid& G, const void* K,
                           const float* mf, const void* vr, const float4* pos4, const int32_t* cell_of,
-                          const uint32_t* nbl, const int32_t* nbc, const double* dt, int kick_on, int write_ad,
-                          void* Rout, void* chi, double* partials, cudaStream_t st, const double* vol = nullptr);
+                          const uint32_t* nbl, const int32_t* nbc, int kick_on, int write_ad,
+                          void* Rout, void* chi, const FinishArgs& F, cudaStream_t st, const double* vol = nullptr);
 
 // k_pair32.cu
 int nbl_capacity(int dim);
@@ -80,15 +102,9 @@ cudaError_t launch_density32(int dim, int n, void* S, const int32_t* start, cons
                              cudaStream_t st, const float4* pos4c, int tiles = 0);
 cudaError_t launch_forces32(int dim, int n, void* S, const int32_t* start, const Grid& G, const void* K,
                             const float* mf, const void* vr, const float4* pos4, const int32_t* cell_of,
-                            const uint32_t* nbl, const int32_t* nbc, const double* dt, int kick_on, int write_ad,
-                            void* Rout, void* chi, double* partials, cudaStream_t st);
-cudaError_t launch_diag_only(int prec, int dim, int n, void* S, double* partials, int sms, cudaStream_t st);
-int reduce_rows_blocks();
-// First level of the fixed-order reduction of per-block partials: returns the
-// number of rows written (0: too few partials, reduce them directly).
-int launch_reduce_rows(int nblocks, const double* partials, double* rows, cudaStream_t st);
-cudaError_t launch_finalize(int nblocks, const double* partials, double* rows, const sph_params& P, double* diag,
-                            double* dt, int count_step, cudaStream_t st);
+                            const uint32_t* nbl, const int32_t* nbc, int kick_on, int write_ad, void* Rout,
+                            void* chi, const FinishArgs& F, cudaStream_t st);
+cudaError_t launch_diag_only(int prec, int dim, int n, void* S, const FinishArgs& F, int sms, cudaStream_t st);
 
 // k_io.cu
 cudaError_t launch_vec_in(int prec, int dim, int n, const double* src3, void* dst, cudaStream_t st);
@@ -118,7 +134,7 @@ cudaError_t launch_scalar_in(int prec, int n, const double* src, const int8_t* k
 // k_dual.cu (dual-criteria time stepping).  Device pointers of one context;
 // S points at the StateSet<Real> of the current (sorted) copy.
 struct DualArgs {
-    int n, cap;
+    int n, cap, sms;
     const void* S;
     void* vr;
     float4* pos4;
@@ -130,16 +146,13 @@ struct DualArgs {
     void* R;
     void* chi;
     double* du;
-    double* partials;
-    double* rows;
+    FinishArgs F;
     uint32_t* err;
 };
-int dual_pair_blocks(int prec, int n, int sms);
 cudaError_t launch_dual_begin(const sph_params& P, const double* diag, double* du, cudaStream_t st);
 cudaError_t launch_dual_advect(int prec, int dim, const DualArgs& a, const Grid& G, const void* K, cudaStream_t st);
 cudaError_t launch_dual_substep(int prec, int dim, const DualArgs& a, const Grid& G, const void* K,
-                                const sph_params& P, double* diag, double* dt_ptr, cudaStream_t st,
-                                int64_t* launches);
+                                cudaStream_t st, int64_t* launches);
 cudaError_t launch_dual_complete(int prec, const DualArgs& a, cudaStream_t st);
 
 // k_adjoint.cu

@@ -87,6 +87,7 @@ struct sph_ctx {
     void* chi;
     double* partials;
     double* rows;        // first-level reduction of the partials
+    unsigned* counters;  // blocks and groups of blocks that have finished (zero between launches)
     double* diag;
     double* dt;
     uint32_t* err;          // [0] the sticky device error word; [1] nonzero when the particles' h, m,
@@ -336,7 +337,8 @@ size_t carve(sph_ctx* c, char* base)
     c->chi = c->density_only ? nullptr : W.take<char>(n * rs);
     // one partials row per block of a pair pass; blocks are never smaller than a warp
     c->partials = W.take<double>(((size_t)n + 31) / 32 * kNPart);
-    c->rows = W.take<double>((size_t)reduce_rows_blocks() * kNPart);
+    c->rows = W.take<double>((size_t)grid_groups() * kNPart);
+    c->counters = W.take<unsigned>((size_t)grid_groups() + 1);
     c->diag = W.take<double>(DG_COUNT);
     c->dt = W.take<double>(1);
     c->err = W.take<uint32_t>(4);
@@ -442,6 +444,11 @@ sph_status run_sort(sph_ctx* c, int drift, int carry_ad)
     return SPH_OK;
 }
 
+FinishArgs finish_args(sph_ctx* c, int count_step)
+{
+    return FinishArgs{c->partials, c->rows, c->counters, &c->P, c->diag, c->dt, count_step};
+}
+
 // Density, fused forces (+ closing kick), reductions and dt.  With
 // pairs == 0 (a and dr supplied by the caller) only the density and the
 // diagnostics run.
@@ -451,10 +458,9 @@ sph_status run_forces(sph_ctx* c, int kick_on, int pairs, int count_step)
     if (!pairs) {
         SPH_CU(launch_density(c->prec, c->dim, n, cur_set(c), c->start, c->G, consts(c), c->vr, c->pos4, c->cell,
                               c->nbl, c->nbc, c->st, c->vol, c->pos4c, c->P.pair_tiles));
-        SPH_CU(launch_diag_only(c->prec, c->dim, n, cur_set(c), c->partials, c->G.sms, c->st));
-        SPH_CU(launch_finalize(pair_blocks(c->prec, n, c->G.sms), c->partials, c->rows, c->P, c->diag, c->dt,
-                               count_step, c->st));
-        c->launches += 3;
+        SPH_CU(launch_diag_only(c->prec, c->dim, n, cur_set(c), finish_args(c, count_step), c->G.sms, c->st));
+        c->launches += 2;
+        SPH_CU(launch_finish_step(c->prec, n, c->G.sms, finish_args(c, count_step), c->st, &c->launches));
         return SPH_OK;
     }
     const int write_ad = 1;
@@ -464,14 +470,13 @@ sph_status run_forces(sph_ctx* c, int kick_on, int pairs, int count_step)
     SPH_MARK(SPH_K_DENSITY, 1);
     SPH_MARK(SPH_K_FORCES, 0);
     SPH_CU(launch_forces(c->prec, c->dim, n, cur_set(c), c->start, c->G, consts(c), c->mf, c->vr, c->pos4, c->cell,
-                         c->nbl, c->nbc, c->dt, kick_on, write_ad, c->R, c->chi, c->partials, c->st,
+                         c->nbl, c->nbc, kick_on, write_ad, c->R, c->chi, finish_args(c, count_step), c->st,
                          c->vol));
     SPH_MARK(SPH_K_FORCES, 1);
+    c->launches += 2;
     SPH_MARK(SPH_K_FINALIZE, 0);
-    SPH_CU(launch_finalize(pair_blocks(c->prec, n, c->G.sms), c->partials, c->rows, c->P, c->diag, c->dt,
-                           count_step, c->st));
+    SPH_CU(launch_finish_step(c->prec, n, c->G.sms, finish_args(c, count_step), c->st, &c->launches));
     SPH_MARK(SPH_K_FINALIZE, 1);
-    c->launches += 3;
     return SPH_OK;
 }
 
@@ -479,6 +484,7 @@ DualArgs dual_args(sph_ctx* c)
 {
     DualArgs a;
     a.n = (int)c->n;
+    a.sms = c->G.sms;
     a.cap = nbl_capacity(c->dim);
     a.S = cur_set(c);
     a.vr = c->vr;
@@ -491,8 +497,7 @@ DualArgs dual_args(sph_ctx* c)
     a.R = c->R;
     a.chi = c->chi;
     a.du = c->du;
-    a.partials = c->partials;
-    a.rows = c->rows;
+    a.F = finish_args(c, 1);
     a.err = c->err;
     return a;
 }
@@ -529,8 +534,7 @@ sph_status run_dual_step(sph_ctx* c)
     constexpr int kMaxSubsteps = 1 << 20;
     for (;;) {
         for (int b = 0; b < batch; ++b)
-            SPH_CU(launch_dual_substep(c->prec, c->dim, a, c->G, consts(c), c->P, c->diag, c->dt, c->st,
-                                       &c->launches));
+            SPH_CU(launch_dual_substep(c->prec, c->dim, a, c->G, consts(c), c->st, &c->launches));
         taken += batch;
         SPH_CU(cudaMemcpyAsync(hb, c->du, sizeof(hb), cudaMemcpyDeviceToHost, c->st));
         SPH_CU(cudaStreamSynchronize(c->st));
@@ -914,6 +918,7 @@ sph_status sph_create(const sph_params* p, int64_t n, void* workspace, size_t by
     carve(c, (char*)workspace);
     if (cudaMemsetAsync(c->err, 0, 4 * sizeof(uint32_t), c->st) != cudaSuccess ||
         cudaMemsetAsync(c->err + 1, 1, 1, c->st) != cudaSuccess ||
+        cudaMemsetAsync(c->counters, 0, ((size_t)grid_groups() + 1) * sizeof(unsigned), c->st) != cudaSuccess ||
         cudaMemsetAsync(c->diag, 0, DG_COUNT * sizeof(double), c->st) != cudaSuccess) {
         delete c;
         return SPH_ERR_CUDA;
@@ -1004,10 +1009,9 @@ sph_status sph_build_cells(sph_ctx* c)
         // sort and the density pass are left to the first step, which does
         // both itself
         const int n = (int)c->n;
-        SPH_CU(launch_diag_only(c->prec, c->dim, n, cur_set(c), c->partials, c->G.sms, c->st));
-        SPH_CU(launch_finalize(pair_blocks(c->prec, n, c->G.sms), c->partials, c->rows, c->P, c->diag, c->dt, 0,
-                               c->st));
-        c->launches += 2;
+        SPH_CU(launch_diag_only(c->prec, c->dim, n, cur_set(c), finish_args(c, 0), c->G.sms, c->st));
+        ++c->launches;
+        SPH_CU(launch_finish_step(c->prec, n, c->G.sms, finish_args(c, 0), c->st, &c->launches));
         c->cells_pending = 1;
         c->have_cells = 1;
         return SPH_OK;
