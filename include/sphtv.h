@@ -317,10 +317,10 @@ SPH_API int64_t sph_launch_count(const sph_ctx* ctx);
 
 /* Kernel classes of one step, for per-kernel timing. */
 enum {
-    SPH_K_KICKDRIFT = 0,   /* kick + drift + cell key + histogram */
+    SPH_K_KICKDRIFT = 0,   /* kick + drift + cell key + histogram and lists of the sort bins */
     SPH_K_SCAN = 1,        /* exclusive scan of the cell counts */
-    SPH_K_ORDER = 2,       /* scatter into cells + per-cell order by id */
-    SPH_K_PERMUTE = 3,     /* permute the particle arrays */
+    SPH_K_ORDER = 2,       /* not timed: the order by id is part of SPH_K_PERMUTE */
+    SPH_K_PERMUTE = 3,     /* order by id within the bins, permute the particle arrays */
     SPH_K_DENSITY = 4,     /* density summation (Eq. 8) */
     SPH_K_FORCES = 5,      /* fused pair pass (Eq. 3, 5-7, 14-16) + closing kick */
     SPH_K_FINALIZE = 6,    /* FP64 reductions and dt (Eq. 9-11) */

@@ -1,10 +1,10 @@
 // k_cells.cu -- the kick-drift stage and the cell-linked list of libsphtv.
 //
-// Per step:  kick + drift + cell key + histogram  ->  exclusive scan of the
-// cell counts  ->  atomic scatter into cell ranges  ->  per-cell ordering by
-// particle id (so the sorted order never depends on atomic timing)  ->
-// permute the particle arrays into the new order (and, in both forms,
-// emit FP32 positions relative to each particle's cell origin).
+// Per step, three kernels:  kick + drift + bin key, with each bin's particles
+// counted and linked into a list  ->  exclusive scan of the bin counts  ->
+// each particle ranks itself by id among its bin's list (so the sorted order
+// never depends on atomic timing) and moves its arrays to the new order (and,
+// in both forms, emits its FP32 position relative to its cell's origin).
 //
 // The kick-drift follows the kick-drift-kick scheme the paper names (Sec. 1,
 // Sec. 3): v += dt/2 a; x += dt v + dr, where dr is the transport-velocity
@@ -75,7 +75,8 @@ __device__ __forceinline__ int wrap_side(const Grid& G, double x, int d)
 
 template <typename Real, int DIM>
 __global__ void k_kick_drift_key(int n, StateSet<Real> S, const double* __restrict__ dt_ptr, int drift, Grid G,
-                                 int32_t* __restrict__ key, int32_t* __restrict__ count, uint32_t* err)
+                                 int32_t* __restrict__ key, int32_t* __restrict__ count,
+                                 int32_t* __restrict__ head, int32_t* __restrict__ next, uint32_t* err)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
@@ -141,173 +142,146 @@ __global__ void k_kick_drift_key(int n, StateSet<Real> S, const double* __restri
     if (e) atomicOr(err, e);
     int k = sort_key<DIM>(G, xs);
     key[i] = k;
-    // one atomic per particle: with the sub-cell bins a warp's lanes seldom
-    // share a bin, and aggregating them by __match_any_sync cost more than
-    // it saved (3 % of this kernel at 128^3)
+    // count the bin, and put the particle at the front of the bin's list (two
+    // atomics per particle: with the sub-cell bins a warp's lanes seldom share
+    // one, and aggregating them by __match_any_sync cost more than it saved).
+    // A list is followed for as many members as its bin counts, so its end and
+    // an empty bin's head need no mark and no clearing.
     atomicAdd(&count[k], 1);
+    next[i] = atomicExch(&head[k], i);
 }
 
 // ------------------------------------------------------- exclusive scan
 
 constexpr int kScanThreads = 512;
-constexpr int kScanItems = 8;
+constexpr int kScanItems = 16;
 constexpr int kScanTile = kScanThreads * kScanItems;
 
-// Exclusive scan of in[0, n) into out (in place allowed); each block scans
-// one tile and writes its total to bsum[blockIdx.x].
-__global__ void __launch_bounds__(kScanThreads) k_scan_tile(const int32_t* in, int32_t* out, int32_t* bsum, int n)
+size_t scan_temp_elems(int n) { return (size_t)(n + kScanTile - 1) / kScanTile; }
+
+// In-place exclusive scan over the block of one value per thread: returns the
+// sum of the threads before, *total the block's sum.
+__device__ __forceinline__ int32_t block_scan(int32_t s, int32_t* warp_tot, int32_t* total)
 {
-    __shared__ int32_t warp_tot[kScanThreads / 32];
+    constexpr int nw = kScanThreads / 32;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int base = blockIdx.x * kScanTile + threadIdx.x * kScanItems;
-    int32_t vals[kScanItems];
-    int32_t s = 0;
-#pragma unroll
-    for (int k = 0; k < kScanItems; ++k) {
-        int idx = base + k;
-        vals[k] = idx < n ? in[idx] : 0;
-        s += vals[k];
-    }
     int32_t incl = s;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
-        int32_t t = __shfl_up_sync(0xffffffffu, incl, off);
+        const int32_t t = __shfl_up_sync(0xffffffffu, incl, off);
         if (lane >= off) incl += t;
     }
     if (lane == 31) warp_tot[w] = incl;
     __syncthreads();
     if (w == 0) {
-        constexpr int nw = kScanThreads / 32;
-        int32_t t = lane < nw ? warp_tot[lane] : 0;
+        const int32_t t = lane < nw ? warp_tot[lane] : 0;
         int32_t ti = t;
 #pragma unroll
         for (int off = 1; off < 32; off <<= 1) {
-            int32_t u = __shfl_up_sync(0xffffffffu, ti, off);
+            const int32_t u = __shfl_up_sync(0xffffffffu, ti, off);
             if (lane >= off) ti += u;
         }
         if (lane < nw) warp_tot[lane] = ti - t;
-        if (lane == nw - 1) bsum[blockIdx.x] = ti;
+        if (lane == nw - 1) warp_tot[nw] = ti;
     }
     __syncthreads();
-    int32_t pre = warp_tot[w] + incl - s;
+    *total = warp_tot[nw];
+    return warp_tot[w] + incl - s;
+}
+
+// The sort's scan: prefix[k] = the sum of count[0, k) within k's tile of
+// kScanTile bins, tile_off[b] the sum of the tiles before tile b, so that the
+// start of bin k is prefix[k] + tile_off[k / kScanTile] (the readers add the
+// two: no pass over the bins for it).  Clears the counts as it reads them.
+// The block that finishes last scans the tiles' sums (one kernel where there
+// were two or three).  Where each reading warp scanned up to 32 sums itself
+// instead, the step of a small problem took as long and the permute 3 us more
+// at 128^3.
+__global__ void __launch_bounds__(kScanThreads) k_bin_scan(int32_t* __restrict__ count, int32_t* __restrict__ prefix,
+                                                           int32_t* tile_off, unsigned* done, int n)
+{
+    __shared__ int32_t warp_tot[kScanThreads / 32 + 1];
+    __shared__ int is_last;
+    const int base = blockIdx.x * kScanTile + threadIdx.x * kScanItems;
+    static_assert(kScanItems % 4 == 0, "16-byte vectors");
+    int32_t vals[kScanItems];
+    const bool whole = base + kScanItems <= n;      // base is a multiple of 16: 64-byte aligned
+    if (whole) {
+        int4* c4 = reinterpret_cast<int4*>(count + base);
+#pragma unroll
+        for (int k = 0; k < kScanItems / 4; ++k) *reinterpret_cast<int4*>(vals + 4 * k) = c4[k];
+#pragma unroll
+        for (int k = 0; k < kScanItems / 4; ++k) c4[k] = make_int4(0, 0, 0, 0);
+    } else {
+#pragma unroll
+        for (int k = 0; k < kScanItems; ++k) {
+            vals[k] = base + k < n ? count[base + k] : 0;
+            if (base + k < n) count[base + k] = 0;
+        }
+    }
+    int32_t s = 0;
 #pragma unroll
     for (int k = 0; k < kScanItems; ++k) {
-        int idx = base + k;
-        if (idx < n) out[idx] = pre;
-        pre += vals[k];
+        const int32_t v = vals[k];
+        vals[k] = s;
+        s += v;
     }
-}
-
-__global__ void k_scan_add(int32_t* out, const int32_t* boff, int n)
-{
-    int idx = blockIdx.x * kScanTile + threadIdx.x;
-    int32_t add = boff[blockIdx.x];
+    int32_t total;
+    const int32_t pre = block_scan(s, warp_tot, &total);
 #pragma unroll
-    for (int k = 0; k < kScanItems; ++k, idx += kScanThreads)
-        if (idx < n) out[idx] += add;
+    for (int k = 0; k < kScanItems; ++k) vals[k] += pre;
+    if (whole) {
+        int4* p4 = reinterpret_cast<int4*>(prefix + base);
+#pragma unroll
+        for (int k = 0; k < kScanItems / 4; ++k) p4[k] = *reinterpret_cast<int4*>(vals + 4 * k);
+    } else {
+#pragma unroll
+        for (int k = 0; k < kScanItems; ++k)
+            if (base + k < n) prefix[base + k] = vals[k];
+    }
+    const int nt = gridDim.x;
+    if (threadIdx.x == 0) {
+        tile_off[blockIdx.x] = total;
+        __threadfence();
+        is_last = atomicAdd(done, 1u) == (unsigned)nt - 1u;
+        if (is_last) *done = 0u;
+    }
+    __syncthreads();
+    if (!is_last) return;
+    __threadfence();
+    int32_t carry = 0;
+    for (int t0 = 0; t0 < nt; t0 += kScanThreads) {
+        const int t = t0 + threadIdx.x;
+        const int32_t v = t < nt ? __ldcg(tile_off + t) : 0;
+        const int32_t p = carry + block_scan(v, warp_tot, &total);
+        if (t < nt) tile_off[t] = p;
+        carry += total;
+        __syncthreads();                        // warp_tot is used again
+    }
 }
 
-size_t scan_temp_elems(int n)
+cudaError_t launch_bin_scan(int32_t* count, int32_t* prefix, int n, int32_t* tile_off, unsigned* done,
+                            cudaStream_t st)
 {
-    size_t tot = 0;
-    while (n > 1) {
-        n = (n + kScanTile - 1) / kScanTile;
-        tot += (size_t)n + 1;
-    }
-    return tot + 1;
-}
-
-cudaError_t launch_exclusive_scan(const int32_t* in, int32_t* out, int n, int32_t* tmp, cudaStream_t st,
-                                  int64_t* launches)
-{
-    int nb = (n + kScanTile - 1) / kScanTile;
-    k_scan_tile<<<nb, kScanThreads, 0, st>>>(in, out, tmp, n);
-    ++*launches;
-    if (nb > 1) {
-        cudaError_t e = launch_exclusive_scan(tmp, tmp, nb, tmp + nb + 1, st, launches);
-        if (e != cudaSuccess) return e;
-        k_scan_add<<<nb, kScanThreads, 0, st>>>(out, tmp, n);
-        ++*launches;
-    }
+    k_bin_scan<<<(n + kScanTile - 1) / kScanTile, kScanThreads, 0, st>>>(count, prefix, tile_off, done, n);
     return cudaGetLastError();
 }
 
-// The sort's scan without its last pass: prefix[k] = the exclusive sum of
-// count[0, k) within k's tile of kScanTile bins, tile_off[b] (tmp) the sum of
-// the tiles before tile b.  The start of bin k is prefix[k] +
-// tile_off[k / kScanTile]; the scatter and the per-bin ordering add the tile
-// offset as they read a start (one pass over the bins fewer).  Returns
-// tile_off, or null for a single tile.
-cudaError_t launch_scan_tiles(const int32_t* count, int32_t* prefix, int n, int32_t* tmp, cudaStream_t st,
-                              int64_t* launches, const int32_t** tile_off)
-{
-    int nb = (n + kScanTile - 1) / kScanTile;
-    k_scan_tile<<<nb, kScanThreads, 0, st>>>(count, prefix, tmp, n);
-    ++*launches;
-    *tile_off = nullptr;
-    if (nb > 1) {
-        cudaError_t e = launch_exclusive_scan(tmp, tmp, nb, tmp + nb + 1, st, launches);
-        if (e != cudaSuccess) return e;
-        *tile_off = tmp;
-    }
-    return cudaGetLastError();
-}
+// ------------------------------------------------------ order and permute
 
-__device__ __forceinline__ int bin_start_of(const int32_t* __restrict__ prefix, const int32_t* __restrict__ tile_off,
-                                            int k)
-{
-    return prefix[k] + (tile_off ? tile_off[k / kScanTile] : 0);
-}
-
-// ------------------------------------------------ scatter and cell order
-
-// Slots by atomics on the bins' counts, counting down: a bin of c particles
-// hands out c - 1 .. 0, so every count is back at zero after the scatter
-// (the next sort needs no clearing).  The order inside a bin is fixed
-// afterwards by k_order_cells.  One atomic per particle: the sub-cell bins
-// are seldom shared within a warp, and aggregating the lanes by
-// __match_any_sync cost more than it saved.
-__global__ void k_scatter(int n, const int32_t* __restrict__ key, const int32_t* __restrict__ prefix,
-                          const int32_t* __restrict__ tile_off, int32_t* __restrict__ count,
-                          int32_t* __restrict__ perm)
-{
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int k = key[i];
-    const int pos = bin_start_of(prefix, tile_off, k) + atomicSub(&count[k], 1) - 1;
-    perm[pos] = i;
-}
-
-// One thread per sort bin (cell, or sub-cell when the sort refines the
-// cells): write the bin's start, and place the bin's particles in
-// increasing caller id (ids are unique, so the rank of each is its slot).
-// Cells hold about two particles (edge >= h_max), so the quadratic rank
-// count is short.  With sub-cells (shift > 0) the thread of each cell's
-// first sub-cell also writes the cell's start (the thread nbin, past the
-// last bin, the end n).
-__global__ void k_order_cells(int nbin, const int32_t* __restrict__ prefix, const int32_t* __restrict__ tile_off,
-                              const int32_t* __restrict__ perm_in, const int32_t* __restrict__ id,
-                              int32_t* __restrict__ perm_out, int32_t* __restrict__ start, int shift,
-                              int32_t* __restrict__ cell_start)
-{
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c > nbin) return;
-    const int s = bin_start_of(prefix, tile_off, c);
-    start[c] = s;
-    if (shift && (c & ((1 << shift) - 1)) == 0) cell_start[c >> shift] = s;
-    if (c == nbin) return;
-    const int e = bin_start_of(prefix, tile_off, c + 1);
-    for (int k = s; k < e; ++k) {
-        const int p = perm_in[k];
-        const int myid = id[p];
-        int rank = 0;
-        for (int t = s; t < e; ++t) rank += id[perm_in[t]] < myid;
-        perm_out[s + rank] = p;
-    }
-}
-
-// --------------------------------------------------------------- permute
-
+// One thread per particle, in the old order: its slot in the new order is its
+// bin's start plus the number of its bin's particles with a smaller id (ids
+// are unique), found by following the bin's list; bins hold less than one
+// particle on average.  The particle's arrays are read in the old order, in
+// which neighbouring threads read neighbouring words, and written to the
+// slots, which are nearly in the same order after one step's motion.  One
+// kernel where there were three (scatter by atomics, order of each bin,
+// permute by gathering), without their passes over two permutations.
+//
+// The threads also write the bins' starts (thread nbin the end, n); with
+// sub-cells (G.sub_shift > 0) the thread of a cell's first sub-cell also
+// writes the cell's start.
+//
 // pos4 = {offset from the cell origin, h} (uniform resolution:
 // {offset, m}, since h is then a constant), mf = m in FP32, cell_out = key;
 // pos4c (when given: the FP32 form at uniform resolution) = {offset, bits of
@@ -315,23 +289,48 @@ __global__ void k_order_cells(int nbin, const int32_t* __restrict__ prefix, cons
 // cell_out.  When *varies is 0 every particle has particle 0's h, m and
 // sigma0 and is a fluid particle, and both state sets hold these arrays
 // (set by sph_set_state): they are left where they are.
-template <typename Real, int DIM, bool CARRY_AD, bool F32POS>
-__global__ void k_permute(int n, const int32_t* __restrict__ perm, StateSet<Real> src, StateSet<Real> dst,
-                          const int32_t* __restrict__ key, Grid G, float4* __restrict__ pos4,
-                          int32_t* __restrict__ cell_out, float* __restrict__ mf, int uniform_h,
-                          float4* __restrict__ pos4c, const uint32_t* __restrict__ varies)
+template <typename Real, int DIM, bool CARRY_AD>
+__global__ void __launch_bounds__(256) k_order_permute(int n, int nbin, const int32_t* __restrict__ key,
+                                const int32_t* __restrict__ prefix, const int32_t* __restrict__ tile_off,
+                                const int32_t* __restrict__ head, const int32_t* __restrict__ next,
+                                int32_t* __restrict__ bin_start, int32_t* __restrict__ cell_start,
+                                StateSet<Real> src, StateSet<Real> dst, Grid G, float4* __restrict__ pos4,
+                                int32_t* __restrict__ cell_out, float* __restrict__ mf, int uniform_h,
+                                float4* __restrict__ pos4c, const uint32_t* __restrict__ varies)
 {
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    auto start_of = [&](int k) { return prefix[k] + tile_off[k / kScanTile]; };
+    if (i <= nbin) {
+        const int s = start_of(i);
+        bin_start[i] = s;
+        if (G.sub_shift && (i & ((1 << G.sub_shift) - 1)) == 0) cell_start[i >> G.sub_shift] = s;
+    }
+    if (i >= n) return;
+    const int bin = key[i];
+    const int id = src.id[i];
     const bool moves = *varies != 0;
-    int i = perm[k];
     double xs[3] = {0.0, 0.0, 0.0};
+    Real vs[3] = {0, 0, 0};
 #pragma unroll
     for (int d = 0; d < DIM; ++d) {
-        size_t so = (size_t)d * n + i, dof = (size_t)d * n + k;
-        xs[d] = src.x[so];
+        xs[d] = src.x[(size_t)d * n + i];
+        vs[d] = src.v[(size_t)d * n + i];
+    }
+    int k = start_of(bin);
+    const int members = start_of(bin + 1) - k;
+    if (members > 1) {
+        int t = head[bin];
+        for (int q = 1; ; ++q) {
+            k += src.id[t] < id;
+            if (q == members) break;
+            t = next[t];
+        }
+    }
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) {
+        const size_t so = (size_t)d * n + i, dof = (size_t)d * n + k;
         dst.x[dof] = xs[d];
-        dst.v[dof] = src.v[so];
+        dst.v[dof] = vs[d];
         if (CARRY_AD) {
             dst.a[dof] = src.a[so];
             dst.dr[dof] = src.dr[so];
@@ -346,22 +345,20 @@ __global__ void k_permute(int n, const int32_t* __restrict__ perm, StateSet<Real
         dst.s0[k] = src.s0[i];
         dst.kind[k] = src.kind[i];
     }
-    dst.id[k] = src.id[i];
-    if (F32POS) {
-        int kk = key[i] >> G.sub_shift;   // the cell of the sort key
-        int c[3];
-        cell_decode(G, kk, c);
-        float o[3] = {0.f, 0.f, 0.f};
-        // the conversions on the integer ALU (the same values as the hardware
-        // conversions, which run on the FP64 pipe)
+    dst.id[k] = id;
+    const int cell = bin >> G.sub_shift;   // the cell of the sort key
+    int c[3];
+    cell_decode(G, cell, c);
+    float o[3] = {0.f, 0.f, 0.f};
+    // the conversions on the integer ALU (the same values as the hardware
+    // conversions, which run on the FP64 pipe)
 #pragma unroll
-        for (int d = 0; d < DIM; ++d) o[d] = d2f_rn(xs[d] - (G.lo[d] + i2d_exact(c[d]) * G.edge[d]));
-        const float m_f = d2f_rn(m);
-        pos4[k] = make_float4(o[0], o[1], o[2], uniform_h ? m_f : d2f_rn(h));
-        if (pos4c) pos4c[k] = make_float4(o[0], o[1], o[2], __int_as_float(kk));
-        cell_out[k] = kk;
-        mf[k] = m_f;
-    }
+    for (int d = 0; d < DIM; ++d) o[d] = d2f_rn(xs[d] - (G.lo[d] + i2d_exact(c[d]) * G.edge[d]));
+    const float m_f = d2f_rn(m);
+    pos4[k] = make_float4(o[0], o[1], o[2], uniform_h ? m_f : d2f_rn(h));
+    if (pos4c) pos4c[k] = make_float4(o[0], o[1], o[2], __int_as_float(cell));
+    cell_out[k] = cell;
+    mf[k] = m_f;
 }
 
 // ------------------------------------------------------------- launchers
@@ -369,63 +366,47 @@ __global__ void k_permute(int n, const int32_t* __restrict__ perm, StateSet<Real
 static inline int nblk(int n, int t) { return (n + t - 1) / t; }
 
 cudaError_t launch_kick_drift_key(int prec, int dim, int n, void* S, const double* dt, int drift, const Grid& G,
-                                  int32_t* key, int32_t* count, uint32_t* err, cudaStream_t st)
+                                  int32_t* key, int32_t* count, int32_t* head, int32_t* next, uint32_t* err,
+                                  cudaStream_t st)
 {
     const int T = 256;
     if (prec == 64) {
         auto s = *(StateSet<double>*)S;
-        if (dim == 2) k_kick_drift_key<double, 2><<<nblk(n, T), T, 0, st>>>(n, s, dt, drift, G, key, count, err);
-        else k_kick_drift_key<double, 3><<<nblk(n, T), T, 0, st>>>(n, s, dt, drift, G, key, count, err);
+        if (dim == 2) k_kick_drift_key<double, 2><<<nblk(n, T), T, 0, st>>>(n, s, dt, drift, G, key, count, head, next, err);
+        else k_kick_drift_key<double, 3><<<nblk(n, T), T, 0, st>>>(n, s, dt, drift, G, key, count, head, next, err);
     } else {
         auto s = *(StateSet<float>*)S;
-        if (dim == 2) k_kick_drift_key<float, 2><<<nblk(n, T), T, 0, st>>>(n, s, dt, drift, G, key, count, err);
-        else k_kick_drift_key<float, 3><<<nblk(n, T), T, 0, st>>>(n, s, dt, drift, G, key, count, err);
+        if (dim == 2) k_kick_drift_key<float, 2><<<nblk(n, T), T, 0, st>>>(n, s, dt, drift, G, key, count, head, next, err);
+        else k_kick_drift_key<float, 3><<<nblk(n, T), T, 0, st>>>(n, s, dt, drift, G, key, count, head, next, err);
     }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_scatter_order(int n, int nbin, const int32_t* key, const int32_t* prefix, const int32_t* tile_off,
-                                 int32_t* count, int32_t* perm_tmp, const int32_t* id, int32_t* perm, int32_t* start,
-                                 int shift, int32_t* cell_start, cudaStream_t st, int64_t* launches)
-{
-    const int T = 256;
-    k_scatter<<<nblk(n, T), T, 0, st>>>(n, key, prefix, tile_off, count, perm_tmp);
-    k_order_cells<<<nblk(nbin + 1, T), T, 0, st>>>(nbin, prefix, tile_off, perm_tmp, id, perm, start, shift,
-                                                   cell_start);
-    *launches += 2;
     return cudaGetLastError();
 }
 
 template <typename Real>
-static void permute_t(int dim, int n, const int32_t* perm, void* src, void* dst, const int32_t* key,
-                      const Grid& G, float4* pos4, int32_t* cell, float* mf, int uh, int carry_ad, cudaStream_t st,
-                      float4* pos4c, const uint32_t* varies)
+static void order_permute_t(int dim, int n, int nbin, const SortBufs& B, void* src, void* dst, const Grid& G,
+                            float4* pos4, int32_t* cell, float* mf, int uh, int carry_ad, cudaStream_t st,
+                            float4* pos4c, const uint32_t* varies)
 {
     const int T = 256;
+    const int nb = nblk(n > nbin ? n : nbin + 1, T);
     auto s = *(StateSet<Real>*)src;
     auto d = *(StateSet<Real>*)dst;
-    constexpr bool F32 = true;   // both forms: the density passes walk the FP32 cell-relative positions
-    if (dim == 2) {
-        if (carry_ad)
-            k_permute<Real, 2, true, F32><<<nblk(n, T), T, 0, st>>>(n, perm, s, d, key, G, pos4, cell, mf, uh, pos4c, varies);
-        else
-            k_permute<Real, 2, false, F32><<<nblk(n, T), T, 0, st>>>(n, perm, s, d, key, G, pos4, cell, mf, uh, pos4c, varies);
-    } else {
-        if (carry_ad)
-            k_permute<Real, 3, true, F32><<<nblk(n, T), T, 0, st>>>(n, perm, s, d, key, G, pos4, cell, mf, uh, pos4c, varies);
-        else
-            k_permute<Real, 3, false, F32><<<nblk(n, T), T, 0, st>>>(n, perm, s, d, key, G, pos4, cell, mf, uh, pos4c, varies);
-    }
+    int32_t* cs = G.sub_shift ? B.cell_start : nullptr;
+    int32_t* bs = G.sub_shift ? B.sub_start : B.cell_start;
+    auto kern = dim == 2 ? (carry_ad ? k_order_permute<Real, 2, true> : k_order_permute<Real, 2, false>)
+                         : (carry_ad ? k_order_permute<Real, 3, true> : k_order_permute<Real, 3, false>);
+    kern<<<nb, T, 0, st>>>(n, nbin, B.key, B.prefix, B.tile_off, B.head, B.next, bs, cs, s, d, G, pos4, cell, mf, uh,
+                           pos4c, varies);
 }
 
-cudaError_t launch_permute(int prec, int dim, int n, const int32_t* perm, void* src, void* dst, const int32_t* key,
-                           const Grid& G, float4* pos4, int32_t* cell, float* mf, int uniform_h, int carry_ad,
-                           cudaStream_t st, const uint32_t* varies, float4* pos4c)
+cudaError_t launch_order_permute(int prec, int dim, int n, int nbin, const SortBufs& B, void* src, void* dst,
+                                 const Grid& G, float4* pos4, int32_t* cell, float* mf, int uniform_h, int carry_ad,
+                                 cudaStream_t st, const uint32_t* varies, float4* pos4c)
 {
     if (prec == 64)
-        permute_t<double>(dim, n, perm, src, dst, key, G, pos4, cell, mf, uniform_h, carry_ad, st, pos4c, varies);
+        order_permute_t<double>(dim, n, nbin, B, src, dst, G, pos4, cell, mf, uniform_h, carry_ad, st, pos4c, varies);
     else
-        permute_t<float>(dim, n, perm, src, dst, key, G, pos4, cell, mf, uniform_h, carry_ad, st, pos4c, varies);
+        order_permute_t<float>(dim, n, nbin, B, src, dst, G, pos4, cell, mf, uniform_h, carry_ad, st, pos4c, varies);
     return cudaGetLastError();
 }
 

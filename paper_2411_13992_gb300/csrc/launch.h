@@ -37,26 +37,26 @@ struct AdjView {
     double* eta;
 };
 
-// k_cells.cu
+// k_cells.cu.  Buffers of the sort: each particle's bin (key), the bins'
+// counts (zero between sorts) and list heads, the lists' links, the scan's
+// within-tile prefixes and tile offsets, and what the sort leaves: the starts
+// of the cells and of their sub-cells along x (null without sub-cells).
+struct SortBufs {
+    int32_t *key, *next;
+    int32_t *count, *head, *prefix;
+    int32_t* tile_off;
+    int32_t *cell_start, *sub_start;
+    unsigned* done;        // zero between launches
+};
 cudaError_t launch_kick_drift_key(int prec, int dim, int n, void* S, const double* dt, int drift, const Grid& G,
-                                  int32_t* key, int32_t* count, uint32_t* err, cudaStream_t st);
+                                  int32_t* key, int32_t* count, int32_t* head, int32_t* next, uint32_t* err,
+                                  cudaStream_t st);
 size_t scan_temp_elems(int n);
-cudaError_t launch_exclusive_scan(const int32_t* in, int32_t* out, int n, int32_t* tmp, cudaStream_t st,
-                                  int64_t* launches);
-// The sort's scan without its last pass (see k_cells.cu): prefix within
-// tiles, *tile_off the tiles' offsets (null for one tile).
-cudaError_t launch_scan_tiles(const int32_t* count, int32_t* prefix, int n, int32_t* tmp, cudaStream_t st,
-                              int64_t* launches, const int32_t** tile_off);
-// nbin sort bins (cells, or sub-cells when shift > 0) whose starts are
-// prefix + tile_off: scatter by the counts (left at zero), order each bin by
-// id, write the bins' starts into start[nbin + 1] and, with shift > 0, the
-// cells' starts into cell_start.
-cudaError_t launch_scatter_order(int n, int nbin, const int32_t* key, const int32_t* prefix, const int32_t* tile_off,
-                                 int32_t* count, int32_t* perm_tmp, const int32_t* id, int32_t* perm, int32_t* start,
-                                 int shift, int32_t* cell_start, cudaStream_t st, int64_t* launches);
-cudaError_t launch_permute(int prec, int dim, int n, const int32_t* perm, void* src, void* dst, const int32_t* key,
-                           const Grid& G, float4* pos4, int32_t* cell, float* mf, int uniform_h, int carry_ad,
-                           cudaStream_t st, const uint32_t* varies, float4* pos4c = nullptr);
+cudaError_t launch_bin_scan(int32_t* count, int32_t* prefix, int n, int32_t* tile_off, unsigned* done,
+                            cudaStream_t st);
+cudaError_t launch_order_permute(int prec, int dim, int n, int nbin, const SortBufs& B, void* src, void* dst,
+                                 const Grid& G, float4* pos4, int32_t* cell, float* mf, int uniform_h, int carry_ad,
+                                 cudaStream_t st, const uint32_t* varies, float4* pos4c = nullptr);
 
 // What the last block of a pass needs to fold the grid's partials and set the
 // next step size: the partials' buffers, the counters (zero between

@@ -53,10 +53,8 @@ struct sph_ctx {
     Consts<float> K32;
     SetPtrs set[2];
     int cur;
-    // the sort: keys, permutations, bin counts (zero between sorts), the
-    // scan's within-tile prefixes, the cells' starts and its scratch
-    int32_t *key, *perm_tmp, *perm, *count, *prefix, *start, *scan_tmp;
-    int32_t* sub_start;  // the sort's sub-cell starts (x_subcells > 1), else null
+    SortBufs sort;
+    int32_t* start;      // the cells' starts (sort.cell_start)
     int count_zero;      // count[] is known to be all zero (a complete sort ran since it was cleared)
     void* vr;
     float4* pos4;
@@ -312,16 +310,18 @@ size_t carve(sph_ctx* c, char* base)
         c->set[s].d = StateSet<double>{x, (double*)v, (double*)a, (double*)dr, (double*)drho, h, m, s0, id, kind};
         c->set[s].f = StateSet<float>{x, (float*)v, (float*)a, (float*)dr, (float*)drho, h, m, s0, id, kind};
     }
-    c->key = W.take<int32_t>(n);
-    c->perm_tmp = W.take<int32_t>(n);
-    c->perm = W.take<int32_t>(n);
+    SortBufs& B = c->sort;
+    B.key = W.take<int32_t>(n);
+    B.next = W.take<int32_t>(n);
     const size_t nb1 = sort_bins(c->G) + 1;
-    c->count = W.take<int32_t>(nb1);
-    c->prefix = W.take<int32_t>(nb1);
-    c->start = W.take<int32_t>(nc1);
-    c->sub_start = c->G.sub_shift ? W.take<int32_t>(nb1) : nullptr;
-    c->G.sub_start = c->sub_start;
-    c->scan_tmp = W.take<int32_t>(scan_temp_elems((int)nb1));
+    B.count = W.take<int32_t>(nb1);
+    B.head = W.take<int32_t>(nb1);
+    B.prefix = W.take<int32_t>(nb1);
+    B.cell_start = c->start = W.take<int32_t>(nc1);
+    B.sub_start = c->G.sub_shift ? W.take<int32_t>(nb1) : nullptr;
+    c->G.sub_start = B.sub_start;
+    B.tile_off = W.take<int32_t>(scan_temp_elems((int)nb1));
+    B.done = W.take<unsigned>(1);
     c->vr = W.take<char>(n * 4 * rs);
     c->pos4 = W.take<float4>(n);     // both forms: FP32 cell-relative positions for the candidate walks
     c->pos4c = c->prec == 32 && c->P.h_min == c->P.h_max ? W.take<float4>(n) : nullptr;
@@ -410,36 +410,32 @@ inline cudaError_t prof_mark(sph_ctx* c, int cls, int end)
         if (s_ != SPH_OK) return s_;     \
     } while (0)
 
-// Kick-drift (optional), cell keys, counting sort, permute.
+// Kick-drift (optional), cell keys, counting sort with the arrays moved.
 sph_status run_sort(sph_ctx* c, int drift, int carry_ad)
 {
     const int n = (int)c->n;
     const size_t nb1 = sort_bins(c->G) + 1;
-    // the bins' starts: the sub-cells' (the cells' then follow from them) or the cells'
-    int32_t* bin_start = c->G.sub_shift ? c->sub_start : c->start;
+    const SortBufs& B = c->sort;
     SPH_MARK(SPH_K_KICKDRIFT, 0);
-    // the scatter counts every bin back down to zero: clear only when a sort
+    // the scan clears the counts as it reads them: clear only when a sort
     // did not complete since the counts were last known to be zero
-    if (!c->count_zero) SPH_CU(cudaMemsetAsync(c->count, 0, nb1 * sizeof(int32_t), c->st));
+    if (!c->count_zero) {
+        SPH_CU(cudaMemsetAsync(B.count, 0, nb1 * sizeof(int32_t), c->st));
+        SPH_CU(cudaMemsetAsync(B.done, 0, sizeof(unsigned), c->st));
+    }
     c->count_zero = 0;
-    SPH_CU(launch_kick_drift_key(c->prec, c->dim, n, cur_set(c), c->dt, drift, c->G, c->key, c->count, c->err, c->st));
-    ++c->launches;
+    SPH_CU(launch_kick_drift_key(c->prec, c->dim, n, cur_set(c), c->dt, drift, c->G, B.key, B.count, B.head, B.next,
+                                 c->err, c->st));
     SPH_MARK(SPH_K_KICKDRIFT, 1);
     SPH_MARK(SPH_K_SCAN, 0);
-    const int32_t* tile_off = nullptr;
-    SPH_CU(launch_scan_tiles(c->count, c->prefix, (int)nb1, c->scan_tmp, c->st, &c->launches, &tile_off));
-    SPH_MARK(SPH_K_SCAN, 1);
-    const int32_t* id = c->prec == 64 ? c->set[c->cur].d.id : c->set[c->cur].f.id;
-    SPH_MARK(SPH_K_ORDER, 0);
-    SPH_CU(launch_scatter_order(n, (int)sort_bins(c->G), c->key, c->prefix, tile_off, c->count, c->perm_tmp, id,
-                                c->perm, bin_start, c->G.sub_shift, c->start, c->st, &c->launches));
+    SPH_CU(launch_bin_scan(B.count, B.prefix, (int)nb1, B.tile_off, B.done, c->st));
     c->count_zero = 1;
-    SPH_MARK(SPH_K_ORDER, 1);
+    SPH_MARK(SPH_K_SCAN, 1);
     SPH_MARK(SPH_K_PERMUTE, 0);
-    SPH_CU(launch_permute(c->prec, c->dim, n, c->perm, cur_set(c), other_set(c), c->key, c->G, c->pos4, c->cell,
-                          c->mf, c->K32.uniform_h, carry_ad, c->st, c->err + 1, c->pos4c));
-    ++c->launches;
+    SPH_CU(launch_order_permute(c->prec, c->dim, n, (int)sort_bins(c->G), B, cur_set(c), other_set(c), c->G, c->pos4,
+                                c->cell, c->mf, c->K32.uniform_h, carry_ad, c->st, c->err + 1, c->pos4c));
     SPH_MARK(SPH_K_PERMUTE, 1);
+    c->launches += 3;
     c->cur = 1 - c->cur;
     return SPH_OK;
 }
@@ -1125,7 +1121,7 @@ sph_status sph_get_state(sph_ctx* c, double* x, double* v, double* a, double* dr
     // the scratch of the sort); written in place into device memory, and
     // through the staging buffer and a copy into host memory (a copy reaches
     // about 3x the rate of kernel stores across the host link)
-    int32_t* pos = c->perm_tmp;
+    int32_t* pos = c->sort.next;
     if (x || v || a || dr || rho) {
         SPH_CU(launch_inverse_perm(n, Sd.id, pos, c->st));
         ++c->launches;
@@ -1455,11 +1451,9 @@ extern "C" sph_status sph_density_noalloc(const sph_params* p, int64_t n, const 
     carve(&c, (char*)base);
 
     const int ni = (int)n;
-    const size_t nc1 = (size_t)G.ncell + 1;
     StateSet<double>& S0 = c.set[0].d;
     // The scratch keeps the previous call's contents: clear what is summed into.
-    SPH_CU(cudaMemsetAsync(c.count, 0, nc1 * sizeof(int32_t), c.st));
-    SPH_CU(cudaMemsetAsync(c.prefix, 0, nc1 * sizeof(int32_t), c.st));
+    // (run_sort clears the bins' counts: the view starts with count_zero = 0.)
     SPH_CU(cudaMemsetAsync(c.err, 0, 4 * sizeof(uint32_t), c.st));
     SPH_CU(cudaMemsetAsync(c.err + 1, 1, 1, c.st));   // the sort moves h, m, sigma0 and kind
     SPH_CU(cudaMemsetAsync(S0.v, 0, (size_t)c.dim * n * sizeof(double), c.st));
