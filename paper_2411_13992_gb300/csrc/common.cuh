@@ -86,6 +86,12 @@ struct Consts {
     Real fr_x[4];
     // h_u = h_max (the h of every pair at uniform resolution)
     Real h_u, inv_h_u, four_h2_u, dwr_coef_u;   // dwr_coef_u: W'(r)/r = dwr_coef_u t^3
+    // products of the above that the FP64 passes would otherwise form in every
+    // thread (a dozen FP64 operations, as many as a third of a pair)
+    Real half_c2, half_c, quarter_c, beta_k;    // c^2/2, c/2, c/4, eta_R/c
+    Real two_h_u, half_inv_h_u, two_inv_h_u;    // 2h, 1/(2h), 2/h
+    Real w_norm_u;                              // a_D h^-D
+    float reach_u, prefilter2_u;                // 2h, and the squared bound of the FP32 prefilter (1e-4 margin)
 };
 
 // Velocity + density deviation packed per particle for the pair pass:

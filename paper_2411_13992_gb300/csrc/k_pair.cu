@@ -34,61 +34,70 @@ namespace sphtv {
 
 // ============================================================== FP64 form
 
-// Candidates come from the clipped FP32 row walk over the cell-relative
-// positions (pos4); a loose FP32 test drops the far ones and the exact FP64
-// test (minimum image, sqrt(r2) < 2 h_ij) decides the rest.  The walk visits
-// candidates in the order of the cell scan (cells by dz, dy, dx, then index),
-// so sigma is summed in the same order as a plain scan would.  With nbl
-// non-null it also writes the particle's neighbour list (j != i,
-// 0 < r < 2 h_ij), transposed (entry k at nbl[k * n + i] = j << kCodeBits),
-// and the count (which may exceed cap); the FP64 force pass walks it.
-template <int DIM>
-__global__ void __launch_bounds__(256) k_density_f64(int n, StateSet<double> S, const int32_t* __restrict__ start,
-                                                     Grid G, Consts<double> K, double4_32a* __restrict__ vr,
-                                                     const float4* __restrict__ pos4,
-                                                     const int32_t* __restrict__ cell_of, uint32_t* __restrict__ nbl,
-                                                     int32_t* __restrict__ nbc, int cap, double* __restrict__ vol)
+// Lanes per particle.  L = 1: one thread per particle, which at 38,912
+// particles or more (256 threads on each of 152 SMs) keeps the FP64 pipe of
+// every SM busy.  L > 1: a group of L consecutive lanes per particle for
+// smaller problems, whose passes are bound by the latency of one thread's
+// chain of FP64 operations (a few hundred per particle, some 60 cycles each):
+// 2,500 particles with one thread each left half the SMs without a warp and
+// one warp on the others.  The lanes of a group share the particle's
+// candidates and neighbours; the per-particle work before and after the sums
+// is done by one thread per particle in full warps, since the FP64 pipe
+// serves a warp instruction whole, however few of its lanes are active.
+// Measured, us a step (start of the comparison -> L = 1 / 4 / 8): 2-D 2,500
+// particles 116 -> 99 / 48 / 42, 8,100: 115 -> 100 / 55 / 55, 20,000: 120 ->
+// 103 / 102 / 113, 40,000: 250 -> 151 / 161 / 186; 3-D 4,096: 391 -> 358 /
+// 122 / 93, 17,576: 397 -> 363 / 259 / 276, 64,000: 889 (now 809) / 823.
+template <int L> struct Lanes {
+    static constexpr int kThreads = L == 1 ? 256 : 512;    // most threads of a block
+};
+
+// Threads of a block with L > 1 lanes per particle: what spreads the particles
+// evenly over the SMs, whole warps; past that, blocks of 128 (L = 4) or 256.
+static int lane_threads(int L, int n, int sms)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    double xi[3] = {0, 0, 0}, vi[3] = {0, 0, 0};
-#pragma unroll
-    for (int d = 0; d < DIM; ++d) {
-        xi[d] = S.x[(size_t)d * n + i];
-        vi[d] = S.v[(size_t)d * n + i];
-    }
-    if (S.kind[i]) {
-        vr[i] = make_double4_32a(vi[0], vi[1], vi[2], __longlong_as_double(0x7ff0000000000000ll));
-        if (nbc) nbc[i] = 0;
-        return;
-    }
-    const double hi = S.h[i];
-    const float4 pi = pos4[i];
-    const float oi[3] = {pi.x, pi.y, pi.z};
-    const int cell_i = cell_of[i];
+    const int64_t t = ((int64_t)n * L + sms - 1) / sms;
+    const int full = L >= 8 ? 512 : 128;          // 64 particles a block: 32 KB of row bounds in 3-D
+    return t > full ? (L >= 8 ? 256 : 128) : (t < 32 ? 32 : (int)((t + 31) / 32 * 32));
+}
+
+// Exact FP64 test and kernel value of the density pass for particle i: the
+// candidate's image (the periodic image of the stencil step, which is the
+// nearest one of every neighbour), r < 2 h_ij, and W added to sigma; true for
+// a force neighbour (j != i, 0 < r < 2 h_ij).  The comparisons of
+// non-negative doubles are made on their bit patterns (same order) by the
+// integer ALU, off the FP64 pipe.  At uniform resolution sigma collects
+// W / (a_D h^-D), the constant applied once at the end.
+template <int DIM>
+struct Density64 {
+    int n, i;
+    const Grid& G;
+    const Consts<double>& K;
+    const StateSet<double>& S;
+    double xi[3];
     int ci[3];
-    cell_decode(G, cell_i, ci);
-    // reach of the walk: the largest support radius 2 h_ij of i (h_j <= h_max)
-    const float reach = (float)(2.0 * pair_h(K, hi, K.h_u));
-    // uniform resolution: h_ij = h for every pair, so the support, the
-    // prefilter bound and a_D h^-D are constants (the same values, computed
-    // once instead of per candidate on the FP64 pipe)
-    const bool uni = K.uniform_h != 0;
-    const double two_hu = 2.0 * K.h_u;
-    const float lim_u = (float)two_hu;
-    const float lim2_u = lim_u * lim_u * 1.0001f;
-    const double wnorm_u = kernel_norm<DIM, double>() * pow_dim<DIM, double>(K.inv_h_u);
-    const double half_inv_hu = 0.5 * K.inv_h_u, two_inv_hu = 2.0 * K.inv_h_u;
-    // sigma; at uniform resolution the sum of W / (a_D h^-D), the constant
-    // applied once at the end
-    double sigma = 0.0;
-    // the exact FP64 test of a candidate that passed the FP32 prefilter: adds
-    // W to sigma; true for a force neighbour (j != i, 0 < r < 2 h_ij).  The
-    // comparisons of non-negative doubles are made on their bit patterns
-    // (same order) by the integer ALU, off the FP64 pipe.
-    auto exact = [&](int j, uint32_t code, double hij) {
-        // x_i - x_j with the periodic image of the stencil step (the nearest
-        // image of every neighbour: the same operations as min_image)
+    double hi;
+    double sigma;
+
+    __device__ __forceinline__ Density64(int n_, int i_, const Grid& G_, const Consts<double>& K_,
+                                         const StateSet<double>& S_, int cell_i)
+        : n(n_), i(i_), G(G_), K(K_), S(S_), sigma(0.0)
+    {
+#pragma unroll
+        for (int d = 0; d < 3; ++d) xi[d] = d < DIM ? S.x[(size_t)d * n + i] : 0.0;
+        hi = S.h[i];
+        cell_decode(G, cell_i, ci);
+    }
+
+    // the largest support radius 2 h_ij of any pair of i (h_j <= h_max)
+    __device__ __forceinline__ float reach() const
+    {
+        return K.uniform_h ? K.reach_u : (float)(2.0 * pair_h(K, hi, K.h_u));
+    }
+
+    __device__ __forceinline__ bool exact(int j, uint32_t code)
+    {
+        const bool uni = K.uniform_h != 0;
         const int step[3] = {(int)(code % kSide) - kStencilR, (int)((code / kSide) % kSide) - kStencilR,
                              (int)(code / (kSide * kSide)) - kStencilR};
         double r2 = 0.0;
@@ -102,48 +111,79 @@ __global__ void __launch_bounds__(256) k_density_f64(int n, StateSet<double> S, 
             }
             r2 += t * t;
         }
-        const double r = sqrt(r2);
+        const bool apart = __double_as_longlong(r2) != 0;                // r2 >= +0
+        const double r = apart ? sqrt_pos(r2) : 0.0;
         // r < 2 h_ij (a NaN has a pattern above every finite value's)
-        if (!((unsigned long long)__double_as_longlong(r) <
-              (unsigned long long)__double_as_longlong(uni ? two_hu : 2.0 * hij)))
-            return false;
+        const unsigned long long rb = (unsigned long long)__double_as_longlong(r);
         if (uni) {
+            if (!(rb < (unsigned long long)__double_as_longlong(K.two_h_u))) return false;
             // t = 1 - q/2 and 2q + 1 with q = r/h, each one fused operation
-            const double t = fma(-half_inv_hu, r, 1.0);
+            const double t = fma(-K.half_inv_h_u, r, 1.0);
             const double t2 = t * t;
-            sigma = fma(t2 * t2, fma(two_inv_hu, r, 1.0), sigma);
+            sigma = fma(t2 * t2, fma(K.two_inv_h_u, r, 1.0), sigma);
         } else {
+            const double hij = pair_h(K, hi, S.h[j]);
+            if (!(rb < (unsigned long long)__double_as_longlong(2.0 * hij))) return false;
             sigma += wendland_W<DIM, double>(r, 1.0 / hij);
         }
-        return j != i && __double_as_longlong(r2) != 0;               // r2 >= +0
-    };
-    // FP32 prefilter bound (1e-4 margin) of the pair (i, j); pj_w = (float)h_j
-    // when h varies
-    const float hi_f = (float)hi;
-    auto prefilter2 = [&](float pj_w) {
-        if (uni) return lim2_u;
-        const float lim = 2.f * (K.h_pair_max ? fmaxf(hi_f, pj_w) : 0.5f * (hi_f + pj_w));
-        return lim * lim * 1.0001f;
-    };
+        return j != i && apart;
+    }
+};
+
+// FP32 prefilter of a candidate (1e-4 margin): the squared bound of the pair
+// (i, j), pj_w = (float)h_j when h varies.
+__device__ __forceinline__ float prefilter2(const Consts<double>& K, float hi_f, float pj_w)
+{
+    if (K.uniform_h) return K.prefilter2_u;
+    const float lim = 2.f * (K.h_pair_max ? fmaxf(hi_f, pj_w) : 0.5f * (hi_f + pj_w));
+    return lim * lim * 1.0001f;
+}
+
+// End of the density pass for particle i: rho_i (Eq. 8), its velocity record
+// {v, rho - rho0} (+inf marks a wall), and V_i = m_i / rho_i for the force
+// pass.
+template <int DIM>
+__device__ __forceinline__ void density64_end(int n, int i, const Consts<double>& K, const StateSet<double>& S,
+                                              double sigma, double4_32a* __restrict__ vr, double* __restrict__ vol)
+{
+    double vi[3] = {0, 0, 0};
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) vi[d] = S.v[(size_t)d * n + i];
+    if (S.kind[i]) {
+        vr[i] = make_double4_32a(vi[0], vi[1], vi[2], __longlong_as_double(0x7ff0000000000000ll));
+        return;
+    }
+    if (K.uniform_h) sigma *= K.w_norm_u;
+    const double rho = __ddiv_rn(__dmul_rn(K.rho0, sigma), S.s0[i]);
+    const double w = __dsub_rn(rho, K.rho0);
+    vr[i] = make_double4_32a(vi[0], vi[1], vi[2], w);
+    if (vol) vol[i] = S.m[i] / (K.rho0 + w);
+}
+
+// Candidates come from the clipped FP32 row walk over the cell-relative
+// positions (pos4); a loose FP32 test drops the far ones and the exact FP64
+// test (minimum image, sqrt(r2) < 2 h_ij) decides the rest.  The walk visits
+// candidates in the order of the cell scan (cells by dz, dy, dx, then index),
+// so sigma is summed in the same order as a plain scan would.  With nbl
+// non-null it also writes the particle's neighbour list (j != i,
+// 0 < r < 2 h_ij), transposed (entry k at nbl[k * n + i] = j << kCodeBits),
+// and the count (which may exceed cap); the FP64 force pass walks it.
+template <int DIM>
+__device__ __forceinline__ double density64_thread(int n, int i, const StateSet<double>& S,
+                                                   const int32_t* __restrict__ start, const Grid& G,
+                                                   const Consts<double>& K, const float4* __restrict__ pos4,
+                                                   const int32_t* __restrict__ cell_of, uint32_t* __restrict__ nbl,
+                                                   int32_t* __restrict__ nbc, int cap, bool two_pass)
+{
+    const float4 pi = pos4[i];
+    const float oi[3] = {pi.x, pi.y, pi.z};
+    const int cell_i = cell_of[i];
+    Density64<DIM> D(n, i, G, K, S, cell_i);
+    const float reach = D.reach();
+    const float hi_f = K.uniform_h ? 0.f : (float)D.hi;      // read at variable resolution only
     int cnt = 0;
-    // one pass: the exact test inside the walk (the lanes whose candidate
-    // passed the prefilter run it while the others wait)
-    auto visit = [&](int j, uint32_t code, const float4&, float r2f, float, float, float) {
-        double hij = K.h_u;
-        float lim2 = lim2_u;
-        if (!uni) {
-            hij = pair_h(K, hi, S.h[j]);
-            const float lim = (float)(2.0 * hij);
-            lim2 = lim * lim * 1.0001f;
-        }
-        if (!(r2f <= lim2)) return;                      // FP32 prefilter, 1e-4 margin
-        if (exact(j, code, hij) && nbl) {
-            if (cnt < cap) nbl[(size_t)cnt * n + i] = ((uint32_t)j << kCodeBits) | code;
-            ++cnt;
-        }
-    };
     bool staged = false;
-    if (nbl) {
+    if (nbl && two_pass) {
         // two passes: the walk stages the candidates that pass the prefilter
         // in the particle's list, then the exact FP64 test runs over them
         // with every lane busy (the FP64 pipe serves a warp instruction
@@ -153,7 +193,7 @@ __global__ void __launch_bounds__(256) k_density_f64(int n, StateSet<double> S, 
         int nf = 0;
         uint32_t* lp = nbl + i;
         auto stage = [&](int j, uint32_t code, const float4& pj, float r2f, float, float, float) {
-            if (!(r2f <= prefilter2(pj.w))) return;
+            if (!(r2f <= prefilter2(K, hi_f, pj.w))) return;
             if (nf < cap) {
                 *lp = ((uint32_t)j << kCodeBits) | code;
                 lp += n;
@@ -166,207 +206,454 @@ __global__ void __launch_bounds__(256) k_density_f64(int n, StateSet<double> S, 
             for (int k = 0; k < nf; ++k) {
                 const uint32_t e = nbl[(size_t)k * n + i];
                 const int j = (int)(e >> kCodeBits);
-                const double hij = uni ? K.h_u : pair_h(K, hi, S.h[j]);
-                if (exact(j, e & ((1u << kCodeBits) - 1u), hij)) {
+                if (D.exact(j, e & ((1u << kCodeBits) - 1u))) {
                     if (cnt != k) nbl[(size_t)cnt * n + i] = e;     // entries before a rejected one stay in place
                     ++cnt;
                 }
             }
         }
     }
-    if (!staged) for_candidates_rows<DIM, false>(oi, reach, cell_i, G, start, cell_of, pos4, visit);
+    if (!staged) {
+        // one pass: the exact test inside the walk (the lanes whose candidate
+        // passed the prefilter run it while the others wait)
+        auto visit = [&](int j, uint32_t code, const float4& pj, float r2f, float, float, float) {
+            if (!(r2f <= prefilter2(K, hi_f, pj.w))) return;
+            if (D.exact(j, code) && nbl) {
+                if (cnt < cap) nbl[(size_t)cnt * n + i] = ((uint32_t)j << kCodeBits) | code;
+                ++cnt;
+            }
+        };
+        for_candidates_rows<DIM, false>(oi, reach, cell_i, G, start, cell_of, pos4, visit);
+    }
     if (nbc) nbc[i] = cnt;
-    if (uni) sigma *= wnorm_u;
-    double rho = __ddiv_rn(__dmul_rn(K.rho0, sigma), S.s0[i]);
-    const double w = __dsub_rn(rho, K.rho0);
-    vr[i] = make_double4_32a(vi[0], vi[1], vi[2], w);
-    // V_i = m_i / rho_i for the force pass, once per particle instead of once
-    // per pair
-    if (vol) vol[i] = S.m[i] / (K.rho0 + w);
+    return D.sigma;
 }
 
+// One stencil row of a particle's walk: two runs of the sort order (the
+// second empty unless the row wraps a periodic x boundary) and the cell index
+// of the row's first cell.
+struct RowRuns {
+    int j0, n0, j1, n1, row;
+};
+
+// Row r = (dy + R) + kSide (dz + R) of the stencil of a particle in cell c at
+// offset oi, cut as for_candidates_rows cuts it.
 template <int DIM>
-__global__ void __launch_bounds__(256, 2) k_forces_f64(int n, StateSet<double> S, const int32_t* __restrict__ start,
-                                                    Grid G, Consts<double> K, const double4_32a* __restrict__ vr,
+__device__ __forceinline__ RowRuns row_runs(int r, const float* oi, float reach, const int* c, const Grid& G,
+                                            const int32_t* __restrict__ start)
+{
+    constexpr int R = kStencilR;
+    RowRuns q = {0, 0, 0, 0, 0};
+    const int dy = r % kSide - R, dz = DIM == 3 ? r / kSide - R : 0;
+    const int cy = cell_step(G, c[1], dy, 1), cz = DIM == 3 ? cell_step(G, c[2], dz, 2) : 0;
+    const float ex = G.edgef[0], ey = G.edgef[1], ez = G.edgef[2];
+    float ry = dy > 0 ? dy * ey - oi[1] : (dy < 0 ? oi[1] + (-dy - 1) * ey : 0.f), rz = 0.f;
+    ry = fmaxf(ry - 1e-3f * ey, 0.f);
+    if (DIM == 3) {
+        rz = dz > 0 ? dz * ez - oi[2] : (dz < 0 ? oi[2] + (-dz - 1) * ez : 0.f);
+        rz = fmaxf(rz - 1e-3f * ez, 0.f);
+    }
+    const float w2 = (reach * reach - rz * rz) - ry * ry;
+    if (cy < 0 || cz < 0 || !(w2 > 0.f)) return q;
+    const int sh = G.sub_shift, nsx = G.nc[0] << sh;
+    const int32_t* __restrict__ rstart = sh ? G.sub_start : start;
+    const float inv_exs = (1.f / ex) * (float)(1 << sh);
+    const float w = sqrt_approx(w2) + 1e-3f * ex;
+    const int slo = max(__float2int_rd((oi[0] - w) * inv_exs), -(R << sh));
+    const int shi = min(__float2int_rd((oi[0] + w) * inv_exs), ((R + 1) << sh) - 1);
+    if (slo > shi) return q;
+    q.row = G.nc[0] * (cy + G.nc[1] * cz);
+    const int rb = q.row << sh;
+    int lo0 = (c[0] << sh) + slo, hi0 = (c[0] << sh) + shi, lo1 = 0, hi1 = -1;
+    if (!G.periodic[0]) {
+        lo0 = max(lo0, 0);
+        hi0 = min(hi0, nsx - 1);
+    } else if (lo0 < 0) {
+        hi1 = hi0;
+        lo0 += nsx;
+        hi0 = min(nsx - 1, nsx + hi1);
+    } else if (lo0 >= nsx) {
+        lo0 -= nsx;
+        hi0 -= nsx;
+    } else if (hi0 >= nsx) {
+        hi1 = hi0 - nsx;
+        hi0 = nsx - 1;
+    }
+    if (lo0 <= hi0) {
+        q.j0 = rstart[rb + lo0];
+        q.n0 = rstart[rb + hi0 + 1] - q.j0;
+    }
+    if (lo1 <= hi1) {
+        q.j1 = rstart[rb + lo1];
+        q.n1 = rstart[rb + hi1 + 1] - q.j1;
+    }
+    return q;
+}
+
+// The density pass of a particle by a group of L lanes: the lanes first find
+// the bounds of the stencil rows (one row per lane at a time, so that the
+// loads of all rows are in flight together), then walk each row L candidates
+// at a time, staging the ones that pass the prefilter in the particle's list
+// in the order of the walk (a ballot gives each its place), then run the
+// exact test over the staged ones L at a time, compacting the list.  Returns
+// the lane's part of sigma.  Called by whole warps; `active` is the same for
+// all lanes of a group.
+template <int DIM, int L>
+__device__ __forceinline__ double density64_group(int n, int i, bool active, RowRuns* __restrict__ rows,
+                                                  const StateSet<double>& S, const int32_t* __restrict__ start,
+                                                  const Grid& G, const Consts<double>& K,
+                                                  const float4* __restrict__ pos4,
+                                                  const int32_t* __restrict__ cell_of, uint32_t* __restrict__ nbl,
+                                                  int32_t* __restrict__ nbc, int cap)
+{
+    constexpr int R = kStencilR, NR = DIM == 3 ? kSide * kSide : kSide;
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31, q = lane & (L - 1);
+    const unsigned below = (1u << lane) - 1u, group = ((L == 32 ? 0u : (1u << L)) - 1u) << (lane - q);
+    const float4 pi = pos4[i];
+    const float oi[3] = {pi.x, pi.y, pi.z};
+    const int cell_i = cell_of[i];
+    Density64<DIM> D(n, i, G, K, S, cell_i);
+    const float reach = D.reach();
+    const float hi_f = K.uniform_h ? 0.f : (float)D.hi;      // read at variable resolution only
+    for (int r = q; r < NR; r += L) {
+        RowRuns rr = {0, 0, 0, 0, 0};
+        if (active) rr = row_runs<DIM>(r, oi, reach, D.ci, G, start);
+        rows[r] = rr;
+    }
+    __syncwarp();
+    const float ex = G.edgef[0], ey = G.edgef[1], ez = G.edgef[2];
+    int nf = 0;
+    for (int r = 0; r < NR; ++r) {
+        const RowRuns rr = rows[r];
+        const int len = rr.n0 + rr.n1;
+        const int most = __reduce_max_sync(kAll, len);
+        const int dy = r % kSide - R, dz = DIM == 3 ? r / kSide - R : 0;
+        for (int f0 = 0; f0 < most; f0 += L) {
+            const int f = f0 + q;
+            bool take = false;
+            uint32_t e = 0;
+            if (f < len) {
+                const int j = f < rr.n0 ? rr.j0 + f : rr.j1 + (f - rr.n0);
+                const float4 pj = pos4[j];
+                int dx = cell_of[j] - rr.row - D.ci[0];
+                if (dx > R) dx -= G.nc[0];                    // across the periodic x boundary
+                else if (dx < -R) dx += G.nc[0];
+                const float rx = (oi[0] - pj.x) - (float)dx * ex;
+                const float ry = (oi[1] - pj.y) - (float)dy * ey;
+                float r2 = rx * rx + ry * ry;
+                if (DIM == 3) {
+                    const float rz = (oi[2] - pj.z) - (float)dz * ez;
+                    r2 += rz * rz;
+                }
+                take = r2 <= prefilter2(K, hi_f, pj.w);
+                e = ((uint32_t)j << kCodeBits) | (uint32_t)((dx + R) + kSide * (dy + R) + kSide * kSide * (dz + R));
+            }
+            const unsigned m = __ballot_sync(kAll, take) & group;
+            const int at = nf + __popc(m & below);
+            if (take && at < cap) nbl[(size_t)at * n + i] = e;
+            nf += __popc(m);
+        }
+    }
+    __syncwarp();
+    int cnt = 0;
+    const bool fits = nf <= cap;
+    const int most = __reduce_max_sync(kAll, fits ? nf : 0);
+    for (int k0 = 0; k0 < most; k0 += L) {
+        const int k = k0 + q;
+        bool keep = false;
+        uint32_t e = 0;
+        if (fits && k < nf) {
+            e = nbl[(size_t)k * n + i];
+            const int j = (int)(e >> kCodeBits);
+            keep = D.exact(j, e & ((1u << kCodeBits) - 1u));
+        }
+        const unsigned m = __ballot_sync(kAll, keep) & group;
+        const int at = cnt + __popc(m & below);
+        if (keep && at != k) nbl[(size_t)at * n + i] = e;
+        cnt += __popc(m);
+    }
+    // more candidates than the list holds: one lane walks them in one pass
+    if (active && !fits) {
+        if (q == 0) return density64_thread<DIM>(n, i, S, start, G, K, pos4, cell_of, nbl, nbc, cap, false);
+        return 0.0;
+    }
+    if (active && q == 0) nbc[i] = cnt;
+    return D.sigma;
+}
+
+template <int DIM, int L>
+__global__ void __launch_bounds__(Lanes<L>::kThreads, L == 1 ? 4 : 1) k_density_f64(int n, StateSet<double> S,
+                                                     const int32_t* __restrict__ start, Grid G, Consts<double> K,
+                                                     double4_32a* __restrict__ vr, const float4* __restrict__ pos4,
+                                                     const int32_t* __restrict__ cell_of, uint32_t* __restrict__ nbl,
+                                                     int32_t* __restrict__ nbc, int cap, double* __restrict__ vol)
+{
+    if constexpr (L == 1) {
+        const int i = blockIdx.x * blockDim.x + threadIdx.x;
+        if (i >= n) return;
+        double sigma = 0.0;
+        if (S.kind[i]) {
+            if (nbc) nbc[i] = 0;
+        } else {
+            sigma = density64_thread<DIM>(n, i, S, start, G, K, pos4, cell_of, nbl, nbc, cap, true);
+        }
+        density64_end<DIM>(n, i, K, S, sigma, vr, vol);
+    } else {
+        // shared memory: each particle's row bounds, then its lanes' sums
+        constexpr int NR = DIM == 3 ? kSide * kSide : kSide;
+        extern __shared__ __align__(16) unsigned char smem64[];
+        RowRuns* rows = reinterpret_cast<RowRuns*>(smem64);
+        double* sums = reinterpret_cast<double*>(smem64 + ((size_t)(blockDim.x / L) * NR * sizeof(RowRuns) + 15) / 16 * 16);
+        const int P = blockDim.x / L, p = threadIdx.x / L;
+        const int i = blockIdx.x * P + p;
+        const bool active = i < n && S.kind[i] == 0;
+        sums[threadIdx.x] = density64_group<DIM, L>(n, min(i, n - 1), active, rows + (size_t)p * NR, S, start, G, K,
+                                                    pos4, cell_of, nbl, nbc, cap);
+        __syncthreads();
+        const int ie = blockIdx.x * P + threadIdx.x;
+        if (threadIdx.x < P && ie < n) {
+            if (S.kind[ie]) nbc[ie] = 0;
+            double sigma = 0.0;
+            for (int k = 0; k < L; ++k) sigma += sums[threadIdx.x * L + k];
+            density64_end<DIM>(n, ie, K, S, sigma, vr, vol);
+        }
+    }
+}
+
+// The pair sums of particle i over its neighbours k0, k0 + dk, ... of the
+// list, or over the cells when there is no list (or more neighbours than it
+// holds) and this thread is the one that scans them.
+template <int DIM>
+__device__ __forceinline__ void forces64_sums(int n, int i, const StateSet<double>& S,
+                                              const int32_t* __restrict__ start, const Grid& G,
+                                              const Consts<double>& K, const double4_32a* __restrict__ vr,
+                                              const int32_t* __restrict__ cell_of,
+                                              const uint32_t* __restrict__ nbl, int cnt, int cap, int k0, int dk,
+                                              const double* __restrict__ vol, PairSums64<DIM>& sums)
+{
+    double xi[3] = {0, 0, 0}, vi[3] = {0, 0, 0};
+    const double4_32a me = vr[i];
+    vi[0] = me.x; vi[1] = me.y; vi[2] = me.z;
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) xi[d] = S.x[(size_t)d * n + i];
+    const double hi = S.h[i];
+    // uniform resolution: h_ij = h for every pair, and W'/r = C t^3 (t = 1 - r
+    // / 2h) leaves C out of the sums
+    const bool uni = K.uniform_h != 0;
+    int ci[3];
+    cell_decode(G, cell_of[i], ci);
+    const PairI64 I = pair_i64(K, me.w);
+    // a neighbour j (0 < r < 2 h_ij) at rv = x_i - x_j, r2 = |rv|^2
+    auto body = [&](int j, const double* rv, double r2) {
+        const double inv_r = rsqrt_pos(r2);
+        const double r = r2 * inv_r;
+        double g;
+        if (uni) {
+            const double t = fma(-K.half_inv_h_u, r, 1.0);
+            g = t * t * t;
+        } else {
+            g = wendland_dW<DIM, double>(r, 1.0 / pair_h(K, hi, S.h[j])) * inv_r;
+        }
+        const double4_32a oj = vr[j];
+        const double vj[3] = {oj.x, oj.y, oj.z};
+        double w_j = oj.w, V_j = vol[j];
+        const bool wall = is_wall(w_j);
+        if (__any_sync(__activemask(), wall)) {
+            // a wall stands in with rho_j = rho_i: w_j = w_i, V_j = m_j / rho_i
+            if (wall) {
+                w_j = me.w;
+                V_j = S.m[j] / (K.rho0 + me.w);
+            }
+        }
+        pair_force64<DIM>(K, I, rv, inv_r, g, vi, vj, w_j, V_j, sums);
+    };
+    if (cnt <= cap) {
+        // the density pass's list: exactly the pairs with 0 < r < 2 h_ij
+        // (its exact FP64 test), in the order of the cell scan below, so
+        // no test is repeated here.  The stencil step of j's cell fixes
+        // the periodic image (the nearest one for every neighbour: the
+        // same operations as min_image).
+        for (int k = k0; k < cnt; k += dk) {
+            const uint32_t e = nbl[(size_t)k * n + i];
+            const int j = (int)(e >> kCodeBits);
+            const int code = (int)(e & ((1u << kCodeBits) - 1u));
+            const int step[3] = {code % kSide - kStencilR, (code / kSide) % kSide - kStencilR,
+                                 code / (kSide * kSide) - kStencilR};
+            double rv[3] = {0, 0, 0};
+            double r2 = 0.0;
+#pragma unroll
+            for (int d = 0; d < DIM; ++d) {
+                double t = __dsub_rn(xi[d], S.x[(size_t)d * n + j]);
+                if (G.periodic[d]) {
+                    const int sc = ci[d] + step[d];
+                    if (sc >= G.nc[d]) t = __dsub_rn(t, G.L[d]);
+                    else if (sc < 0) t = __dadd_rn(t, G.L[d]);
+                }
+                rv[d] = t;
+                r2 += t * t;
+            }
+            body(j, rv, r2);
+        }
+    } else if (k0 == 0) {
+        // no list (or more neighbours than it holds): scan the cells with
+        // the minimum image and the support test
+        const int SR = G.R, zr = DIM == 3 ? SR : 0;
+        for (int dz = -zr; dz <= zr; ++dz) {
+            int cz = DIM == 3 ? cell_step(G, ci[2], dz, 2) : 0;
+            if (cz < 0) continue;
+            for (int dy = -SR; dy <= SR; ++dy) {
+                int cy = cell_step(G, ci[1], dy, 1);
+                if (cy < 0) continue;
+                for (int dx = -SR; dx <= SR; ++dx) {
+                    int cx = cell_step(G, ci[0], dx, 0);
+                    if (cx < 0) continue;
+                    int cell = cx + G.nc[0] * (cy + G.nc[1] * cz);
+                    for (int j = start[cell]; j < start[cell + 1]; ++j) {
+                        if (j == i) continue;
+                        double rv[3] = {0, 0, 0};
+                        double r2 = 0.0;
+#pragma unroll
+                        for (int d = 0; d < DIM; ++d) {
+                            rv[d] = min_image(G, xi[d], S.x[(size_t)d * n + j], d);
+                            r2 += rv[d] * rv[d];
+                        }
+                        const double hij = uni ? K.h_u : pair_h(K, hi, S.h[j]);
+                        if (r2 > 4.0 * hij * hij * (1.0 + 1e-12)) continue;
+                        if (!(r2 > 0.0)) continue;
+                        if (!(sqrt(r2) < 2.0 * hij)) continue;
+                        body(j, rv, r2);
+                    }
+                }
+            }
+        }
+    }
+}
+
+// L lanes per particle (see Lanes): lane q of a group takes the neighbours
+// q, q + L, ...; their sums meet in shared memory, where one thread per
+// particle adds them in lane order and ends the particle's step.
+template <int DIM, int L>
+__global__ void __launch_bounds__(Lanes<L>::kThreads, L == 1 ? 2 : 1) k_forces_f64(int n, StateSet<double> S,
+                                                    const int32_t* __restrict__ start, Grid G, Consts<double> K,
+                                                    const double4_32a* __restrict__ vr,
+                                                    const int32_t* __restrict__ cell_of,
                                                     const uint32_t* __restrict__ nbl, const int32_t* __restrict__ nbc,
                                                     int cap, const double* dt_ptr, int kick_on,
                                                     int write_ad, double* __restrict__ Rout,
-                                                    double* __restrict__ chi_out, GridSum B, DtConsts D,
+                                                    double* __restrict__ chi_out, GridSum B, DtConsts Dc,
                                                     double* __restrict__ diag, double* dt_next, int count_step,
                                                     const double* __restrict__ vol)
 {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int P = blockDim.x / L;
+    PairSums64<DIM> sums;
+    if constexpr (L == 1) {
+        const int i = blockIdx.x * blockDim.x + threadIdx.x;
+        if (i < n && S.kind[i] == 0)
+            forces64_sums<DIM>(n, i, S, start, G, K, vr, cell_of, nbl, nbl ? nbc[i] : cap + 1, cap, 0, 1, vol, sums);
+    } else {
+        extern __shared__ __align__(16) unsigned char smem64[];
+        double* part = reinterpret_cast<double*>(smem64);       // [3 DIM][blockDim.x]
+        const int i = blockIdx.x * P + threadIdx.x / L;
+        if (i < n && S.kind[i] == 0)
+            forces64_sums<DIM>(n, i, S, start, G, K, vr, cell_of, nbl, nbc[i], cap, threadIdx.x % L, L, vol, sums);
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) {
+            part[(3 * d + 0) * blockDim.x + threadIdx.x] = sums.P[d];
+            part[(3 * d + 1) * blockDim.x + threadIdx.x] = sums.V[d];
+            part[(3 * d + 2) * blockDim.x + threadIdx.x] = sums.R[d];
+        }
+        __syncthreads();
+        sums = PairSums64<DIM>();
+        if (threadIdx.x < P) {
+#pragma unroll
+            for (int d = 0; d < DIM; ++d)
+                for (int q = 0; q < L; ++q) {
+                    sums.P[d] += part[(3 * d + 0) * blockDim.x + threadIdx.x * L + q];
+                    sums.V[d] += part[(3 * d + 1) * blockDim.x + threadIdx.x * L + q];
+                    sums.R[d] += part[(3 * d + 2) * blockDim.x + threadIdx.x * L + q];
+                }
+        }
+    }
+    // the end of the step, one thread per particle
+    const int i = blockIdx.x * P + threadIdx.x;
     double part[kNPart];
 #pragma unroll
     for (int k = 0; k < kNPart; ++k) part[k] = 0.0;
     const double dt = *dt_ptr;
     const double hdt = kick_on ? 0.5 * dt : 0.0;
-    if (i < n && S.kind[i] == 0) {
-        double xi[3] = {0, 0, 0}, vi[3] = {0, 0, 0};
-        double4_32a me = vr[i];
-        vi[0] = me.x; vi[1] = me.y; vi[2] = me.z;
+    if (threadIdx.x < P && i < n) {
+        if (S.kind[i] == 0) {
+            const double4_32a me = vr[i];
+            const double vi[3] = {me.x, me.y, me.z};
+            const double rho_i = K.rho0 + me.w;
+            const double inv_rho_i = 1.0 / rho_i;
+            const double hi = S.h[i];
+            // W'/r = C t^3 at uniform resolution, C = -5 a_D h^-(D+2): C leaves the sums
+            const double C = K.uniform_h ? K.dwr_coef_u : 1.0;
+            const double fp = (-2.0 * C) * inv_rho_i, fv = (K.two_eta * C) * inv_rho_i;
+            double a[3] = {0, 0, 0}, R[3] = {0, 0, 0};
+            double R2 = 0.0;
+            const double m_i = S.m[i];
+            // free-stream forcing lambda(x) (U_inf - v) of the fringe region
+            const double lam = K.fr_on ? fringe_rate<double>(K, S.x[i]) : 0.0;
 #pragma unroll
-        for (int d = 0; d < DIM; ++d) xi[d] = S.x[(size_t)d * n + i];
-        const double hi = S.h[i];
-        const double rho_i = K.rho0 + me.w;
-        const double inv_rho_i = 1.0 / rho_i;
-        PlainD acc_a[DIM], acc_R[DIM];
-        // uniform resolution: h_ij = h for every pair, so the support bounds
-        // and -5 a_D h^-(D+2) are constants
-        const bool uni = K.uniform_h != 0;
-        const double far_u = 4.0 * K.h_u * K.h_u * (1.0 + 1e-12), two_hu = 2.0 * K.h_u;
-        const double dwrnorm_u = -5.0 * kernel_norm<DIM, double>() * pow_dim<DIM, double>(K.inv_h_u) * K.inv_h_u *
-                                 K.inv_h_u;
-        // the cell of i (as the sort computed it from these positions)
-        const int ci[3] = {cell_coord(G, xi[0], 0), cell_coord(G, xi[1], 1), DIM == 3 ? cell_coord(G, xi[2], 2) : 0};
-        // W'/r = C t^3 at uniform resolution (t = 1 - r / 2h): C leaves the sums
-        const double C = uni ? dwrnorm_u : 1.0;
-        const double half_inv_h = 0.5 * K.inv_h_u;
-        const PairI64 I = pair_i64(K, me.w, inv_rho_i, C);
-        // a neighbour j (0 < r < 2 h_ij) at rv = x_i - x_j, r2 = |rv|^2
-        auto body = [&](int j, const double* rv, double r2) {
-            const double inv_r = rsqrt(r2);
-            const double r = r2 * inv_r;
-            double g;
-            if (uni) {
-                const double t = fma(-half_inv_h, r, 1.0);
-                g = t * t * t;
-            } else {
-                g = wendland_dW<DIM, double>(r, 1.0 / pair_h(K, hi, S.h[j])) * inv_r;
+            for (int d = 0; d < DIM; ++d) {
+                const double pair_a = fma(fp, sums.P[d], fv * sums.V[d]);
+                // the fluid's momentum rate from its pair terms: minus the force on the walls
+                if (K.body_force) part[9 + d] = m_i * pair_a;
+                a[d] = K.g[d] + pair_a;
+                if (K.fr_on) a[d] += lam * (K.fr_u[d] - vi[d]);
+                R[d] = C * sums.R[d];
+                R2 += R[d] * R[d];
             }
-            const double4_32a oj = vr[j];
-            const double vj[3] = {oj.x, oj.y, oj.z};
-            double w_j = oj.w, V_j = vol[j];
-            const bool wall = is_wall(w_j);
-            if (__any_sync(__activemask(), wall)) {
-                // a wall stands in with rho_j = rho_i: w_j = w_i, V_j = m_j / rho_i
-                if (wall) {
-                    w_j = me.w;
-                    V_j = S.m[j] * inv_rho_i;
-                }
-            }
-            pair_force64<DIM>(K, I, rv, inv_r, g, vi, vj, w_j, V_j, acc_a, acc_R);
-        };
-        const int cnt = nbl ? nbc[i] : cap + 1;
-        if (cnt <= cap) {
-            // the density pass's list: exactly the pairs with 0 < r < 2 h_ij
-            // (its exact FP64 test), in the order of the cell scan below, so
-            // no test is repeated here.  The stencil step of j's cell fixes
-            // the periodic image (the nearest one for every neighbour: the
-            // same operations as min_image).
-            for (int k = 0; k < cnt; ++k) {
-                const uint32_t e = nbl[(size_t)k * n + i];
-                const int j = (int)(e >> kCodeBits);
-                const int code = (int)(e & ((1u << kCodeBits) - 1u));
-                const int step[3] = {code % kSide - kStencilR, (code / kSide) % kSide - kStencilR,
-                                     code / (kSide * kSide) - kStencilR};
-                double rv[3] = {0, 0, 0};
-                double r2 = 0.0;
+            const double htv = K.tv_h_particle ? hi : K.h_min;
+            const double htv2 = htv * htv;
+            const double chi = tv_limiter(K, htv2 * R2);
+            // Eq. 12 (background pressure p0 = rho0 c^2): dr = dt^2/2 a_bg = -(dt^2 p0 / rho_i) R_i
+            const bool bgmode = K.tv_mode == SPH_TV_BACKGROUND;
+            const double bg = bgmode ? -(dt * dt * (K.rho0 * K.c2) / rho_i) : 0.0;
+            // 1/dt once per particle: the transport speed is a diagnostic
+            const double inv_dt = dt > 0.0 ? 1.0 / dt : 0.0;
+            double v2 = 0.0, vt2 = 0.0, dr2 = 0.0;
 #pragma unroll
-                for (int d = 0; d < DIM; ++d) {
-                    double t = __dsub_rn(xi[d], S.x[(size_t)d * n + j]);
-                    if (G.periodic[d]) {
-                        const int sc = ci[d] + step[d];
-                        if (sc >= G.nc[d]) t = __dsub_rn(t, G.L[d]);
-                        else if (sc < 0) t = __dadd_rn(t, G.L[d]);
-                    }
-                    rv[d] = t;
-                    r2 += t * t;
+            for (int d = 0; d < DIM; ++d) {
+                size_t o = (size_t)d * n + i;
+                double dr = bgmode ? bg * R[d] : K.tv_xi * chi * htv2 * R[d];
+                double vn = __dadd_rn(vi[d], __dmul_rn(hdt, a[d]));
+                if (write_ad) {
+                    S.a[o] = a[d];
+                    S.dr[o] = dr;
                 }
-                body(j, rv, r2);
+                S.v[o] = vn;
+                Rout[o] = R[d];
+                part[1 + d] = m_i * vn;
+                v2 += vn * vn;
+                dr2 += dr * dr;
+                const double vt = fma(dr, inv_dt, vn);
+                vt2 += vt * vt;
             }
+            chi_out[i] = chi;
+            part[0] = m_i;
+            part[4] = 0.5 * m_i * v2;
+            part[5] = chi > 0.0 ? 1.0 : 0.0;
+            part[6] = v2;                 // squares: the roots are taken at the very end
+            part[7] = vt2;
+            part[8] = dr2;
         } else {
-            // no list (or more neighbours than it holds): scan the cells with
-            // the minimum image and the support test
-            const int SR = G.R, zr = DIM == 3 ? SR : 0;
-            for (int dz = -zr; dz <= zr; ++dz) {
-                int cz = DIM == 3 ? cell_step(G, ci[2], dz, 2) : 0;
-                if (cz < 0) continue;
-                for (int dy = -SR; dy <= SR; ++dy) {
-                    int cy = cell_step(G, ci[1], dy, 1);
-                    if (cy < 0) continue;
-                    for (int dx = -SR; dx <= SR; ++dx) {
-                        int cx = cell_step(G, ci[0], dx, 0);
-                        if (cx < 0) continue;
-                        int cell = cx + G.nc[0] * (cy + G.nc[1] * cz);
-                        for (int j = start[cell]; j < start[cell + 1]; ++j) {
-                            if (j == i) continue;
-                            double rv[3] = {0, 0, 0};
-                            double r2 = 0.0;
 #pragma unroll
-                            for (int d = 0; d < DIM; ++d) {
-                                rv[d] = min_image(G, xi[d], S.x[(size_t)d * n + j], d);
-                                r2 += rv[d] * rv[d];
-                            }
-                            const double hij = uni ? K.h_u : pair_h(K, hi, S.h[j]);
-                            if (r2 > (uni ? far_u : 4.0 * hij * hij * (1.0 + 1e-12))) continue;
-                            if (!(r2 > 0.0)) continue;
-                            if (!(sqrt(r2) < (uni ? two_hu : 2.0 * hij))) continue;
-                            body(j, rv, r2);
-                        }
-                    }
+            for (int d = 0; d < DIM; ++d) {
+                if (write_ad) {
+                    S.a[(size_t)d * n + i] = 0.0;
+                    S.dr[(size_t)d * n + i] = 0.0;
                 }
+                Rout[(size_t)d * n + i] = 0.0;
             }
+            chi_out[i] = 0.0;
         }
-        double a[3] = {0, 0, 0}, R[3] = {0, 0, 0};
-        double R2 = 0.0;
-        const double m_i = S.m[i];
-        // free-stream forcing lambda(x) (U_inf - v) of the fringe region
-        const double lam = K.fr_on ? fringe_rate<double>(K, xi[0]) : 0.0;
-#pragma unroll
-        for (int d = 0; d < DIM; ++d) {
-            const double pair_a = acc_a[d].value();
-            // the fluid's momentum rate from its pair terms: minus the force on the walls
-            if (K.body_force) part[9 + d] = m_i * pair_a;
-            a[d] = K.g[d] + pair_a;
-            if (K.fr_on) a[d] += lam * (K.fr_u[d] - vi[d]);
-            R[d] = C * acc_R[d].value();
-            R2 += R[d] * R[d];
-        }
-        const double htv = K.tv_h_particle ? hi : K.h_min;
-        const double htv2 = htv * htv;
-        const double chi = tv_limiter(K, htv2 * R2);
-        // Eq. 12 (background pressure p0 = rho0 c^2): dr = dt^2/2 a_bg = -(dt^2 p0 / rho_i) R_i
-        const bool bgmode = K.tv_mode == SPH_TV_BACKGROUND;
-        const double bg = bgmode ? -(dt * dt * (K.rho0 * K.c2) / rho_i) : 0.0;
-        double v2 = 0.0, vt2 = 0.0, dr2 = 0.0;
-#pragma unroll
-        for (int d = 0; d < DIM; ++d) {
-            size_t o = (size_t)d * n + i;
-            double dr = bgmode ? bg * R[d] : K.tv_xi * chi * htv2 * R[d];
-            double vn = __dadd_rn(vi[d], __dmul_rn(hdt, a[d]));
-            if (write_ad) {
-                S.a[o] = a[d];
-                S.dr[o] = dr;
-            }
-            S.v[o] = vn;
-            Rout[o] = R[d];
-            part[1 + d] = m_i * vn;
-            v2 += vn * vn;
-            dr2 += dr * dr;
-            double vt = dt > 0.0 ? vn + dr / dt : vn;
-            vt2 += vt * vt;
-        }
-        chi_out[i] = chi;
-        part[0] = m_i;
-        part[4] = 0.5 * m_i * v2;
-        part[5] = chi > 0.0 ? 1.0 : 0.0;
-        part[6] = v2;                 // squares: block_partials takes the roots
-        part[7] = vt2;
-        part[8] = dr2;
-    } else if (i < n) {
-#pragma unroll
-        for (int d = 0; d < DIM; ++d) {
-            if (write_ad) {
-                S.a[(size_t)d * n + i] = 0.0;
-                S.dr[(size_t)d * n + i] = 0.0;
-            }
-            Rout[(size_t)d * n + i] = 0.0;
-        }
-        chi_out[i] = 0.0;
     }
     __shared__ double total[kNPart];
-    if (grid_partials(part, B, total, true, K.body_force != 0)) finish_step(total, D, diag, dt_next, count_step);
+    if (grid_partials(part, B, total, true, K.body_force != 0)) finish_step(total, Dc, diag, dt_next, count_step);
 }
 
 // ================================================ diagnostics only
@@ -417,15 +704,36 @@ static inline int nblk(int n, int t) { return (n + t - 1) / t; }
 // Threads per block of the pair passes: 256 (FP64) or 128 (FP32) when the
 // particles fill every SM at that size; smaller blocks (down to one warp)
 // when they do not, so that a small problem still spreads over all SMs
-// instead of queueing its FP64 work on a few.
+// instead of queueing its FP64 work on a few.  FP64 between one and eight
+// full blocks per SM: 64, since the FP64 pipe is the bound and a pass takes
+// as long as the SM with the most blocks (40,000 particles: 157 blocks of 256
+// on 152 SMs, 208 us a step against 151 with 64; 64,000 in 3-D: 889 against
+// 809 us; 96^3: the same).
 int pair_threads(int prec, int n, int sms)
 {
     const int full = prec == 64 ? 256 : 128;
     if (sms <= 0) sms = 152;
-    if ((int64_t)n >= (int64_t)sms * full) return full;
+    if ((int64_t)n >= (int64_t)sms * full) return prec == 64 && (int64_t)n < (int64_t)sms * full * 8 ? 64 : full;
     int t = ((n + sms - 1) / sms + 31) / 32 * 32;
     return t < 32 ? 32 : (t > full ? full : t);
 }
+
+// The FP64 pair passes with neighbour lists: lanes per particle (see Lanes),
+// threads per block and blocks.
+struct Lane64 {
+    int L, T, blocks;
+};
+
+static Lane64 lanes64(int dim, int n, int sms)
+{
+    if (sms <= 0) sms = 152;
+    const int L = n >= sms * 256 ? 1 : (n >= sms * 64 ? 4 : (dim == 2 || n >= sms * 16 ? 8 : 16));
+    const int T = L == 1 ? pair_threads(64, n, sms) : lane_threads(L, n, sms);
+    return Lane64{L, T, nblk(n, T / L)};
+}
+
+#define SPH_LANES64(kernel, DIM, L) \
+    ((L) == 1 ? kernel<DIM, 1> : (L) == 4 ? kernel<DIM, 4> : (L) == 8 ? kernel<DIM, 8> : kernel<DIM, 16>)
 
 int pair_blocks(int prec, int n, int sms) { return nblk(n, pair_threads(prec, n, sms)); }
 
@@ -449,17 +757,15 @@ cudaError_t launch_density(int prec, int dim, int n, void* S, const int32_t* sta
                            void* vr, const float4* pos4, const int32_t* cell_of, uint32_t* nbl, int32_t* nbc,
                            cudaStream_t st, double* vol, const float4* pos4c, int tiles)
 {
-    const int T = pair_threads(prec, n, G.sms);
     if (prec == 32) return launch_density32(dim, n, S, start, G, K, vr, pos4, cell_of, nbl, nbc, st, pos4c, tiles);
     auto s = *(StateSet<double>*)S;
     auto k = *(const Consts<double>*)K;
     const int cap = nbl_capacity(dim);
-    if (dim == 2)
-        k_density_f64<2><<<nblk(n, T), T, 0, st>>>(n, s, start, G, k, (double4_32a*)vr, pos4, cell_of, nbl, nbc, cap,
-                                                   vol);
-    else
-        k_density_f64<3><<<nblk(n, T), T, 0, st>>>(n, s, start, G, k, (double4_32a*)vr, pos4, cell_of, nbl, nbc, cap,
-                                                   vol);
+    const Lane64 Q = nbl ? lanes64(dim, n, G.sms) : Lane64{1, pair_threads(64, n, G.sms), nblk(n, pair_threads(64, n, G.sms))};
+    const size_t smem = Q.L == 1 ? 0 : ((size_t)(Q.T / Q.L) * (dim == 3 ? kSide * kSide : kSide) * sizeof(RowRuns) + 15) / 16 * 16 +
+                                           Q.T * sizeof(double);
+    auto kern = dim == 2 ? SPH_LANES64(k_density_f64, 2, Q.L) : SPH_LANES64(k_density_f64, 3, Q.L);
+    kern<<<Q.blocks, Q.T, smem, st>>>(n, s, start, G, k, (double4_32a*)vr, pos4, cell_of, nbl, nbc, cap, vol);
     return cudaGetLastError();
 }
 
@@ -468,28 +774,25 @@ cudaError_t launch_forces(int prec, int dim, int n, void* S, const int32_t* star
                           const uint32_t* nbl, const int32_t* nbc, int kick_on, int write_ad,
                           void* Rout, void* chi, const FinishArgs& F, cudaStream_t st, const double* vol)
 {
-    const int T = pair_threads(prec, n, G.sms);
     if (prec == 32)
         return launch_forces32(dim, n, S, start, G, K, mf, vr, pos4, cell_of, nbl, nbc, kick_on, write_ad, Rout, chi,
                                F, st);
     auto s = *(StateSet<double>*)S;
     auto k = *(const Consts<double>*)K;
     const int cap = nbl_capacity(dim);
-    const GridSum B = grid_sum(F, nblk(n, T));
+    const Lane64 Q = lanes64(dim, n, G.sms);
+    const GridSum B = grid_sum(F, Q.blocks);
     const DtConsts D = dt_consts(*F.P);
-    if (dim == 2)
-        k_forces_f64<2><<<nblk(n, T), T, 0, st>>>(n, s, start, G, k, (const double4_32a*)vr, nbl, nbc, cap, F.dt,
-                                                  kick_on, write_ad, (double*)Rout, (double*)chi, B, D, F.diag, F.dt,
-                                                  F.count_step, vol);
-    else
-        k_forces_f64<3><<<nblk(n, T), T, 0, st>>>(n, s, start, G, k, (const double4_32a*)vr, nbl, nbc, cap, F.dt,
-                                                  kick_on, write_ad, (double*)Rout, (double*)chi, B, D, F.diag, F.dt,
-                                                  F.count_step, vol);
+    const size_t smem = Q.L == 1 ? 0 : (size_t)3 * dim * Q.T * sizeof(double);
+    auto kern = dim == 2 ? SPH_LANES64(k_forces_f64, 2, Q.L) : SPH_LANES64(k_forces_f64, 3, Q.L);
+    kern<<<Q.blocks, Q.T, smem, st>>>(n, s, start, G, k, (const double4_32a*)vr, cell_of, nbl, nbc, cap, F.dt, kick_on,
+                                      write_ad, (double*)Rout, (double*)chi, B, D, F.diag, F.dt, F.count_step, vol);
     return cudaGetLastError();
 }
 
 cudaError_t launch_finish_step(int prec, int n, int sms, const FinishArgs& F, cudaStream_t st, int64_t* launches)
 {
+    // (the FP64 passes of more than kInlineBlocks blocks have one lane per particle)
     const int nb = pair_blocks(prec, n, sms);
     const GridSum B = grid_sum(F, nb);
     if (B.group) return cudaSuccess;      // the pass folded its partials itself

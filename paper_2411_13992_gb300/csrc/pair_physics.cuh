@@ -33,29 +33,63 @@ __device__ __forceinline__ Real tv_limiter(const Consts<Real>& K, Real s)
     return Real(0);
 }
 
+// 1/sqrt(x) and sqrt(x) for a normal x > 0 in six FP64 operations: the
+// hardware's approximation y0 (its upper word only), then one step of
+// Householder's third-order iteration for x^(-1/2), y0 (1 + e/2 + 3 e^2/8)
+// with e = 1 - x y0^2.  The error left by the iteration is O(e^3) < 2^-58, so
+// that both results are within one rounding of the exact values.
+__device__ __forceinline__ double rsqrt_seed(double x)
+{
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    return y;
+}
+
+__device__ __forceinline__ double sqrt_pos(double x)
+{
+    const double y0 = rsqrt_seed(x);
+    const double g = x * y0;
+    const double e = fma(-g, y0, 1.0);
+    return fma(g * e, fma(0.375, e, 0.5), g);
+}
+
+__device__ __forceinline__ double rsqrt_pos(double x)
+{
+    const double y0 = rsqrt_seed(x);
+    const double e = fma(-(x * y0), y0, 1.0);
+    return fma(y0 * e, fma(0.375, e, 0.5), y0);
+}
+
 // Per-particle values of i shared by all pairs of i in the FP64 force pass.
-// C is a constant factor of W'/r that the pass takes out of the pair sums
-// (-5 a_D h^-(D+2) at uniform resolution, where W'/r = C t^3; else 1).
 struct PairI64 {
     double w;          // rho_i - rho0
-    double inv_rho;    // 1 / rho_i
     double hp;         // p_i / 2 = (c^2 / 2) w_i
     double crho;       // (c/2)(rho0 + w_i / 2): (c/2) rho_bar = crho + (c/4) w_j
-    double m2_ir;      // -2 C / rho_i
-    double eta_ir;     // 2 eta C / rho_i
 };
 
-__device__ __forceinline__ PairI64 pair_i64(const Consts<double>& K, double w, double inv_rho, double C)
+__device__ __forceinline__ PairI64 pair_i64(const Consts<double>& K, double w)
 {
     PairI64 I;
     I.w = w;
-    I.inv_rho = inv_rho;
-    I.hp = (0.5 * K.c2) * w;
-    I.crho = (0.5 * K.c) * (K.rho0 + 0.5 * w);
-    I.m2_ir = (-2.0 * C) * inv_rho;
-    I.eta_ir = (K.two_eta * C) * inv_rho;
+    I.hp = K.half_c2 * w;
+    I.crho = K.half_c * fma(0.5, w, K.rho0);
     return I;
 }
+
+// The pair sums of particle i in the FP64 force pass, without the factors
+// that all pairs of i share: P = sum V_j g P*_ij r_ij, V = sum V_j g v_ij,
+// R = sum V_j g r_ij, where W'/r = C g (C a constant of the particle's
+// resolution, 1 at variable resolution).  Then a_i = -2 C / rho_i P + 2 eta C
+// / rho_i V and R_i = C R.
+template <int DIM>
+struct PairSums64 {
+    double P[DIM], V[DIM], R[DIM];
+    __device__ __forceinline__ PairSums64()
+    {
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) P[d] = V[d] = R[d] = 0.0;
+    }
+};
 
 // min(max(x, 0), 1) by the sign and order of the binary64 bit pattern (the
 // order of non-negative doubles is that of their patterns): integer selects
@@ -75,19 +109,19 @@ __device__ __forceinline__ bool is_wall(double w)
     return (__double_as_longlong(w) & 0x7fffffffffffffffLL) == 0x7ff0000000000000LL;
 }
 
-// Contribution of neighbour j to a_i and R_i in the FP64 form: Eq. 3
+// Contribution of neighbour j to the sums of i in the FP64 form: Eq. 3
 // (pressure, with P* of Eq. 5-6), Eq. 7 (viscous) and the residual of
 // Eq. 14, arranged for the FP64 pipe (1/74 of the FP32 rate here): P* from
 // the density deviations (p_i + p_j = c^2 (w_i + w_j), rho_bar = rho0 +
-// (w_i + w_j)/2), the limiter's clamp on the integer ALU, and one product
-// V_j g that the pressure, viscous and residual terms share.  rv = x_i -
-// x_j, inv_r = 1/r, g = W'(r, h_ij) / (r C); w_j = rho_j - rho0 and V_j =
-// m_j / rho_j, for a wall neighbour w_i and m_j / rho_i (the caller
-// substitutes them).  acc_R collects R_i / C.
+// (w_i + w_j)/2), the limiter's clamp on the integer ALU, one product V_j g
+// that the three sums share, and every factor of i alone out of the pair
+// (39 FP64 operations in 3-D).  rv = x_i - x_j, inv_r = 1/r, g = W'(r, h_ij)
+// / (r C); w_j = rho_j - rho0 and V_j = m_j / rho_j, for a wall neighbour w_i
+// and m_j / rho_i (the caller substitutes them).
 template <int DIM>
 __device__ __forceinline__ void pair_force64(const Consts<double>& K, const PairI64& I, const double* rv,
                                              double inv_r, double g, const double* vi, const double* vj,
-                                             double w_j, double V_j, PlainD* acc_a, PlainD* acc_R)
+                                             double w_j, double V_j, PairSums64<DIM>& S)
 {
     double dv[3] = {0.0, 0.0, 0.0};
     double dvr = 0.0;
@@ -97,18 +131,17 @@ __device__ __forceinline__ void pair_force64(const Consts<double>& K, const Pair
         dvr += dv[d] * rv[d];
     }
     const double du = -dvr * inv_r;                                   // U_l - U_r
-    const double beta = clamp01((K.beta_slope * K.inv_c) * du);
-    const double hpsum = fma(0.5 * K.c2, w_j, I.hp);                   // (p_i + p_j) / 2
-    const double crhobar = fma(0.25 * K.c, w_j, I.crho);               // (c/2) rho_bar
+    const double beta = clamp01(K.beta_k * du);
+    const double hpsum = fma(K.half_c2, w_j, I.hp);                   // (p_i + p_j) / 2
+    const double crhobar = fma(K.quarter_c, w_j, I.crho);               // (c/2) rho_bar
     const double pstar = fma(beta * du, crhobar, hpsum);
     const double vw = V_j * g;                                        // V_j W'/(r C)
-    const double cpw = I.m2_ir * (vw * pstar);                        // -2 m_j P* / (rho_i rho_j) W'/r
-    const double cv = I.eta_ir * vw;                                  // 2 eta m_j / (rho_i rho_j) W'/r
+    const double vwp = vw * pstar;
 #pragma unroll
     for (int d = 0; d < DIM; ++d) {
-        acc_a[d].s = fma(cpw, rv[d], acc_a[d].s);
-        acc_a[d].s = fma(cv, dv[d], acc_a[d].s);
-        acc_R[d].s = fma(vw, rv[d], acc_R[d].s);
+        S.P[d] = fma(vwp, rv[d], S.P[d]);
+        S.V[d] = fma(vw, dv[d], S.V[d]);
+        S.R[d] = fma(vw, rv[d], S.R[d]);
     }
 }
 
@@ -144,15 +177,16 @@ __device__ __forceinline__ Real fringe_rate(const Consts<Real>& K, Real x)
 // integer maxima of their bit patterns (a NaN counts as 0, as fmax ignores
 // it), which keeps both off the FP64 pipe (1/74 of the FP32 rate on this
 // part).  sums = false (the same for every thread of the grid) when the
-// caller's sums are all zero: they are skipped.
-constexpr int kMaxWarps = 8;         // warps of a block of any pass that writes partials
+// caller's sums are all zero: they are skipped, as in a warp without mass.
+constexpr int kMaxWarps = 16;         // warps of a block of any pass that writes partials
 
 __device__ __forceinline__ void block_partials(double* vals, double* out_block, bool sums = true, bool body = false)
 {
     __shared__ double sh[kMaxWarps][kNPart];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    if (!sums) {
-        // the caller's sums are all zero (uniform over the grid): skip them
+    // slot 0 is a mass: a warp in which it is zero everywhere holds no fluid particle
+    if (!sums || !__any_sync(0xffffffffu, __double_as_longlong(vals[0]) != 0)) {
+        // the caller's sums are all zero: skip them
         if (lane == 0)
             for (int k = 0; k < 5; ++k) sh[w][k] = 0.0;
     } else {

@@ -282,7 +282,17 @@ Consts<Real> make_consts(const sph_params* p)
         const double pi = 3.14159265358979323846;
         const double norm = p->dim == 2 ? 7.0 / (4.0 * pi) : 21.0 / (16.0 * pi);
         K.dwr_coef_u = (Real)(-5.0 * norm * std::pow(1.0 / p->h_max, p->dim + 2));
+        K.w_norm_u = (Real)(norm * std::pow(1.0 / p->h_max, p->dim));
     }
+    K.half_c2 = (Real)(0.5 * c2);
+    K.half_c = (Real)(0.5 * p->c0);
+    K.quarter_c = (Real)(0.25 * p->c0);
+    K.beta_k = (Real)(p->riemann_eta / p->c0);
+    K.two_h_u = (Real)(2.0 * p->h_max);
+    K.half_inv_h_u = (Real)(0.5 / p->h_max);
+    K.two_inv_h_u = (Real)(2.0 / p->h_max);
+    K.reach_u = (float)(2.0 * p->h_max);
+    K.prefilter2_u = K.reach_u * K.reach_u * 1.0001f;
     return K;
 }
 
@@ -335,8 +345,9 @@ size_t carve(sph_ctx* c, char* base)
     c->du = dual ? W.take<double>(DU_COUNT) : nullptr;
     c->R = c->density_only ? nullptr : W.take<char>(D * n * rs);
     c->chi = c->density_only ? nullptr : W.take<char>(n * rs);
-    // one partials row per block of a pair pass; blocks are never smaller than a warp
-    c->partials = W.take<double>(((size_t)n + 31) / 32 * kNPart);
+    // one partials row per block of a pair pass: blocks hold 32 particles or
+    // more, or (several lanes per particle) there is at most one per SM
+    c->partials = W.take<double>((((size_t)n + 31) / 32 + 1024) * kNPart);
     c->rows = W.take<double>((size_t)grid_groups() * kNPart);
     c->counters = W.take<unsigned>((size_t)grid_groups() + 1);
     c->diag = W.take<double>(DG_COUNT);
