@@ -170,6 +170,16 @@ struct KSum {
     __device__ __forceinline__ float value() const { return s; }
 };
 
+// Compensated partial sums combined exactly: (s, c) holds s - c.
+__device__ __forceinline__ void ksum_merge(float& s, float& c, float s2, float c2)
+{
+    const float t = __fadd_rn(s, s2);
+    const float bb = __fsub_rn(t, s);
+    const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bb)), __fsub_rn(s2, bb));   // s + s2 = t + e exactly
+    c = __fsub_rn(__fadd_rn(c, c2), e);
+    s = t;
+}
+
 struct PlainF {
     float s;
     __device__ __forceinline__ PlainF() : s(0.f) {}

@@ -16,6 +16,13 @@
 //                   the reverse of the drift and the opening kick; its first
 //                   block adds the step's d/d(eta) (fixed-order reduction)
 //
+// Both walks run over the neighbour list that the step's density pass left in
+// the tape (the FP64 form scanned the 5^D cells with its exact test before:
+// 570 and 176 us per reverse step of 4,096 particles), and in the FP64 form
+// with a group of L lanes per particle (adj_lanes64 below), since one thread's
+// chain of FP64 operations is the bound of a problem of some thousand
+// particles.
+//
 // Subgradients: d beta/d dU = eta_R / c inside 0 < eta_R dU / c < 1, else 0
 // (Eq. 6); d chi/d s = C inside thresh < s < 1/C, else 0 (Eq. 15).
 #include <type_traits>
@@ -29,6 +36,33 @@ namespace sphtv {
 
 template <typename Real>
 using AccOf = typename std::conditional<sizeof(Real) == 4, KSum, PlainD>::type;
+
+// Sum of a group's accumulators, in every lane of the group (a fixed tree).
+template <int L>
+__device__ __forceinline__ void group_sum(KSum& a)
+{
+#pragma unroll
+    for (int o = L / 2; o >= 1; o >>= 1) {
+        const float s2 = __shfl_xor_sync(0xffffffffu, a.s, o);
+        const float c2 = __shfl_xor_sync(0xffffffffu, a.c, o);
+        ksum_merge(a.s, a.c, s2, c2);
+    }
+    if (L > 1) {
+        a.s = __fsub_rn(a.s, a.c);
+        a.c = 0.f;
+    }
+}
+
+template <int L>
+__device__ __forceinline__ void group_sum(PlainD& a)
+{
+#pragma unroll
+    for (int o = L / 2; o >= 1; o >>= 1) a.s += __shfl_xor_sync(0xffffffffu, a.s, o);
+}
+
+// A compensated sum as a double keeps its compensation: s - c.
+__device__ __forceinline__ double wide_value(const KSum& a) { return (double)a.s - (double)a.c; }
+__device__ __forceinline__ double wide_value(const PlainD& a) { return a.s; }
 
 // The cotangents Abar_k and Rbar_k of a particle as one record of
 // kAbStride<DIM> values ({Abar, Rbar}, padded to a whole number of 16-byte
@@ -70,41 +104,46 @@ struct Tape {
     const Real* R;         // [DIM][n] residual
     const int32_t* start;  // cell ranges
     const float4* pos4;    // FP32 form: cell-relative positions
-    const int32_t* cell;   // FP32 form: cell of each particle
+    const int32_t* cell;   // cell of each particle
     const double* dt;      // step size of the step
-    const uint32_t* nbl;   // FP32 form: the step's force-neighbour list (transposed), or null
+    const uint32_t* nbl;   // the step's force-neighbour list (transposed)
     const int32_t* nbc;    // and its counts
 };
 
 // Visit the neighbours j != k of particle k with 0 < r < 2 h_kj, decided
-// exactly as the forward pass decided them: f(j, rv[3] = x_k - x_j, r, 1/r)
-// (FP32 form: 1/r from rsqrt and r = r^2/r, as the forward force pass takes
-// them; FP64 form: r = sqrt(r^2), 1/r = 1/r).
-template <typename Real, int DIM, typename F>
-__device__ __forceinline__ void adj_visit(int n, int k, const Grid& G, const Consts<Real>& K, const Tape<Real>& T,
-                                          F& f)
+// exactly as the forward pass decided them: f(j, rv[3] = x_k - x_j, r, 1/r,
+// w_j) with w_j = pos4[j].w (FP32 form: m_j at uniform resolution, else h_j).
+// Lane q of a group of L takes the list's entries q, q + L, ...; a particle
+// with more neighbours than the list holds is walked over its cells by lane 0.
+// FP32 form: 1/r from rsqrt and r = r^2/r, as the forward force pass takes
+// them; FP64 form: 1/r within one rounding, r = r^2 (1/r).
+template <typename Real, int DIM, int L, typename F>
+__device__ __forceinline__ void adj_visit(int n, int k, int q, const Grid& G, const Consts<Real>& K,
+                                          const Tape<Real>& T, F& f)
 {
+    const int cnt = T.nbc[k];
+    const bool listed = cnt <= list_capacity(DIM);
     if constexpr (sizeof(Real) == 4) {
         const float4 pk = T.pos4[k];
         const float ok[3] = {pk.x, pk.y, pk.z};
-        const int cnt = T.nbl ? T.nbc[k] : 0;
-        if (T.nbl && cnt <= list_capacity(DIM)) {
-            // FP32 form: the forward density pass's list of the step, which
-            // holds exactly the pairs its walk accepted, in the walk's order;
-            // the pair vector and r^2 with the walk's arithmetic
+        if (listed) {
+            // the list holds exactly the pairs the density pass's walk
+            // accepted, in the walk's order; the pair vector and r^2 with the
+            // walk's arithmetic
             const float ex = G.edgef[0], ey = G.edgef[1], ez = G.edgef[2];
-            // the entry two ahead and the neighbour's position one ahead in flight
-            const uint32_t* lp = T.nbl + k;
-            uint32_t e_n = cnt > 0 ? lp[0] : 0u;
-            uint32_t e_nn = cnt > 1 ? lp[n] : 0u;
+            // the lane's entry two ahead and the neighbour's position one ahead in flight
+            const size_t row = (size_t)L * n;
+            const uint32_t* lp = T.nbl + k + (size_t)q * n;
+            uint32_t e_n = q < cnt ? lp[0] : 0u;
+            uint32_t e_nn = q + L < cnt ? lp[row] : 0u;
             float4 p_n = T.pos4[e_n >> kCodeBits];
-            lp += 2 * (size_t)n;
-            for (int q = 0; q < cnt; ++q, lp += n) {
+            lp += 2 * row;
+            for (int t = q; t < cnt; t += L, lp += row) {
                 const uint32_t e = e_n;
                 const float4 pj = p_n;
                 e_n = e_nn;
-                if (q + 1 < cnt) p_n = T.pos4[e_n >> kCodeBits];
-                e_nn = q + 2 < cnt ? *lp : 0u;
+                if (t + L < cnt) p_n = T.pos4[e_n >> kCodeBits];
+                e_nn = t + 2 * L < cnt ? *lp : 0u;
                 const int j = (int)(e >> kCodeBits);
                 const uint32_t code = e & ((1u << kCodeBits) - 1u);
                 const int dx = (int)(code % kSide) - kStencilR, dy = (int)((code / kSide) % kSide) - kStencilR,
@@ -121,35 +160,65 @@ __device__ __forceinline__ void adj_visit(int n, int k, const Grid& G, const Con
                 }
                 const Real rv[3] = {rxy.x, rxy.y, rz};
                 const float inv_r = rsqrtf(r2);
-                f(j, rv, r2 * inv_r, inv_r);
+                f(j, rv, r2 * inv_r, inv_r, pj.w);
             }
             return;
         }
-        // more neighbours than the list holds (or no list): the clipped row
-        // walk of the forward density pass, with its arithmetic for r^2, so
-        // the pairs are exactly the forward's (same order as the cell scan
-        // below)
+        if (q) return;
+        // the clipped row walk of the forward density pass, with its
+        // arithmetic for r^2, so the pairs are exactly the forward's
         const float hk = (float)T.h[k];
         const float reach = K.uniform_h ? 2.f * K.h_u : 2.f * pair_h(K, hk, K.h_u);
-        auto g = [&](int j, uint32_t, const float4&, float r2, float rx, float ry, float rz) {
+        auto g = [&](int j, uint32_t, const float4& pj, float r2, float rx, float ry, float rz) {
             float lim;
             if (K.uniform_h) lim = K.four_h2_u;
             else {
-                const float hh = pair_h(K, hk, (float)T.h[j]);
+                const float hh = pair_h(K, hk, pj.w);
                 lim = 4.f * hh * hh;
             }
             if (!(r2 < lim) || !(r2 > 0.f)) return;
             const Real rv[3] = {rx, ry, rz};
             const float inv_r = rsqrtf(r2);
-            f(j, rv, r2 * inv_r, inv_r);
+            f(j, rv, r2 * inv_r, inv_r, pj.w);
         };
         for_candidates_rows<DIM, false>(ok, reach, T.cell[k], G, T.start, T.cell, T.pos4, g);
     } else {
-        // FP64 form: the exact test of the forward pass (minimum image,
+        double xk[3] = {0, 0, 0};
+#pragma unroll
+        for (int d = 0; d < DIM; ++d) xk[d] = T.x[(size_t)d * n + k];
+        int c[3];
+        cell_decode(G, T.cell[k], c);
+        if (listed) {
+            // the list of the density pass's exact test; the stencil step of
+            // j's cell fixes the periodic image
+            for (int t = q; t < cnt; t += L) {
+                const uint32_t e = T.nbl[(size_t)t * n + k];
+                const int j = (int)(e >> kCodeBits);
+                const int code = (int)(e & ((1u << kCodeBits) - 1u));
+                const int step[3] = {code % kSide - kStencilR, (code / kSide) % kSide - kStencilR,
+                                     code / (kSide * kSide) - kStencilR};
+                Real rv[3] = {0, 0, 0};
+                double r2 = 0.0;
+#pragma unroll
+                for (int d = 0; d < DIM; ++d) {
+                    double y = __dsub_rn(xk[d], T.x[(size_t)d * n + j]);
+                    if (G.periodic[d]) {
+                        const int sc = c[d] + step[d];
+                        if (sc >= G.nc[d]) y = __dsub_rn(y, G.L[d]);
+                        else if (sc < 0) y = __dadd_rn(y, G.L[d]);
+                    }
+                    rv[d] = y;
+                    r2 += y * y;
+                }
+                const double inv_r = rsqrt_pos(r2);
+                f(j, rv, r2 * inv_r, inv_r, 0.f);
+            }
+            return;
+        }
+        if (q) return;
+        // the exact test of the forward pass over the cells (minimum image,
         // sqrt(r^2) < 2 h_kj)
         const int SR = G.R, zr = DIM == 3 ? SR : 0;
-        int c[3];
-        for (int d = 0; d < 3; ++d) c[d] = d < DIM ? cell_coord(G, T.x[(size_t)d * n + k], d) : 0;
         for (int dz = -zr; dz <= zr; ++dz) {
             int cz = DIM == 3 ? cell_step(G, c[2], dz, 2) : 0;
             if (cz < 0) continue;
@@ -165,13 +234,13 @@ __device__ __forceinline__ void adj_visit(int n, int k, const Grid& G, const Con
                         Real rv[3] = {0, 0, 0};
                         double r2 = 0.0;
                         for (int d = 0; d < DIM; ++d) {
-                            rv[d] = min_image(G, T.x[(size_t)d * n + k], T.x[(size_t)d * n + j], d);
+                            rv[d] = min_image(G, xk[d], T.x[(size_t)d * n + j], d);
                             r2 += rv[d] * rv[d];
                         }
                         const double r = sqrt(r2);
                         const double hij = pair_h(K, T.h[k], T.h[j]);
                         if (!(r < 2.0 * hij) || r == 0.0) continue;
-                        f(j, rv, (Real)r, Real(1) / (Real)r);
+                        f(j, rv, (Real)r, Real(1) / (Real)r, 0.f);
                     }
                 }
             }
@@ -241,15 +310,37 @@ __device__ __forceinline__ void pair_adjoint(const Consts<Real>& K, const Real* 
 __device__ __forceinline__ float recip(float x) { return rcp_approx(x); }
 __device__ __forceinline__ double recip(double x) { return 1.0 / x; }
 
-template <typename Real>
-__device__ __forceinline__ Real inv_pair_h(const Consts<Real>& K, const Tape<Real>& T, int k, int j)
+// W'(r) and W''(r) of the pair (k, j); w_j = pos4[j].w of the FP32 form (h_j
+// at variable resolution).  The FP64 form at uniform resolution takes them
+// from the constant C = -5 a_D h^-(D+2): W' = C r t^3 and W'' = C t^2 (1 - 2q)
+// with t = 1 - q/2.
+template <typename Real, int DIM>
+__device__ __forceinline__ void pair_kernels(const Consts<Real>& K, const Tape<Real>& T, int k, int j, Real hk,
+                                             float w_j, Real r, Real& w, Real& w2)
 {
+    Real inv_h;
     if constexpr (sizeof(Real) == 4) {
-        if (K.uniform_h) return K.inv_h_u;
-        return 1.f / pair_h(K, (float)T.h[k], (float)T.h[j]);
+        inv_h = K.uniform_h ? K.inv_h_u : 1.f / pair_h(K, hk, w_j);
     } else {
-        return 1.0 / pair_h(K, T.h[k], T.h[j]);
+        if (K.uniform_h) {
+            const double t = fma(-K.half_inv_h_u, r, 1.0), t2 = t * t;
+            w = K.dwr_coef_u * r * (t2 * t);
+            w2 = K.dwr_coef_u * t2 * fma(-K.two_inv_h_u, r, 1.0);
+            return;
+        }
+        inv_h = 1.0 / pair_h(K, hk, T.h[j]);
     }
+    w = wendland_dW<DIM, Real>(r, inv_h);
+    w2 = wendland_d2W<DIM, Real>(r, inv_h);
+}
+
+template <typename Real>
+__device__ __forceinline__ Real mass_of(const Consts<Real>& K, const Tape<Real>& T, int j, float w_j)
+{
+    // at uniform resolution the position record of the FP32 form holds the
+    // same FP32 mass (a conversion fewer on the FP64 pipe per pair)
+    if constexpr (sizeof(Real) == 4) return K.uniform_h ? w_j : (float)T.m[j];
+    else return T.m[j];
 }
 
 // ------------------------------------------------------------------- prep
@@ -290,32 +381,31 @@ __global__ void __launch_bounds__(256) k_adj_prep(int n, Tape<Real> T, Consts<Re
 
 // ------------------------------------------------------------------ pairs
 
-template <typename Real, int DIM>
-__global__ void __launch_bounds__(128) k_adj_pairs(int n, Tape<Real> T, Grid G, Consts<Real> K,
+constexpr int kAdjTPB = 128;
+
+template <typename Real, int DIM, int L>
+__global__ void __launch_bounds__(kAdjTPB) k_adj_pairs(int n, Tape<Real> T, Grid G, Consts<Real> K,
                                                    const Real* __restrict__ AR,
                                                    Real* __restrict__ xbp, Real* __restrict__ vbp,
                                                    Real* __restrict__ sigb, double* __restrict__ partials)
 {
     using Acc = AccOf<Real>;
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    double part[kNPart];
-#pragma unroll
-    for (int q = 0; q < kNPart; ++q) part[q] = 0.0;
-    if (k < n && !T.kind[k]) {
+    const int k = (blockIdx.x * blockDim.x + threadIdx.x) / L, q = threadIdx.x % L;
+    const bool fluid = k < n && !T.kind[k];
+    Acc ax[DIM], av[DIM], arho, aeta;
+    if (fluid) {
         const auto mk = T.vr[k];
         const Real vk[3] = {mk.x, mk.y, mk.z};
         const Real rho_k = K.rho0 + mk.w;
         const Real p_k = K.c2 * mk.w;
         const Real inv_rho_k = Real(1) / rho_k;
         const Real m_k = (Real)T.m[k];
+        const Real h_k = K.uniform_h ? K.h_u : (Real)T.h[k];
         Real Ak[3] = {0, 0, 0}, Rk[3] = {0, 0, 0};
         load_ab<Real, DIM>(AR, k, Ak, Rk);
-        Acc ax[DIM], av[DIM], arho;
-        double eta_acc = 0.0;
-        auto pair = [&](int j, const Real* rv, Real r, Real inv_r) {
-            const Real inv_h = inv_pair_h(K, T, k, j);
-            const Real w = wendland_dW<DIM, Real>(r, inv_h);
-            const Real w2 = wendland_d2W<DIM, Real>(r, inv_h);
+        auto pair = [&](int j, const Real* rv, Real r, Real inv_r, float w_j) {
+            Real w, w2;
+            pair_kernels<Real, DIM>(K, T, k, j, h_k, w_j, r, w, w2);
             const auto mj = T.vr[j];
             const Real vj[3] = {mj.x, mj.y, mj.z};
             const bool wall = isinf(mj.w);
@@ -325,13 +415,13 @@ __global__ void __launch_bounds__(128) k_adj_pairs(int n, Tape<Real> T, Grid G, 
             Real rb[3], dvb[3], rib, rjb, eb;
             // k's own sums (k as i)
             pair_adjoint<Real, DIM>(K, rv, r, inv_r, w, w2, vk, rho_k, inv_rho_k, p_k, vj, rho_j, inv_rho_j, p_j,
-                                    (Real)T.m[j], Ak, Rk, rb, dvb, rib, rjb, eb);
+                                    mass_of(K, T, j, w_j), Ak, Rk, rb, dvb, rib, rjb, eb);
             for (int d = 0; d < DIM; ++d) {
                 ax[d].add(rb[d]);
                 av[d].add(dvb[d]);
             }
             arho.add(wall ? rib + rjb : rib);
-            eta_acc += (double)eb;
+            aeta.add(eb);
             if (wall) return;
             // the fluid neighbour's sums (j as i, k as j): r_jk = -r_kj
             Real Aj[3] = {0, 0, 0}, Rj[3] = {0, 0, 0}, mrv[3] = {0, 0, 0};
@@ -345,24 +435,39 @@ __global__ void __launch_bounds__(128) k_adj_pairs(int n, Tape<Real> T, Grid G, 
             }
             arho.add(rjb);
         };
-        adj_visit<Real, DIM>(n, k, G, K, T, pair);
+        adj_visit<Real, DIM, L>(n, k, q, G, K, T, pair);
+    }
+    __syncwarp();
+    double eta = wide_value(aeta);          // every lane's own part
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) {
+        group_sum<L>(ax[d]);
+        group_sum<L>(av[d]);
+    }
+    group_sum<L>(arho);
+    if (k < n && q == 0) {
         for (int d = 0; d < DIM; ++d) {
             xbp[(size_t)d * n + k] = ax[d].value();
             vbp[(size_t)d * n + k] = av[d].value();
         }
-        sigb[k] = arho.value() * K.rho0 / (Real)T.s0[k];
-        part[0] = eta_acc;
-    } else if (k < n) {
-        for (int d = 0; d < DIM; ++d) xbp[(size_t)d * n + k] = vbp[(size_t)d * n + k] = Real(0);
-        sigb[k] = Real(0);
+        sigb[k] = fluid ? arho.value() * K.rho0 / (Real)T.s0[k] : Real(0);
     }
-    block_partials(part, partials + (size_t)blockIdx.x * kNPart);
+    // the block's d/d(eta), in a fixed order
+    __shared__ double wsum[kAdjTPB / 32];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) eta += __shfl_down_sync(0xffffffffu, eta, off);
+    if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = eta;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int w = 1; w < (int)blockDim.x / 32; ++w) eta += wsum[w];
+        partials[blockIdx.x] = eta;
+    }
 }
 
 // ------------------------------------------------- density + drift / kick
 
-template <typename Real, int DIM>
-__global__ void __launch_bounds__(128) k_adj_density(int n, Tape<Real> T, Grid G, Consts<Real> K,
+template <typename Real, int DIM, int L>
+__global__ void __launch_bounds__(kAdjTPB) k_adj_density(int n, Tape<Real> T, Grid G, Consts<Real> K,
                                                      const Real* __restrict__ sigb, const Real* __restrict__ xbp,
                                                      const Real* __restrict__ vbp, int step_mode,
                                                      double* __restrict__ xc, double* __restrict__ vc,
@@ -375,23 +480,39 @@ __global__ void __launch_bounds__(128) k_adj_density(int n, Tape<Real> T, Grid G
         // block 0 first adds the pair kernel's per-block d/d(eta) partials to
         // eta (a fixed order: strided per thread, then the warps, then the
         // block's warps by thread 0)
-        __shared__ double wsum[32];
+        __shared__ double wsum[kAdjTPB / 32];
         double v = 0.0;
-        for (int b = threadIdx.x; b < nblocks; b += blockDim.x) v += partials[(size_t)b * kNPart];
+        for (int b = threadIdx.x; b < nblocks; b += blockDim.x) v += partials[b];
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
         if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = v;
         __syncthreads();
         if (threadIdx.x == 0) {
             double t = 0.0;
-            for (int w = 0; w < (int)(blockDim.x + 31) / 32; ++w) t += wsum[w];
+            for (int w = 0; w < (int)blockDim.x / 32; ++w) t += wsum[w];
             *eta += t;
         }
     }
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
+    const int k = (blockIdx.x * blockDim.x + threadIdx.x) / L, q = threadIdx.x % L;
+    const bool fluid = k < n && !T.kind[k];
+    Acc acc[DIM];
+    if (fluid) {
+        const Real sk = sigb[k];
+        const Real h_k = K.uniform_h ? K.h_u : (Real)T.h[k];
+        auto pair = [&](int j, const Real* rv, Real r, Real inv_r, float w_j) {
+            Real w, w2;
+            pair_kernels<Real, DIM>(K, T, k, j, h_k, w_j, r, w, w2);
+            const Real g = (sk + sigb[j]) * w * inv_r;        // sigb is 0 for a wall
+            for (int d = 0; d < DIM; ++d) acc[d].add(g * rv[d]);
+        };
+        adj_visit<Real, DIM, L>(n, k, q, G, K, T, pair);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) group_sum<L>(acc[d]);
+    if (k >= n || q) return;
     const int i = T.id[k];
-    if (T.kind[k]) {
+    if (!fluid) {
         if (step_mode)
             for (int d = 0; d < 3; ++d) {
                 const size_t o = (size_t)d * n + i;
@@ -399,16 +520,6 @@ __global__ void __launch_bounds__(128) k_adj_density(int n, Tape<Real> T, Grid G
             }
         return;
     }
-    const Real sk = sigb[k];
-    Acc acc[DIM];
-    auto pair = [&](int j, const Real* rv, Real r, Real inv_r) {
-        const Real inv_h = inv_pair_h(K, T, k, j);
-        const Real w = wendland_dW<DIM, Real>(r, inv_h);
-        const Real sj = T.kind[j] ? Real(0) : sigb[j];
-        const Real g = sizeof(Real) == 4 ? (sk + sj) * w * inv_r : (sk + sj) * w / r;
-        for (int d = 0; d < DIM; ++d) acc[d].add(g * rv[d]);
-    };
-    adj_visit<Real, DIM>(n, k, G, K, T, pair);
     const double dt = step_mode ? *T.dt : 0.0;
     const double hdt = 0.5 * dt;
     for (int d = 0; d < DIM; ++d) {
@@ -423,6 +534,37 @@ __global__ void __launch_bounds__(128) k_adj_density(int n, Tape<Real> T, Grid G
         xc[o] = xb;
         vc[o] = vh;
     }
+}
+
+// -------------------------------------------------------------- the tape
+
+// The forward values of a step that the reverse sweep reads, from the
+// context's buffers into a tape slot: one kernel for what eleven copies did
+// (each a node of the segment's graph).
+template <typename Real, int DIM>
+__global__ void __launch_bounds__(256) k_save_tape(int n, int nstart, StateSet<Real> S,
+                                                   const typename Vec4<Real>::T* __restrict__ vr,
+                                                   const Real* __restrict__ R, const int32_t* __restrict__ start,
+                                                   const float4* __restrict__ pos4, const int32_t* __restrict__ cell,
+                                                   Tape<Real> T)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < nstart) const_cast<int32_t*>(T.start)[i] = start[i];
+    if (i >= n) return;
+    const_cast<int32_t*>(T.id)[i] = S.id[i];
+    const_cast<int8_t*>(T.kind)[i] = S.kind[i];
+    const_cast<double*>(T.h)[i] = S.h[i];
+    const_cast<double*>(T.m)[i] = S.m[i];
+    const_cast<double*>(T.s0)[i] = S.s0[i];
+    const_cast<typename Vec4<Real>::T*>(T.vr)[i] = vr[i];
+    const_cast<int32_t*>(T.cell)[i] = cell[i];
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) {
+        const size_t o = (size_t)d * n + i;
+        const_cast<Real*>(T.R)[o] = R[o];
+        if (sizeof(Real) == 8) const_cast<double*>(T.x)[o] = S.x[o];
+    }
+    if (sizeof(Real) == 4) const_cast<float4*>(T.pos4)[i] = pos4[i];
 }
 
 // ----------------------------------------------------- cotangent layouts
@@ -457,7 +599,17 @@ cudaError_t launch_soa_to_aos(int n, const double* src, double* dst3, cudaStream
 
 static inline int nblk(int n, int t) { return (n + t - 1) / t; }
 
-int adj_pair_blocks(int n) { return nblk(n, 128); }
+// Lanes per particle of the reverse kernels in the FP64 form: as many as give
+// every SM some 500 threads (the FP64 pipe is full with few warps).  The FP32
+// form keeps one: its compensated sums stay in the order of the list.
+static int adj_lanes64(int n, int sms)
+{
+    if (sms <= 0) sms = 152;
+    return n >= sms * 512 ? 1 : (n >= sms * 128 ? 4 : 8);
+}
+
+// Blocks of the pair kernel at most (eight lanes per particle).
+size_t adj_partials(int n) { return ((size_t)n + kAdjTPB / 8 - 1) / (kAdjTPB / 8); }
 
 template <typename Real>
 static Tape<Real> make_tape(const TapeView& V)
@@ -471,17 +623,52 @@ static Tape<Real> make_tape(const TapeView& V)
     return T;
 }
 
+template <typename Real, int DIM, int L>
+static void adjoint_step_l(int n, const Tape<Real>& T, const Grid& G, const Consts<Real>& K, const AdjView& A,
+                           int step_mode, cudaStream_t st)
+{
+    const int nb = nblk(n, kAdjTPB / L);
+    k_adj_pairs<Real, DIM, L><<<nb, kAdjTPB, 0, st>>>(n, T, G, K, (const Real*)A.AR, (Real*)A.xbp, (Real*)A.vbp,
+                                                      (Real*)A.sigb, A.partials);
+    k_adj_density<Real, DIM, L><<<nb, kAdjTPB, 0, st>>>(n, T, G, K, (const Real*)A.sigb, (const Real*)A.xbp,
+                                                        (const Real*)A.vbp, step_mode, A.xc, A.vc, A.ac, A.drc,
+                                                        A.partials, nb, A.eta);
+}
+
 template <typename Real, int DIM>
 static void adjoint_step_t(int n, const TapeView& V, const Grid& G, const Consts<Real>& K, const AdjView& A,
                            int step_mode, cudaStream_t st)
 {
-    Tape<Real> T = make_tape<Real>(V);
+    const Tape<Real> T = make_tape<Real>(V);
     k_adj_prep<Real, DIM><<<nblk(n, 256), 256, 0, st>>>(n, T, K, step_mode, A.vc, A.ac, A.drc, (Real*)A.AR);
-    k_adj_pairs<Real, DIM><<<nblk(n, 128), 128, 0, st>>>(n, T, G, K, (const Real*)A.AR,
-                                                         (Real*)A.xbp, (Real*)A.vbp, (Real*)A.sigb, A.partials);
-    k_adj_density<Real, DIM><<<nblk(n, 128), 128, 0, st>>>(n, T, G, K, (const Real*)A.sigb, (const Real*)A.xbp,
-                                                           (const Real*)A.vbp, step_mode, A.xc, A.vc, A.ac, A.drc,
-                                                           A.partials, nblk(n, 128), A.eta);
+    if constexpr (sizeof(Real) == 8) {
+        const int L = adj_lanes64(n, G.sms);
+        if (L == 8) return adjoint_step_l<Real, DIM, 8>(n, T, G, K, A, step_mode, st);
+        if (L == 4) return adjoint_step_l<Real, DIM, 4>(n, T, G, K, A, step_mode, st);
+    }
+    adjoint_step_l<Real, DIM, 1>(n, T, G, K, A, step_mode, st);
+}
+
+template <typename Real>
+static void save_tape_t(int dim, int n, int nstart, const void* S, const void* vr, const void* R,
+                        const int32_t* start, const float4* pos4, const int32_t* cell, const TapeView& V,
+                        cudaStream_t st)
+{
+    const Tape<Real> T = make_tape<Real>(V);
+    const auto s = *(const StateSet<Real>*)S;
+    const auto v = (const typename Vec4<Real>::T*)vr;
+    const int nb = nblk(n > nstart ? n : nstart, 256);
+    if (dim == 2) k_save_tape<Real, 2><<<nb, 256, 0, st>>>(n, nstart, s, v, (const Real*)R, start, pos4, cell, T);
+    else k_save_tape<Real, 3><<<nb, 256, 0, st>>>(n, nstart, s, v, (const Real*)R, start, pos4, cell, T);
+}
+
+cudaError_t launch_save_tape(int prec, int dim, int n, int nstart, const void* S, const void* vr, const void* R,
+                             const int32_t* start, const float4* pos4, const int32_t* cell, const TapeView& V,
+                             cudaStream_t st)
+{
+    if (prec == 64) save_tape_t<double>(dim, n, nstart, S, vr, R, start, pos4, cell, V, st);
+    else save_tape_t<float>(dim, n, nstart, S, vr, R, start, pos4, cell, V, st);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_adjoint_step(int prec, int dim, int n, const TapeView& V, const Grid& G, const void* K,

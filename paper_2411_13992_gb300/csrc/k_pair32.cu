@@ -905,16 +905,6 @@ __host__ __device__ constexpr size_t coop_table_bytes()
     return (size_t)C::NG * (C::NR * sizeof(CoopRow) + (C::NR + 1) * sizeof(int));
 }
 
-// Compensated partial sums combined exactly: (s, c) holds s - c.
-__device__ __forceinline__ void ksum_merge(float& s, float& c, float s2, float c2)
-{
-    const float t = __fadd_rn(s, s2);
-    const float bb = __fsub_rn(t, s);
-    const float e = __fadd_rn(__fsub_rn(s, __fsub_rn(t, bb)), __fsub_rn(s2, bb));   // s + s2 = t + e exactly
-    c = __fsub_rn(__fadd_rn(c, c2), e);
-    s = t;
-}
-
 template <typename Acc> struct PartialSum;
 template <> struct PartialSum<KSum> {
     static __device__ __forceinline__ void get(const KSum& a, float& s, float& c) { s = a.s; c = a.c; }

@@ -24,7 +24,7 @@ struct TapeView {
     const float4* pos4;
     const int32_t* cell;
     const double* dt;
-    const uint32_t* nbl;   // FP32 form: the step's force-neighbour list (transposed, nbl_capacity rows)
+    const uint32_t* nbl;   // the step's force-neighbour list (transposed, nbl_capacity rows)
     const int32_t* nbc;    // and its counts
 };
 
@@ -156,7 +156,10 @@ cudaError_t launch_dual_substep(int prec, int dim, const DualArgs& a, const Grid
 cudaError_t launch_dual_complete(int prec, const DualArgs& a, cudaStream_t st);
 
 // k_adjoint.cu
-int adj_pair_blocks(int n);
+size_t adj_partials(int n);
+cudaError_t launch_save_tape(int prec, int dim, int n, int nstart, const void* S, const void* vr, const void* R,
+                             const int32_t* start, const float4* pos4, const int32_t* cell, const TapeView& V,
+                             cudaStream_t st);
 cudaError_t launch_adjoint_step(int prec, int dim, int n, const TapeView& V, const Grid& G, const void* K,
                                 const AdjView& A, int step_mode, cudaStream_t st);
 cudaError_t launch_aos_to_soa(int n, const double* src3, double* dst, cudaStream_t st);

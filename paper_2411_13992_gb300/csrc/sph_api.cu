@@ -39,7 +39,7 @@ struct TapeSlot {
     float4* pos4;
     int32_t* cell;
     double* dt;
-    uint32_t* nbl;      // FP32 form: the step's force-neighbour list (the density pass's, transposed)
+    uint32_t* nbl;      // the step's force-neighbour list (the density pass's, transposed)
     int32_t* nbc;       // and its counts
 };
 
@@ -365,7 +365,7 @@ size_t carve(sph_ctx* c, char* base)
             TapeSlot sl;
             sl.id = W.take<int32_t>(n);
             sl.kind = W.take<int8_t>(n);
-            sl.x = W.take<double>(D * n);
+            sl.x = c->prec == 64 ? W.take<double>(D * n) : nullptr;   // (the FP32 form reads pos4)
             sl.h = W.take<double>(n);
             sl.m = W.take<double>(n);
             sl.s0 = W.take<double>(n);
@@ -373,10 +373,10 @@ size_t carve(sph_ctx* c, char* base)
             sl.R = W.take<char>(D * n * rs);
             sl.start = W.take<int32_t>(nc1);
             sl.pos4 = c->prec == 32 ? W.take<float4>(n) : nullptr;
-            sl.cell = c->prec == 32 ? W.take<int32_t>(n) : nullptr;
+            sl.cell = W.take<int32_t>(n);
             sl.dt = W.take<double>(1);
-            sl.nbl = c->prec == 32 ? W.take<uint32_t>((size_t)nbl_capacity(D) * n) : nullptr;
-            sl.nbc = c->prec == 32 ? W.take<int32_t>(n) : nullptr;
+            sl.nbl = W.take<uint32_t>((size_t)nbl_capacity(D) * n);
+            sl.nbc = W.take<int32_t>(n);
             if (base && c->tape) c->tape[t] = sl;
         }
         AdjView& A = c->adj;
@@ -388,7 +388,7 @@ size_t carve(sph_ctx* c, char* base)
         A.xbp = W.take<char>(D * n * rs);
         A.vbp = W.take<char>(D * n * rs);
         A.sigb = W.take<char>(n * rs);
-        A.partials = W.take<double>((size_t)adj_pair_blocks((int)n) * kNPart);
+        A.partials = W.take<double>(adj_partials((int)n));
         A.eta = W.take<double>(1);
     }
     return (W.off + kAlign - 1) & ~(kAlign - 1);
@@ -727,42 +727,20 @@ sph_status reload_state(sph_ctx* c, const double* x, const double* v, const doub
     return SPH_OK;
 }
 
-// Copy the current step's forward values into tape slot t (dt is copied by
-// the caller before the step runs).  list_in_slot: the step's density pass
-// wrote its neighbour list into the slot's own list buffers (the FP32
-// form's adjoint walks that list); otherwise the list is copied from the
-// context's buffers.
-sph_status save_tape(sph_ctx* c, int t, bool list_in_slot = false)
-{
-    const size_t n = (size_t)c->n;
-    const size_t rs = c->prec == 64 ? 8 : 4;
-    const size_t nc1 = (size_t)c->G.ncell + 1;
-    const StateSet<double>& S = c->set[c->cur].d;
-    TapeSlot& T = c->tape[t];
-    SPH_CU(cudaMemcpyAsync(T.id, S.id, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, c->st));
-    SPH_CU(cudaMemcpyAsync(T.kind, S.kind, n, cudaMemcpyDeviceToDevice, c->st));
-    SPH_CU(cudaMemcpyAsync(T.x, S.x, c->dim * n * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
-    SPH_CU(cudaMemcpyAsync(T.h, S.h, n * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
-    SPH_CU(cudaMemcpyAsync(T.m, S.m, n * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
-    SPH_CU(cudaMemcpyAsync(T.s0, S.s0, n * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
-    SPH_CU(cudaMemcpyAsync(T.vr, c->vr, n * 4 * rs, cudaMemcpyDeviceToDevice, c->st));
-    SPH_CU(cudaMemcpyAsync(T.R, c->R, c->dim * n * rs, cudaMemcpyDeviceToDevice, c->st));
-    SPH_CU(cudaMemcpyAsync(T.start, c->start, nc1 * sizeof(int32_t), cudaMemcpyDeviceToDevice, c->st));
-    if (c->prec == 32) {
-        SPH_CU(cudaMemcpyAsync(T.pos4, c->pos4, n * sizeof(float4), cudaMemcpyDeviceToDevice, c->st));
-        SPH_CU(cudaMemcpyAsync(T.cell, c->cell, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, c->st));
-        if (!list_in_slot) {
-            SPH_CU(cudaMemcpyAsync(T.nbl, c->nbl, (size_t)nbl_capacity(c->dim) * n * sizeof(uint32_t),
-                                   cudaMemcpyDeviceToDevice, c->st));
-            SPH_CU(cudaMemcpyAsync(T.nbc, c->nbc, n * sizeof(int32_t), cudaMemcpyDeviceToDevice, c->st));
-        }
-    }
-    return SPH_OK;
-}
-
 TapeView tape_view(const TapeSlot& T)
 {
     return TapeView{T.id, T.kind, T.x, T.h, T.m, T.s0, T.vr, T.R, T.start, T.pos4, T.cell, T.dt, T.nbl, T.nbc};
+}
+
+// Copy the current step's forward values into tape slot t (dt is copied by
+// the caller before the step runs; the step's density pass wrote its
+// neighbour list into the slot's own list buffers).
+sph_status save_tape(sph_ctx* c, int t)
+{
+    SPH_CU(launch_save_tape(c->prec, c->dim, (int)c->n, c->G.ncell + 1, cur_set(c), c->vr, c->R, c->start, c->pos4,
+                            c->cell, tape_view(c->tape[t]), c->st));
+    ++c->launches;
+    return SPH_OK;
 }
 
 // Caller [n][3] cotangents -> [3][n] FP64 (z row zeroed in 2-D), and back.
@@ -785,6 +763,23 @@ sph_status cot_out(sph_ctx* c, const double* src, double* dst)
     return SPH_OK;
 }
 
+// While it lives, the context's neighbour list is that of tape slot t.
+struct ListInSlot {
+    sph_ctx* c;
+    uint32_t* nbl;
+    int32_t* nbc;
+    ListInSlot(sph_ctx* c_, int t) : c(c_), nbl(c_->nbl), nbc(c_->nbc)
+    {
+        c->nbl = c->tape[t].nbl;
+        c->nbc = c->tape[t].nbc;
+    }
+    ~ListInSlot()
+    {
+        c->nbl = nbl;
+        c->nbc = nbc;
+    }
+};
+
 // One segment of the adjoint after the cotangents are in: nsteps forward
 // steps from the reloaded state that record the tape (with the step sizes
 // taken), then the reverse sweep over them.  No host work between the
@@ -794,20 +789,13 @@ sph_status adjoint_segment(sph_ctx* c, int nsteps)
     for (int t = 0; t < nsteps; ++t) {
         SPH_CU(cudaMemcpyAsync(c->tape[t].dt, c->dt, sizeof(double), cudaMemcpyDeviceToDevice, c->st));
         SPH_TRY(run_sort(c, 1, 0));
-        // FP32 form: the step's density pass writes its neighbour list
-        // straight into the tape slot (no copy), the force pass reads it there
-        uint32_t* const nbl = c->nbl;
-        int32_t* const nbc = c->nbc;
-        const bool in_slot = c->prec == 32;
-        if (in_slot) {
-            c->nbl = c->tape[t].nbl;
-            c->nbc = c->tape[t].nbc;
+        {
+            // the step's density pass writes its neighbour list straight into
+            // the tape slot (no copy), the force pass reads it there
+            ListInSlot in_slot(c, t);
+            SPH_TRY(run_forces(c, 1, 1, 1));
         }
-        const sph_status s = run_forces(c, 1, 1, 1);
-        c->nbl = nbl;
-        c->nbc = nbc;
-        SPH_TRY(s);
-        SPH_TRY(save_tape(c, t, in_slot));
+        SPH_TRY(save_tape(c, t));
     }
     AdjView& A = c->adj;
     SPH_CU(cudaMemsetAsync(A.eta, 0, sizeof(double), c->st));
@@ -1348,7 +1336,10 @@ sph_status sph_force_pass_adjoint(sph_ctx* c, const double* x, const double* v, 
     if (c->P.adjoint_steps < 1 || c->P.tv_mode == SPH_TV_BACKGROUND) return SPH_ERR_ARG;
     if (!c->have_state) return SPH_ERR_STATE;
     SPH_TRY(reload_state(c, x, v, nullptr, nullptr));
-    SPH_TRY(sph_build_cells(c));
+    {
+        ListInSlot in_slot(c, 0);
+        SPH_TRY(sph_build_cells(c));
+    }
     SPH_TRY(save_tape(c, 0));
     SPH_CU(cudaMemsetAsync(c->tape[0].dt, 0, sizeof(double), c->st));
     AdjView& A = c->adj;
