@@ -13,6 +13,20 @@ namespace sphtv {
 
 constexpr double kPi = 3.14159265358979323846;
 
+// Start of a kernel launched with launch() (launch.h): wait until the kernel
+// before this one has ended and its writes can be read.  Every thread calls it
+// before its first access to memory, so that the end of a kernel implies the
+// end of all before it.  The kernels' pointers carry no __restrict__: the
+// loads of a const __restrict__ parameter count as invariant for the whole
+// kernel, and the compiler moved some of them ahead of the wait.  No kernel
+// releases the next one early (griddepcontrol.launch_dependents): blocks
+// placed while the kernel before still held most SMs crowded onto the free
+// ones and then ran two or three to an SM (3-D 16^3 FP64 step 93 -> 138 us).
+__device__ __forceinline__ void pdl_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // Device error word bits (sticky; read back by sph_sync).
 enum : uint32_t { ERRB_OVERFLOW = 1u, ERRB_NAN = 2u, ERRB_DOMAIN = 4u, ERRB_INPUT = 8u };
 

@@ -71,7 +71,7 @@ __device__ __forceinline__ double wide_value(const PlainD& a) { return a.s; }
 template <int DIM> constexpr int kAbStride = DIM == 3 ? 8 : 4;
 
 template <typename Real, int DIM>
-__device__ __forceinline__ void load_ab(const Real* __restrict__ AR, int k, Real* Ab, Real* Rb)
+__device__ __forceinline__ void load_ab(const Real* AR, int k, Real* Ab, Real* Rb)
 {
     const Real* p = AR + (size_t)k * kAbStride<DIM>;
     if constexpr (sizeof(Real) == 4) {
@@ -347,9 +347,10 @@ __device__ __forceinline__ Real mass_of(const Consts<Real>& K, const Tape<Real>&
 
 template <typename Real, int DIM>
 __global__ void __launch_bounds__(256) k_adj_prep(int n, Tape<Real> T, Consts<Real> K, int step_mode,
-                                                  const double* __restrict__ vc, const double* __restrict__ ac,
-                                                  const double* __restrict__ drc, Real* __restrict__ AR)
+                                                  const double* vc, const double* ac,
+                                                  const double* drc, Real* AR)
 {
+    pdl_wait();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
     const int i = T.id[k];
@@ -385,10 +386,11 @@ constexpr int kAdjTPB = 128;
 
 template <typename Real, int DIM, int L>
 __global__ void __launch_bounds__(kAdjTPB) k_adj_pairs(int n, Tape<Real> T, Grid G, Consts<Real> K,
-                                                   const Real* __restrict__ AR,
-                                                   Real* __restrict__ xbp, Real* __restrict__ vbp,
-                                                   Real* __restrict__ sigb, double* __restrict__ partials)
+                                                   const Real* AR,
+                                                   Real* xbp, Real* vbp,
+                                                   Real* sigb, double* partials)
 {
+    pdl_wait();
     using Acc = AccOf<Real>;
     const int k = (blockIdx.x * blockDim.x + threadIdx.x) / L, q = threadIdx.x % L;
     const bool fluid = k < n && !T.kind[k];
@@ -468,13 +470,14 @@ __global__ void __launch_bounds__(kAdjTPB) k_adj_pairs(int n, Tape<Real> T, Grid
 
 template <typename Real, int DIM, int L>
 __global__ void __launch_bounds__(kAdjTPB) k_adj_density(int n, Tape<Real> T, Grid G, Consts<Real> K,
-                                                     const Real* __restrict__ sigb, const Real* __restrict__ xbp,
-                                                     const Real* __restrict__ vbp, int step_mode,
-                                                     double* __restrict__ xc, double* __restrict__ vc,
-                                                     double* __restrict__ ac, double* __restrict__ drc,
-                                                     const double* __restrict__ partials, int nblocks,
-                                                     double* __restrict__ eta)
+                                                     const Real* sigb, const Real* xbp,
+                                                     const Real* vbp, int step_mode,
+                                                     double* xc, double* vc,
+                                                     double* ac, double* drc,
+                                                     const double* partials, int nblocks,
+                                                     double* eta)
 {
+    pdl_wait();
     using Acc = AccOf<Real>;
     if (blockIdx.x == 0) {
         // block 0 first adds the pair kernel's per-block d/d(eta) partials to
@@ -543,11 +546,12 @@ __global__ void __launch_bounds__(kAdjTPB) k_adj_density(int n, Tape<Real> T, Gr
 // (each a node of the segment's graph).
 template <typename Real, int DIM>
 __global__ void __launch_bounds__(256) k_save_tape(int n, int nstart, StateSet<Real> S,
-                                                   const typename Vec4<Real>::T* __restrict__ vr,
-                                                   const Real* __restrict__ R, const int32_t* __restrict__ start,
-                                                   const float4* __restrict__ pos4, const int32_t* __restrict__ cell,
+                                                   const typename Vec4<Real>::T* vr,
+                                                   const Real* R, const int32_t* start,
+                                                   const float4* pos4, const int32_t* cell,
                                                    Tape<Real> T)
 {
+    pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < nstart) const_cast<int32_t*>(T.start)[i] = start[i];
     if (i >= n) return;
@@ -569,15 +573,17 @@ __global__ void __launch_bounds__(256) k_save_tape(int n, int nstart, StateSet<R
 
 // ----------------------------------------------------- cotangent layouts
 
-__global__ void k_aos_to_soa(int n, const double* __restrict__ src3, double* __restrict__ dst)
+__global__ void k_aos_to_soa(int n, const double* src3, double* dst)
 {
+    pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     for (int d = 0; d < 3; ++d) dst[(size_t)d * n + i] = src3[3 * (size_t)i + d];
 }
 
-__global__ void k_soa_to_aos(int n, const double* __restrict__ src, double* __restrict__ dst3)
+__global__ void k_soa_to_aos(int n, const double* src, double* dst3)
 {
+    pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     for (int d = 0; d < 3; ++d) dst3[3 * (size_t)i + d] = src[(size_t)d * n + i];
@@ -587,13 +593,13 @@ __global__ void k_soa_to_aos(int n, const double* __restrict__ src, double* __re
 
 cudaError_t launch_aos_to_soa(int n, const double* src3, double* dst, cudaStream_t st)
 {
-    k_aos_to_soa<<<(n + 255) / 256, 256, 0, st>>>(n, src3, dst);
+    launch(k_aos_to_soa, (n + 255) / 256, 256, 0, st, n, src3, dst);
     return cudaGetLastError();
 }
 
 cudaError_t launch_soa_to_aos(int n, const double* src, double* dst3, cudaStream_t st)
 {
-    k_soa_to_aos<<<(n + 255) / 256, 256, 0, st>>>(n, src, dst3);
+    launch(k_soa_to_aos, (n + 255) / 256, 256, 0, st, n, src, dst3);
     return cudaGetLastError();
 }
 
@@ -628,9 +634,9 @@ static void adjoint_step_l(int n, const Tape<Real>& T, const Grid& G, const Cons
                            int step_mode, cudaStream_t st)
 {
     const int nb = nblk(n, kAdjTPB / L);
-    k_adj_pairs<Real, DIM, L><<<nb, kAdjTPB, 0, st>>>(n, T, G, K, (const Real*)A.AR, (Real*)A.xbp, (Real*)A.vbp,
+    launch(k_adj_pairs<Real, DIM, L>, nb, kAdjTPB, 0, st, n, T, G, K, (const Real*)A.AR, (Real*)A.xbp, (Real*)A.vbp,
                                                       (Real*)A.sigb, A.partials);
-    k_adj_density<Real, DIM, L><<<nb, kAdjTPB, 0, st>>>(n, T, G, K, (const Real*)A.sigb, (const Real*)A.xbp,
+    launch(k_adj_density<Real, DIM, L>, nb, kAdjTPB, 0, st, n, T, G, K, (const Real*)A.sigb, (const Real*)A.xbp,
                                                         (const Real*)A.vbp, step_mode, A.xc, A.vc, A.ac, A.drc,
                                                         A.partials, nb, A.eta);
 }
@@ -640,7 +646,7 @@ static void adjoint_step_t(int n, const TapeView& V, const Grid& G, const Consts
                            int step_mode, cudaStream_t st)
 {
     const Tape<Real> T = make_tape<Real>(V);
-    k_adj_prep<Real, DIM><<<nblk(n, 256), 256, 0, st>>>(n, T, K, step_mode, A.vc, A.ac, A.drc, (Real*)A.AR);
+    launch(k_adj_prep<Real, DIM>, nblk(n, 256), 256, 0, st, n, T, K, step_mode, A.vc, A.ac, A.drc, (Real*)A.AR);
     if constexpr (sizeof(Real) == 8) {
         const int L = adj_lanes64(n, G.sms);
         if (L == 8) return adjoint_step_l<Real, DIM, 8>(n, T, G, K, A, step_mode, st);
@@ -658,8 +664,8 @@ static void save_tape_t(int dim, int n, int nstart, const void* S, const void* v
     const auto s = *(const StateSet<Real>*)S;
     const auto v = (const typename Vec4<Real>::T*)vr;
     const int nb = nblk(n > nstart ? n : nstart, 256);
-    if (dim == 2) k_save_tape<Real, 2><<<nb, 256, 0, st>>>(n, nstart, s, v, (const Real*)R, start, pos4, cell, T);
-    else k_save_tape<Real, 3><<<nb, 256, 0, st>>>(n, nstart, s, v, (const Real*)R, start, pos4, cell, T);
+    if (dim == 2) launch(k_save_tape<Real, 2>, nb, 256, 0, st, n, nstart, s, v, (const Real*)R, start, pos4, cell, T);
+    else launch(k_save_tape<Real, 3>, nb, 256, 0, st, n, nstart, s, v, (const Real*)R, start, pos4, cell, T);
 }
 
 cudaError_t launch_save_tape(int prec, int dim, int n, int nstart, const void* S, const void* vr, const void* R,

@@ -74,10 +74,11 @@ __device__ __forceinline__ int wrap_side(const Grid& G, double x, int d)
 }
 
 template <typename Real, int DIM>
-__global__ void k_kick_drift_key(int n, StateSet<Real> S, const double* __restrict__ dt_ptr, int drift, Grid G,
-                                 int32_t* __restrict__ key, int32_t* __restrict__ count,
-                                 int32_t* __restrict__ head, int32_t* __restrict__ next, uint32_t* err)
+__global__ void k_kick_drift_key(int n, StateSet<Real> S, const double* dt_ptr, int drift, Grid G,
+                                 int32_t* key, int32_t* count,
+                                 int32_t* head, int32_t* next, uint32_t* err)
 {
+    pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     double xs[3] = {0.0, 0.0, 0.0};
@@ -197,9 +198,10 @@ __device__ __forceinline__ int32_t block_scan(int32_t s, int32_t* warp_tot, int3
 // were two or three).  Where each reading warp scanned up to 32 sums itself
 // instead, the step of a small problem took as long and the permute 3 us more
 // at 128^3.
-__global__ void __launch_bounds__(kScanThreads) k_bin_scan(int32_t* __restrict__ count, int32_t* __restrict__ prefix,
+__global__ void __launch_bounds__(kScanThreads) k_bin_scan(int32_t* count, int32_t* prefix,
                                                            int32_t* tile_off, unsigned* done, int n)
 {
+    pdl_wait();
     __shared__ int32_t warp_tot[kScanThreads / 32 + 1];
     __shared__ int is_last;
     const int base = blockIdx.x * kScanTile + threadIdx.x * kScanItems;
@@ -263,7 +265,7 @@ __global__ void __launch_bounds__(kScanThreads) k_bin_scan(int32_t* __restrict__
 cudaError_t launch_bin_scan(int32_t* count, int32_t* prefix, int n, int32_t* tile_off, unsigned* done,
                             cudaStream_t st)
 {
-    k_bin_scan<<<(n + kScanTile - 1) / kScanTile, kScanThreads, 0, st>>>(count, prefix, tile_off, done, n);
+    launch(k_bin_scan, (n + kScanTile - 1) / kScanTile, kScanThreads, 0, st, count, prefix, tile_off, done, n);
     return cudaGetLastError();
 }
 
@@ -290,14 +292,15 @@ cudaError_t launch_bin_scan(int32_t* count, int32_t* prefix, int n, int32_t* til
 // sigma0 and is a fluid particle, and both state sets hold these arrays
 // (set by sph_set_state): they are left where they are.
 template <typename Real, int DIM, bool CARRY_AD>
-__global__ void __launch_bounds__(256) k_order_permute(int n, int nbin, const int32_t* __restrict__ key,
-                                const int32_t* __restrict__ prefix, const int32_t* __restrict__ tile_off,
-                                const int32_t* __restrict__ head, const int32_t* __restrict__ next,
-                                int32_t* __restrict__ bin_start, int32_t* __restrict__ cell_start,
-                                StateSet<Real> src, StateSet<Real> dst, Grid G, float4* __restrict__ pos4,
-                                int32_t* __restrict__ cell_out, float* __restrict__ mf, int uniform_h,
-                                float4* __restrict__ pos4c, const uint32_t* __restrict__ varies)
+__global__ void __launch_bounds__(256) k_order_permute(int n, int nbin, const int32_t* key,
+                                const int32_t* prefix, const int32_t* tile_off,
+                                const int32_t* head, const int32_t* next,
+                                int32_t* bin_start, int32_t* cell_start,
+                                StateSet<Real> src, StateSet<Real> dst, Grid G, float4* pos4,
+                                int32_t* cell_out, float* mf, int uniform_h,
+                                float4* pos4c, const uint32_t* varies)
 {
+    pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     auto start_of = [&](int k) { return prefix[k] + tile_off[k / kScanTile]; };
     if (i <= nbin) {
@@ -372,12 +375,12 @@ cudaError_t launch_kick_drift_key(int prec, int dim, int n, void* S, const doubl
     const int T = 256;
     if (prec == 64) {
         auto s = *(StateSet<double>*)S;
-        if (dim == 2) k_kick_drift_key<double, 2><<<nblk(n, T), T, 0, st>>>(n, s, dt, drift, G, key, count, head, next, err);
-        else k_kick_drift_key<double, 3><<<nblk(n, T), T, 0, st>>>(n, s, dt, drift, G, key, count, head, next, err);
+        if (dim == 2) launch(k_kick_drift_key<double, 2>, nblk(n, T), T, 0, st, n, s, dt, drift, G, key, count, head, next, err);
+        else launch(k_kick_drift_key<double, 3>, nblk(n, T), T, 0, st, n, s, dt, drift, G, key, count, head, next, err);
     } else {
         auto s = *(StateSet<float>*)S;
-        if (dim == 2) k_kick_drift_key<float, 2><<<nblk(n, T), T, 0, st>>>(n, s, dt, drift, G, key, count, head, next, err);
-        else k_kick_drift_key<float, 3><<<nblk(n, T), T, 0, st>>>(n, s, dt, drift, G, key, count, head, next, err);
+        if (dim == 2) launch(k_kick_drift_key<float, 2>, nblk(n, T), T, 0, st, n, s, dt, drift, G, key, count, head, next, err);
+        else launch(k_kick_drift_key<float, 3>, nblk(n, T), T, 0, st, n, s, dt, drift, G, key, count, head, next, err);
     }
     return cudaGetLastError();
 }
@@ -395,7 +398,7 @@ static void order_permute_t(int dim, int n, int nbin, const SortBufs& B, void* s
     int32_t* bs = G.sub_shift ? B.sub_start : B.cell_start;
     auto kern = dim == 2 ? (carry_ad ? k_order_permute<Real, 2, true> : k_order_permute<Real, 2, false>)
                          : (carry_ad ? k_order_permute<Real, 3, true> : k_order_permute<Real, 3, false>);
-    kern<<<nb, T, 0, st>>>(n, nbin, B.key, B.prefix, B.tile_off, B.head, B.next, bs, cs, s, d, G, pos4, cell, mf, uh,
+    launch(kern, nb, T, 0, st, n, nbin, B.key, B.prefix, B.tile_off, B.head, B.next, bs, cs, s, d, G, pos4, cell, mf, uh,
                            pos4c, varies);
 }
 

@@ -219,8 +219,9 @@ template <> __device__ __forceinline__ float fma_free_mul<float>(float a, float 
 
 // Eq. 9-11 with h = h_min from max |v| of the fluid (the diagnostics of the
 // previous step or of sph_build_cells; the sort does not change v).
-__global__ void k_dual_begin(DtConsts D, const double* __restrict__ diag, double* __restrict__ du)
+__global__ void k_dual_begin(DtConsts D, const double* diag, double* du)
 {
+    pdl_wait();
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     const double vmax = diag[DG_VMAX];
     const double vad = fmax(vmax, D.v_floor);
@@ -245,6 +246,7 @@ __global__ void k_dual_begin(DtConsts D, const double* __restrict__ diag, double
 template <typename Real, int DIM, typename Acc, bool UNIFORM>
 __global__ void __launch_bounds__(sizeof(Real) == 8 ? 256 : 128) k_dual_advect(DualK<Real> A, Grid G, Consts<Real> K)
 {
+    pdl_wait();
     __shared__ float4 tab[kCodes];
     fill_shift_table<Real>(G, tab);
     const int n = A.n;
@@ -321,6 +323,7 @@ __global__ void __launch_bounds__(sizeof(Real) == 8 ? 256 : 128) k_dual_advect(D
 template <typename Real, int DIM>
 __global__ void __launch_bounds__(256) k_dual_first_half(DualK<Real> A, Grid G)
 {
+    pdl_wait();
     if (dual_done(A.du)) return;
     const int n = A.n;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -362,6 +365,7 @@ __global__ void __launch_bounds__(256) k_dual_first_half(DualK<Real> A, Grid G)
 template <typename Real, int DIM, typename Acc, bool UNIFORM>
 __global__ void __launch_bounds__(sizeof(Real) == 8 ? 256 : 128) k_dual_pressure(DualK<Real> A, Grid G, Consts<Real> K)
 {
+    pdl_wait();
     __shared__ float4 tab[kCodes];
     if (dual_done(A.du)) return;
     fill_shift_table<Real>(G, tab);
@@ -416,6 +420,7 @@ __global__ void __launch_bounds__(sizeof(Real) == 8 ? 256 : 128) k_dual_pressure
 template <typename Real, int DIM>
 __global__ void __launch_bounds__(256) k_dual_drift(DualK<Real> A, Grid G)
 {
+    pdl_wait();
     if (dual_done(A.du)) return;
     const int n = A.n;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -439,8 +444,8 @@ __global__ void __launch_bounds__(256) k_dual_drift(DualK<Real> A, Grid G)
 
 // The end of a substep, from the grid's totals: advance t; pick the next
 // substep size, or finish the advection step and write the diagnostics.
-__device__ __forceinline__ void finish_substep(const double* out, const DtConsts& D, double* __restrict__ du,
-                                               double* __restrict__ diag, double* __restrict__ dt_ptr)
+__device__ __forceinline__ void finish_substep(const double* out, const DtConsts& D, double* du,
+                                               double* diag, double* dt_ptr)
 {
     if (threadIdx.x != 0) return;
     const double vmax = out[6];
@@ -482,6 +487,7 @@ __device__ __forceinline__ void finish_substep(const double* out, const DtConsts
 template <typename Real, int DIM, typename Acc, bool UNIFORM>
 __global__ void __launch_bounds__(sizeof(Real) == 8 ? 256 : 128) k_dual_continuity(DualK<Real> A, Grid G, Consts<Real> K, DtConsts D)
 {
+    pdl_wait();
     __shared__ float4 tab[kCodes];
     if (dual_done(A.du)) return;
     fill_shift_table<Real>(G, tab);
@@ -572,8 +578,9 @@ __global__ void __launch_bounds__(sizeof(Real) == 8 ? 256 : 128) k_dual_continui
 
 // The rows of a large grid (see GridSum), and the end of the substep.
 __global__ void __launch_bounds__(256) k_fold_substep(GridSum B, int nrows, DtConsts D, double* du,
-                                                      double* __restrict__ diag, double* __restrict__ dt_ptr)
+                                                      double* diag, double* dt_ptr)
 {
+    pdl_wait();
     if (dual_done(du)) return;
     __shared__ double total[kNPart];
     if (fold_grid(B, nrows, total)) finish_substep(total, D, du, diag, dt_ptr);
@@ -583,6 +590,7 @@ __global__ void __launch_bounds__(256) k_fold_substep(GridSum B, int nrows, DtCo
 template <typename Real>
 __global__ void __launch_bounds__(256) k_dual_complete(DualK<Real> A)
 {
+    pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= A.n || A.S.kind[i]) return;
     auto me = A.vr[i];
@@ -631,7 +639,7 @@ template <template <typename, int, typename, bool> class Kern> struct Dispatch;
         {                                                                                                  \
             const int T = pair_threads(sizeof(Real) == 8 ? 64 : 32, A.n, G.sms);                            \
             (void)D;                                                                                       \
-            name<Real, DIM, Acc, U><<<nblk(A.n, T), T, 0, st>>>(A, G, K, ##__VA_ARGS__);                     \
+            launch(name<Real, DIM, Acc, U>, nblk(A.n, T), T, 0, st, A, G, K, ##__VA_ARGS__);                     \
         }                                                                                                  \
     };
 SPH_DUAL_PAIR_KERNEL(k_dual_advect)
@@ -668,13 +676,13 @@ void run_elem(int dim, const DualArgs& a, const Grid& G, int which, cudaStream_t
     const auto A = dual_k<Real>(a);
     const int T = 256, B = nblk(A.n, T);
     if (which == 0) {
-        if (dim == 2) k_dual_first_half<Real, 2><<<B, T, 0, st>>>(A, G);
-        else k_dual_first_half<Real, 3><<<B, T, 0, st>>>(A, G);
+        if (dim == 2) launch(k_dual_first_half<Real, 2>, B, T, 0, st, A, G);
+        else launch(k_dual_first_half<Real, 3>, B, T, 0, st, A, G);
     } else if (which == 1) {
-        if (dim == 2) k_dual_drift<Real, 2><<<B, T, 0, st>>>(A, G);
-        else k_dual_drift<Real, 3><<<B, T, 0, st>>>(A, G);
+        if (dim == 2) launch(k_dual_drift<Real, 2>, B, T, 0, st, A, G);
+        else launch(k_dual_drift<Real, 3>, B, T, 0, st, A, G);
     } else {
-        k_dual_complete<Real><<<B, T, 0, st>>>(A);
+        launch(k_dual_complete<Real>, B, T, 0, st, A);
     }
 }
 
@@ -682,7 +690,7 @@ void run_elem(int dim, const DualArgs& a, const Grid& G, int which, cudaStream_t
 
 cudaError_t launch_dual_begin(const sph_params& P, const double* diag, double* du, cudaStream_t st)
 {
-    k_dual_begin<<<1, 32, 0, st>>>(dt_consts(P), diag, du);
+    launch(k_dual_begin, 1, 32, 0, st, dt_consts(P), diag, du);
     return cudaGetLastError();
 }
 
@@ -705,7 +713,7 @@ cudaError_t launch_dual_substep(int prec, int dim, const DualArgs& a, const Grid
     const int nb = pair_blocks(prec, a.n, a.sms);
     const GridSum B = grid_sum(a.F, nb);
     if (B.group == 0) {
-        k_fold_substep<<<kFoldBlocks, 256, 0, st>>>(B, nb, dt_consts(*a.F.P), a.du, a.F.diag, a.F.dt);
+        launch(k_fold_substep, kFoldBlocks, 256, 0, st, B, nb, dt_consts(*a.F.P), a.du, a.F.diag, a.F.dt);
         ++*launches;
     }
     return cudaGetLastError();

@@ -9,8 +9,9 @@
 namespace sphtv {
 
 template <typename Real, int DIM>
-__global__ void k_vec_in(int n, const double* __restrict__ src3, Real* __restrict__ dst)
+__global__ void k_vec_in(int n, const double* src3, Real* dst)
 {
+    pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
 #pragma unroll
@@ -18,9 +19,10 @@ __global__ void k_vec_in(int n, const double* __restrict__ src3, Real* __restric
 }
 
 template <typename Real, int DIM>
-__global__ void k_vec_out(int n, const Real* __restrict__ src, const int32_t* __restrict__ id,
-                          double* __restrict__ dst3)
+__global__ void k_vec_out(int n, const Real* src, const int32_t* id,
+                          double* dst3)
 {
+    pdl_wait();
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
     size_t o = 3 * (size_t)id[k];
@@ -30,8 +32,9 @@ __global__ void k_vec_out(int n, const Real* __restrict__ src, const int32_t* __
 
 // pos[id[k]] = k: where the particle the caller gave as number i sits in
 // the cell order.
-__global__ void k_inverse_perm(int n, const int32_t* __restrict__ id, int32_t* __restrict__ pos)
+__global__ void k_inverse_perm(int n, const int32_t* id, int32_t* pos)
 {
+    pdl_wait();
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < n) pos[id[k]] = k;
 }
@@ -40,9 +43,10 @@ __global__ void k_inverse_perm(int n, const int32_t* __restrict__ id, int32_t* _
 // position pos[i], so the writes of a warp are contiguous (the destination
 // may be page-locked host memory written across the host link).
 template <typename Real, int DIM>
-__global__ void k_vec_out_gather(int n, const Real* __restrict__ src, const int32_t* __restrict__ pos,
-                                 double* __restrict__ dst3)
+__global__ void k_vec_out_gather(int n, const Real* src, const int32_t* pos,
+                                 double* dst3)
 {
+    pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const size_t k = (size_t)pos[i];
@@ -51,9 +55,10 @@ __global__ void k_vec_out_gather(int n, const Real* __restrict__ src, const int3
 }
 
 template <typename V4>
-__global__ void k_rho_out_gather(int n, const V4* __restrict__ vr, const int8_t* __restrict__ kind,
-                                 const int32_t* __restrict__ pos, double rho0, double* __restrict__ dst)
+__global__ void k_rho_out_gather(int n, const V4* vr, const int8_t* kind,
+                                 const int32_t* pos, double rho0, double* dst)
 {
+    pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int k = pos[i];
@@ -61,9 +66,10 @@ __global__ void k_rho_out_gather(int n, const V4* __restrict__ vr, const int8_t*
 }
 
 template <typename Real, int DIM>
-__global__ void k_walls_velocity(int n, const int8_t* __restrict__ kind, const double* __restrict__ vw3,
-                                 Real* __restrict__ v)
+__global__ void k_walls_velocity(int n, const int8_t* kind, const double* vw3,
+                                 Real* v)
 {
+    pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n || !kind[i]) return;
 #pragma unroll
@@ -72,6 +78,7 @@ __global__ void k_walls_velocity(int n, const int8_t* __restrict__ kind, const d
 
 __global__ void k_init_ids(int n, int32_t* id)
 {
+    pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) id[i] = i;
 }
@@ -105,25 +112,28 @@ __device__ double sigma0_of(double h, double m, double rho0)
 // the others compute their own (the lattice sum is FP64 work, and FP64 runs
 // at 1/74 of the FP32 rate).
 template <int DIM>
-__global__ void k_sigma0_first(const double* __restrict__ h, const double* __restrict__ m, double rho0,
-                               double* __restrict__ s0)
+__global__ void k_sigma0_first(const double* h, const double* m, double rho0,
+                               double* s0)
 {
+    pdl_wait();
     if (blockIdx.x == 0 && threadIdx.x == 0) s0[0] = sigma0_of<DIM>(h[0], m[0], rho0);
 }
 
 template <int DIM>
-__global__ void k_sigma0(int n, const double* __restrict__ h, const double* __restrict__ m, double rho0,
-                         double* __restrict__ s0)
+__global__ void k_sigma0(int n, const double* h, const double* m, double rho0,
+                         double* s0)
 {
+    pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < 1 || i >= n) return;
     s0[i] = (h[i] == h[0] && m[i] == m[0]) ? s0[0] : sigma0_of<DIM>(h[i], m[i], rho0);
 }
 
 template <typename V4>
-__global__ void k_rho_out(int n, const V4* __restrict__ vr, const int8_t* __restrict__ kind,
-                          const int32_t* __restrict__ id, double rho0, double* __restrict__ dst)
+__global__ void k_rho_out(int n, const V4* vr, const int8_t* kind,
+                          const int32_t* id, double rho0, double* dst)
 {
+    pdl_wait();
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
     dst[id[k]] = kind[k] ? rho0 : rho0 + (double)vr[k].w;
@@ -131,9 +141,10 @@ __global__ void k_rho_out(int n, const V4* __restrict__ vr, const int8_t* __rest
 
 // Every h must lie in [h_min, h_max] (the cell edge is sized by h_max) and
 // every mass must be positive and finite.
-__global__ void k_check_input(int n, const double* __restrict__ h, const double* __restrict__ m, double h_min,
+__global__ void k_check_input(int n, const double* h, const double* m, double h_min,
                               double h_max, uint32_t* err)
 {
+    pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     bool ok = h[i] >= h_min && h[i] <= h_max && m[i] > 0.0 && isfinite(m[i]);
@@ -142,9 +153,10 @@ __global__ void k_check_input(int n, const double* __restrict__ h, const double*
 
 // Sets *varies (cleared by the caller) when a particle's h, m or sigma0
 // differs from particle 0's or a particle is a wall particle.
-__global__ void k_check_constants(int n, const double* __restrict__ h, const double* __restrict__ m,
-                                  const double* __restrict__ s0, const int8_t* __restrict__ kind, uint32_t* varies)
+__global__ void k_check_constants(int n, const double* h, const double* m,
+                                  const double* s0, const int8_t* kind, uint32_t* varies)
 {
+    pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const bool v = kind[i] != 0 || h[i] != h[0] || m[i] != m[0] || s0[i] != s0[0];
@@ -153,9 +165,10 @@ __global__ void k_check_constants(int n, const double* __restrict__ h, const dou
 }
 
 template <typename Real>
-__global__ void k_scalar_out(int n, const Real* __restrict__ src, const int32_t* __restrict__ id,
-                             double* __restrict__ dst)
+__global__ void k_scalar_out(int n, const Real* src, const int32_t* id,
+                             double* dst)
 {
+    pdl_wait();
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k < n) dst[id[k]] = (double)src[k];
 }
@@ -163,9 +176,10 @@ __global__ void k_scalar_out(int n, const Real* __restrict__ src, const int32_t*
 // Caller-order scalar in (walls get 0); used before the first sort, when the
 // internal order is the caller's.
 template <typename Real>
-__global__ void k_scalar_in(int n, const double* __restrict__ src, const int8_t* __restrict__ kind,
-                            Real* __restrict__ dst)
+__global__ void k_scalar_in(int n, const double* src, const int8_t* kind,
+                            Real* dst)
 {
+    pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < n) dst[i] = kind[i] ? Real(0) : (Real)src[i];
 }
@@ -176,11 +190,11 @@ cudaError_t launch_vec_in(int prec, int dim, int n, const double* src3, void* ds
 {
     const int T = 256;
     if (prec == 64) {
-        if (dim == 2) k_vec_in<double, 2><<<nblk(n, T), T, 0, st>>>(n, src3, (double*)dst);
-        else k_vec_in<double, 3><<<nblk(n, T), T, 0, st>>>(n, src3, (double*)dst);
+        if (dim == 2) launch(k_vec_in<double, 2>, nblk(n, T), T, 0, st, n, src3, (double*)dst);
+        else launch(k_vec_in<double, 3>, nblk(n, T), T, 0, st, n, src3, (double*)dst);
     } else {
-        if (dim == 2) k_vec_in<float, 2><<<nblk(n, T), T, 0, st>>>(n, src3, (float*)dst);
-        else k_vec_in<float, 3><<<nblk(n, T), T, 0, st>>>(n, src3, (float*)dst);
+        if (dim == 2) launch(k_vec_in<float, 2>, nblk(n, T), T, 0, st, n, src3, (float*)dst);
+        else launch(k_vec_in<float, 3>, nblk(n, T), T, 0, st, n, src3, (float*)dst);
     }
     return cudaGetLastError();
 }
@@ -190,11 +204,11 @@ cudaError_t launch_vec_out(int prec, int dim, int n, const void* src, const int3
 {
     const int T = 256;
     if (prec == 64) {
-        if (dim == 2) k_vec_out<double, 2><<<nblk(n, T), T, 0, st>>>(n, (const double*)src, id, dst3);
-        else k_vec_out<double, 3><<<nblk(n, T), T, 0, st>>>(n, (const double*)src, id, dst3);
+        if (dim == 2) launch(k_vec_out<double, 2>, nblk(n, T), T, 0, st, n, (const double*)src, id, dst3);
+        else launch(k_vec_out<double, 3>, nblk(n, T), T, 0, st, n, (const double*)src, id, dst3);
     } else {
-        if (dim == 2) k_vec_out<float, 2><<<nblk(n, T), T, 0, st>>>(n, (const float*)src, id, dst3);
-        else k_vec_out<float, 3><<<nblk(n, T), T, 0, st>>>(n, (const float*)src, id, dst3);
+        if (dim == 2) launch(k_vec_out<float, 2>, nblk(n, T), T, 0, st, n, (const float*)src, id, dst3);
+        else launch(k_vec_out<float, 3>, nblk(n, T), T, 0, st, n, (const float*)src, id, dst3);
     }
     return cudaGetLastError();
 }
@@ -204,18 +218,18 @@ cudaError_t launch_walls_velocity(int prec, int dim, int n, const int8_t* kind, 
 {
     const int T = 256;
     if (prec == 64) {
-        if (dim == 2) k_walls_velocity<double, 2><<<nblk(n, T), T, 0, st>>>(n, kind, vw3, (double*)v);
-        else k_walls_velocity<double, 3><<<nblk(n, T), T, 0, st>>>(n, kind, vw3, (double*)v);
+        if (dim == 2) launch(k_walls_velocity<double, 2>, nblk(n, T), T, 0, st, n, kind, vw3, (double*)v);
+        else launch(k_walls_velocity<double, 3>, nblk(n, T), T, 0, st, n, kind, vw3, (double*)v);
     } else {
-        if (dim == 2) k_walls_velocity<float, 2><<<nblk(n, T), T, 0, st>>>(n, kind, vw3, (float*)v);
-        else k_walls_velocity<float, 3><<<nblk(n, T), T, 0, st>>>(n, kind, vw3, (float*)v);
+        if (dim == 2) launch(k_walls_velocity<float, 2>, nblk(n, T), T, 0, st, n, kind, vw3, (float*)v);
+        else launch(k_walls_velocity<float, 3>, nblk(n, T), T, 0, st, n, kind, vw3, (float*)v);
     }
     return cudaGetLastError();
 }
 
 cudaError_t launch_init_ids(int n, int32_t* id, cudaStream_t st)
 {
-    k_init_ids<<<nblk(n, 256), 256, 0, st>>>(n, id);
+    launch(k_init_ids, nblk(n, 256), 256, 0, st, n, id);
     return cudaGetLastError();
 }
 
@@ -223,11 +237,11 @@ cudaError_t launch_sigma0(int dim, int n, const double* h, const double* m, doub
                           cudaStream_t st)
 {
     if (dim == 2) {
-        k_sigma0_first<2><<<1, 32, 0, st>>>(h, m, rho0, s0);
-        k_sigma0<2><<<nblk(n, 128), 128, 0, st>>>(n, h, m, rho0, s0);
+        launch(k_sigma0_first<2>, 1, 32, 0, st, h, m, rho0, s0);
+        launch(k_sigma0<2>, nblk(n, 128), 128, 0, st, n, h, m, rho0, s0);
     } else {
-        k_sigma0_first<3><<<1, 32, 0, st>>>(h, m, rho0, s0);
-        k_sigma0<3><<<nblk(n, 128), 128, 0, st>>>(n, h, m, rho0, s0);
+        launch(k_sigma0_first<3>, 1, 32, 0, st, h, m, rho0, s0);
+        launch(k_sigma0<3>, nblk(n, 128), 128, 0, st, n, h, m, rho0, s0);
     }
     return cudaGetLastError();
 }
@@ -235,14 +249,14 @@ cudaError_t launch_sigma0(int dim, int n, const double* h, const double* m, doub
 cudaError_t launch_rho_out(int prec, int n, const void* vr, const int8_t* kind, const int32_t* id, double rho0,
                            double* dst, cudaStream_t st)
 {
-    if (prec == 64) k_rho_out<double4_32a><<<nblk(n, 256), 256, 0, st>>>(n, (const double4_32a*)vr, kind, id, rho0, dst);
-    else k_rho_out<float4><<<nblk(n, 256), 256, 0, st>>>(n, (const float4*)vr, kind, id, rho0, dst);
+    if (prec == 64) launch(k_rho_out<double4_32a>, nblk(n, 256), 256, 0, st, n, (const double4_32a*)vr, kind, id, rho0, dst);
+    else launch(k_rho_out<float4>, nblk(n, 256), 256, 0, st, n, (const float4*)vr, kind, id, rho0, dst);
     return cudaGetLastError();
 }
 
 cudaError_t launch_inverse_perm(int n, const int32_t* id, int32_t* pos, cudaStream_t st)
 {
-    k_inverse_perm<<<nblk(n, 256), 256, 0, st>>>(n, id, pos);
+    launch(k_inverse_perm, nblk(n, 256), 256, 0, st, n, id, pos);
     return cudaGetLastError();
 }
 
@@ -251,11 +265,11 @@ cudaError_t launch_vec_out_gather(int prec, int dim, int n, const void* src, con
 {
     const int T = 256;
     if (prec == 64) {
-        if (dim == 2) k_vec_out_gather<double, 2><<<nblk(n, T), T, 0, st>>>(n, (const double*)src, pos, dst3);
-        else k_vec_out_gather<double, 3><<<nblk(n, T), T, 0, st>>>(n, (const double*)src, pos, dst3);
+        if (dim == 2) launch(k_vec_out_gather<double, 2>, nblk(n, T), T, 0, st, n, (const double*)src, pos, dst3);
+        else launch(k_vec_out_gather<double, 3>, nblk(n, T), T, 0, st, n, (const double*)src, pos, dst3);
     } else {
-        if (dim == 2) k_vec_out_gather<float, 2><<<nblk(n, T), T, 0, st>>>(n, (const float*)src, pos, dst3);
-        else k_vec_out_gather<float, 3><<<nblk(n, T), T, 0, st>>>(n, (const float*)src, pos, dst3);
+        if (dim == 2) launch(k_vec_out_gather<float, 2>, nblk(n, T), T, 0, st, n, (const float*)src, pos, dst3);
+        else launch(k_vec_out_gather<float, 3>, nblk(n, T), T, 0, st, n, (const float*)src, pos, dst3);
     }
     return cudaGetLastError();
 }
@@ -264,36 +278,36 @@ cudaError_t launch_rho_out_gather(int prec, int n, const void* vr, const int8_t*
                                   double rho0, double* dst, cudaStream_t st)
 {
     if (prec == 64)
-        k_rho_out_gather<double4_32a><<<nblk(n, 256), 256, 0, st>>>(n, (const double4_32a*)vr, kind, pos, rho0, dst);
-    else k_rho_out_gather<float4><<<nblk(n, 256), 256, 0, st>>>(n, (const float4*)vr, kind, pos, rho0, dst);
+        launch(k_rho_out_gather<double4_32a>, nblk(n, 256), 256, 0, st, n, (const double4_32a*)vr, kind, pos, rho0, dst);
+    else launch(k_rho_out_gather<float4>, nblk(n, 256), 256, 0, st, n, (const float4*)vr, kind, pos, rho0, dst);
     return cudaGetLastError();
 }
 
 cudaError_t launch_check_input(int n, const double* h, const double* m, double h_min, double h_max, uint32_t* err,
                                cudaStream_t st)
 {
-    k_check_input<<<nblk(n, 256), 256, 0, st>>>(n, h, m, h_min, h_max, err);
+    launch(k_check_input, nblk(n, 256), 256, 0, st, n, h, m, h_min, h_max, err);
     return cudaGetLastError();
 }
 
 cudaError_t launch_check_constants(int n, const double* h, const double* m, const double* s0, const int8_t* kind,
                                    uint32_t* varies, cudaStream_t st)
 {
-    k_check_constants<<<nblk(n, 256), 256, 0, st>>>(n, h, m, s0, kind, varies);
+    launch(k_check_constants, nblk(n, 256), 256, 0, st, n, h, m, s0, kind, varies);
     return cudaGetLastError();
 }
 
 cudaError_t launch_scalar_in(int prec, int n, const double* src, const int8_t* kind, void* dst, cudaStream_t st)
 {
-    if (prec == 64) k_scalar_in<double><<<nblk(n, 256), 256, 0, st>>>(n, src, kind, (double*)dst);
-    else k_scalar_in<float><<<nblk(n, 256), 256, 0, st>>>(n, src, kind, (float*)dst);
+    if (prec == 64) launch(k_scalar_in<double>, nblk(n, 256), 256, 0, st, n, src, kind, (double*)dst);
+    else launch(k_scalar_in<float>, nblk(n, 256), 256, 0, st, n, src, kind, (float*)dst);
     return cudaGetLastError();
 }
 
 cudaError_t launch_scalar_out(int prec, int n, const void* src, const int32_t* id, double* dst, cudaStream_t st)
 {
-    if (prec == 64) k_scalar_out<double><<<nblk(n, 256), 256, 0, st>>>(n, (const double*)src, id, dst);
-    else k_scalar_out<float><<<nblk(n, 256), 256, 0, st>>>(n, (const float*)src, id, dst);
+    if (prec == 64) launch(k_scalar_out<double>, nblk(n, 256), 256, 0, st, n, (const double*)src, id, dst);
+    else launch(k_scalar_out<float>, nblk(n, 256), 256, 0, st, n, (const float*)src, id, dst);
     return cudaGetLastError();
 }
 

@@ -144,7 +144,7 @@ __device__ __forceinline__ float prefilter2(const Consts<double>& K, float hi_f,
 // pass.
 template <int DIM>
 __device__ __forceinline__ void density64_end(int n, int i, const Consts<double>& K, const StateSet<double>& S,
-                                              double sigma, double4_32a* __restrict__ vr, double* __restrict__ vol)
+                                              double sigma, double4_32a* vr, double* vol)
 {
     double vi[3] = {0, 0, 0};
 #pragma unroll
@@ -170,10 +170,10 @@ __device__ __forceinline__ void density64_end(int n, int i, const Consts<double>
 // and the count (which may exceed cap); the FP64 force pass walks it.
 template <int DIM>
 __device__ __forceinline__ double density64_thread(int n, int i, const StateSet<double>& S,
-                                                   const int32_t* __restrict__ start, const Grid& G,
-                                                   const Consts<double>& K, const float4* __restrict__ pos4,
-                                                   const int32_t* __restrict__ cell_of, uint32_t* __restrict__ nbl,
-                                                   int32_t* __restrict__ nbc, int cap, bool two_pass)
+                                                   const int32_t* start, const Grid& G,
+                                                   const Consts<double>& K, const float4* pos4,
+                                                   const int32_t* cell_of, uint32_t* nbl,
+                                                   int32_t* nbc, int cap, bool two_pass)
 {
     const float4 pi = pos4[i];
     const float oi[3] = {pi.x, pi.y, pi.z};
@@ -240,7 +240,7 @@ struct RowRuns {
 // offset oi, cut as for_candidates_rows cuts it.
 template <int DIM>
 __device__ __forceinline__ RowRuns row_runs(int r, const float* oi, float reach, const int* c, const Grid& G,
-                                            const int32_t* __restrict__ start)
+                                            const int32_t* start)
 {
     constexpr int R = kStencilR;
     RowRuns q = {0, 0, 0, 0, 0};
@@ -256,7 +256,7 @@ __device__ __forceinline__ RowRuns row_runs(int r, const float* oi, float reach,
     const float w2 = (reach * reach - rz * rz) - ry * ry;
     if (cy < 0 || cz < 0 || !(w2 > 0.f)) return q;
     const int sh = G.sub_shift, nsx = G.nc[0] << sh;
-    const int32_t* __restrict__ rstart = sh ? G.sub_start : start;
+    const int32_t* rstart = sh ? G.sub_start : start;
     const float inv_exs = (1.f / ex) * (float)(1 << sh);
     const float w = sqrt_approx(w2) + 1e-3f * ex;
     const int slo = max(__float2int_rd((oi[0] - w) * inv_exs), -(R << sh));
@@ -299,12 +299,12 @@ __device__ __forceinline__ RowRuns row_runs(int r, const float* oi, float reach,
 // the lane's part of sigma.  Called by whole warps; `active` is the same for
 // all lanes of a group.
 template <int DIM, int L>
-__device__ __forceinline__ double density64_group(int n, int i, bool active, RowRuns* __restrict__ rows,
-                                                  const StateSet<double>& S, const int32_t* __restrict__ start,
+__device__ __forceinline__ double density64_group(int n, int i, bool active, RowRuns* rows,
+                                                  const StateSet<double>& S, const int32_t* start,
                                                   const Grid& G, const Consts<double>& K,
-                                                  const float4* __restrict__ pos4,
-                                                  const int32_t* __restrict__ cell_of, uint32_t* __restrict__ nbl,
-                                                  int32_t* __restrict__ nbc, int cap)
+                                                  const float4* pos4,
+                                                  const int32_t* cell_of, uint32_t* nbl,
+                                                  int32_t* nbc, int cap)
 {
     constexpr int R = kStencilR, NR = DIM == 3 ? kSide * kSide : kSide;
     constexpr unsigned kAll = 0xffffffffu;
@@ -384,11 +384,12 @@ __device__ __forceinline__ double density64_group(int n, int i, bool active, Row
 
 template <int DIM, int L>
 __global__ void __launch_bounds__(Lanes<L>::kThreads, L == 1 ? 4 : 1) k_density_f64(int n, StateSet<double> S,
-                                                     const int32_t* __restrict__ start, Grid G, Consts<double> K,
-                                                     double4_32a* __restrict__ vr, const float4* __restrict__ pos4,
-                                                     const int32_t* __restrict__ cell_of, uint32_t* __restrict__ nbl,
-                                                     int32_t* __restrict__ nbc, int cap, double* __restrict__ vol)
+                                                     const int32_t* start, Grid G, Consts<double> K,
+                                                     double4_32a* vr, const float4* pos4,
+                                                     const int32_t* cell_of, uint32_t* nbl,
+                                                     int32_t* nbc, int cap, double* vol)
 {
+    pdl_wait();
     if constexpr (L == 1) {
         const int i = blockIdx.x * blockDim.x + threadIdx.x;
         if (i >= n) return;
@@ -426,11 +427,11 @@ __global__ void __launch_bounds__(Lanes<L>::kThreads, L == 1 ? 4 : 1) k_density_
 // holds) and this thread is the one that scans them.
 template <int DIM>
 __device__ __forceinline__ void forces64_sums(int n, int i, const StateSet<double>& S,
-                                              const int32_t* __restrict__ start, const Grid& G,
-                                              const Consts<double>& K, const double4_32a* __restrict__ vr,
-                                              const int32_t* __restrict__ cell_of,
-                                              const uint32_t* __restrict__ nbl, int cnt, int cap, int k0, int dk,
-                                              const double* __restrict__ vol, PairSums64<DIM>& sums)
+                                              const int32_t* start, const Grid& G,
+                                              const Consts<double>& K, const double4_32a* vr,
+                                              const int32_t* cell_of,
+                                              const uint32_t* nbl, int cnt, int cap, int k0, int dk,
+                                              const double* vol, PairSums64<DIM>& sums)
 {
     double xi[3] = {0, 0, 0}, vi[3] = {0, 0, 0};
     const double4_32a me = vr[i];
@@ -535,16 +536,17 @@ __device__ __forceinline__ void forces64_sums(int n, int i, const StateSet<doubl
 // particle adds them in lane order and ends the particle's step.
 template <int DIM, int L>
 __global__ void __launch_bounds__(Lanes<L>::kThreads, L == 1 ? 2 : 1) k_forces_f64(int n, StateSet<double> S,
-                                                    const int32_t* __restrict__ start, Grid G, Consts<double> K,
-                                                    const double4_32a* __restrict__ vr,
-                                                    const int32_t* __restrict__ cell_of,
-                                                    const uint32_t* __restrict__ nbl, const int32_t* __restrict__ nbc,
+                                                    const int32_t* start, Grid G, Consts<double> K,
+                                                    const double4_32a* vr,
+                                                    const int32_t* cell_of,
+                                                    const uint32_t* nbl, const int32_t* nbc,
                                                     int cap, const double* dt_ptr, int kick_on,
-                                                    int write_ad, double* __restrict__ Rout,
-                                                    double* __restrict__ chi_out, GridSum B, DtConsts Dc,
-                                                    double* __restrict__ diag, double* dt_next, int count_step,
-                                                    const double* __restrict__ vol)
+                                                    int write_ad, double* Rout,
+                                                    double* chi_out, GridSum B, DtConsts Dc,
+                                                    double* diag, double* dt_next, int count_step,
+                                                    const double* vol)
 {
+    pdl_wait();
     const int P = blockDim.x / L;
     PairSums64<DIM> sums;
     if constexpr (L == 1) {
@@ -662,8 +664,9 @@ __global__ void __launch_bounds__(Lanes<L>::kThreads, L == 1 ? 2 : 1) k_forces_f
 // used when the caller supplied a and dr, so no force pass is needed.
 template <typename Real, int DIM>
 __global__ void __launch_bounds__(256) k_diag_only(int n, StateSet<Real> S, GridSum B, DtConsts D,
-                                                   double* __restrict__ diag, double* dt_next, int count_step)
+                                                   double* diag, double* dt_next, int count_step)
 {
+    pdl_wait();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     double part[kNPart];
 #pragma unroll
@@ -690,9 +693,10 @@ __global__ void __launch_bounds__(256) k_diag_only(int n, StateSet<Real> S, Grid
 }
 
 // The rows of a large grid (see GridSum), and the end of the step.
-__global__ void __launch_bounds__(256) k_fold_step(GridSum B, int nrows, DtConsts D, double* __restrict__ diag,
+__global__ void __launch_bounds__(256) k_fold_step(GridSum B, int nrows, DtConsts D, double* diag,
                                                    double* dt_ptr, int count_step)
 {
+    pdl_wait();
     __shared__ double total[kNPart];
     if (fold_grid(B, nrows, total)) finish_step(total, D, diag, dt_ptr, count_step);
 }
@@ -765,7 +769,7 @@ cudaError_t launch_density(int prec, int dim, int n, void* S, const int32_t* sta
     const size_t smem = Q.L == 1 ? 0 : ((size_t)(Q.T / Q.L) * (dim == 3 ? kSide * kSide : kSide) * sizeof(RowRuns) + 15) / 16 * 16 +
                                            Q.T * sizeof(double);
     auto kern = dim == 2 ? SPH_LANES64(k_density_f64, 2, Q.L) : SPH_LANES64(k_density_f64, 3, Q.L);
-    kern<<<Q.blocks, Q.T, smem, st>>>(n, s, start, G, k, (double4_32a*)vr, pos4, cell_of, nbl, nbc, cap, vol);
+    launch(kern, Q.blocks, Q.T, smem, st, n, s, start, G, k, (double4_32a*)vr, pos4, cell_of, nbl, nbc, cap, vol);
     return cudaGetLastError();
 }
 
@@ -785,7 +789,7 @@ cudaError_t launch_forces(int prec, int dim, int n, void* S, const int32_t* star
     const DtConsts D = dt_consts(*F.P);
     const size_t smem = Q.L == 1 ? 0 : (size_t)3 * dim * Q.T * sizeof(double);
     auto kern = dim == 2 ? SPH_LANES64(k_forces_f64, 2, Q.L) : SPH_LANES64(k_forces_f64, 3, Q.L);
-    kern<<<Q.blocks, Q.T, smem, st>>>(n, s, start, G, k, (const double4_32a*)vr, cell_of, nbl, nbc, cap, F.dt, kick_on,
+    launch(kern, Q.blocks, Q.T, smem, st, n, s, start, G, k, (const double4_32a*)vr, cell_of, nbl, nbc, cap, F.dt, kick_on,
                                       write_ad, (double*)Rout, (double*)chi, B, D, F.diag, F.dt, F.count_step, vol);
     return cudaGetLastError();
 }
@@ -796,7 +800,7 @@ cudaError_t launch_finish_step(int prec, int n, int sms, const FinishArgs& F, cu
     const int nb = pair_blocks(prec, n, sms);
     const GridSum B = grid_sum(F, nb);
     if (B.group) return cudaSuccess;      // the pass folded its partials itself
-    k_fold_step<<<kFoldBlocks, 256, 0, st>>>(B, nb, dt_consts(*F.P), F.diag, F.dt, F.count_step);
+    launch(k_fold_step, kFoldBlocks, 256, 0, st, B, nb, dt_consts(*F.P), F.diag, F.dt, F.count_step);
     ++*launches;
     return cudaGetLastError();
 }
@@ -808,12 +812,12 @@ cudaError_t launch_diag_only(int prec, int dim, int n, void* S, const FinishArgs
     const DtConsts D = dt_consts(*F.P);
     if (prec == 64) {
         auto s = *(StateSet<double>*)S;
-        if (dim == 2) k_diag_only<double, 2><<<nblk(n, T), T, 0, st>>>(n, s, B, D, F.diag, F.dt, F.count_step);
-        else k_diag_only<double, 3><<<nblk(n, T), T, 0, st>>>(n, s, B, D, F.diag, F.dt, F.count_step);
+        if (dim == 2) launch(k_diag_only<double, 2>, nblk(n, T), T, 0, st, n, s, B, D, F.diag, F.dt, F.count_step);
+        else launch(k_diag_only<double, 3>, nblk(n, T), T, 0, st, n, s, B, D, F.diag, F.dt, F.count_step);
     } else {
         auto s = *(StateSet<float>*)S;
-        if (dim == 2) k_diag_only<float, 2><<<nblk(n, T), T, 0, st>>>(n, s, B, D, F.diag, F.dt, F.count_step);
-        else k_diag_only<float, 3><<<nblk(n, T), T, 0, st>>>(n, s, B, D, F.diag, F.dt, F.count_step);
+        if (dim == 2) launch(k_diag_only<float, 2>, nblk(n, T), T, 0, st, n, s, B, D, F.diag, F.dt, F.count_step);
+        else launch(k_diag_only<float, 3>, nblk(n, T), T, 0, st, n, s, B, D, F.diag, F.dt, F.count_step);
     }
     return cudaGetLastError();
 }

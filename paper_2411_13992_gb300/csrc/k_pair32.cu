@@ -188,8 +188,8 @@ __device__ __forceinline__ void list_take(const uint32_t* base_i, int& cnt, floa
 // along x and the run bounds need no case analysis.
 template <int DIM, typename Acc, bool INNER>
 __device__ __forceinline__ void density_rows(const float* oi, const int* c, const Grid& G, const Consts<float>& K,
-                                             float wnorm, const int32_t* __restrict__ rstart,
-                                             const float4* __restrict__ pos4c, Acc& sigma, int& cnt,
+                                             float wnorm, const int32_t* rstart,
+                                             const float4* pos4c, Acc& sigma, int& cnt,
                                              const uint32_t* base_i, int n, int cap)
 {
     constexpr int R = kStencilR, zr = DIM == 3 ? R : 0;
@@ -321,13 +321,14 @@ __device__ __forceinline__ void density_rows(const float* oi, const int* c, cons
 // 7 % longer early in the run and 25 % longer after step 400.
 constexpr int kDensityTPB32 = 512;
 template <int DIM, typename Acc, bool UNIFORM>
-__global__ void __launch_bounds__(kDensityTPB32, 2) k_density32(int n, const float4* __restrict__ pos4,
-                                                      const int32_t* __restrict__ cell_of,
-                                                      const int32_t* __restrict__ start, Grid G, Consts<float> K,
-                                                      StateSet<float> S, float4* __restrict__ vr,
-                                                      uint32_t* __restrict__ nbl, int32_t* __restrict__ nbc, int cap,
-                                                      const float4* __restrict__ pos4c)
+__global__ void __launch_bounds__(kDensityTPB32, 2) k_density32(int n, const float4* pos4,
+                                                      const int32_t* cell_of,
+                                                      const int32_t* start, Grid G, Consts<float> K,
+                                                      StateSet<float> S, float4* vr,
+                                                      uint32_t* nbl, int32_t* nbc, int cap,
+                                                      const float4* pos4c)
 {
+    pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     // every load of the particle's own data first: they are independent
@@ -501,8 +502,8 @@ struct TileView {
 // particles' offsets (when they fit), and the home-row prefix counts.  Every
 // thread of the block calls it; it ends with a barrier.
 template <int DIM, int T>
-__device__ __forceinline__ void stage_tile(TileView& V, const Grid& G, const int32_t* __restrict__ start,
-                                           const float4* __restrict__ pos4c, int nb0, int nb1, int tile_cap,
+__device__ __forceinline__ void stage_tile(TileView& V, const Grid& G, const int32_t* start,
+                                           const float4* pos4c, int nb0, int nb1, int tile_cap,
                                            int* s_warp)
 {
     using TD = TileDims<DIM>;
@@ -629,9 +630,9 @@ __device__ __forceinline__ float tile_r2(const float* oi, int hx_i, const float4
 
 template <int DIM, typename Acc>
 __global__ void __launch_bounds__(TileThreads<DIM>::WALK) k_density32_tile(
-    int n, const float4* __restrict__ pos4c, const int32_t* __restrict__ cell_of, const int32_t* __restrict__ start,
-    Grid G, Consts<float> K, StateSet<float> S, float4* __restrict__ vr, uint32_t* __restrict__ nbl,
-    int32_t* __restrict__ nbc, int cap, int nb0, int nb1, int tile_cap)
+    int n, const float4* pos4c, const int32_t* cell_of, const int32_t* start,
+    Grid G, Consts<float> K, StateSet<float> S, float4* vr, uint32_t* nbl,
+    int32_t* nbc, int cap, int nb0, int nb1, int tile_cap)
 {
     using TD = TileDims<DIM>;
     constexpr int T = TileThreads<DIM>::WALK, R = TD::R, H0 = TD::H0, H1 = TD::H1, NHC = TD::NHC;
@@ -749,9 +750,9 @@ __host__ __device__ constexpr size_t flat_table_bytes()
 
 template <int DIM, typename Acc>
 __global__ void __launch_bounds__(FlatShape<DIM>::T) k_density32_flat(
-    int n, const float4* __restrict__ pos4c, const int32_t* __restrict__ cell_of, const int32_t* __restrict__ start,
-    Grid G, Consts<float> K, StateSet<float> S, float4* __restrict__ vr, uint32_t* __restrict__ nbl,
-    int32_t* __restrict__ nbc, int cap, int nb0, int nb1, int tile_cap)
+    int n, const float4* pos4c, const int32_t* cell_of, const int32_t* start,
+    Grid G, Consts<float> K, StateSet<float> S, float4* vr, uint32_t* nbl,
+    int32_t* nbc, int cap, int nb0, int nb1, int tile_cap)
 {
     using TD = TileDims<DIM>;
     constexpr int T = FlatShape<DIM>::T, NR = FlatShape<DIM>::NR, R = TD::R, H0 = TD::H0, H1 = TD::H1, NHC = TD::NHC;
@@ -917,9 +918,9 @@ template <> struct PartialSum<PlainF> {
 
 template <int DIM, typename Acc>
 __global__ void __launch_bounds__(TileThreads<DIM>::COOP, 4) k_density32_coop(
-    int n, const float4* __restrict__ pos4c, const int32_t* __restrict__ cell_of, const int32_t* __restrict__ start,
-    Grid G, Consts<float> K, StateSet<float> S, float4* __restrict__ vr, uint32_t* __restrict__ nbl,
-    int32_t* __restrict__ nbc, int cap, int nb0, int nb1, int tile_cap)
+    int n, const float4* pos4c, const int32_t* cell_of, const int32_t* start,
+    Grid G, Consts<float> K, StateSet<float> S, float4* vr, uint32_t* nbl,
+    int32_t* nbc, int cap, int nb0, int nb1, int tile_cap)
 {
     using TD = TileDims<DIM>;
     using C = CoopShape<DIM>;
@@ -1126,17 +1127,18 @@ __global__ void __launch_bounds__(TileThreads<DIM>::COOP, 4) k_density32_coop(
 // Variable resolution keeps eight blocks (64 registers) and one pair ahead:
 // at six blocks its pass ran 10 % longer.
 template <int DIM, typename Acc, bool UNIFORM>
-__global__ void __launch_bounds__(kTPB32, UNIFORM ? 6 : 8) k_forces32(int n, const float4* __restrict__ pos4,
-                                                     const int32_t* __restrict__ cell_of,
-                                                     const int32_t* __restrict__ start, Grid G, Consts<float> K,
-                                                     StateSet<float> S, const float* __restrict__ mf,
-                                                     const float4* __restrict__ vr, const uint32_t* __restrict__ nbl,
-                                                     const int32_t* __restrict__ nbc, int cap,
+__global__ void __launch_bounds__(kTPB32, UNIFORM ? 6 : 8) k_forces32(int n, const float4* pos4,
+                                                     const int32_t* cell_of,
+                                                     const int32_t* start, Grid G, Consts<float> K,
+                                                     StateSet<float> S, const float* mf,
+                                                     const float4* vr, const uint32_t* nbl,
+                                                     const int32_t* nbc, int cap,
                                                      const double* dt_ptr, int kick_on, int write_ad,
-                                                     float* __restrict__ Rout, float* __restrict__ chi_out,
-                                                     GridSum B, DtConsts D, double* __restrict__ diag,
+                                                     float* Rout, float* chi_out,
+                                                     GridSum B, DtConsts D, double* diag,
                                                      double* dt_next, int count_step)
 {
+    pdl_wait();
     __shared__ float4 tab[kCodes];
     for (int t = threadIdx.x; t < kCodes; t += blockDim.x) {
         float sh[3];
@@ -1353,7 +1355,7 @@ static void density_t(int n, const float4* pos4, const int32_t* cell_of, const i
                       cudaStream_t st, const float4* pos4c)
 {
     const int T = n >= G.sms * kDensityTPB32 ? kDensityTPB32 : pair_threads(32, n, G.sms);
-    k_density32<DIM, Acc, U><<<nblk(n, T), T, 0, st>>>(n, pos4, cell_of, start, G, K, S, vr, nbl, nbc,
+    launch(k_density32<DIM, Acc, U>, nblk(n, T), T, 0, st, n, pos4, cell_of, start, G, K, S, vr, nbl, nbc,
                                                        nbl_capacity(DIM), pos4c);
 }
 
@@ -1402,7 +1404,7 @@ static void forces_t(int n, const float4* pos4, const int32_t* cell_of, const in
                      const FinishArgs& F, cudaStream_t st)
 {
     const int T = pair_threads(32, n, G.sms);
-    k_forces32<DIM, Acc, U><<<nblk(n, T), T, 0, st>>>(n, pos4, cell_of, start, G, K, S, mf, vr, nbl, nbc,
+    launch(k_forces32<DIM, Acc, U>, nblk(n, T), T, 0, st, n, pos4, cell_of, start, G, K, S, mf, vr, nbl, nbc,
                                                       nbl_capacity(DIM), F.dt, kick_on, write_ad, Rout, chi,
                                                       grid_sum(F, nblk(n, T)), dt_consts(*F.P), F.diag, F.dt,
                                                       F.count_step);

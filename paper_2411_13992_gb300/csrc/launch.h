@@ -10,6 +10,29 @@
 
 namespace sphtv {
 
+// Launch with programmatic stream serialization: the kernel is placed as the
+// blocks of the one before it exit, without the full drain and flush of a
+// plain launch in between, and waits for that kernel's end in pdl_wait(),
+// which every kernel launched this way calls before anything else.  Measured
+// against plain launches of the same kernels: dual-criteria advection step of
+// the 200^2 cavity 192 -> 144 us, rollout 256^2 3.71 -> 3.51 ms, steps
+// replayed from a graph 1-3 % (cavity 256^2 43.2 -> 42.2 us).
+template <typename... P, typename... A>
+inline cudaError_t launch(void (*kern)(P...), int grid, int block, size_t smem, cudaStream_t st, A&&... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
 // Forward values of one step kept for the adjoint (device pointers).
 struct TapeView {
     const int32_t* id;

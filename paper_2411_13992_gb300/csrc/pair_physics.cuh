@@ -410,8 +410,8 @@ struct DtConsts {
 
 // Diagnostics and the next step size of a kick-drift-kick step (or of
 // sph_build_cells, count_step = 0) from the grid's totals.
-__device__ __forceinline__ void finish_step(const double* out, const DtConsts& D, double* __restrict__ diag,
-                                            double* __restrict__ dt_ptr, int count_step)
+__device__ __forceinline__ void finish_step(const double* out, const DtConsts& D, double* diag,
+                                            double* dt_ptr, int count_step)
 {
     const double dt_used = *dt_ptr;
     __syncthreads();                      // thread 0 writes *dt_ptr below

@@ -19,8 +19,8 @@ namespace sphtv {
 // the loads of pos4 are warp broadcasts.
 template <int DIM, typename F>
 __device__ __forceinline__ void for_candidates(const float* oi, int cell_i, const Grid& G,
-                                               const int32_t* __restrict__ start,
-                                               const float4* __restrict__ pos4, F& f)
+                                               const int32_t* start,
+                                               const float4* pos4, F& f)
 {
     int c[3];
     cell_decode(G, cell_i, c);
@@ -84,9 +84,9 @@ __device__ __forceinline__ void for_candidates(const float* oi, int cell_i, cons
 // from cell_of.
 template <int DIM, bool TWO = true, bool CELL_IN_W = false, typename F>
 __device__ __forceinline__ void for_candidates_rows(const float* oi, float reach, int cell_i, const Grid& G,
-                                                    const int32_t* __restrict__ start,
-                                                    const int32_t* __restrict__ cell_of,
-                                                    const float4* __restrict__ pos4, F& f)
+                                                    const int32_t* start,
+                                                    const int32_t* cell_of,
+                                                    const float4* pos4, F& f)
 {
     int c[3];
     cell_decode(G, cell_i, c);
@@ -98,7 +98,7 @@ __device__ __forceinline__ void for_candidates_rows(const float* oi, float reach
     // the x cut in sub-cells (s = 0: cells): nsx along a row, the stencil's
     // sub-cells -R 2^s .. (R + 1) 2^s - 1 around the first of cell c[0]
     const int sh = G.sub_shift;
-    const int32_t* __restrict__ rstart = sh ? G.sub_start : start;
+    const int32_t* rstart = sh ? G.sub_start : start;
     const int nsx = ncx << sh;
     const float inv_exs = inv_ex * (float)(1 << sh);   // exact: a power of two
     for (int dz = -zr; dz <= zr; ++dz) {
