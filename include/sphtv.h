@@ -137,7 +137,8 @@ typedef struct sph_params {
     int32_t integrator;     /* SPH_INT_*: kick-drift-kick (default) or dual-criteria;
                                SPH_INT_DUAL requires fixed_dt = 0 */
     int32_t graphs;         /* 1 (default): sph_step replays kick-drift-kick steps two at a
-                               time from a captured CUDA graph on a library-owned stream,
+                               time (8 at a time in calls of 16 steps or more)
+                               from a captured CUDA graph on a library-owned stream,
                                ordered after and before the context's stream by events
                                (same results, fewer launches); 0: always launch directly */
     int32_t pair_tiles;     /* FP32 form at uniform resolution (h_min == h_max), the density

@@ -60,10 +60,6 @@ __device__ __forceinline__ void group_sum(PlainD& a)
     for (int o = L / 2; o >= 1; o >>= 1) a.s += __shfl_xor_sync(0xffffffffu, a.s, o);
 }
 
-// A compensated sum as a double keeps its compensation: s - c.
-__device__ __forceinline__ double wide_value(const KSum& a) { return (double)a.s - (double)a.c; }
-__device__ __forceinline__ double wide_value(const PlainD& a) { return a.s; }
-
 // The cotangents Abar_k and Rbar_k of a particle as one record of
 // kAbStride<DIM> values ({Abar, Rbar}, padded to a whole number of 16-byte
 // vectors in the FP32 form), so that the pair kernel gathers a neighbour's
@@ -394,7 +390,8 @@ __global__ void __launch_bounds__(kAdjTPB) k_adj_pairs(int n, Tape<Real> T, Grid
     using Acc = AccOf<Real>;
     const int k = (blockIdx.x * blockDim.x + threadIdx.x) / L, q = threadIdx.x % L;
     const bool fluid = k < n && !T.kind[k];
-    Acc ax[DIM], av[DIM], arho, aeta;
+    Acc ax[DIM], av[DIM], arho;
+    double eta = 0.0;
     if (fluid) {
         const auto mk = T.vr[k];
         const Real vk[3] = {mk.x, mk.y, mk.z};
@@ -423,7 +420,7 @@ __global__ void __launch_bounds__(kAdjTPB) k_adj_pairs(int n, Tape<Real> T, Grid
                 av[d].add(dvb[d]);
             }
             arho.add(wall ? rib + rjb : rib);
-            aeta.add(eb);
+            eta += (double)eb;
             if (wall) return;
             // the fluid neighbour's sums (j as i, k as j): r_jk = -r_kj
             Real Aj[3] = {0, 0, 0}, Rj[3] = {0, 0, 0}, mrv[3] = {0, 0, 0};
@@ -440,7 +437,6 @@ __global__ void __launch_bounds__(kAdjTPB) k_adj_pairs(int n, Tape<Real> T, Grid
         adj_visit<Real, DIM, L>(n, k, q, G, K, T, pair);
     }
     __syncwarp();
-    double eta = wide_value(aeta);          // every lane's own part
 #pragma unroll
     for (int d = 0; d < DIM; ++d) {
         group_sum<L>(ax[d]);
@@ -571,37 +567,7 @@ __global__ void __launch_bounds__(256) k_save_tape(int n, int nstart, StateSet<R
     if (sizeof(Real) == 4) const_cast<float4*>(T.pos4)[i] = pos4[i];
 }
 
-// ----------------------------------------------------- cotangent layouts
-
-__global__ void k_aos_to_soa(int n, const double* src3, double* dst)
-{
-    pdl_wait();
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    for (int d = 0; d < 3; ++d) dst[(size_t)d * n + i] = src3[3 * (size_t)i + d];
-}
-
-__global__ void k_soa_to_aos(int n, const double* src, double* dst3)
-{
-    pdl_wait();
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    for (int d = 0; d < 3; ++d) dst3[3 * (size_t)i + d] = src[(size_t)d * n + i];
-}
-
 // -------------------------------------------------------------- launchers
-
-cudaError_t launch_aos_to_soa(int n, const double* src3, double* dst, cudaStream_t st)
-{
-    launch(k_aos_to_soa, (n + 255) / 256, 256, 0, st, n, src3, dst);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_soa_to_aos(int n, const double* src, double* dst3, cudaStream_t st)
-{
-    launch(k_soa_to_aos, (n + 255) / 256, 256, 0, st, n, src, dst3);
-    return cudaGetLastError();
-}
 
 static inline int nblk(int n, int t) { return (n + t - 1) / t; }
 

@@ -1,7 +1,7 @@
-// k_io.cu -- state transfer kernels of libsphtv: caller [n][3] rows <->
-// per-component arrays, un-permuting from the cell order back to the
-// caller's order, wall velocities, and the per-particle reference sums
-// sigma0 of Eq. 8 (the perfect-lattice sum at the particle's own spacing
+// k_io.cu -- state transfer kernels of libsphtv: the load of a state in the
+// caller's order ([n][3] rows into per-component arrays, wall velocities, the
+// input checks), the way back from the cell order, the adjoint's cotangents,
+// and the per-particle reference sums sigma0 of Eq. 8 (the perfect-lattice sum at the particle's own spacing
 // dp = (m/rho0)^(1/D) and smoothing length h).
 #include "common.cuh"
 #include "launch.h"
@@ -16,18 +16,6 @@ __global__ void k_vec_in(int n, const double* src3, Real* dst)
     if (i >= n) return;
 #pragma unroll
     for (int d = 0; d < DIM; ++d) dst[(size_t)d * n + i] = (Real)src3[3 * (size_t)i + d];
-}
-
-template <typename Real, int DIM>
-__global__ void k_vec_out(int n, const Real* src, const int32_t* id,
-                          double* dst3)
-{
-    pdl_wait();
-    int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n) return;
-    size_t o = 3 * (size_t)id[k];
-#pragma unroll
-    for (int d = 0; d < 3; ++d) dst3[o + d] = d < DIM ? (double)src[(size_t)d * n + k] : 0.0;
 }
 
 // pos[id[k]] = k: where the particle the caller gave as number i sits in
@@ -65,24 +53,6 @@ __global__ void k_rho_out_gather(int n, const V4* vr, const int8_t* kind,
     dst[i] = kind[k] ? rho0 : rho0 + (double)vr[k].w;
 }
 
-template <typename Real, int DIM>
-__global__ void k_walls_velocity(int n, const int8_t* kind, const double* vw3,
-                                 Real* v)
-{
-    pdl_wait();
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || !kind[i]) return;
-#pragma unroll
-    for (int d = 0; d < DIM; ++d) v[(size_t)d * n + i] = vw3 ? (Real)vw3[3 * (size_t)i + d] : Real(0);
-}
-
-__global__ void k_init_ids(int n, int32_t* id)
-{
-    pdl_wait();
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) id[i] = i;
-}
-
 template <int DIM>
 __device__ double sigma0_of(double h, double m, double rho0)
 {
@@ -107,26 +77,187 @@ __device__ double sigma0_of(double h, double m, double rho0)
     return s / (DIM == 2 ? dp * dp : dp * dp * dp);
 }
 
-// The reference sum depends on (h, m) only: particle 0's value is computed
-// once (k_sigma0_first) and copied to every particle with the same h and m;
-// the others compute their own (the lattice sum is FP64 work, and FP64 runs
-// at 1/74 of the FP32 rate).
+// sigma0_of by a whole warp for one (h, m): one lattice point per lane, the
+// terms added in sigma0_of's order (the products by 2, 4 and 8 are exact, so
+// the sum is sigma0_of's bit for bit).  FP64 work: a thread's own sum takes
+// some 400 operations, a warp's shared one about 60.
 template <int DIM>
-__global__ void k_sigma0_first(const double* h, const double* m, double rho0,
-                               double* s0)
+__device__ __forceinline__ double sigma0_shared(double h, double m, double rho0)
 {
-    pdl_wait();
-    if (blockIdx.x == 0 && threadIdx.x == 0) s0[0] = sigma0_of<DIM>(h[0], m[0], rho0);
+    const double vol = m / rho0;
+    const double dp = DIM == 2 ? sqrt(vol) : cbrt(vol);
+    const double ratio = h / dp;
+    const double reach2 = 4.0 * ratio * ratio;
+    const int side = (int)ceil(2.0 * ratio) + 1;
+    const double inv = 1.0 / ratio;
+    const int points = DIM == 3 ? side * side * side : side * side, lane = threadIdx.x & 31;
+    double s = 0.0;
+    for (int base = 0; base < points; base += 32) {
+        const int p = base + lane;
+        const int kx = p % side, ky = (p / side) % side, kz = p / (side * side);
+        const double r2 = (double)(kx * kx + ky * ky + kz * kz);
+        double term = 0.0;
+        if (p < points && r2 < reach2) {
+            const double mult = (kx ? 2.0 : 1.0) * (ky ? 2.0 : 1.0) * (kz ? 2.0 : 1.0);
+            term = mult * wendland_W<DIM, double>(sqrt(r2), inv);
+        }
+        for (int t = 0; t < min(32, points - base); ++t) s += __shfl_sync(0xffffffffu, term, t);
+    }
+    return s / (DIM == 2 ? dp * dp : dp * dp * dp);
+}
+
+// The reference sum depends on (h, m) only: particle 0's value is computed
+// once, by one warp, and stands for every particle with the same h and m; the
+// others share theirs among the lanes of a warp that want the same one, or,
+// where a warp wants more than four, compute their own.
+template <int DIM>
+__device__ __forceinline__ double sigma0_in_warp(double h, double m, double rho0, bool want)
+{
+    const int lane = threadIdx.x & 31;
+    const unsigned same = __match_any_sync(0xffffffffu, __double_as_longlong(h)) &
+                          __match_any_sync(0xffffffffu, __double_as_longlong(m)) &
+                          __ballot_sync(0xffffffffu, want);
+    unsigned leaders = __ballot_sync(0xffffffffu, want && lane == __ffs(same) - 1);
+    double s0 = 0.0;
+    if (__popc(leaders) > 4) {
+        if (want) s0 = sigma0_of<DIM>(h, m, rho0);
+        return s0;
+    }
+    while (leaders) {
+        const int l = __ffs(leaders) - 1;
+        leaders &= leaders - 1;
+        const double v = sigma0_shared<DIM>(__shfl_sync(0xffffffffu, h, l), __shfl_sync(0xffffffffu, m, l), rho0);
+        if (want && (same >> l & 1u)) s0 = v;
+    }
+    return s0;
 }
 
 template <int DIM>
-__global__ void k_sigma0(int n, const double* h, const double* m, double rho0,
-                         double* s0)
+__global__ void k_sigma0_first(const double* h, const double* m, double rho0, double* s0_first, uint32_t* varies)
 {
     pdl_wait();
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < 1 || i >= n) return;
-    s0[i] = (h[i] == h[0] && m[i] == m[0]) ? s0[0] : sigma0_of<DIM>(h[i], m[i], rho0);
+    const double v = sigma0_shared<DIM>(h[0], m[0], rho0);
+    if (threadIdx.x == 0) {
+        *s0_first = v;
+        *varies = 0u;
+    }
+}
+
+// One particle's load, everything sph_set_state (or the adjoint's reload)
+// brings, in the caller's order: positions and velocities (walls: the
+// prescribed velocity) into the components, accelerations and displacements
+// or zeros, h, m, sigma0 and kind into both state sets (the sort leaves them
+// where they are when they do not vary), ids, the adjoint's copies; checks h
+// and m (h in [h_min, h_max], which sizes the cell edge; m positive and
+// finite) and sets *varies (cleared before) when a particle's h, m or sigma0
+// differs from particle 0's or a particle is a wall particle.  One kernel for
+// eight and the copies between them: loading 3,000 particles is launches, not
+// bytes.
+template <typename Real, int DIM>
+__global__ void __launch_bounds__(256) k_load_state(int n, LoadArgs A, StateSet<Real> S0, StateSet<Real> S1,
+                                                    double rho0, double h_min, double h_max, uint32_t* err)
+{
+    pdl_wait();
+    const int at = blockIdx.x * blockDim.x + threadIdx.x, i = min(at, n - 1);
+    const double h = A.h[i], m = A.m[i], h0 = A.h[0], m0 = A.m[0];
+    const int8_t kind = A.kind ? A.kind[i] : 0;
+    double s0, s00;
+    if (A.sigma0) {
+        s0 = A.sigma0[i];
+        s00 = A.sigma0[0];
+    } else {
+        s00 = s0 = *A.s0_first;
+        const bool other = h != h0 || m != m0;
+        if (__any_sync(0xffffffffu, other)) {
+            const double own = sigma0_in_warp<DIM>(h, m, rho0, other);
+            if (other) s0 = own;
+        }
+    }
+    const bool varies = kind != 0 || h != h0 || m != m0 || s0 != s00;
+    const unsigned b = __ballot_sync(0xffffffffu, varies);
+    if (b && (threadIdx.x & 31) == 0) atomicOr(err + 1, 1u);
+    if (at >= n) return;
+    if (!(h >= h_min && h <= h_max && m > 0.0 && isfinite(m))) atomicOr(err, ERRB_INPUT);
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) {
+        const size_t o = (size_t)d * n + i;
+        if (A.x) S0.x[o] = A.x[3 * (size_t)i + d];
+        if (kind) S0.v[o] = A.vw ? (Real)A.vw[3 * (size_t)i + d] : Real(0);
+        else if (A.v) S0.v[o] = (Real)A.v[3 * (size_t)i + d];
+        else if (A.zero_v) S0.v[o] = Real(0);
+        if (A.a) {
+            S0.a[o] = (Real)A.a[3 * (size_t)i + d];
+            S0.dr[o] = (Real)A.dr[3 * (size_t)i + d];
+        } else if (A.zero_ad) {
+            S0.a[o] = Real(0);
+            S0.dr[o] = Real(0);
+        }
+    }
+    S0.h[i] = S1.h[i] = h;
+    S0.m[i] = S1.m[i] = m;
+    S0.s0[i] = S1.s0[i] = s0;
+    S0.kind[i] = S1.kind[i] = kind;
+    S0.id[i] = i;
+    if (S0.drho) S0.drho[i] = Real(0);
+    if (A.orig_h) {
+        A.orig_h[i] = h;
+        A.orig_m[i] = m;
+        A.orig_s0[i] = s0;
+        A.orig_kind[i] = kind;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) A.orig_vw[3 * (size_t)i + d] = A.vw ? A.vw[3 * (size_t)i + d] : 0.0;
+    }
+}
+
+// The whole state out into device memory, in the caller's order (each of the
+// outputs may be null): one kernel for an inverse permutation and five
+// gathers.  The reads are in the sorted order, each particle's rows of 24
+// bytes go where its id says.
+template <typename Real, int DIM>
+__global__ void __launch_bounds__(256) k_store_state(int n, StateSet<Real> S, const typename Vec4<Real>::T* vr,
+                                                     double rho0, double* x, double* v, double* a, double* dr,
+                                                     double* rho)
+{
+    pdl_wait();
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    const size_t i = (size_t)S.id[k];
+    auto row = [&](double* dst, const auto* src) {
+        if (!dst) return;
+#pragma unroll
+        for (int d = 0; d < 3; ++d) dst[3 * i + d] = d < DIM ? (double)src[(size_t)d * n + k] : 0.0;
+    };
+    row(x, S.x);
+    row(v, S.v);
+    row(a, S.a);
+    row(dr, S.dr);
+    if (rho) rho[i] = S.kind[k] ? rho0 : rho0 + (double)vr[k].w;
+}
+
+// The adjoint's four cotangents between the caller's rows and [3][n]
+// (components past DIM are zero on the way in).
+__global__ void __launch_bounds__(256) k_cotangents_in(int n, int dim, Four<const double> src, Four<double> dst)
+{
+    pdl_wait();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        if (!src.p[q]) continue;
+        for (int d = 0; d < 3; ++d) dst.p[q][(size_t)d * n + i] = d < dim ? src.p[q][3 * (size_t)i + d] : 0.0;
+    }
+}
+
+__global__ void __launch_bounds__(256) k_cotangents_out(int n, Four<const double> src, Four<double> dst)
+{
+    pdl_wait();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        if (!dst.p[q]) continue;
+        for (int d = 0; d < 3; ++d) dst.p[q][3 * (size_t)i + d] = src.p[q][(size_t)d * n + i];
+    }
 }
 
 template <typename V4>
@@ -137,31 +268,6 @@ __global__ void k_rho_out(int n, const V4* vr, const int8_t* kind,
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
     dst[id[k]] = kind[k] ? rho0 : rho0 + (double)vr[k].w;
-}
-
-// Every h must lie in [h_min, h_max] (the cell edge is sized by h_max) and
-// every mass must be positive and finite.
-__global__ void k_check_input(int n, const double* h, const double* m, double h_min,
-                              double h_max, uint32_t* err)
-{
-    pdl_wait();
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    bool ok = h[i] >= h_min && h[i] <= h_max && m[i] > 0.0 && isfinite(m[i]);
-    if (!ok) atomicOr(err, ERRB_INPUT);
-}
-
-// Sets *varies (cleared by the caller) when a particle's h, m or sigma0
-// differs from particle 0's or a particle is a wall particle.
-__global__ void k_check_constants(int n, const double* h, const double* m,
-                                  const double* s0, const int8_t* kind, uint32_t* varies)
-{
-    pdl_wait();
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const bool v = kind[i] != 0 || h[i] != h[0] || m[i] != m[0] || s0[i] != s0[0];
-    const unsigned b = __ballot_sync(__activemask(), v);
-    if (b && (threadIdx.x & 31) == __ffs(b) - 1) atomicOr(varies, 1u);
 }
 
 template <typename Real>
@@ -199,50 +305,53 @@ cudaError_t launch_vec_in(int prec, int dim, int n, const double* src3, void* ds
     return cudaGetLastError();
 }
 
-cudaError_t launch_vec_out(int prec, int dim, int n, const void* src, const int32_t* id, double* dst3,
-                           cudaStream_t st)
+cudaError_t launch_load_state(int prec, int dim, int n, const LoadArgs& A, void* S0, void* S1, double rho0,
+                              double h_min, double h_max, uint32_t* err, cudaStream_t st, int64_t* launches)
 {
-    const int T = 256;
+    if (A.sigma0) {
+        const cudaError_t e = cudaMemsetAsync(err + 1, 0, sizeof(uint32_t), st);
+        if (e != cudaSuccess) return e;
+    } else {
+        launch(dim == 2 ? k_sigma0_first<2> : k_sigma0_first<3>, 1, 32, 0, st, A.h, A.m, rho0, A.s0_first, err + 1);
+        ++*launches;
+    }
+    const int T = 256, nb = nblk(n, T);
     if (prec == 64) {
-        if (dim == 2) launch(k_vec_out<double, 2>, nblk(n, T), T, 0, st, n, (const double*)src, id, dst3);
-        else launch(k_vec_out<double, 3>, nblk(n, T), T, 0, st, n, (const double*)src, id, dst3);
+        const auto a = *(const StateSet<double>*)S0, b = *(const StateSet<double>*)S1;
+        launch(dim == 2 ? k_load_state<double, 2> : k_load_state<double, 3>, nb, T, 0, st, n, A, a, b, rho0, h_min,
+               h_max, err);
     } else {
-        if (dim == 2) launch(k_vec_out<float, 2>, nblk(n, T), T, 0, st, n, (const float*)src, id, dst3);
-        else launch(k_vec_out<float, 3>, nblk(n, T), T, 0, st, n, (const float*)src, id, dst3);
+        const auto a = *(const StateSet<float>*)S0, b = *(const StateSet<float>*)S1;
+        launch(dim == 2 ? k_load_state<float, 2> : k_load_state<float, 3>, nb, T, 0, st, n, A, a, b, rho0, h_min,
+               h_max, err);
     }
+    ++*launches;
     return cudaGetLastError();
 }
 
-cudaError_t launch_walls_velocity(int prec, int dim, int n, const int8_t* kind, const double* vw3, void* v,
-                                  cudaStream_t st)
+cudaError_t launch_store_state(int prec, int dim, int n, const void* S, const void* vr, double rho0, double* x,
+                               double* v, double* a, double* dr, double* rho, cudaStream_t st)
 {
-    const int T = 256;
-    if (prec == 64) {
-        if (dim == 2) launch(k_walls_velocity<double, 2>, nblk(n, T), T, 0, st, n, kind, vw3, (double*)v);
-        else launch(k_walls_velocity<double, 3>, nblk(n, T), T, 0, st, n, kind, vw3, (double*)v);
-    } else {
-        if (dim == 2) launch(k_walls_velocity<float, 2>, nblk(n, T), T, 0, st, n, kind, vw3, (float*)v);
-        else launch(k_walls_velocity<float, 3>, nblk(n, T), T, 0, st, n, kind, vw3, (float*)v);
-    }
+    const int T = 256, nb = nblk(n, T);
+    if (prec == 64)
+        launch(dim == 2 ? k_store_state<double, 2> : k_store_state<double, 3>, nb, T, 0, st, n,
+               *(const StateSet<double>*)S, (const double4_32a*)vr, rho0, x, v, a, dr, rho);
+    else
+        launch(dim == 2 ? k_store_state<float, 2> : k_store_state<float, 3>, nb, T, 0, st, n,
+               *(const StateSet<float>*)S, (const float4*)vr, rho0, x, v, a, dr, rho);
     return cudaGetLastError();
 }
 
-cudaError_t launch_init_ids(int n, int32_t* id, cudaStream_t st)
+cudaError_t launch_cotangents_in(int n, int dim, const Four<const double>& src, const Four<double>& dst,
+                                 cudaStream_t st)
 {
-    launch(k_init_ids, nblk(n, 256), 256, 0, st, n, id);
+    launch(k_cotangents_in, nblk(n, 256), 256, 0, st, n, dim, src, dst);
     return cudaGetLastError();
 }
 
-cudaError_t launch_sigma0(int dim, int n, const double* h, const double* m, double rho0, double* s0,
-                          cudaStream_t st)
+cudaError_t launch_cotangents_out(int n, const Four<const double>& src, const Four<double>& dst, cudaStream_t st)
 {
-    if (dim == 2) {
-        launch(k_sigma0_first<2>, 1, 32, 0, st, h, m, rho0, s0);
-        launch(k_sigma0<2>, nblk(n, 128), 128, 0, st, n, h, m, rho0, s0);
-    } else {
-        launch(k_sigma0_first<3>, 1, 32, 0, st, h, m, rho0, s0);
-        launch(k_sigma0<3>, nblk(n, 128), 128, 0, st, n, h, m, rho0, s0);
-    }
+    launch(k_cotangents_out, nblk(n, 256), 256, 0, st, n, src, dst);
     return cudaGetLastError();
 }
 
@@ -280,20 +389,6 @@ cudaError_t launch_rho_out_gather(int prec, int n, const void* vr, const int8_t*
     if (prec == 64)
         launch(k_rho_out_gather<double4_32a>, nblk(n, 256), 256, 0, st, n, (const double4_32a*)vr, kind, pos, rho0, dst);
     else launch(k_rho_out_gather<float4>, nblk(n, 256), 256, 0, st, n, (const float4*)vr, kind, pos, rho0, dst);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_check_input(int n, const double* h, const double* m, double h_min, double h_max, uint32_t* err,
-                               cudaStream_t st)
-{
-    launch(k_check_input, nblk(n, 256), 256, 0, st, n, h, m, h_min, h_max, err);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_check_constants(int n, const double* h, const double* m, const double* s0, const int8_t* kind,
-                                   uint32_t* varies, cudaStream_t st)
-{
-    launch(k_check_constants, nblk(n, 256), 256, 0, st, n, h, m, s0, kind, varies);
     return cudaGetLastError();
 }
 

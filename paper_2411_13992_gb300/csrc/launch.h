@@ -131,13 +131,29 @@ cudaError_t launch_diag_only(int prec, int dim, int n, void* S, const FinishArgs
 
 // k_io.cu
 cudaError_t launch_vec_in(int prec, int dim, int n, const double* src3, void* dst, cudaStream_t st);
-cudaError_t launch_vec_out(int prec, int dim, int n, const void* src, const int32_t* id, double* dst3,
-                           cudaStream_t st);
-cudaError_t launch_walls_velocity(int prec, int dim, int n, const int8_t* kind, const double* vw3, void* v,
-                                  cudaStream_t st);
-cudaError_t launch_init_ids(int n, int32_t* id, cudaStream_t st);
-cudaError_t launch_sigma0(int dim, int n, const double* h, const double* m, double rho0, double* s0,
-                          cudaStream_t st);
+// Sources of a state load, in the caller's order, readable by this device's
+// kernels.  Null x, v or a, dr: already in the state set, or (zero_v, zero_ad)
+// zero; null kind: all fluid; null vw: walls at rest; null sigma0: computed,
+// through s0_first.  orig_*: the adjoint's copies, or null.
+struct LoadArgs {
+    const double *x, *v, *a, *dr, *h, *m, *vw, *sigma0;
+    const int8_t* kind;
+    int zero_v, zero_ad;
+    double* s0_first;
+    double *orig_h, *orig_m, *orig_s0, *orig_vw;
+    int8_t* orig_kind;
+};
+cudaError_t launch_load_state(int prec, int dim, int n, const LoadArgs& A, void* S0, void* S1, double rho0,
+                              double h_min, double h_max, uint32_t* err, cudaStream_t st, int64_t* launches);
+cudaError_t launch_store_state(int prec, int dim, int n, const void* S, const void* vr, double rho0, double* x,
+                               double* v, double* a, double* dr, double* rho, cudaStream_t st);
+template <typename T>
+struct Four {
+    T* p[4];
+};
+cudaError_t launch_cotangents_in(int n, int dim, const Four<const double>& src, const Four<double>& dst,
+                                 cudaStream_t st);
+cudaError_t launch_cotangents_out(int n, const Four<const double>& src, const Four<double>& dst, cudaStream_t st);
 // Output by gathering (coalesced writes in the caller's order): pos from
 // launch_inverse_perm of the sorted ids.
 cudaError_t launch_inverse_perm(int n, const int32_t* id, int32_t* pos, cudaStream_t st);
@@ -147,11 +163,7 @@ cudaError_t launch_rho_out_gather(int prec, int n, const void* vr, const int8_t*
                                   double rho0, double* dst, cudaStream_t st);
 cudaError_t launch_rho_out(int prec, int n, const void* vr, const int8_t* kind, const int32_t* id, double rho0,
                            double* dst, cudaStream_t st);
-cudaError_t launch_check_input(int n, const double* h, const double* m, double h_min, double h_max, uint32_t* err,
-                               cudaStream_t st);
 cudaError_t launch_scalar_out(int prec, int n, const void* src, const int32_t* id, double* dst, cudaStream_t st);
-cudaError_t launch_check_constants(int n, const double* h, const double* m, const double* s0, const int8_t* kind,
-                                   uint32_t* varies, cudaStream_t st);
 cudaError_t launch_scalar_in(int prec, int n, const double* src, const int8_t* kind, void* dst, cudaStream_t st);
 
 // k_dual.cu (dual-criteria time stepping).  Device pointers of one context;
@@ -185,7 +197,5 @@ cudaError_t launch_save_tape(int prec, int dim, int n, int nstart, const void* S
                              cudaStream_t st);
 cudaError_t launch_adjoint_step(int prec, int dim, int n, const TapeView& V, const Grid& G, const void* K,
                                 const AdjView& A, int step_mode, cudaStream_t st);
-cudaError_t launch_aos_to_soa(int n, const double* src3, double* dst, cudaStream_t st);
-cudaError_t launch_soa_to_aos(int n, const double* src, double* dst3, cudaStream_t st);
 
 }  // namespace sphtv

@@ -68,13 +68,14 @@ struct sph_ctx {
     double* du;         // dual integrator: device state (DU_*)
     int dual_est;       // dual integrator: substeps to launch before the first check
     int density_only;   // sph_density_noalloc's view: no neighbour lists
-    // CUDA graph replay of kick-drift-kick steps (params.graphs): two steps
-    // per graph, one graph per parity of the ping-pong state sets
+    // CUDA graph replay of kick-drift-kick steps (params.graphs): kGraphSteps
+    // steps per graph, one graph of each length per parity of the ping-pong
+    // state sets ([length][parity])
     cudaStream_t gst;           // library-owned stream of the replays
     cudaEvent_t gev[2];         // context stream -> gst, gst -> context stream
-    cudaGraphExec_t gexec[2];
-    int gstate[2];              // 0 not captured, 1 ready, -1 capture failed (launch directly)
-    int64_t glaunches[2];       // kernels in one replay
+    cudaGraphExec_t gexec[2][2];
+    int gstate[2][2];           // 0 not captured, 1 ready, -1 capture failed (launch directly)
+    int64_t glaunches[2][2];    // kernels in one replay
     // the adjoint's segment (forward replay recording the tape, then the
     // reverse sweep) for one segment length, captured on first use
     cudaGraphExec_t aexec;
@@ -88,6 +89,7 @@ struct sph_ctx {
     unsigned* counters;  // blocks and groups of blocks that have finished (zero between launches)
     double* diag;
     double* dt;
+    double* s0_first;       // sigma0 of particle 0 during a load
     uint32_t* err;          // [0] the sticky device error word; [1] nonzero when the particles' h, m,
                             // sigma0 or kind vary (else the sort leaves these arrays where they are)
     double* stage;
@@ -352,6 +354,7 @@ size_t carve(sph_ctx* c, char* base)
     c->counters = W.take<unsigned>((size_t)grid_groups() + 1);
     c->diag = W.take<double>(DG_COUNT);
     c->dt = W.take<double>(1);
+    c->s0_first = W.take<double>(1);
     c->err = W.take<uint32_t>(4);
     c->stage = W.take<double>(3 * n);
     const int K = c->P.adjoint_steps;
@@ -556,10 +559,18 @@ sph_status run_dual_step(sph_ctx* c)
     return SPH_OK;
 }
 
-// Capture two kick-drift-kick steps starting from state-set parity par into
-// a graph on the library stream.  Nothing runs during the capture (the sets
-// and counters are left as they were); on any failure the context falls
-// back to direct launches for that parity.
+// Steps per graph, and the steps a call must still have to take for a graph to
+// be used.  The gap between two replays is about 3 us: two steps per graph
+// leave half of it on each step of a small problem (2-D 50^2 FP64: 40.3 us a
+// step, 40.6 with direct launches, 39.3 with eight, 38.9 with sixteen).  A
+// capture costs 3 us per kernel once, so short calls take the short graph.
+constexpr int kGraphSteps[2] = {2, 8};
+constexpr int kGraphFrom[2] = {2, 16};
+
+// Capture kGraphSteps[len] kick-drift-kick steps starting from state-set
+// parity par into a graph on the library stream.  Nothing runs during the
+// capture (the sets and counters are left as they were); on any failure the
+// context falls back to direct launches for that parity.
 // The library stream of the replays and the two events that fence it
 // against the context's stream; false if they cannot be created.
 bool graph_stream(sph_ctx* c)
@@ -580,9 +591,9 @@ bool graph_stream(sph_ctx* c)
     return true;
 }
 
-void graph_capture(sph_ctx* c, int par)
+void graph_capture(sph_ctx* c, int len, int par)
 {
-    c->gstate[par] = -1;
+    c->gstate[len][par] = -1;
     if (!graph_stream(c)) return;
     cudaStream_t user = c->st;
     const int cur0 = c->cur;
@@ -591,24 +602,26 @@ void graph_capture(sph_ctx* c, int par)
     bool ok = cudaStreamBeginCapture(c->gst, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
     if (ok) {
         c->st = c->gst;
-        for (int k = 0; k < 2 && ok; ++k) ok = run_sort(c, 1, 0) == SPH_OK && run_forces(c, 1, 1, 1) == SPH_OK;
+        for (int k = 0; k < kGraphSteps[len] && ok; ++k)
+            ok = run_sort(c, 1, 0) == SPH_OK && run_forces(c, 1, 1, 1) == SPH_OK;
         c->st = user;
         ok = cudaStreamEndCapture(c->gst, &g) == cudaSuccess && ok && g;
     }
     c->cur = cur0;
-    c->glaunches[par] = c->launches - l0;
+    c->glaunches[len][par] = c->launches - l0;
     c->launches = l0;
-    if (ok && cudaGraphInstantiate(&c->gexec[par], g, 0) == cudaSuccess) c->gstate[par] = 1;
+    if (ok && cudaGraphInstantiate(&c->gexec[len][par], g, 0) == cudaSuccess) c->gstate[len][par] = 1;
     if (g) cudaGraphDestroy(g);
     cudaGetLastError();
 }
 
 void graph_release(sph_ctx* c)
 {
-    for (int par = 0; par < 2; ++par) {
-        if (c->gstate[par] == 1) cudaGraphExecDestroy(c->gexec[par]);
-        c->gstate[par] = 0;
-    }
+    for (int len = 0; len < 2; ++len)
+        for (int par = 0; par < 2; ++par) {
+            if (c->gstate[len][par] == 1) cudaGraphExecDestroy(c->gexec[len][par]);
+            c->gstate[len][par] = 0;
+        }
     if (c->astate == 1) cudaGraphExecDestroy(c->aexec);
     c->astate = 0;
     c->asteps = 0;
@@ -639,8 +652,6 @@ bool is_host_ptr(const void* p)
 
 // ------------------------------------------------------------------ adjoint
 
-// Load a state (caller order) with the per-particle constants of the last
-// sph_set_state.  a and dr may be NULL (then computed by the force pass).
 // Address through which this device's kernels can reach p directly: p for
 // memory of the current device (or managed memory), the mapped alias of
 // page-locked host memory; nullptr otherwise (pageable host memory, another
@@ -664,67 +675,79 @@ void* device_view(const void* p)
 }
 
 // [n][3] rows of src (host or device) into the per-component array dst of
-// precision prec: read in place when the device can reach src (page-locked
-// host memory streams across the host link inside the conversion kernel),
-// else copied to the staging buffer first.
-sph_status vec_in(sph_ctx* c, int prec, const double* src, void* dst)
+// precision prec: *in_place is src as the load kernel can read it (device
+// memory, or page-locked host memory, which streams across the host link
+// inside the kernel); else src is copied to the staging buffer, converted
+// into dst, and *in_place is null.
+sph_status vec_in(sph_ctx* c, int prec, const double* src, void* dst, const double** in_place)
 {
     const size_t n = (size_t)c->n;
-    const double* dv = (const double*)device_view(src);
-    if (!dv) {
-        SPH_CU(cudaMemcpyAsync(c->stage, src, 3 * n * sizeof(double), cudaMemcpyDefault, c->st));
-        dv = c->stage;
-    }
-    SPH_CU(launch_vec_in(prec, c->dim, (int)n, dv, dst, c->st));
+    *in_place = (const double*)device_view(src);
+    if (*in_place) return SPH_OK;
+    SPH_CU(cudaMemcpyAsync(c->stage, src, 3 * n * sizeof(double), cudaMemcpyDefault, c->st));
+    SPH_CU(launch_vec_in(prec, c->dim, (int)n, c->stage, dst, c->st));
     ++c->launches;
     return SPH_OK;
 }
 
-// h, m, sigma0 and kind of state set 0 into state set 1: the sort leaves these
-// arrays where they are when they do not vary over the particles, so both
-// sets must hold them.
-sph_status copy_constants(sph_ctx* c)
+// count elements of src as the load kernel can read them: in place, or copied
+// into dst.
+template <typename T>
+sph_status scalar_in(sph_ctx* c, const T* src, T* dst, const T** view)
 {
-    const size_t n = (size_t)c->n;
-    const StateSet<double>& A = c->set[0].d;
-    const StateSet<double>& B = c->set[1].d;
-    SPH_CU(cudaMemcpyAsync(B.h, A.h, n * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
-    SPH_CU(cudaMemcpyAsync(B.m, A.m, n * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
-    SPH_CU(cudaMemcpyAsync(B.s0, A.s0, n * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
-    SPH_CU(cudaMemcpyAsync(B.kind, A.kind, n, cudaMemcpyDeviceToDevice, c->st));
+    *view = (const T*)device_view(src);
+    if (*view) return SPH_OK;
+    SPH_CU(cudaMemcpyAsync(dst, src, (size_t)c->n * sizeof(T), cudaMemcpyDefault, c->st));
+    *view = dst;
     return SPH_OK;
 }
 
-sph_status reload_state(sph_ctx* c, const double* x, const double* v, const double* a, const double* dr)
+// Load a state (caller's order): the vectors x, v and (or zeros) a, dr, and
+// the per-particle constants of A, whose pointers the device can read.
+sph_status load_state(sph_ctx* c, const double* x, const double* v, const double* a, const double* dr, LoadArgs A)
 {
-    const size_t n = (size_t)c->n;
-    const size_t rs = c->prec == 64 ? 8 : 4;
     c->cur = 0;
     StateSet<double>& Sd = c->set[0].d;
     void* sv = c->prec == 64 ? (void*)c->set[0].d.v : (void*)c->set[0].f.v;
     void* sa = c->prec == 64 ? (void*)c->set[0].d.a : (void*)c->set[0].f.a;
     void* sdr = c->prec == 64 ? (void*)c->set[0].d.dr : (void*)c->set[0].f.dr;
-    SPH_TRY(vec_in(c, 64, x, Sd.x));
-    SPH_TRY(vec_in(c, c->prec, v, sv));
+    SPH_TRY(vec_in(c, 64, x, Sd.x, &A.x));
+    SPH_TRY(vec_in(c, c->prec, v, sv, &A.v));
+    A.zero_v = 0;
+    A.a = A.dr = nullptr;
+    A.zero_ad = a == nullptr;
     if (a) {
-        SPH_TRY(vec_in(c, c->prec, a, sa));
-        SPH_TRY(vec_in(c, c->prec, dr, sdr));
-    } else {
-        SPH_CU(cudaMemsetAsync(sa, 0, c->dim * n * rs, c->st));
-        SPH_CU(cudaMemsetAsync(sdr, 0, c->dim * n * rs, c->st));
+        SPH_TRY(vec_in(c, c->prec, a, sa, &A.a));
+        SPH_TRY(vec_in(c, c->prec, dr, sdr, &A.dr));
+        if (!A.a != !A.dr) {          // one readable in place, the other staged: convert the first by itself
+            const double* src = A.a ? A.a : A.dr;
+            SPH_CU(launch_vec_in(c->prec, c->dim, (int)c->n, src, A.a ? sa : sdr, c->st));
+            ++c->launches;
+            A.a = A.dr = nullptr;
+        }
     }
-    SPH_CU(cudaMemcpyAsync(Sd.h, c->orig_h, n * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
-    SPH_CU(cudaMemcpyAsync(Sd.m, c->orig_m, n * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
-    SPH_CU(cudaMemcpyAsync(Sd.s0, c->orig_s0, n * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
-    SPH_CU(cudaMemcpyAsync(Sd.kind, c->orig_kind, n, cudaMemcpyDeviceToDevice, c->st));
-    SPH_TRY(copy_constants(c));
-    SPH_CU(launch_walls_velocity(c->prec, c->dim, (int)n, Sd.kind, c->orig_vw, sv, c->st));
-    SPH_CU(launch_init_ids((int)n, Sd.id, c->st));
-    c->launches += 2;
+    A.s0_first = c->s0_first;
+    void* S0 = c->prec == 64 ? (void*)&c->set[0].d : (void*)&c->set[0].f;
+    void* S1 = c->prec == 64 ? (void*)&c->set[1].d : (void*)&c->set[1].f;
+    SPH_CU(launch_load_state(c->prec, c->dim, (int)c->n, A, S0, S1, c->P.rho0, c->P.h_min, c->P.h_max, c->err, c->st,
+                             &c->launches));
     c->have_state = 1;
     c->have_cells = 0;
     c->ad_given = a != nullptr;
     return SPH_OK;
+}
+
+// Load a state with the per-particle constants of the last sph_set_state.
+// a and dr may be NULL (then computed by the force pass).
+sph_status reload_state(sph_ctx* c, const double* x, const double* v, const double* a, const double* dr)
+{
+    LoadArgs A = {};
+    A.h = c->orig_h;
+    A.m = c->orig_m;
+    A.sigma0 = c->orig_s0;
+    A.kind = c->orig_kind;
+    A.vw = c->orig_vw;
+    return load_state(c, x, v, a, dr, A);
 }
 
 TapeView tape_view(const TapeSlot& T)
@@ -743,23 +766,61 @@ sph_status save_tape(sph_ctx* c, int t)
     return SPH_OK;
 }
 
-// Caller [n][3] cotangents -> [3][n] FP64 (z row zeroed in 2-D), and back.
-sph_status cot_in(sph_ctx* c, const double* src, double* dst)
+// The caller's [n][3] cotangents (xbar, vbar, abar, drbar) into the adjoint's
+// [3][n] (z row zeroed in 2-D): in one kernel what the device can read in
+// place, the others through the staging buffer.
+sph_status cotangents_in(sph_ctx* c, const double* xb, const double* vb, const double* ab, const double* db)
 {
-    const size_t n = (size_t)c->n;
-    SPH_CU(cudaMemcpyAsync(c->stage, src, 3 * n * sizeof(double), cudaMemcpyDefault, c->st));
-    SPH_CU(launch_aos_to_soa((int)n, c->stage, dst, c->st));
-    if (c->dim == 2) SPH_CU(cudaMemsetAsync(dst + 2 * n, 0, n * sizeof(double), c->st));
-    ++c->launches;
+    const AdjView& A = c->adj;
+    const double* src[4] = {xb, vb, ab, db};
+    const Four<double> dst = {{A.xc, A.vc, A.ac, A.drc}};
+    Four<const double> direct = {{nullptr, nullptr, nullptr, nullptr}};
+    bool any = false;
+    for (int q = 0; q < 4; ++q) {
+        direct.p[q] = (const double*)device_view(src[q]);
+        if (direct.p[q]) {
+            any = true;
+            continue;
+        }
+        SPH_CU(cudaMemcpyAsync(c->stage, src[q], 3 * (size_t)c->n * sizeof(double), cudaMemcpyDefault, c->st));
+        Four<const double> one = {{nullptr, nullptr, nullptr, nullptr}};
+        one.p[q] = c->stage;
+        SPH_CU(launch_cotangents_in((int)c->n, c->dim, one, dst, c->st));
+        ++c->launches;
+    }
+    if (any) {
+        SPH_CU(launch_cotangents_in((int)c->n, c->dim, direct, dst, c->st));
+        ++c->launches;
+    }
     return SPH_OK;
 }
 
-sph_status cot_out(sph_ctx* c, const double* src, double* dst)
+// And back, the ones asked for (not NULL); host memory through the staging
+// buffer and a copy.
+sph_status cotangents_out(sph_ctx* c, double* xb, double* vb, double* ab, double* db)
 {
-    const size_t n = (size_t)c->n;
-    SPH_CU(launch_soa_to_aos((int)n, src, c->stage, c->st));
-    SPH_CU(cudaMemcpyAsync(dst, c->stage, 3 * n * sizeof(double), cudaMemcpyDefault, c->st));
-    ++c->launches;
+    const AdjView& A = c->adj;
+    double* out[4] = {xb, vb, ab, db};
+    const Four<const double> src = {{A.xc, A.vc, A.ac, A.drc}};
+    Four<double> direct = {{nullptr, nullptr, nullptr, nullptr}};
+    bool any = false;
+    for (int q = 0; q < 4; ++q) {
+        if (!out[q]) continue;
+        direct.p[q] = is_host_ptr(out[q]) ? nullptr : (double*)device_view(out[q]);
+        any = any || direct.p[q];
+    }
+    if (any) {
+        SPH_CU(launch_cotangents_out((int)c->n, src, direct, c->st));
+        ++c->launches;
+    }
+    for (int q = 0; q < 4; ++q) {
+        if (!out[q] || direct.p[q]) continue;
+        Four<double> one = {{nullptr, nullptr, nullptr, nullptr}};
+        one.p[q] = c->stage;
+        SPH_CU(launch_cotangents_out((int)c->n, src, one, c->st));
+        ++c->launches;
+        SPH_CU(cudaMemcpyAsync(out[q], c->stage, 3 * (size_t)c->n * sizeof(double), cudaMemcpyDefault, c->st));
+    }
     return SPH_OK;
 }
 
@@ -932,58 +993,30 @@ sph_status sph_set_state(sph_ctx* c, const double* x, const double* v, const dou
 {
     if (!c || !x || !v || !h || !m) return SPH_ERR_ARG;
     if ((a == nullptr) != (dr == nullptr)) return SPH_ERR_ARG;
-    const size_t n = (size_t)c->n;
-    const size_t vb = 3 * n * sizeof(double);
-    c->cur = 0;
     StateSet<double>& Sd = c->set[0].d;
-    void* S = cur_set(c);
-    void* sv = c->prec == 64 ? (void*)c->set[0].d.v : (void*)c->set[0].f.v;
-    void* sa = c->prec == 64 ? (void*)c->set[0].d.a : (void*)c->set[0].f.a;
-    void* sdr = c->prec == 64 ? (void*)c->set[0].d.dr : (void*)c->set[0].f.dr;
-    (void)S;
-    const size_t rs = c->prec == 64 ? 8 : 4;
-    SPH_TRY(vec_in(c, 64, x, Sd.x));
-    SPH_TRY(vec_in(c, c->prec, v, sv));
-    if (a) {
-        SPH_TRY(vec_in(c, c->prec, a, sa));
-        SPH_TRY(vec_in(c, c->prec, dr, sdr));
-    } else {
-        SPH_CU(cudaMemsetAsync(sa, 0, c->dim * n * rs, c->st));
-        SPH_CU(cudaMemsetAsync(sdr, 0, c->dim * n * rs, c->st));
+    LoadArgs A = {};
+    SPH_TRY(scalar_in(c, h, Sd.h, &A.h));
+    SPH_TRY(scalar_in(c, m, Sd.m, &A.m));
+    if (kind) SPH_TRY(scalar_in(c, kind, Sd.kind, &A.kind));
+    if (sigma0) SPH_TRY(scalar_in(c, sigma0, Sd.s0, &A.sigma0));
+    if (vw) {
+        A.vw = (const double*)device_view(vw);
+        if (!A.vw) {
+            // not readable in place: the neighbour list's buffer (96 entries a
+            // particle or more, free until the next density pass) holds the
+            // rows for the load, while the staging buffer serves the vectors
+            SPH_CU(cudaMemcpyAsync(c->nbl, vw, 3 * (size_t)c->n * sizeof(double), cudaMemcpyDefault, c->st));
+            A.vw = (const double*)c->nbl;
+        }
     }
-    SPH_CU(cudaMemcpyAsync(Sd.h, h, n * sizeof(double), cudaMemcpyDefault, c->st));
-    SPH_CU(cudaMemcpyAsync(Sd.m, m, n * sizeof(double), cudaMemcpyDefault, c->st));
-    if (kind) SPH_CU(cudaMemcpyAsync(Sd.kind, kind, n, cudaMemcpyDefault, c->st));
-    else SPH_CU(cudaMemsetAsync(Sd.kind, 0, n, c->st));
-    if (vw) SPH_CU(cudaMemcpyAsync(c->stage, vw, vb, cudaMemcpyDefault, c->st));
-    SPH_CU(launch_walls_velocity(c->prec, c->dim, (int)n, Sd.kind, vw ? c->stage : nullptr, sv, c->st));
     if (c->P.adjoint_steps > 0) {
-        if (vw) SPH_CU(cudaMemcpyAsync(c->orig_vw, c->stage, vb, cudaMemcpyDeviceToDevice, c->st));
-        else SPH_CU(cudaMemsetAsync(c->orig_vw, 0, vb, c->st));
+        A.orig_h = c->orig_h;
+        A.orig_m = c->orig_m;
+        A.orig_s0 = c->orig_s0;
+        A.orig_kind = c->orig_kind;
+        A.orig_vw = c->orig_vw;
     }
-    if (sigma0) SPH_CU(cudaMemcpyAsync(Sd.s0, sigma0, n * sizeof(double), cudaMemcpyDefault, c->st));
-    else {
-        SPH_CU(launch_sigma0(c->dim, (int)n, Sd.h, Sd.m, c->P.rho0, Sd.s0, c->st));
-        c->launches += 2;
-    }
-    SPH_CU(launch_init_ids((int)n, Sd.id, c->st));
-    SPH_CU(launch_check_input((int)n, Sd.h, Sd.m, c->P.h_min, c->P.h_max, c->err, c->st));
-    SPH_CU(cudaMemsetAsync(c->err + 1, 0, sizeof(uint32_t), c->st));
-    SPH_CU(launch_check_constants((int)n, Sd.h, Sd.m, Sd.s0, Sd.kind, c->err + 1, c->st));
-    SPH_TRY(copy_constants(c));
-    ++c->launches;
-    if (Sd.drho) SPH_CU(cudaMemsetAsync(Sd.drho, 0, n * rs, c->st));
-    c->launches += 3;
-    if (c->P.adjoint_steps > 0) {
-        SPH_CU(cudaMemcpyAsync(c->orig_h, Sd.h, n * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
-        SPH_CU(cudaMemcpyAsync(c->orig_m, Sd.m, n * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
-        SPH_CU(cudaMemcpyAsync(c->orig_s0, Sd.s0, n * sizeof(double), cudaMemcpyDeviceToDevice, c->st));
-        SPH_CU(cudaMemcpyAsync(c->orig_kind, Sd.kind, n, cudaMemcpyDeviceToDevice, c->st));
-    }
-    c->have_state = 1;
-    c->have_cells = 0;
-    c->ad_given = a != nullptr;
-    return SPH_OK;
+    return load_state(c, x, v, a, dr, A);
 }
 
 sph_status sph_build_cells(sph_ctx* c)
@@ -1025,13 +1058,16 @@ sph_status sph_step(sph_ctx* c, int32_t nsteps)
     if (!c || nsteps < 0) return SPH_ERR_ARG;
     const int32_t nsteps_in = nsteps;
     if (!c->have_cells) return SPH_ERR_STATE;
-    if (c->P.integrator == SPH_INT_KDK && c->P.graphs && !c->prof_ev && nsteps >= 2) {
-        const int par = c->cur;
-        if (c->gstate[par] == 0) graph_capture(c, par);
-        if (c->gstate[par] == 1) {
-            SPH_TRY(graph_launch(c, c->gexec[par], nsteps / 2));
-            c->launches += (int64_t)(nsteps / 2) * c->glaunches[par];
-            nsteps &= 1;     // two steps per replay bring the sets back to this parity
+    if (c->P.integrator == SPH_INT_KDK && c->P.graphs && !c->prof_ev) {
+        const int par = c->cur;      // an even number of steps brings the sets back to this parity
+        for (int len = 1; len >= 0; --len) {
+            if (nsteps < kGraphFrom[len]) continue;
+            if (c->gstate[len][par] == 0) graph_capture(c, len, par);
+            if (c->gstate[len][par] != 1) continue;
+            const int times = nsteps / kGraphSteps[len];
+            SPH_TRY(graph_launch(c, c->gexec[len][par], times));
+            c->launches += (int64_t)times * c->glaunches[len][par];
+            nsteps -= times * kGraphSteps[len];
         }
     }
     for (int32_t k = 0; k < nsteps; ++k) {
@@ -1113,6 +1149,15 @@ sph_status sph_get_state(sph_ctx* c, double* x, double* v, double* a, double* dr
     const void* sa = c->prec == 64 ? (void*)c->set[c->cur].d.a : (void*)c->set[c->cur].f.a;
     const void* sdr = c->prec == 64 ? (void*)c->set[c->cur].d.dr : (void*)c->set[c->cur].f.dr;
     if (rho && !c->have_cells) return SPH_ERR_STATE;
+    // every output in memory of this device: one kernel
+    bool direct = x || v || a || dr || rho;
+    for (double* o : {x, v, a, dr, rho})
+        if (o && (is_host_ptr(o) || device_view(o) != o)) direct = false;
+    if (direct) {
+        SPH_CU(launch_store_state(c->prec, c->dim, n, cur_set(c), c->vr, c->P.rho0, x, v, a, dr, rho, c->st));
+        ++c->launches;
+        return SPH_OK;
+    }
     bool host = false;
     struct Out { double* dst; const void* src; int prec; } outs[4] = {{x, Sd.x, 64}, {v, sv, c->prec},
                                                                     {a, sa, c->prec}, {dr, sdr, c->prec}};
@@ -1303,10 +1348,7 @@ sph_status sph_step_adjoint(sph_ctx* c, const double* x0, const double* v0, cons
     SPH_TRY(reload_state(c, x0, v0, a0, dr0));
     SPH_TRY(sph_build_cells(c));
     AdjView& A = c->adj;
-    SPH_TRY(cot_in(c, xbar, A.xc));      // the forward replay leaves the cotangents alone
-    SPH_TRY(cot_in(c, vbar, A.vc));
-    SPH_TRY(cot_in(c, abar, A.ac));
-    SPH_TRY(cot_in(c, drbar, A.drc));
+    SPH_TRY(cotangents_in(c, xbar, vbar, abar, drbar));     // the forward replay leaves the cotangents alone
     bool replayed = false;
     if (c->P.graphs && !c->prof_ev) {
         if (c->astate == 0 || c->asteps != nsteps || c->acur0 != c->cur) adjoint_capture(c, nsteps);
@@ -1318,10 +1360,7 @@ sph_status sph_step_adjoint(sph_ctx* c, const double* x0, const double* v0, cons
         }
     }
     if (!replayed) SPH_TRY(adjoint_segment(c, nsteps));
-    SPH_TRY(cot_out(c, A.xc, xbar));
-    SPH_TRY(cot_out(c, A.vc, vbar));
-    SPH_TRY(cot_out(c, A.ac, abar));
-    SPH_TRY(cot_out(c, A.drc, drbar));
+    SPH_TRY(cotangents_out(c, xbar, vbar, abar, drbar));
     double eta = 0.0;
     SPH_CU(cudaMemcpyAsync(&eta, A.eta, sizeof(double), cudaMemcpyDeviceToHost, c->st));
     SPH_CU(cudaStreamSynchronize(c->st));
@@ -1344,15 +1383,11 @@ sph_status sph_force_pass_adjoint(sph_ctx* c, const double* x, const double* v, 
     SPH_CU(cudaMemsetAsync(c->tape[0].dt, 0, sizeof(double), c->st));
     AdjView& A = c->adj;
     SPH_CU(cudaMemsetAsync(A.eta, 0, sizeof(double), c->st));
-    SPH_TRY(cot_in(c, xbar, A.xc));
-    SPH_TRY(cot_in(c, vbar, A.vc));
-    SPH_TRY(cot_in(c, abar, A.ac));
-    SPH_TRY(cot_in(c, drbar, A.drc));
+    SPH_TRY(cotangents_in(c, xbar, vbar, abar, drbar));
     SPH_CU(launch_adjoint_step(c->prec, c->dim, (int)c->n, tape_view(c->tape[0]), cells_only(c->G), consts(c), A, 0,
                               c->st));
     c->launches += 3;
-    SPH_TRY(cot_out(c, A.xc, xbar));
-    SPH_TRY(cot_out(c, A.vc, vbar));
+    SPH_TRY(cotangents_out(c, xbar, vbar, nullptr, nullptr));
     double eta = 0.0;
     SPH_CU(cudaMemcpyAsync(&eta, A.eta, sizeof(double), cudaMemcpyDeviceToHost, c->st));
     SPH_CU(cudaStreamSynchronize(c->st));
@@ -1453,20 +1488,18 @@ extern "C" sph_status sph_density_noalloc(const sph_params* p, int64_t n, const 
     carve(&c, (char*)base);
 
     const int ni = (int)n;
-    StateSet<double>& S0 = c.set[0].d;
     // The scratch keeps the previous call's contents: clear what is summed into.
     // (run_sort clears the bins' counts: the view starts with count_zero = 0.)
-    SPH_CU(cudaMemsetAsync(c.err, 0, 4 * sizeof(uint32_t), c.st));
-    SPH_CU(cudaMemsetAsync(c.err + 1, 1, 1, c.st));   // the sort moves h, m, sigma0 and kind
-    SPH_CU(cudaMemsetAsync(S0.v, 0, (size_t)c.dim * n * sizeof(double), c.st));
-    SPH_CU(launch_vec_in(64, c.dim, ni, x, S0.x, c.st));
-    SPH_CU(cudaMemcpyAsync(S0.h, h, n * sizeof(double), cudaMemcpyDeviceToDevice, c.st));
-    SPH_CU(cudaMemcpyAsync(S0.m, m, n * sizeof(double), cudaMemcpyDeviceToDevice, c.st));
-    if (kind) SPH_CU(cudaMemcpyAsync(S0.kind, kind, n, cudaMemcpyDeviceToDevice, c.st));
-    else SPH_CU(cudaMemsetAsync(S0.kind, 0, n, c.st));
-    if (sigma0) SPH_CU(cudaMemcpyAsync(S0.s0, sigma0, n * sizeof(double), cudaMemcpyDeviceToDevice, c.st));
-    else SPH_CU(launch_sigma0(c.dim, ni, S0.h, S0.m, p->rho0, S0.s0, c.st));
-    SPH_CU(launch_init_ids(ni, S0.id, c.st));
+    LoadArgs A = {};
+    A.x = x;
+    A.h = h;
+    A.m = m;
+    A.kind = kind;
+    A.sigma0 = sigma0;
+    A.zero_v = 1;
+    A.s0_first = c.s0_first;
+    SPH_CU(launch_load_state(64, c.dim, ni, A, &c.set[0].d, &c.set[1].d, p->rho0, p->h_min, p->h_max, c.err, c.st,
+                             &c.launches));
     c.cur = 0;
     s = run_sort(&c, 0, 0);
     if (s != SPH_OK) return s;
