@@ -13,8 +13,9 @@
 //                       substep's second half), x += dr (first substep of the
 //                       advection step only), x += dt/2 v
 //   k_dual_pressure   : Riemann pressure force (Eq. 3 row 2, Eq. 5-6) + the
-//                       held viscous force + g; v += dt a
-//   k_dual_drift      : x += dt/2 v
+//                       held viscous force + g; v += dt a; in the FP32 form
+//                       also x += dt/2 v
+//   k_dual_drift      : x += dt/2 v (FP64 form)
 //   k_dual_continuity : drho_i = 2 rho_i sum_j V_j (U* - U_l) dW/dr (Eq. 3
 //                       row 1, U* of Eq. 5 row 1), diagnostics partials; its
 //                       last block folds them, sets the next substep size and
@@ -56,6 +57,12 @@ struct DualK {
     StateSet<Real> S;
     typename V4<Real>::T* vr;
     float4* pos4;            // cell-relative offsets (the FP32 form's drifts keep them current), m or h
+    // FP32 form: the velocity records and offsets after the second half drift,
+    // in buffers of their own: the pressure pass gathers its neighbours from
+    // vr and pos4 and writes the drifted particle here (the FP64 form's second
+    // pair of pointers is vr and pos4 again)
+    typename V4<Real>::T* vr_b;
+    float4* pos4_b;
     const float* mf;         // FP32 form: masses
     const uint32_t* nbl;
     const int32_t* nbc;
@@ -90,7 +97,8 @@ __device__ __forceinline__ void fill_shift_table(const Grid& G, float4* tab)
 // form: m or h) and oj = vr[j].  The FP32 walk keeps the list entries four
 // ahead and the neighbour data two ahead in flight.
 template <typename Real, int DIM, typename F>
-__device__ __forceinline__ void for_list(const DualK<Real>& A, const Grid& G, const float4* tab, int i, int cnt, F& f)
+__device__ __forceinline__ void for_list(const DualK<Real>& A, const Grid& G, const float4* tab, int i, int cnt,
+                                         const typename V4<Real>::T* vr, const float4* pos4, F& f)
 {
     const int n = A.n;
     if constexpr (std::is_same<Real, double>::value) {
@@ -106,10 +114,10 @@ __device__ __forceinline__ void for_list(const DualK<Real>& A, const Grid& G, co
                 rv[d] = min_image(G, xi[d], A.S.x[(size_t)d * n + j], d);
                 r2 += rv[d] * rv[d];
             }
-            f(j, rv, r2, 0.f, A.vr[j]);
+            f(j, rv, r2, 0.f, vr[j]);
         }
     } else {
-        const float4 pi = A.pos4[i];
+        const float4 pi = pos4[i];
         const float oi[3] = {pi.x, pi.y, pi.z};
         const uint32_t* lp = A.nbl + i;
         auto one = [&](uint32_t ec, const float4& pj, const float4& oj) {
@@ -131,14 +139,14 @@ __device__ __forceinline__ void for_list(const DualK<Real>& A, const Grid& G, co
         uint32_t e1 = cnt > 1 ? lp[(size_t)n] : 0u;
         uint32_t e2 = cnt > 2 ? lp[2 * (size_t)n] : 0u;
         uint32_t e3 = cnt > 3 ? lp[3 * (size_t)n] : 0u;
-        float4 p0 = A.pos4[e0 >> kCodeBits], o0 = A.vr[e0 >> kCodeBits];
-        float4 p1 = A.pos4[e1 >> kCodeBits], o1 = A.vr[e1 >> kCodeBits];
+        float4 p0 = pos4[e0 >> kCodeBits], o0 = vr[e0 >> kCodeBits];
+        float4 p1 = pos4[e1 >> kCodeBits], o1 = vr[e1 >> kCodeBits];
         int k = 0;
         const uint32_t* lq = lp + 4 * (size_t)n;
         const size_t n2 = 2 * (size_t)n;
         for (; k + 1 < cnt; k += 2, lq += n2) {
-            const float4 p2 = A.pos4[e2 >> kCodeBits], o2 = A.vr[e2 >> kCodeBits];
-            const float4 p3 = A.pos4[e3 >> kCodeBits], o3 = A.vr[e3 >> kCodeBits];
+            const float4 p2 = pos4[e2 >> kCodeBits], o2 = vr[e2 >> kCodeBits];
+            const float4 p3 = pos4[e3 >> kCodeBits], o3 = vr[e3 >> kCodeBits];
             const uint32_t e4 = k + 4 < cnt ? lq[0] : 0u;
             const uint32_t e5 = k + 5 < cnt ? lq[n] : 0u;
             one(e0, p0, o0);
@@ -294,7 +302,7 @@ __global__ void __launch_bounds__(sizeof(Real) == 8 ? 256 : 128) k_dual_advect(D
             acc_R[d].add(vw * rv[d]);
         }
     };
-    for_list<Real, DIM>(A, G, tab, i, cnt, pair);
+    for_list<Real, DIM>(A, G, tab, i, cnt, A.vr, A.pos4, pair);
     Real R[3] = {0, 0, 0}, R2 = 0;
 #pragma unroll
     for (int d = 0; d < DIM; ++d) {
@@ -331,7 +339,8 @@ __global__ void __launch_bounds__(256) k_dual_first_half(DualK<Real> A, Grid G)
     const double dt = A.du[DU_DT];
     const double hdt = 0.5 * dt;
     const bool first = A.du[DU_FIRST] != 0.0;
-    auto me = A.vr[i];
+    // the last substep left the particle in the second pair of buffers
+    auto me = first ? A.vr[i] : A.vr_b[i];
     Real w = me.w;
     const Real dr = A.S.drho[i];
     if (!first) w = fma_free_add<Real>(w, fma_free_mul<Real>((Real)A.du[DU_HDT_PREV], dr));
@@ -342,7 +351,8 @@ __global__ void __launch_bounds__(256) k_dual_first_half(DualK<Real> A, Grid G)
     // FP32 (the permute recomputes them from the FP64 positions at the next
     // advection step), which keeps the FP64 origin arithmetic off the
     // substeps
-    float4 p = sizeof(Real) == 4 ? A.pos4[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (sizeof(Real) == 4) p = first ? A.pos4[i] : A.pos4_b[i];
     float of[3] = {p.x, p.y, p.z};
     const float hdtf = (float)hdt;
 #pragma unroll
@@ -371,7 +381,14 @@ __global__ void __launch_bounds__(sizeof(Real) == 8 ? 256 : 128) k_dual_pressure
     fill_shift_table<Real>(G, tab);
     const int n = A.n;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n || A.S.kind[i]) return;
+    if (i >= n) return;
+    if (A.S.kind[i]) {
+        if (sizeof(Real) == 4) {
+            A.vr_b[i] = A.vr[i];
+            A.pos4_b[i] = A.pos4[i];
+        }
+        return;
+    }
     const int cnt = min(A.nbc[i], A.cap);
     const double dt = A.du[DU_DT];
     const auto me = A.vr[i];
@@ -407,18 +424,38 @@ __global__ void __launch_bounds__(sizeof(Real) == 8 ? 256 : 128) k_dual_pressure
 #pragma unroll
         for (int d = 0; d < DIM; ++d) acc[d].add(cpw * rv[d]);
     };
-    for_list<Real, DIM>(A, G, tab, i, cnt, pair);
+    for_list<Real, DIM>(A, G, tab, i, cnt, A.vr, A.pos4, pair);
+    // v += dt a, and in the FP32 form the second half drift x += dt/2 v (the
+    // FP64 positions, which only their own thread reads, in place; the offsets
+    // follow in FP32), as the arithmetic of k_dual_drift
+    const double hdt = 0.5 * dt;
+    const float hdtf = (float)hdt;
+    float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (sizeof(Real) == 4) p = A.pos4[i];
+    float of[3] = {p.x, p.y, p.z};
+    Real vn[3] = {0, 0, 0};
 #pragma unroll
     for (int d = 0; d < DIM; ++d) {
         const size_t o = (size_t)d * n + i;
         const Real a = (acc[d].value() + A.anu[o]) + K.g[d];
         A.S.a[o] = a;
-        A.S.v[o] = fma_free_add<Real>(A.S.v[o], fma_free_mul<Real>((Real)dt, a));
+        vn[d] = fma_free_add<Real>(A.S.v[o], fma_free_mul<Real>((Real)dt, a));
+        A.S.v[o] = vn[d];
+        if (sizeof(Real) == 4) {
+            A.S.x[o] = __dadd_rn(A.S.x[o], __dmul_rn(hdt, (double)vn[d]));
+            of[d] = __fmaf_rn(hdtf, (float)vn[d], of[d]);
+        }
+    }
+    if (sizeof(Real) == 4) {
+        A.vr_b[i] = V4<Real>::make(vn[0], vn[1], vn[2], me.w);
+        A.pos4_b[i] = make_float4(of[0], of[1], of[2], p.w);
     }
 }
 
-template <typename Real, int DIM>
-__global__ void __launch_bounds__(256) k_dual_drift(DualK<Real> A, Grid G)
+// The second half drift of the FP64 form, whose pressure pass gathers the
+// neighbours' positions that this kernel moves.
+template <int DIM>
+__global__ void __launch_bounds__(256) k_dual_drift(DualK<double> A, Grid G)
 {
     pdl_wait();
     if (dual_done(A.du)) return;
@@ -426,20 +463,15 @@ __global__ void __launch_bounds__(256) k_dual_drift(DualK<Real> A, Grid G)
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n || A.S.kind[i]) return;
     const double hdt = 0.5 * A.du[DU_DT];
-    const float hdtf = (float)hdt;
-    float4 p = sizeof(Real) == 4 ? A.pos4[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-    float of[3] = {p.x, p.y, p.z};
-    Real v[3] = {0, 0, 0};
+    double v[3] = {0, 0, 0};
 #pragma unroll
     for (int d = 0; d < DIM; ++d) {
         const size_t o = (size_t)d * n + i;
         v[d] = A.S.v[o];
-        A.S.x[o] = __dadd_rn(A.S.x[o], __dmul_rn(hdt, (double)v[d]));
-        of[d] = __fmaf_rn(hdtf, (float)v[d], of[d]);    // the offsets follow in FP32 (k_dual_first_half)
+        A.S.x[o] = __dadd_rn(A.S.x[o], __dmul_rn(hdt, v[d]));
     }
-    const Real w = A.vr[i].w;
-    A.vr[i] = V4<Real>::make(v[0], v[1], v[2], w);
-    if (sizeof(Real) == 4) A.pos4[i] = make_float4(of[0], of[1], of[2], p.w);
+    const double w = A.vr[i].w;
+    A.vr[i] = V4<double>::make(v[0], v[1], v[2], w);
 }
 
 // The end of a substep, from the grid's totals: advance t; pick the next
@@ -498,7 +530,7 @@ __global__ void __launch_bounds__(sizeof(Real) == 8 ? 256 : 128) k_dual_continui
     for (int k = 0; k < kNPart; ++k) part[k] = 0.0;
     if (i < n && A.S.kind[i] == 0) {
         const int cnt = min(A.nbc[i], A.cap);
-        const auto me = A.vr[i];
+        const auto me = A.vr_b[i];
         const Real vi[3] = {me.x, me.y, me.z};
         const Real rho_i = K.rho0 + me.w;
         const Real inv_rho_i = recip(rho_i);
@@ -506,7 +538,7 @@ __global__ void __launch_bounds__(sizeof(Real) == 8 ? 256 : 128) k_dual_continui
         Real hi, mi;
         {
             float wi = 0.f;
-            if constexpr (!std::is_same<Real, double>::value) wi = A.pos4[i].w;
+            if constexpr (!std::is_same<Real, double>::value) wi = A.pos4_b[i].w;
             h_m_of<Real, UNIFORM>(A, K, i, wi, hi, mi);
         }
         Acc s;
@@ -527,7 +559,7 @@ __global__ void __launch_bounds__(sizeof(Real) == 8 ? 256 : 128) k_dual_continui
             // V_j (U* - U_l) dW/dr, dW/dr = (W'/r) r
             s.add(mj * inv_rho_j * dus * (g.dwr * g.r));
         };
-        for_list<Real, DIM>(A, G, tab, i, cnt, pair);
+        for_list<Real, DIM>(A, G, tab, i, cnt, A.vr_b, A.pos4_b, pair);
         A.S.drho[i] = Real(2) * rho_i * s.value();
         // max |v| for the next substep size, from |v|^2 in the precision of v;
         // the other diagnostics (and |v|^2 in FP64 for the kinetic energy) only
@@ -593,7 +625,7 @@ __global__ void __launch_bounds__(256) k_dual_complete(DualK<Real> A)
     pdl_wait();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= A.n || A.S.kind[i]) return;
-    auto me = A.vr[i];
+    auto me = A.vr_b[i];
     me.w = fma_free_add<Real>(me.w, fma_free_mul<Real>((Real)A.du[DU_HDT_PREV], A.S.drho[i]));
     A.vr[i] = me;
 }
@@ -613,6 +645,8 @@ DualK<Real> dual_k(const DualArgs& a)
     k.S = *(const StateSet<Real>*)a.S;
     k.vr = (typename V4<Real>::T*)a.vr;
     k.pos4 = a.pos4;
+    k.vr_b = (typename V4<Real>::T*)(sizeof(Real) == 4 ? a.vr_b : a.vr);
+    k.pos4_b = sizeof(Real) == 4 ? a.pos4_b : a.pos4;
     k.mf = a.mf;
     k.nbl = a.nbl;
     k.nbc = a.nbc;
@@ -671,19 +705,10 @@ void run_pair(int prec, int dim, const DualArgs& a, const Grid& G, const void* K
 }
 
 template <typename Real>
-void run_elem(int dim, const DualArgs& a, const Grid& G, int which, cudaStream_t st)
+void run_first_half(int dim, const DualArgs& a, const Grid& G, cudaStream_t st)
 {
     const auto A = dual_k<Real>(a);
-    const int T = 256, B = nblk(A.n, T);
-    if (which == 0) {
-        if (dim == 2) launch(k_dual_first_half<Real, 2>, B, T, 0, st, A, G);
-        else launch(k_dual_first_half<Real, 3>, B, T, 0, st, A, G);
-    } else if (which == 1) {
-        if (dim == 2) launch(k_dual_drift<Real, 2>, B, T, 0, st, A, G);
-        else launch(k_dual_drift<Real, 3>, B, T, 0, st, A, G);
-    } else {
-        launch(k_dual_complete<Real>, B, T, 0, st, A);
-    }
+    launch(dim == 2 ? k_dual_first_half<Real, 2> : k_dual_first_half<Real, 3>, nblk(A.n, 256), 256, 0, st, A, G);
 }
 
 }  // namespace
@@ -703,13 +728,15 @@ cudaError_t launch_dual_advect(int prec, int dim, const DualArgs& a, const Grid&
 cudaError_t launch_dual_substep(int prec, int dim, const DualArgs& a, const Grid& G, const void* K,
                                 cudaStream_t st, int64_t* launches)
 {
-    if (prec == 64) run_elem<double>(dim, a, G, 0, st);
-    else run_elem<float>(dim, a, G, 0, st);
+    if (prec == 64) run_first_half<double>(dim, a, G, st);
+    else run_first_half<float>(dim, a, G, st);
     run_pair<k_dual_pressure_t>(prec, dim, a, G, K, st);
-    if (prec == 64) run_elem<double>(dim, a, G, 1, st);
-    else run_elem<float>(dim, a, G, 1, st);
+    if (prec == 64) {
+        launch(dim == 2 ? k_dual_drift<2> : k_dual_drift<3>, nblk(a.n, 256), 256, 0, st, dual_k<double>(a), G);
+        ++*launches;
+    }
     run_pair<k_dual_continuity_t>(prec, dim, a, G, K, st);
-    *launches += 4;
+    *launches += 3;
     const int nb = pair_blocks(prec, a.n, a.sms);
     const GridSum B = grid_sum(a.F, nb);
     if (B.group == 0) {
@@ -721,8 +748,8 @@ cudaError_t launch_dual_substep(int prec, int dim, const DualArgs& a, const Grid
 
 cudaError_t launch_dual_complete(int prec, const DualArgs& a, cudaStream_t st)
 {
-    if (prec == 64) run_elem<double>(2, a, Grid{}, 2, st);
-    else run_elem<float>(2, a, Grid{}, 2, st);
+    if (prec == 64) launch(k_dual_complete<double>, nblk(a.n, 256), 256, 0, st, dual_k<double>(a));
+    else launch(k_dual_complete<float>, nblk(a.n, 256), 256, 0, st, dual_k<float>(a));
     return cudaGetLastError();
 }
 

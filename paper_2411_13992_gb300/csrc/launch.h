@@ -173,6 +173,8 @@ struct DualArgs {
     const void* S;
     void* vr;
     float4* pos4;
+    void* vr_b;            // FP32 form: second pair of buffers (see k_dual.cu)
+    float4* pos4_b;
     const int32_t* cell_of;
     const float* mf;
     const uint32_t* nbl;

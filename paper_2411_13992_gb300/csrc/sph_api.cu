@@ -65,6 +65,8 @@ struct sph_ctx {
     int32_t* nbc;       // neighbour count per particle (with nbl)
     double* vol;        // FP64 form: V = m/rho per particle, written by the density pass for the force pass
     void* anu;          // dual integrator: viscous acceleration held for an advection step
+    void* vr_b;         // dual integrator, FP32 form: velocity records and offsets after the
+    float4* pos4_b;     // pressure pass's drift
     double* du;         // dual integrator: device state (DU_*)
     int dual_est;       // dual integrator: substeps to launch before the first check
     int density_only;   // sph_density_noalloc's view: no neighbour lists
@@ -345,6 +347,8 @@ size_t carve(sph_ctx* c, char* base)
     c->vol = lists && c->prec == 64 ? W.take<double>(n) : nullptr;
     c->anu = dual ? W.take<char>(D * n * rs) : nullptr;
     c->du = dual ? W.take<double>(DU_COUNT) : nullptr;
+    c->vr_b = dual && c->prec == 32 ? W.take<char>(n * 4 * rs) : nullptr;
+    c->pos4_b = dual && c->prec == 32 ? W.take<float4>(n) : nullptr;
     c->R = c->density_only ? nullptr : W.take<char>(D * n * rs);
     c->chi = c->density_only ? nullptr : W.take<char>(n * rs);
     // one partials row per block of a pair pass: blocks hold 32 particles or
@@ -499,6 +503,8 @@ DualArgs dual_args(sph_ctx* c)
     a.S = cur_set(c);
     a.vr = c->vr;
     a.pos4 = c->pos4;
+    a.vr_b = c->vr_b;
+    a.pos4_b = c->pos4_b;
     a.cell_of = c->cell;
     a.mf = c->mf;
     a.nbl = c->nbl;
