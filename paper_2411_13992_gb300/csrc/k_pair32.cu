@@ -1118,16 +1118,22 @@ __global__ void __launch_bounds__(TileThreads<DIM>::COOP, 4) k_density32_coop(
 
 // ------------------------------------------------------------------ forces
 
-// Register budget at uniform resolution: six blocks of 128 threads per SM
-// (at most 85 registers; 80 used, no spills), for the three pairs of neighbour
-// data in flight ahead of the three being computed.  The pass waits on these
-// gathers (L1/L2 hits): with eight blocks and one pair of data ahead it ran
-// 12 % longer early in a 128^3 run and 11 % longer after step 400; with three
-// pairs per iteration at seven or eight blocks the registers spill (+35-75 %).
+// U pairs per iteration, the next U pairs' neighbour data in flight.  At
+// uniform resolution U = 3 with six blocks of 128 threads per SM (at most 85
+// registers; 80 used, no spills): the pass waits on these gathers (L1/L2
+// hits); with eight blocks and one pair of data ahead it ran 12 % longer early
+// in a 128^3 run and 11 % longer after step 400; with three pairs per
+// iteration at seven or eight blocks the registers spill (+35-75 %).  A grid
+// of at most kDeepBlocks blocks per SM leaves registers over and too few
+// warps to cover the gathers, and takes U = 5 (step of the 2,900-particle
+// cavity 35.1 -> 33.5 us, of the 69,000-particle one 41.9 -> 41.4, rollout
+// 256^2 3.21 -> 3.16 ms; U = 4 the same within 1 %, 6 slower).
 // Variable resolution keeps eight blocks (64 registers) and one pair ahead:
 // at six blocks its pass ran 10 % longer.
-template <int DIM, typename Acc, bool UNIFORM>
-__global__ void __launch_bounds__(kTPB32, UNIFORM ? 6 : 8) k_forces32(int n, const float4* pos4,
+constexpr int kDeepBlocks = 4, kDeepPairs = 5;
+constexpr int forces_blocks(bool uniform, int U) { return !uniform ? 8 : (U == 3 ? 6 : kDeepBlocks); }
+template <int DIM, typename Acc, bool UNIFORM, int U>
+__global__ void __launch_bounds__(kTPB32, forces_blocks(UNIFORM, U)) k_forces32(int n, const float4* pos4,
                                                      const int32_t* cell_of,
                                                      const int32_t* start, Grid G, Consts<float> K,
                                                      StateSet<float> S, const float* mf,
@@ -1198,47 +1204,47 @@ __global__ void __launch_bounds__(kTPB32, UNIFORM ? 6 : 8) k_forces32(int n, con
                 }
                 pair((int)(ec >> kCodeBits), pj, oj, rv, r2);
             };
-            // uniform resolution: three pairs per iteration, the next
-            // iteration's three pairs of neighbour data and the entries of the
-            // one after in flight (the entries read once, as streaming loads,
-            // through a pointer that advances by three list rows per
-            // iteration); the pairs in list order, so the sums are those of a
-            // pair-by-pair walk
+            // uniform resolution: U pairs per iteration, the next iteration's U
+            // pairs of neighbour data and the entries of the one after in flight
+            // (the entries read once, as streaming loads, through a pointer that
+            // advances by U list rows per iteration); the pairs in list order,
+            // so the sums are those of a pair-by-pair walk
             if constexpr (UNIFORM) {
-                uint32_t e[6];
+                uint32_t e[2 * U];
 #pragma unroll
-                for (int t = 0; t < 6; ++t) e[t] = cnt > t ? __ldcs(lp + (size_t)t * n) : 0u;
-                float4 pc[3], oc[3];
+                for (int t = 0; t < 2 * U; ++t) e[t] = cnt > t ? __ldcs(lp + (size_t)t * n) : 0u;
+                float4 pc[U], oc[U];
 #pragma unroll
-                for (int t = 0; t < 3; ++t) {
+                for (int t = 0; t < U; ++t) {
                     pc[t] = pos4[e[t] >> kCodeBits];
                     oc[t] = vr[e[t] >> kCodeBits];
                 }
                 int k = 0;
-                const uint32_t* lq = lp + 6 * (size_t)n;
-                const size_t n3 = 3 * (size_t)n;
-                for (; k + 2 < cnt; k += 3, lq += n3) {
-                    float4 pn[3], on[3];
+                const uint32_t* lq = lp + 2 * U * (size_t)n;
+                const size_t nu = U * (size_t)n;
+                for (; k + U - 1 < cnt; k += U, lq += nu) {
+                    float4 pn[U], on[U];
 #pragma unroll
-                    for (int t = 0; t < 3; ++t) {
-                        pn[t] = pos4[e[3 + t] >> kCodeBits];
-                        on[t] = vr[e[3 + t] >> kCodeBits];
+                    for (int t = 0; t < U; ++t) {
+                        pn[t] = pos4[e[U + t] >> kCodeBits];
+                        on[t] = vr[e[U + t] >> kCodeBits];
                     }
-                    uint32_t en[3];
+                    uint32_t en[U];
 #pragma unroll
-                    for (int t = 0; t < 3; ++t) en[t] = k + 6 + t < cnt ? __ldcs(lq + (size_t)t * n) : 0u;
+                    for (int t = 0; t < U; ++t) en[t] = k + 2 * U + t < cnt ? __ldcs(lq + (size_t)t * n) : 0u;
 #pragma unroll
-                    for (int t = 0; t < 3; ++t) one(e[t], pc[t], oc[t]);
+                    for (int t = 0; t < U; ++t) one(e[t], pc[t], oc[t]);
 #pragma unroll
-                    for (int t = 0; t < 3; ++t) {
+                    for (int t = 0; t < U; ++t) {
                         pc[t] = pn[t];
                         oc[t] = on[t];
-                        e[t] = e[3 + t];
-                        e[3 + t] = en[t];
+                        e[t] = e[U + t];
+                        e[U + t] = en[t];
                     }
                 }
-                if (k < cnt) one(e[0], pc[0], oc[0]);
-                if (k + 1 < cnt) one(e[1], pc[1], oc[1]);
+#pragma unroll
+                for (int t = 0; t < U - 1; ++t)
+                    if (k + t < cnt) one(e[t], pc[t], oc[t]);
             } else {
                 // variable resolution (the pair's h per pair: more registers):
                 // two pairs per iteration, the neighbour data one pair ahead
@@ -1404,10 +1410,10 @@ static void forces_t(int n, const float4* pos4, const int32_t* cell_of, const in
                      const FinishArgs& F, cudaStream_t st)
 {
     const int T = pair_threads(32, n, G.sms);
-    launch(k_forces32<DIM, Acc, U>, nblk(n, T), T, 0, st, n, pos4, cell_of, start, G, K, S, mf, vr, nbl, nbc,
-                                                      nbl_capacity(DIM), F.dt, kick_on, write_ad, Rout, chi,
-                                                      grid_sum(F, nblk(n, T)), dt_consts(*F.P), F.diag, F.dt,
-                                                      F.count_step);
+    const bool deep = U && nblk(n, T) <= kDeepBlocks * G.sms;
+    launch(deep ? k_forces32<DIM, Acc, U, U ? kDeepPairs : 3> : k_forces32<DIM, Acc, U, 3>, nblk(n, T), T, 0, st, n,
+           pos4, cell_of, start, G, K, S, mf, vr, nbl, nbc, nbl_capacity(DIM), F.dt, kick_on, write_ad, Rout, chi,
+           grid_sum(F, nblk(n, T)), dt_consts(*F.P), F.diag, F.dt, F.count_step);
 }
 
 #define SPH_DISPATCH32(FN, ...)                                                   \
