@@ -108,14 +108,16 @@ struct Tape {
 
 // Visit the neighbours j != k of particle k with 0 < r < 2 h_kj, decided
 // exactly as the forward pass decided them: f(j, rv[3] = x_k - x_j, r, 1/r,
-// w_j) with w_j = pos4[j].w (FP32 form: m_j at uniform resolution, else h_j).
+// w_j, load(j)) with w_j = pos4[j].w (FP32 form: m_j at uniform resolution,
+// else h_j) and load(j) whatever else of j the caller gathers, which the FP32
+// list walk requests one neighbour ahead.
 // Lane q of a group of L takes the list's entries q, q + L, ...; a particle
 // with more neighbours than the list holds is walked over its cells by lane 0.
 // FP32 form: 1/r from rsqrt and r = r^2/r, as the forward force pass takes
 // them; FP64 form: 1/r within one rounding, r = r^2 (1/r).
-template <typename Real, int DIM, int L, typename F>
+template <typename Real, int DIM, int L, typename Load, typename F>
 __device__ __forceinline__ void adj_visit(int n, int k, int q, const Grid& G, const Consts<Real>& K,
-                                          const Tape<Real>& T, F& f)
+                                          const Tape<Real>& T, Load& load, F& f)
 {
     const int cnt = T.nbc[k];
     const bool listed = cnt <= list_capacity(DIM);
@@ -127,18 +129,23 @@ __device__ __forceinline__ void adj_visit(int n, int k, int q, const Grid& G, co
             // accepted, in the walk's order; the pair vector and r^2 with the
             // walk's arithmetic
             const float ex = G.edgef[0], ey = G.edgef[1], ez = G.edgef[2];
-            // the lane's entry two ahead and the neighbour's position one ahead in flight
+            // the lane's entry two ahead and the neighbour's data one ahead in flight
             const size_t row = (size_t)L * n;
             const uint32_t* lp = T.nbl + k + (size_t)q * n;
             uint32_t e_n = q < cnt ? lp[0] : 0u;
             uint32_t e_nn = q + L < cnt ? lp[row] : 0u;
             float4 p_n = T.pos4[e_n >> kCodeBits];
+            auto d_n = load((int)(e_n >> kCodeBits));
             lp += 2 * row;
             for (int t = q; t < cnt; t += L, lp += row) {
                 const uint32_t e = e_n;
                 const float4 pj = p_n;
+                const auto dj = d_n;
                 e_n = e_nn;
-                if (t + L < cnt) p_n = T.pos4[e_n >> kCodeBits];
+                if (t + L < cnt) {
+                    p_n = T.pos4[e_n >> kCodeBits];
+                    d_n = load((int)(e_n >> kCodeBits));
+                }
                 e_nn = t + 2 * L < cnt ? *lp : 0u;
                 const int j = (int)(e >> kCodeBits);
                 const uint32_t code = e & ((1u << kCodeBits) - 1u);
@@ -156,7 +163,7 @@ __device__ __forceinline__ void adj_visit(int n, int k, int q, const Grid& G, co
                 }
                 const Real rv[3] = {rxy.x, rxy.y, rz};
                 const float inv_r = rsqrtf(r2);
-                f(j, rv, r2 * inv_r, inv_r, pj.w);
+                f(j, rv, r2 * inv_r, inv_r, pj.w, dj);
             }
             return;
         }
@@ -175,7 +182,7 @@ __device__ __forceinline__ void adj_visit(int n, int k, int q, const Grid& G, co
             if (!(r2 < lim) || !(r2 > 0.f)) return;
             const Real rv[3] = {rx, ry, rz};
             const float inv_r = rsqrtf(r2);
-            f(j, rv, r2 * inv_r, inv_r, pj.w);
+            f(j, rv, r2 * inv_r, inv_r, pj.w, load(j));
         };
         for_candidates_rows<DIM, false>(ok, reach, T.cell[k], G, T.start, T.cell, T.pos4, g);
     } else {
@@ -207,7 +214,7 @@ __device__ __forceinline__ void adj_visit(int n, int k, int q, const Grid& G, co
                     r2 += y * y;
                 }
                 const double inv_r = rsqrt_pos(r2);
-                f(j, rv, r2 * inv_r, inv_r, 0.f);
+                f(j, rv, r2 * inv_r, inv_r, 0.f, load(j));
             }
             return;
         }
@@ -236,7 +243,7 @@ __device__ __forceinline__ void adj_visit(int n, int k, int q, const Grid& G, co
                         const double r = sqrt(r2);
                         const double hij = pair_h(K, T.h[k], T.h[j]);
                         if (!(r < 2.0 * hij) || r == 0.0) continue;
-                        f(j, rv, (Real)r, Real(1) / (Real)r, 0.f);
+                        f(j, rv, (Real)r, Real(1) / (Real)r, 0.f, load(j));
                     }
                 }
             }
@@ -380,6 +387,13 @@ __global__ void __launch_bounds__(256) k_adj_prep(int n, Tape<Real> T, Consts<Re
 
 constexpr int kAdjTPB = 128;
 
+// What the pair kernel gathers of a neighbour besides its position.
+template <typename Real>
+struct Neighbour {
+    typename Vec4<Real>::T vr;
+    Real Ab[3], Rb[3];
+};
+
 template <typename Real, int DIM, int L>
 __global__ void __launch_bounds__(kAdjTPB) k_adj_pairs(int n, Tape<Real> T, Grid G, Consts<Real> K,
                                                    const Real* AR,
@@ -402,10 +416,16 @@ __global__ void __launch_bounds__(kAdjTPB) k_adj_pairs(int n, Tape<Real> T, Grid
         const Real h_k = K.uniform_h ? K.h_u : (Real)T.h[k];
         Real Ak[3] = {0, 0, 0}, Rk[3] = {0, 0, 0};
         load_ab<Real, DIM>(AR, k, Ak, Rk);
-        auto pair = [&](int j, const Real* rv, Real r, Real inv_r, float w_j) {
+        auto load = [&](int j) {
+            Neighbour<Real> d = {};
+            d.vr = T.vr[j];
+            load_ab<Real, DIM>(AR, j, d.Ab, d.Rb);       // zero for a wall
+            return d;
+        };
+        auto pair = [&](int j, const Real* rv, Real r, Real inv_r, float w_j, const Neighbour<Real>& nb) {
             Real w, w2;
             pair_kernels<Real, DIM>(K, T, k, j, h_k, w_j, r, w, w2);
-            const auto mj = T.vr[j];
+            const auto mj = nb.vr;
             const Real vj[3] = {mj.x, mj.y, mj.z};
             const bool wall = isinf(mj.w);
             const Real rho_j = wall ? rho_k : K.rho0 + mj.w;
@@ -423,8 +443,8 @@ __global__ void __launch_bounds__(kAdjTPB) k_adj_pairs(int n, Tape<Real> T, Grid
             eta += (double)eb;
             if (wall) return;
             // the fluid neighbour's sums (j as i, k as j): r_jk = -r_kj
-            Real Aj[3] = {0, 0, 0}, Rj[3] = {0, 0, 0}, mrv[3] = {0, 0, 0};
-            load_ab<Real, DIM>(AR, j, Aj, Rj);
+            const Real *Aj = nb.Ab, *Rj = nb.Rb;
+            Real mrv[3] = {0, 0, 0};
             for (int d = 0; d < DIM; ++d) mrv[d] = -rv[d];
             pair_adjoint<Real, DIM>(K, mrv, r, inv_r, w, w2, vj, rho_j, inv_rho_j, p_j, vk, rho_k, inv_rho_k, p_k,
                                     m_k, Aj, Rj, rb, dvb, rib, rjb, eb);
@@ -434,7 +454,7 @@ __global__ void __launch_bounds__(kAdjTPB) k_adj_pairs(int n, Tape<Real> T, Grid
             }
             arho.add(rjb);
         };
-        adj_visit<Real, DIM, L>(n, k, q, G, K, T, pair);
+        adj_visit<Real, DIM, L>(n, k, q, G, K, T, load, pair);
     }
     __syncwarp();
 #pragma unroll
@@ -498,13 +518,14 @@ __global__ void __launch_bounds__(kAdjTPB) k_adj_density(int n, Tape<Real> T, Gr
     if (fluid) {
         const Real sk = sigb[k];
         const Real h_k = K.uniform_h ? K.h_u : (Real)T.h[k];
-        auto pair = [&](int j, const Real* rv, Real r, Real inv_r, float w_j) {
+        auto load = [&](int j) { return sigb[j]; };           // 0 for a wall
+        auto pair = [&](int j, const Real* rv, Real r, Real inv_r, float w_j, Real sj) {
             Real w, w2;
             pair_kernels<Real, DIM>(K, T, k, j, h_k, w_j, r, w, w2);
-            const Real g = (sk + sigb[j]) * w * inv_r;        // sigb is 0 for a wall
+            const Real g = (sk + sj) * w * inv_r;
             for (int d = 0; d < DIM; ++d) acc[d].add(g * rv[d]);
         };
-        adj_visit<Real, DIM, L>(n, k, q, G, K, T, pair);
+        adj_visit<Real, DIM, L>(n, k, q, G, K, T, load, pair);
     }
     __syncwarp();
 #pragma unroll
