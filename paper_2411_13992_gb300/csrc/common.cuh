@@ -351,6 +351,17 @@ __device__ __forceinline__ float sqrt_approx(float x)
     return y;
 }
 
+// 1/sqrt(x) of the special-function unit for a normal x > 0: rsqrtf's value
+// there, without the scaling of subnormal arguments that rsqrtf wraps around
+// it (a test and two multiplications per pair; the density pass takes the
+// distances of the same pairs from sqrt_approx, which flushes them too).
+__device__ __forceinline__ float rsqrt_approx(float x)
+{
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 // Neighbour-list entries: (j << kCodeBits) | stencil code of j's cell, the
 // code being (dx + R) + S (dy + R) + S^2 (dz + R) with S = 2R + 1.
 constexpr int kSide = 2 * kStencilR + 1;                 // stencil cells per axis

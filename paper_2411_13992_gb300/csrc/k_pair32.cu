@@ -1171,7 +1171,7 @@ __global__ void __launch_bounds__(kTPB32, forces_blocks(UNIFORM, U)) k_forces32(
         // W'/r = coef t^3, coef = -5 a_D h^-(D+2) (uniform h: one constant)
         const float norm = kernel_norm<DIM, float>();
         auto pair = [&](int j, const float4& pj, const float4& oj, const float* rv, float r2) {
-            const float inv_r = rsqrtf(r2);
+            const float inv_r = rsqrt_approx(r2);
             const float r = r2 * inv_r;
             float inv_h, m_j;
             if (UNIFORM) {
