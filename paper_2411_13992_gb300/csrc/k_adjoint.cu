@@ -162,7 +162,7 @@ __device__ __forceinline__ void adj_visit(int n, int k, int q, const Grid& G, co
                     r2 = fmaf(rz, rz, r2);
                 }
                 const Real rv[3] = {rxy.x, rxy.y, rz};
-                const float inv_r = rsqrt_approx(r2);
+                const float inv_r = rsqrtf(r2);
                 f(j, rv, r2 * inv_r, inv_r, pj.w, dj);
             }
             return;
@@ -181,7 +181,7 @@ __device__ __forceinline__ void adj_visit(int n, int k, int q, const Grid& G, co
             }
             if (!(r2 < lim) || !(r2 > 0.f)) return;
             const Real rv[3] = {rx, ry, rz};
-            const float inv_r = rsqrt_approx(r2);
+            const float inv_r = rsqrtf(r2);
             f(j, rv, r2 * inv_r, inv_r, pj.w, load(j));
         };
         for_candidates_rows<DIM, false>(ok, reach, T.cell[k], G, T.start, T.cell, T.pos4, g);

@@ -34,14 +34,18 @@ __device__ __forceinline__ Real tv_limiter(const Consts<Real>& K, Real s)
 }
 
 // 1/sqrt(x) and sqrt(x) for a normal x > 0 in six FP64 operations: the
-// hardware's approximation y0 (its upper word only), then one step of
-// Householder's third-order iteration for x^(-1/2), y0 (1 + e/2 + 3 e^2/8)
+// hardware's approximation y0 (from the upper word of x only), then one step
+// of Householder's third-order iteration for x^(-1/2), y0 (1 + e/2 + 3 e^2/8)
 // with e = 1 - x y0^2.  The error left by the iteration is O(e^3) < 2^-58, so
-// that both results are within one rounding of the exact values.
+// that both results are within one rounding of the exact values.  For a
+// subnormal x (a pair closer than 1.5e-154) the seed is that of the smallest
+// normal number (an integer maximum on the upper word), and both results are
+// finite.
 __device__ __forceinline__ double rsqrt_seed(double x)
 {
     double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double xn = __hiloint2double(max(__double2hiint(x), 0x00100000), __double2loint(x));
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(xn));
     return y;
 }
 
