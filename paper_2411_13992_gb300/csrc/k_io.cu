@@ -87,6 +87,7 @@ __device__ __forceinline__ double sigma0_shared(double h, double m, double rho0)
     const double vol = m / rho0;
     const double dp = DIM == 2 ? sqrt(vol) : cbrt(vol);
     const double ratio = h / dp;
+    if (!(ratio < 500.0)) return sigma0_of<DIM>(h, m, rho0);     // the points' count would pass 32 bits
     const double reach2 = 4.0 * ratio * ratio;
     const int side = (int)ceil(2.0 * ratio) + 1;
     const double inv = 1.0 / ratio;

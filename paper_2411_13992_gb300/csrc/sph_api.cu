@@ -661,9 +661,11 @@ bool is_host_ptr(const void* p)
 // Address through which this device's kernels can reach p directly: p for
 // memory of the current device (or managed memory), the mapped alias of
 // page-locked host memory; nullptr otherwise (pageable host memory, another
-// device), which then goes through the staging buffer by a copy.
-void* device_view(const void* p)
+// device, values off their natural alignment), which then goes through the
+// staging buffer by a copy.
+void* device_view(const void* p, size_t align = sizeof(double))
 {
+    if ((uintptr_t)p % align) return nullptr;
     cudaPointerAttributes attr;
     if (cudaPointerGetAttributes(&attr, p) != cudaSuccess) {
         cudaGetLastError();
@@ -701,7 +703,7 @@ sph_status vec_in(sph_ctx* c, int prec, const double* src, void* dst, const doub
 template <typename T>
 sph_status scalar_in(sph_ctx* c, const T* src, T* dst, const T** view)
 {
-    *view = (const T*)device_view(src);
+    *view = (const T*)device_view(src, alignof(T));
     if (*view) return SPH_OK;
     SPH_CU(cudaMemcpyAsync(dst, src, (size_t)c->n * sizeof(T), cudaMemcpyDefault, c->st));
     *view = dst;
