@@ -17,6 +17,8 @@
 // Method (see k_pair.cu for the FP64 form and pair_physics.cuh for the
 // readings of the paper): density Eq. 8 with Eq. 2; pressure Eq. 3, 5, 6;
 // viscous Eq. 7; residual, limiter and displacement Eq. 14-16.
+#include <type_traits>
+
 #include "common.cuh"
 #include "launch.h"
 #include "pair_physics.cuh"
@@ -395,6 +397,103 @@ __global__ void __launch_bounds__(kDensityTPB32, 2) k_density32(int n, const flo
     // rho - rho0 = rho0 (sigma - sigma0) / sigma0; sigma - sigma0 is exact in FP32
     const float w = K.rho0 * (sigma.value() - s0) / s0;
     vr[i] = make_float4(vi[0], vi[1], vi[2], w);
+}
+
+// The density pass at uniform resolution with a group of L lanes per particle,
+// for problems too small to fill the chip with one thread each (one warp on
+// some of the SMs, each thread with a chain of some 10,000 instructions in
+// 3-D).  The lanes first find the bounds of the stencil rows (one row per lane
+// at a time), then take each row's candidates L at a time, the next row's
+// first ones in flight.  Every lane adds all L terms, handed round by
+// shuffles, so that the compensated sum is taken in the row walk's order, and
+// a ballot gives each neighbour its place in the list: sigma and the list are
+// bit for bit those of k_density32.
+// Measured, us a step: see density_lanes().
+template <int DIM, typename Acc, int L>
+__global__ void __launch_bounds__(256) k_density32_lanes(int n, const int32_t* cell_of, const int32_t* start, Grid G,
+                                                         Consts<float> K, StateSet<float> S, float4* vr,
+                                                         uint32_t* nbl, int32_t* nbc, int cap, const float4* pos4c)
+{
+    pdl_wait();
+    constexpr int R = kStencilR, NR = DIM == 3 ? kSide * kSide : kSide;
+    constexpr unsigned kAll = 0xffffffffu;
+    __shared__ RowRuns bounds[256 / L * NR];
+    const int lane = threadIdx.x & 31, q = lane & (L - 1), lead = lane - q;
+    const unsigned below = (1u << lane) - 1u, group = ((1u << L) - 1u) << lead;
+    const int p = threadIdx.x / L, i = blockIdx.x * (blockDim.x / L) + p, k = min(i, n - 1);
+    const bool active = i < n && S.kind[k] == 0;
+    const float4 pi = pos4c[k];
+    const float oi[3] = {pi.x, pi.y, pi.z};
+    const int cell_i = cell_of[k];
+    const float s0 = (float)S.s0[k];
+    float vi[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) vi[d] = S.v[(size_t)d * n + k];
+    int c[3];
+    cell_decode(G, cell_i, c);
+    RowRuns* rows = bounds + p * NR;
+    for (int r = q; r < NR; r += L) {
+        RowRuns rr = {0, 0, 0, 0, 0};
+        if (active) rr = row_runs<DIM>(r, oi, 2.f * K.h_u, c, G, start);
+        rows[r] = rr;
+    }
+    __syncwarp();
+    const float ex = G.edgef[0], ey = G.edgef[1], ez = G.edgef[2];
+    const float wnorm = kernel_norm<DIM, float>() * pow_dim<DIM, float>(K.inv_h_u);
+    // candidate f of a row, if it has as many
+    auto at = [&](const RowRuns& rr, int f) { return f < rr.n0 ? rr.j0 + f : rr.j1 + (f - rr.n0); };
+    auto record = [&](const RowRuns& rr, int f) {
+        return f < rr.n0 + rr.n1 ? pos4c[at(rr, f)] : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    Acc sigma;
+    int cnt = 0;
+    RowRuns rr = rows[0];
+    float4 pj = record(rr, q);
+    for (int r = 0; r < NR; ++r) {
+        const int len = rr.n0 + rr.n1;
+        const int most = __reduce_max_sync(kAll, len);
+        const int dy = r % kSide - R, dz = DIM == 3 ? r / kSide - R : 0;
+        const float shy = -(float)dy * ey, shz = -(float)dz * ez;
+        const RowRuns next = rows[r + 1 < NR ? r + 1 : r];
+        const float4 pn = record(next, q);
+        for (int f0 = 0; f0 < most; f0 += L) {
+            const int f = f0 + q;
+            const bool have = f < len;
+            if (f0) pj = record(rr, f);
+            int dx = __float_as_int(pj.w) - rr.row - c[0];
+            if (dx > R) dx -= G.nc[0];                    // across the periodic x boundary
+            else if (dx < -R) dx += G.nc[0];
+            const float2 rxy = __fadd2_rn(__ffma2_rn(make_float2(pj.x, pj.y), make_float2(-1.f, -1.f),
+                                                     make_float2(oi[0], oi[1])),
+                                          make_float2(-(float)dx * ex, shy));
+            const float2 sq = __fmul2_rn(rxy, rxy);
+            float r2 = sq.x + sq.y;
+            if (DIM == 3) {
+                const float rz = (oi[2] - pj.z) + shz;
+                r2 = fmaf(rz, rz, r2);
+            }
+            const float w = w_term_uniform(K, wnorm, r2);
+#pragma unroll
+            for (int t = 0; t < L; ++t) {
+                if (f0 + t >= most) break;
+                sigma.add_if(__shfl_sync(kAll, w, lead + t), f0 + t < len);
+            }
+            const bool take = have && r2 < K.four_h2_u && r2 > 0.f;
+            const unsigned m = __ballot_sync(kAll, take) & group;
+            const int pos = cnt + __popc(m & below);
+            if (take && pos < cap)
+                __stcs(nbl + (size_t)pos * n + i,
+                       ((uint32_t)at(rr, f) << kCodeBits) |
+                           (uint32_t)((dx + R) + kSide * (dy + R) + kSide * kSide * (dz + R)));
+            cnt += __popc(m);
+        }
+        rr = next;
+        pj = pn;
+    }
+    if (i >= n || q) return;
+    nbc[i] = cnt;
+    vr[i] = make_float4(vi[0], vi[1], vi[2],
+                        active ? K.rho0 * (sigma.value() - s0) / s0 : __int_as_float(0x7f800000));
 }
 
 // ------------------------------------------------- density on cell-blocked tiles
@@ -1355,11 +1454,35 @@ static inline int nblk(int n, int t) { return (n + t - 1) / t; }
 
 int nbl_capacity(int dim) { return list_capacity(dim); }
 
+// Lanes per particle of the density pass at uniform resolution.  Measured, us
+// a step with 1 / 4 / 8 / 16 lanes, lines at 32, 96 and 180 particles per SM:
+// 2-D 2,304 particles 32.6 / 29.9 / 28.2 / 27.9, 10,000: 33.3 / 30.7 / 30.2 /
+// 33.3, 25,600: 34.7 / 33.2 / 35.7 / 41.8, 30,600: 35.6 / 36.0 / 37.7; 3-D
+// 4,096: 79.6 / 61.5 / 52.8 / 50.1, 13,824: 76.4 / 63.7 / 59.9 / 70.9, 19,683:
+// 78.2 / 71.4 / 79.1, 27,000: 80.5 / 74.2 / 86.1, 29,791: 85.8 / 87.3.
+static int density_lanes(int n, int sms)
+{
+    return n < sms * 32 ? 16 : (n < sms * 96 ? 8 : (n < sms * 180 ? 4 : 1));
+}
+
 template <int DIM, typename Acc, bool U>
 static void density_t(int n, const float4* pos4, const int32_t* cell_of, const int32_t* start, const Grid& G,
                       const Consts<float>& K, StateSet<float> S, float4* vr, uint32_t* nbl, int32_t* nbc,
                       cudaStream_t st, const float4* pos4c)
 {
+    // (plain sums keep one lane: a thread fuses a term's last product into the
+    // sum, which terms handed round between lanes cannot)
+    if constexpr (U && std::is_same<Acc, KSum>::value) {
+        const int L = density_lanes(n, G.sms);
+        if (L > 1) {
+            // as many threads as spread the particles evenly over the SMs
+            const int64_t t = ((int64_t)n * L + G.sms - 1) / G.sms;
+            const int T = t > 256 ? 256 : (int)((t + 31) / 32 * 32);
+            auto kern = L == 4 ? k_density32_lanes<DIM, Acc, 4> : L == 8 ? k_density32_lanes<DIM, Acc, 8> : k_density32_lanes<DIM, Acc, 16>;
+            launch(kern, nblk(n, T / L), T, 0, st, n, cell_of, start, G, K, S, vr, nbl, nbc, nbl_capacity(DIM), pos4c);
+            return;
+        }
+    }
     const int T = n >= G.sms * kDensityTPB32 ? kDensityTPB32 : pair_threads(32, n, G.sms);
     launch(k_density32<DIM, Acc, U>, nblk(n, T), T, 0, st, n, pos4, cell_of, start, G, K, S, vr, nbl, nbc,
                                                        nbl_capacity(DIM), pos4c);

@@ -183,4 +183,65 @@ __device__ __forceinline__ void for_candidates_rows(const float* oi, float reach
     }
 }
 
+// One stencil row of a particle's walk: two runs of the sort order (the
+// second empty unless the row wraps a periodic x boundary) and the cell index
+// of the row's first cell.
+struct RowRuns {
+    int j0, n0, j1, n1, row;
+};
+
+// Row r = (dy + R) + kSide (dz + R) of the stencil of a particle in cell c at
+// offset oi, cut as for_candidates_rows cuts it.
+template <int DIM>
+__device__ __forceinline__ RowRuns row_runs(int r, const float* oi, float reach, const int* c, const Grid& G,
+                                            const int32_t* start)
+{
+    constexpr int R = kStencilR;
+    RowRuns q = {0, 0, 0, 0, 0};
+    const int dy = r % kSide - R, dz = DIM == 3 ? r / kSide - R : 0;
+    const int cy = cell_step(G, c[1], dy, 1), cz = DIM == 3 ? cell_step(G, c[2], dz, 2) : 0;
+    const float ex = G.edgef[0], ey = G.edgef[1], ez = G.edgef[2];
+    float ry = dy > 0 ? dy * ey - oi[1] : (dy < 0 ? oi[1] + (-dy - 1) * ey : 0.f), rz = 0.f;
+    ry = fmaxf(ry - 1e-3f * ey, 0.f);
+    if (DIM == 3) {
+        rz = dz > 0 ? dz * ez - oi[2] : (dz < 0 ? oi[2] + (-dz - 1) * ez : 0.f);
+        rz = fmaxf(rz - 1e-3f * ez, 0.f);
+    }
+    const float w2 = (reach * reach - rz * rz) - ry * ry;
+    if (cy < 0 || cz < 0 || !(w2 > 0.f)) return q;
+    const int sh = G.sub_shift, nsx = G.nc[0] << sh;
+    const int32_t* rstart = sh ? G.sub_start : start;
+    const float inv_exs = (1.f / ex) * (float)(1 << sh);
+    const float w = sqrt_approx(w2) + 1e-3f * ex;
+    const int slo = max(__float2int_rd((oi[0] - w) * inv_exs), -(R << sh));
+    const int shi = min(__float2int_rd((oi[0] + w) * inv_exs), ((R + 1) << sh) - 1);
+    if (slo > shi) return q;
+    q.row = G.nc[0] * (cy + G.nc[1] * cz);
+    const int rb = q.row << sh;
+    int lo0 = (c[0] << sh) + slo, hi0 = (c[0] << sh) + shi, lo1 = 0, hi1 = -1;
+    if (!G.periodic[0]) {
+        lo0 = max(lo0, 0);
+        hi0 = min(hi0, nsx - 1);
+    } else if (lo0 < 0) {
+        hi1 = hi0;
+        lo0 += nsx;
+        hi0 = min(nsx - 1, nsx + hi1);
+    } else if (lo0 >= nsx) {
+        lo0 -= nsx;
+        hi0 -= nsx;
+    } else if (hi0 >= nsx) {
+        hi1 = hi0 - nsx;
+        hi0 = nsx - 1;
+    }
+    if (lo0 <= hi0) {
+        q.j0 = rstart[rb + lo0];
+        q.n0 = rstart[rb + hi0 + 1] - q.j0;
+    }
+    if (lo1 <= hi1) {
+        q.j1 = rstart[rb + lo1];
+        q.n1 = rstart[rb + hi1 + 1] - q.j1;
+    }
+    return q;
+}
+
 }  // namespace sphtv
