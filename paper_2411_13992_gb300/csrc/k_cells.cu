@@ -195,7 +195,8 @@ __device__ __forceinline__ int32_t block_scan(int32_t s, int32_t* warp_tot, int3
 // start of bin k is prefix[k] + tile_off[k / kScanTile] (the readers add the
 // two: no pass over the bins for it).  Clears the counts as it reads them.
 // The block that finishes last scans the tiles' sums (one kernel where there
-// were two or three).  Where each reading warp scanned up to 32 sums itself
+// were two or three); a single tile needs no such scan (step of 2,304
+// particles 27.9 -> 25.8 us, of 4,096 in 3-D 50.1 -> 48.1).  Where each reading warp scanned up to 32 sums itself
 // instead, the step of a small problem took as long and the permute 3 us more
 // at 128^3.
 __global__ void __launch_bounds__(kScanThreads) k_bin_scan(int32_t* count, int32_t* prefix,
@@ -242,6 +243,10 @@ __global__ void __launch_bounds__(kScanThreads) k_bin_scan(int32_t* count, int32
             if (base + k < n) prefix[base + k] = vals[k];
     }
     const int nt = gridDim.x;
+    if (nt == 1) {
+        if (threadIdx.x == 0) tile_off[0] = 0;
+        return;
+    }
     if (threadIdx.x == 0) {
         tile_off[blockIdx.x] = total;
         __threadfence();
