@@ -191,7 +191,12 @@ def _ptr(a, keep: list, dtype, shape_tail=None):
     try:
         import torch
         if isinstance(a, torch.Tensor):
-            tdt = {np.float64: torch.float64, np.int8: torch.int8}[dtype]
+            tdt = torch.float64 if dtype is np.float64 else torch.int8
+            if a.dtype is tdt and a.is_contiguous() and not (shape_tail == 3 and a.dim() == 2 and a.shape[1] == 2):
+                # as it is: no conversion to ask for (three calls a tensor, a
+                # sixth of a one-step call of 3,000 particles)
+                keep.append(a)
+                return a.data_ptr()
             t = a.detach().to(tdt).contiguous()
             if shape_tail == 3 and t.dim() == 2 and t.shape[1] == 2:
                 t = torch.nn.functional.pad(t, (0, 1))
