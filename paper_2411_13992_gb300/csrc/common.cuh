@@ -245,6 +245,34 @@ __device__ __forceinline__ double f2d_exact(float f)
                                             ((unsigned long long)(u & 0x7fffffu) << 29)));
 }
 
+// A double rounded to the nearest float (ties to even), as the hardware
+// conversion rounds it, on the integer ALU for results that are normal
+// floats: the 52-bit fraction is cut to 23 bits and rounded up when the cut
+// part is above half an ulp, or exactly half with an odd last kept bit (a
+// carry out of the fraction raises the exponent, and past the largest float
+// gives infinity, as rounding does).  Zeros, subnormal results, infinities
+// and NaN take the hardware conversion.
+__device__ __forceinline__ float d2f_rn(double x)
+{
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+    const int E = (int)((b >> 52) & 0x7ff) - 1023;
+    if (E < -126 || E > 127) return (float)x;
+    const unsigned long long frac = b & 0xfffffffffffffULL;
+    const unsigned keep = (unsigned)(frac >> 29);
+    const unsigned long long cut = frac & 0x1fffffffULL;               // the 29 bits cut off
+    const unsigned up = (cut > 0x10000000ULL || (cut == 0x10000000ULL && (keep & 1u))) ? 1u : 0u;
+    const unsigned f = (((unsigned)(E + 127) << 23) + keep + up) | ((unsigned)(b >> 32) & 0x80000000u);
+    return __uint_as_float(f);
+}
+
+// x / 2 on the integer ALU for a normal x whose half is normal.
+__device__ __forceinline__ double half_exact(double x)
+{
+    const int hi = __double2hiint(x), e = hi & 0x7ff00000;
+    if (e < 0x00200000 || e == 0x7ff00000) return 0.5 * x;
+    return __hiloint2double(hi - 0x00100000, __double2loint(x));
+}
+
 // max(trunc(t), 0) on the integer ALU for the cell index (the callers clamp
 // it to [0, nc - 1]), as the hardware conversion toward zero then the clamp
 // would give it: 0 for t < 1 (and -0.0, negative t, NaN), the integer part

@@ -26,26 +26,6 @@ __device__ __forceinline__ double i2d_exact(int c)
     return __longlong_as_double((long long)(((unsigned long long)(e + 1023) << 52) | frac));
 }
 
-// A double rounded to the nearest float (ties to even), as the hardware
-// conversion rounds it, on the integer ALU for results that are normal
-// floats: the 52-bit fraction is cut to 23 bits and rounded up when the cut
-// part is above half an ulp, or exactly half with an odd last kept bit (a
-// carry out of the fraction raises the exponent, and past the largest float
-// gives infinity, as rounding does).  Zeros, subnormal results, infinities
-// and NaN take the hardware conversion.
-__device__ __forceinline__ float d2f_rn(double x)
-{
-    const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-    const int E = (int)((b >> 52) & 0x7ff) - 1023;
-    if (E < -126 || E > 127) return (float)x;
-    const unsigned long long frac = b & 0xfffffffffffffULL;
-    const unsigned keep = (unsigned)(frac >> 29);
-    const unsigned long long cut = frac & 0x1fffffffULL;               // the 29 bits cut off
-    const unsigned up = (cut > 0x10000000ULL || (cut == 0x10000000ULL && (keep & 1u))) ? 1u : 0u;
-    const unsigned f = (((unsigned)(E + 127) << 23) + keep + up) | ((unsigned)(b >> 32) & 0x80000000u);
-    return __uint_as_float(f);
-}
-
 template <typename Real>
 __device__ __forceinline__ Real kick(Real v, double hdt, Real a);
 

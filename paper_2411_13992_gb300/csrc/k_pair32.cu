@@ -1256,7 +1256,14 @@ __global__ void __launch_bounds__(kTPB32, forces_blocks(UNIFORM, U)) k_forces32(
 #pragma unroll
     for (int k = 0; k < kNPart; ++k) part[k] = 0.0;
     const double dt = *dt_ptr;
-    const double hdt = kick_on ? 0.5 * dt : 0.0;
+    // The FP64 pipe bounds the end of the step in 2-D on a grid of several
+    // waves (some 26 operations of 19 SM cycles a warp, against 20 neighbours a
+    // particle): conversions and factors of 1/2 go to the integer ALU there
+    // (pass of 490,000 particles 56.2 -> 51.6 us, same bits).  In 3-D and on
+    // small grids the longer integer chains cost 0.2-2 us a step instead.
+    constexpr bool kOffPipe = DIM == 2 && U == 3;
+    auto wide = [](float f) { return kOffPipe ? f2d_exact(f) : (double)f; };
+    const float dtf = kOffPipe ? d2f_rn(dt) : (float)dt;
     if (i < n && S.kind[i] == 0) {
         const float4 pi = pos4[i];
         const float oi[3] = {pi.x, pi.y, pi.z};
@@ -1405,8 +1412,8 @@ __global__ void __launch_bounds__(kTPB32, forces_blocks(UNIFORM, U)) k_forces32(
         // momentum and kinetic energy in FP64; the maxima of the transport
         // speed |v + dr/dt| and of |dr| (diagnostics of the correction) from
         // FP32 squares, to keep this epilogue off the FP64 pipe
-        const float inv_dt = dt > 0.0 ? 1.f / (float)dt : 0.f;
-        const float hdtf = (float)hdt;
+        const float inv_dt = dtf > 0.f ? 1.f / dtf : 0.f;
+        const float hdtf = kick_on ? 0.5f * dtf : 0.f;
         double v2 = 0.0;
         float vt2 = 0.f, dr2 = 0.f;
 #pragma unroll
@@ -1420,19 +1427,20 @@ __global__ void __launch_bounds__(kTPB32, forces_blocks(UNIFORM, U)) k_forces32(
             }
             S.v[o] = vn;
             Rout[o] = R[d];
-            part[1 + d] = m_i * (double)vn;
-            v2 += (double)vn * vn;
+            const double vd = wide(vn);
+            part[1 + d] = m_i * vd;
+            v2 = d ? v2 + vd * vd : vd * vd;
             dr2 += dr * dr;
             const float vt = fmaf(dr, inv_dt, vn);
             vt2 += vt * vt;
         }
         chi_out[i] = chi;
         part[0] = m_i;
-        part[4] = 0.5 * m_i * v2;
+        part[4] = (kOffPipe ? half_exact(m_i) : 0.5 * m_i) * v2;
         part[5] = chi > 0.f ? 1.0 : 0.0;
         part[6] = v2;                 // squares: block_partials takes the roots
-        part[7] = (double)vt2;
-        part[8] = (double)dr2;
+        part[7] = wide(vt2);
+        part[8] = wide(dr2);
     } else if (i < n) {
 #pragma unroll
         for (int d = 0; d < DIM; ++d) {
