@@ -662,9 +662,10 @@ bool is_host_ptr(const void* p)
 // memory of the current device (or managed memory), the mapped alias of
 // page-locked host memory; nullptr otherwise (pageable host memory, another
 // device, values off their natural alignment), which then goes through the
-// staging buffer by a copy.
-void* device_view(const void* p, size_t align = sizeof(double))
+// staging buffer by a copy.  *host: whether p is page-locked host memory.
+void* device_view(const void* p, size_t align = sizeof(double), bool* host = nullptr)
 {
+    if (host) *host = false;
     if ((uintptr_t)p % align) return nullptr;
     cudaPointerAttributes attr;
     if (cudaPointerGetAttributes(&attr, p) != cudaSuccess) {
@@ -678,32 +679,51 @@ void* device_view(const void* p, size_t align = sizeof(double))
     }
     if (attr.type == cudaMemoryTypeManaged) return const_cast<void*>(p);
     if (attr.type == cudaMemoryTypeDevice) return attr.device == dev ? const_cast<void*>(p) : nullptr;
-    if (attr.type == cudaMemoryTypeHost && attr.devicePointer) return attr.devicePointer;
+    if (attr.type == cudaMemoryTypeHost && attr.devicePointer) {
+        if (host) *host = true;
+        return attr.devicePointer;
+    }
     return nullptr;
 }
 
+// The same for memory on the device's side alone: nullptr for host memory too,
+// which a copy brings across the link faster than a kernel that reads several
+// arrays at once (end-to-end step of 128^3 from page-locked buffers 4.24 ms
+// with copies and one conversion kernel per vector, 4.31 ms with the load
+// kernel reading them all).
+const void* device_side(const void* p, size_t align = sizeof(double))
+{
+    bool host;
+    const void* v = device_view(p, align, &host);
+    return host ? nullptr : v;
+}
+
 // [n][3] rows of src (host or device) into the per-component array dst of
-// precision prec: *in_place is src as the load kernel can read it (device
-// memory, or page-locked host memory, which streams across the host link
-// inside the kernel); else src is copied to the staging buffer, converted
-// into dst, and *in_place is null.
+// precision prec: *in_place is src as the load kernel reads it, if it is memory
+// on the device's side.  Page-locked host memory streams across the link inside
+// a conversion kernel of its own, the rest is copied to the staging buffer and
+// converted from there; *in_place is then null.
 sph_status vec_in(sph_ctx* c, int prec, const double* src, void* dst, const double** in_place)
 {
-    const size_t n = (size_t)c->n;
-    *in_place = (const double*)device_view(src);
+    bool host;
+    const double* dv = (const double*)device_view(src, sizeof(double), &host);
+    *in_place = host ? nullptr : dv;
     if (*in_place) return SPH_OK;
-    SPH_CU(cudaMemcpyAsync(c->stage, src, 3 * n * sizeof(double), cudaMemcpyDefault, c->st));
-    SPH_CU(launch_vec_in(prec, c->dim, (int)n, c->stage, dst, c->st));
+    if (!dv) {
+        SPH_CU(cudaMemcpyAsync(c->stage, src, 3 * (size_t)c->n * sizeof(double), cudaMemcpyDefault, c->st));
+        dv = c->stage;
+    }
+    SPH_CU(launch_vec_in(prec, c->dim, (int)c->n, dv, dst, c->st));
     ++c->launches;
     return SPH_OK;
 }
 
-// count elements of src as the load kernel can read them: in place, or copied
-// into dst.
+// count elements of src as the load kernel can read them: in place on the
+// device's side, or copied into dst.
 template <typename T>
 sph_status scalar_in(sph_ctx* c, const T* src, T* dst, const T** view)
 {
-    *view = (const T*)device_view(src, alignof(T));
+    *view = (const T*)device_side(src, alignof(T));
     if (*view) return SPH_OK;
     SPH_CU(cudaMemcpyAsync(dst, src, (size_t)c->n * sizeof(T), cudaMemcpyDefault, c->st));
     *view = dst;
@@ -727,7 +747,7 @@ sph_status load_state(sph_ctx* c, const double* x, const double* v, const double
     if (a) {
         SPH_TRY(vec_in(c, c->prec, a, sa, &A.a));
         SPH_TRY(vec_in(c, c->prec, dr, sdr, &A.dr));
-        if (!A.a != !A.dr) {          // one readable in place, the other staged: convert the first by itself
+        if (!A.a != !A.dr) {          // one in place, the other converted already: convert the first by itself
             const double* src = A.a ? A.a : A.dr;
             SPH_CU(launch_vec_in(c->prec, c->dim, (int)c->n, src, A.a ? sa : sdr, c->st));
             ++c->launches;
@@ -775,8 +795,8 @@ sph_status save_tape(sph_ctx* c, int t)
 }
 
 // The caller's [n][3] cotangents (xbar, vbar, abar, drbar) into the adjoint's
-// [3][n] (z row zeroed in 2-D): in one kernel what the device can read in
-// place, the others through the staging buffer.
+// [3][n] (z row zeroed in 2-D): in one kernel what lies on the device's side,
+// the others through the staging buffer.
 sph_status cotangents_in(sph_ctx* c, const double* xb, const double* vb, const double* ab, const double* db)
 {
     const AdjView& A = c->adj;
@@ -785,7 +805,7 @@ sph_status cotangents_in(sph_ctx* c, const double* xb, const double* vb, const d
     Four<const double> direct = {{nullptr, nullptr, nullptr, nullptr}};
     bool any = false;
     for (int q = 0; q < 4; ++q) {
-        direct.p[q] = (const double*)device_view(src[q]);
+        direct.p[q] = (const double*)device_side(src[q]);
         if (direct.p[q]) {
             any = true;
             continue;
@@ -1008,9 +1028,9 @@ sph_status sph_set_state(sph_ctx* c, const double* x, const double* v, const dou
     if (kind) SPH_TRY(scalar_in(c, kind, Sd.kind, &A.kind));
     if (sigma0) SPH_TRY(scalar_in(c, sigma0, Sd.s0, &A.sigma0));
     if (vw) {
-        A.vw = (const double*)device_view(vw);
+        A.vw = (const double*)device_side(vw);
         if (!A.vw) {
-            // not readable in place: the neighbour list's buffer (96 entries a
+            // to be copied: the neighbour list's buffer (96 entries a
             // particle or more, free until the next density pass) holds the
             // rows for the load, while the staging buffer serves the vectors
             SPH_CU(cudaMemcpyAsync(c->nbl, vw, 3 * (size_t)c->n * sizeof(double), cudaMemcpyDefault, c->st));
