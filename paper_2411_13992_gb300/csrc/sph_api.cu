@@ -688,7 +688,7 @@ void* device_view(const void* p, size_t align = sizeof(double), bool* host = nul
 
 // The same for memory on the device's side alone: nullptr for host memory too,
 // which a copy brings across the link faster than a kernel that reads several
-// arrays at once (end-to-end step of 128^3 from page-locked buffers 4.24 ms
+// arrays at once (end-to-end step of 128^3 from page-locked buffers 4.16 ms
 // with copies and one conversion kernel per vector, 4.31 ms with the load
 // kernel reading them all).
 const void* device_side(const void* p, size_t align = sizeof(double))
