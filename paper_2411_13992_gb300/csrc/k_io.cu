@@ -53,12 +53,23 @@ __global__ void k_rho_out_gather(int n, const V4* vr, const int8_t* kind,
     dst[i] = kind[k] ? rho0 : rho0 + (double)vr[k].w;
 }
 
+// Smoothing lengths (in units of dp) from which the lattice sum is taken at its
+// limit, the kernel's integral: sigma0 = dp^-D.  The two differ by 1.2e-15 of
+// the value at 500 in 2-D and 4e-14 at 100 in 3-D, falling with the 5th and 6th
+// power (the decay of the kernel's transform), below the rounding of the sum's
+// million and eight million terms.  Without the line the sum over the lattice
+// of a mass near or at 0 or of an infinite h has no end in practice, and the
+// load would never come to the check that reports them.
+template <int DIM> constexpr double kLatticeMax = DIM == 2 ? 500.0 : 100.0;
+
 template <int DIM>
 __device__ double sigma0_of(double h, double m, double rho0)
 {
     const double vol = m / rho0;
     const double dp = DIM == 2 ? sqrt(vol) : cbrt(vol);
     const double ratio = h / dp;               // smoothing length in units of dp
+    if (ratio >= kLatticeMax<DIM>) return 1.0 / (DIM == 2 ? dp * dp : dp * dp * dp);
+    // (a negative ratio or NaN, whose particle the load rejects: no point, or one)
     const double reach2 = 4.0 * ratio * ratio;
     const int K = (int)ceil(2.0 * ratio);
     const double inv = 1.0 / ratio;
@@ -87,7 +98,7 @@ __device__ __forceinline__ double sigma0_shared(double h, double m, double rho0)
     const double vol = m / rho0;
     const double dp = DIM == 2 ? sqrt(vol) : cbrt(vol);
     const double ratio = h / dp;
-    if (!(ratio < 500.0)) return sigma0_of<DIM>(h, m, rho0);     // the points' count would pass 32 bits
+    if (!(ratio > 0.0 && ratio < kLatticeMax<DIM>)) return sigma0_of<DIM>(h, m, rho0);   // at most 8 million points below
     const double reach2 = 4.0 * ratio * ratio;
     const int side = (int)ceil(2.0 * ratio) + 1;
     const double inv = 1.0 / ratio;
