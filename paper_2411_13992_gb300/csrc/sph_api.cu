@@ -721,11 +721,11 @@ sph_status vec_in(sph_ctx* c, int prec, const double* src, void* dst, const doub
 // count elements of src as the load kernel can read them: in place on the
 // device's side, or copied into dst.
 template <typename T>
-sph_status scalar_in(sph_ctx* c, const T* src, T* dst, const T** view)
+sph_status scalar_in(sph_ctx* c, const T* src, T* dst, const T** view, cudaMemcpyKind kind = cudaMemcpyDefault)
 {
     *view = (const T*)device_side(src, alignof(T));
     if (*view) return SPH_OK;
-    SPH_CU(cudaMemcpyAsync(dst, src, (size_t)c->n * sizeof(T), cudaMemcpyDefault, c->st));
+    SPH_CU(cudaMemcpyAsync(dst, src, (size_t)c->n * sizeof(T), kind, c->st));
     *view = dst;
     return SPH_OK;
 }
@@ -1518,12 +1518,15 @@ extern "C" sph_status sph_density_noalloc(const sph_params* p, int64_t n, const 
     const int ni = (int)n;
     // The scratch keeps the previous call's contents: clear what is summed into.
     // (run_sort clears the bins' counts: the view starts with count_zero = 0.)
+    // The constants are read in place where the load kernel can read them, else
+    // copied first as device memory (another device's, or off its alignment).
+    StateSet<double>& S0 = c.set[0].d;
     LoadArgs A = {};
     A.x = x;
-    A.h = h;
-    A.m = m;
-    A.kind = kind;
-    A.sigma0 = sigma0;
+    SPH_TRY(scalar_in(&c, h, S0.h, &A.h, cudaMemcpyDeviceToDevice));
+    SPH_TRY(scalar_in(&c, m, S0.m, &A.m, cudaMemcpyDeviceToDevice));
+    if (kind) SPH_TRY(scalar_in(&c, kind, S0.kind, &A.kind, cudaMemcpyDeviceToDevice));
+    if (sigma0) SPH_TRY(scalar_in(&c, sigma0, S0.s0, &A.sigma0, cudaMemcpyDeviceToDevice));
     A.zero_v = 1;
     A.s0_first = c.s0_first;
     SPH_CU(launch_load_state(64, c.dim, ni, A, &c.set[0].d, &c.set[1].d, p->rho0, p->h_min, p->h_max, c.err, c.st,
