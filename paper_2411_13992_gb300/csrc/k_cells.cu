@@ -187,7 +187,7 @@ __global__ void __launch_bounds__(kScanThreads) k_bin_scan(int32_t* count, int32
     __shared__ int is_last;
     const int base = blockIdx.x * kScanTile + threadIdx.x * kScanItems;
     static_assert(kScanItems % 4 == 0, "16-byte vectors");
-    int32_t vals[kScanItems];
+    __align__(16) int32_t vals[kScanItems];          // moved as int4, wherever the compiler keeps it
     const bool whole = base + kScanItems <= n;      // base is a multiple of 16: 64-byte aligned
     if (whole) {
         int4* c4 = reinterpret_cast<int4*>(count + base);
