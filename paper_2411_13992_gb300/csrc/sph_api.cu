@@ -602,7 +602,7 @@ void graph_capture(sph_ctx* c, int len, int par)
     c->gstate[len][par] = -1;
     if (!graph_stream(c)) return;
     cudaStream_t user = c->st;
-    const int cur0 = c->cur;
+    const int cur0 = c->cur, count_zero0 = c->count_zero;
     const int64_t l0 = c->launches;
     cudaGraph_t g = nullptr;
     bool ok = cudaStreamBeginCapture(c->gst, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
@@ -617,6 +617,7 @@ void graph_capture(sph_ctx* c, int len, int par)
     c->glaunches[len][par] = c->launches - l0;
     c->launches = l0;
     if (ok && cudaGraphInstantiate(&c->gexec[len][par], g, 0) == cudaSuccess) c->gstate[len][par] = 1;
+    else c->count_zero = count_zero0;      // nothing ran: a clearing of the counts is still to be done
     if (g) cudaGraphDestroy(g);
     cudaGetLastError();
 }
@@ -906,6 +907,7 @@ void adjoint_capture(sph_ctx* c, int nsteps)
     c->acur0 = c->cur;
     if (!graph_stream(c)) return;
     cudaStream_t user = c->st;
+    const int count_zero0 = c->count_zero;
     const int64_t l0 = c->launches;
     cudaGraph_t g = nullptr;
     bool ok = cudaStreamBeginCapture(c->gst, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
@@ -920,6 +922,7 @@ void adjoint_capture(sph_ctx* c, int nsteps)
     c->alaunches = c->launches - l0;
     c->launches = l0;
     if (ok && cudaGraphInstantiate(&c->aexec, g, 0) == cudaSuccess) c->astate = 1;
+    else c->count_zero = count_zero0;
     if (g) cudaGraphDestroy(g);
     cudaGetLastError();
 }
