@@ -1227,12 +1227,18 @@ __global__ void __launch_bounds__(TileThreads<DIM>::COOP, 4) k_density32_coop(
 // warps to cover the gathers, and takes U = 5 (step of the 2,900-particle
 // cavity 35.1 -> 33.5 us, of the 69,000-particle one 41.9 -> 41.4, rollout
 // 256^2 3.21 -> 3.16 ms; U = 4 the same within 1 %, 6 slower).
-// Variable resolution keeps eight blocks (64 registers) and one pair ahead:
-// at six blocks its pass ran 10 % longer.
+// Variable resolution keeps one pair ahead, and as many blocks as its registers
+// allow without spills: eight (64 registers) in 2-D, where its pass ran 10 %
+// longer at six, seven (72) in 3-D.  Step of 96^3 with varying h at 8 / 7 / 6 /
+// 5 blocks: 1449 / 1378 / 1439 / 1492 us, of 16^3 186 / 175 / 176 / 173 (44
+// bytes of spilled registers loaded a thread at 8).
 constexpr int kDeepBlocks = 4, kDeepPairs = 5;
-constexpr int forces_blocks(bool uniform, int U) { return !uniform ? 8 : (U == 3 ? 6 : kDeepBlocks); }
+constexpr int forces_blocks(int dim, bool uniform, int U)
+{
+    return !uniform ? (dim == 3 ? 7 : 8) : (U == 3 ? 6 : kDeepBlocks);
+}
 template <int DIM, typename Acc, bool UNIFORM, int U>
-__global__ void __launch_bounds__(kTPB32, forces_blocks(UNIFORM, U)) k_forces32(int n, const float4* pos4,
+__global__ void __launch_bounds__(kTPB32, forces_blocks(DIM, UNIFORM, U)) k_forces32(int n, const float4* pos4,
                                                      const int32_t* cell_of,
                                                      const int32_t* start, Grid G, Consts<float> K,
                                                      StateSet<float> S, const float* mf,
