@@ -1266,7 +1266,10 @@ __global__ void __launch_bounds__(kTPB32, forces_blocks(DIM, UNIFORM, U)) k_forc
     // waves (some 26 operations of 19 SM cycles a warp, against 20 neighbours a
     // particle): conversions and factors of 1/2 go to the integer ALU there
     // (pass of 490,000 particles 56.2 -> 51.6 us, same bits).  In 3-D and on
-    // small grids the longer integer chains cost 0.2-2 us a step instead.
+    // grids of at most kDeepBlocks blocks per SM the longer integer chains cost
+    // 0.2-2 us a step instead: such a grid has U = 5, or in 2-D at variable
+    // resolution, whose walk does not depend on U, U = 1 (step of 773 / 12,283
+    // particles 48.2 -> 47.9 / 53.6 -> 53.2 us).
     constexpr bool kOffPipe = DIM == 2 && U == 3;
     auto wide = [](float f) { return kOffPipe ? f2d_exact(f) : (double)f; };
     const float dtf = kOffPipe ? d2f_rn(dt) : (float)dt;
@@ -1547,9 +1550,10 @@ static void forces_t(int n, const float4* pos4, const int32_t* cell_of, const in
                      const FinishArgs& F, cudaStream_t st)
 {
     const int T = pair_threads(32, n, G.sms);
-    const bool deep = U && nblk(n, T) <= kDeepBlocks * G.sms;
-    launch(deep ? k_forces32<DIM, Acc, U, U ? kDeepPairs : 3> : k_forces32<DIM, Acc, U, 3>, nblk(n, T), T, 0, st, n,
-           pos4, cell_of, start, G, K, S, mf, vr, nbl, nbc, nbl_capacity(DIM), F.dt, kick_on, write_ad, Rout, chi,
+    const bool deep = nblk(n, T) <= kDeepBlocks * G.sms;
+    constexpr int kSmall = U ? kDeepPairs : (DIM == 2 ? 1 : 3);
+    launch(deep ? k_forces32<DIM, Acc, U, kSmall> : k_forces32<DIM, Acc, U, 3>, nblk(n, T), T, 0, st, n, pos4, cell_of,
+           start, G, K, S, mf, vr, nbl, nbc, nbl_capacity(DIM), F.dt, kick_on, write_ad, Rout, chi,
            grid_sum(F, nblk(n, T)), dt_consts(*F.P), F.diag, F.dt, F.count_step);
 }
 
