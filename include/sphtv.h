@@ -133,7 +133,11 @@ typedef struct sph_params {
                                with SPH_INT_DUAL); each step of it takes a tape
                                slot in the workspace, which also holds that
                                step's neighbour list (128 entries per particle
-                               in 3-D, 96 in 2-D, 4 bytes each) */
+                               in 3-D, 96 in 2-D, 4 bytes each); in the FP64
+                               form only while the lists of all slots take at
+                               most 1 GiB, beyond which the reverse sweep builds
+                               each list again (the same results, 111 bytes per
+                               particle and step in 3-D instead of 631) */
     int32_t integrator;     /* SPH_INT_*: kick-drift-kick (default) or dual-criteria;
                                SPH_INT_DUAL requires fixed_dt = 0 */
     int32_t graphs;         /* 1 (default): sph_step replays kick-drift-kick steps two at a

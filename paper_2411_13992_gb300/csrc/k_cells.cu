@@ -349,6 +349,24 @@ __global__ void __launch_bounds__(256) k_order_permute(int n, int nbin, const in
     mf[k] = m_f;
 }
 
+// The cell-relative FP32 records of sorted particles by themselves, as
+// k_order_permute writes them (the FP64 form's adjoint, whose tape does not
+// hold them).
+template <int DIM>
+__global__ void __launch_bounds__(256) k_offsets(int n, const double* x, const double* h, const double* m,
+                                                 const int32_t* cell, Grid G, int uniform_h, float4* pos4)
+{
+    pdl_wait();
+    const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= n) return;
+    int c[3];
+    cell_decode(G, cell[k], c);
+    float o[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+    for (int d = 0; d < DIM; ++d) o[d] = d2f_rn(x[(size_t)d * n + k] - (G.lo[d] + i2d_exact(c[d]) * G.edge[d]));
+    pos4[k] = make_float4(o[0], o[1], o[2], d2f_rn(uniform_h ? m[k] : h[k]));
+}
+
 // ------------------------------------------------------------- launchers
 
 static inline int nblk(int n, int t) { return (n + t - 1) / t; }
@@ -395,6 +413,13 @@ cudaError_t launch_order_permute(int prec, int dim, int n, int nbin, const SortB
         order_permute_t<double>(dim, n, nbin, B, src, dst, G, pos4, cell, mf, uniform_h, carry_ad, st, pos4c, varies);
     else
         order_permute_t<float>(dim, n, nbin, B, src, dst, G, pos4, cell, mf, uniform_h, carry_ad, st, pos4c, varies);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_offsets(int dim, int n, const double* x, const double* h, const double* m, const int32_t* cell,
+                           const Grid& G, int uniform_h, float4* pos4, cudaStream_t st)
+{
+    launch(dim == 2 ? k_offsets<2> : k_offsets<3>, nblk(n, 256), 256, 0, st, n, x, h, m, cell, G, uniform_h, pos4);
     return cudaGetLastError();
 }
 

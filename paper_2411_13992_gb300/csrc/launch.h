@@ -80,6 +80,8 @@ cudaError_t launch_bin_scan(int32_t* count, int32_t* prefix, int n, int32_t* til
 cudaError_t launch_order_permute(int prec, int dim, int n, int nbin, const SortBufs& B, void* src, void* dst,
                                  const Grid& G, float4* pos4, int32_t* cell, float* mf, int uniform_h, int carry_ad,
                                  cudaStream_t st, const uint32_t* varies, float4* pos4c = nullptr);
+cudaError_t launch_offsets(int dim, int n, const double* x, const double* h, const double* m, const int32_t* cell,
+                           const Grid& G, int uniform_h, float4* pos4, cudaStream_t st);
 
 // What the last block of a pass needs to fold the grid's partials and set the
 // next step size: the partials' buffers, the counters (zero between

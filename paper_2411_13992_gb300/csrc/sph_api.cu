@@ -40,7 +40,7 @@ struct TapeSlot {
     int32_t* cell;
     double* dt;
     uint32_t* nbl;      // the step's force-neighbour list (the density pass's, transposed)
-    int32_t* nbc;       // and its counts
+    int32_t* nbc;       // and its counts; both the context's own without lists in the slots (tape_lists)
 };
 
 struct sph_ctx {
@@ -300,6 +300,22 @@ Consts<Real> make_consts(const sph_params* p)
     return K;
 }
 
+// Whether the adjoint's tape slots hold their steps' neighbour lists.  The FP32
+// form's always do.  The FP64 form's do while the lists of all slots take at
+// most kTapeListBytes; a longer or larger tape, which they would make five to
+// six times as large (631 against 111 bytes a particle and step in 3-D), leaves
+// them out, and the reverse sweep builds each step's list again from its tape
+// (rebuild_list).  A step of the segment, replay and reverse, with the list in
+// the slot / built again: 2-D 4,096 particles 118 / 128 us, 262,144 2.94 / 3.10
+// ms; 3-D 4,096 314 / 345 us, 262,144 13.6 / 14.3 ms, 96^3 44.3 / 45.8 ms.
+constexpr size_t kTapeListBytes = (size_t)1 << 30;
+
+bool tape_lists(const sph_ctx* c)
+{
+    const size_t per_slot = (size_t)c->n * (nbl_capacity(c->dim) + 1) * sizeof(uint32_t);
+    return c->prec == 32 || per_slot * (size_t)c->P.adjoint_steps <= kTapeListBytes;
+}
+
 // Lay the buffers out in the workspace (base == nullptr: only measure).
 size_t carve(sph_ctx* c, char* base)
 {
@@ -382,8 +398,8 @@ size_t carve(sph_ctx* c, char* base)
             sl.pos4 = c->prec == 32 ? W.take<float4>(n) : nullptr;
             sl.cell = W.take<int32_t>(n);
             sl.dt = W.take<double>(1);
-            sl.nbl = W.take<uint32_t>((size_t)nbl_capacity(D) * n);
-            sl.nbc = W.take<int32_t>(n);
+            sl.nbl = tape_lists(c) ? W.take<uint32_t>((size_t)nbl_capacity(D) * n) : c->nbl;
+            sl.nbc = tape_lists(c) ? W.take<int32_t>(n) : c->nbc;
             if (base && c->tape) c->tape[t] = sl;
         }
         AdjView& A = c->adj;
@@ -870,6 +886,24 @@ struct ListInSlot {
     }
 };
 
+// The neighbour list of tape slot t in the context's list, from the slot's
+// positions, by the density pass that wrote it in the forward step: the same
+// tests in the same order (the cut at the sub-cells only leaves out candidates
+// that fail them).  What else the pass writes, the velocity records, goes to
+// the cotangent records' buffer, which the reverse step fills afterwards; the
+// velocities it reads are those of no step (R in their place).
+sph_status rebuild_list(sph_ctx* c, int t)
+{
+    const TapeSlot& T = c->tape[t];
+    const int n = (int)c->n;
+    const Grid G = cells_only(c->G);
+    StateSet<double> S{T.x, (double*)T.R, nullptr, nullptr, nullptr, T.h, T.m, T.s0, T.id, T.kind};
+    SPH_CU(launch_offsets(c->dim, n, T.x, T.h, T.m, T.cell, G, c->K64.uniform_h, c->pos4, c->st));
+    SPH_CU(launch_density(64, c->dim, n, &S, T.start, G, consts(c), c->adj.AR, c->pos4, T.cell, c->nbl, c->nbc, c->st));
+    c->launches += 2;
+    return SPH_OK;
+}
+
 // One segment of the adjoint after the cotangents are in: nsteps forward
 // steps from the reloaded state that record the tape (with the step sizes
 // taken), then the reverse sweep over them.  No host work between the
@@ -890,6 +924,8 @@ sph_status adjoint_segment(sph_ctx* c, int nsteps)
     AdjView& A = c->adj;
     SPH_CU(cudaMemsetAsync(A.eta, 0, sizeof(double), c->st));
     for (int t = nsteps - 1; t >= 0; --t) {
+        // (the last step's list is still the context's)
+        if (!tape_lists(c) && t < nsteps - 1) SPH_TRY(rebuild_list(c, t));
         SPH_CU(launch_adjoint_step(c->prec, c->dim, (int)c->n, tape_view(c->tape[t]), cells_only(c->G), consts(c), A, 1,
                                       c->st));
         c->launches += 3;
