@@ -585,9 +585,15 @@ sph_status run_dual_step(sph_ctx* c)
 // be used.  The gap between two replays is about 3 us: two steps per graph
 // leave half of it on each step of a small problem (2-D 50^2 FP64: 40.3 us a
 // step, 40.6 with direct launches, 39.3 with eight, 38.9 with sixteen).  A
-// capture costs 3 us per kernel once, so short calls take the short graph.
+// capture costs the host 40-55 us once for two steps and some 120 for eight, so
+// short calls take the short graph, and the long graph is captured behind
+// kGraphLead steps replayed from the short one, whose 200 us or more on the
+// device cover it.  First call of 20 steps on a new context with the long
+// graph captured before them / behind: cavity 256^2 942 / 888 us, 48^2 692 /
+// 635, 2-D 50^2 FP64 902 / 847 (later calls 820, 580, 786 either way).
 constexpr int kGraphSteps[2] = {2, 8};
 constexpr int kGraphFrom[2] = {2, 16};
+constexpr int kGraphLead = 8;
 
 // Capture kGraphSteps[len] kick-drift-kick steps starting from state-set
 // parity par into a graph on the library stream.  Nothing runs during the
@@ -1127,15 +1133,20 @@ sph_status sph_step(sph_ctx* c, int32_t nsteps)
     if (!c->have_cells) return SPH_ERR_STATE;
     if (c->P.integrator == SPH_INT_KDK && c->P.graphs && !c->prof_ev) {
         const int par = c->cur;      // an even number of steps brings the sets back to this parity
-        for (int len = 1; len >= 0; --len) {
-            if (nsteps < kGraphFrom[len]) continue;
+        auto replay = [&](int len, int steps) {
             if (c->gstate[len][par] == 0) graph_capture(c, len, par);
-            if (c->gstate[len][par] != 1) continue;
-            const int times = nsteps / kGraphSteps[len];
+            if (c->gstate[len][par] != 1) return SPH_OK;
+            const int times = steps / kGraphSteps[len];
             SPH_TRY(graph_launch(c, c->gexec[len][par], times));
             c->launches += (int64_t)times * c->glaunches[len][par];
             nsteps -= times * kGraphSteps[len];
+            return SPH_OK;
+        };
+        if (nsteps >= kGraphFrom[1]) {
+            if (c->gstate[1][par] == 0) SPH_TRY(replay(0, kGraphLead));
+            SPH_TRY(replay(1, nsteps));
         }
+        if (nsteps >= kGraphFrom[0]) SPH_TRY(replay(0, nsteps));
     }
     for (int32_t k = 0; k < nsteps; ++k) {
         if (c->P.integrator == SPH_INT_DUAL) {
