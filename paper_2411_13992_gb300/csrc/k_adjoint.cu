@@ -220,7 +220,7 @@ __device__ __forceinline__ void adj_visit(int n, int k, int q, const Grid& G, co
         }
         if (q) return;
         // the exact test of the forward pass over the cells (minimum image,
-        // sqrt(r^2) < 2 h_kj)
+        // sqrt(r^2) < 2 h_kj by the same root)
         const int SR = G.R, zr = DIM == 3 ? SR : 0;
         for (int dz = -zr; dz <= zr; ++dz) {
             int cz = DIM == 3 ? cell_step(G, c[2], dz, 2) : 0;
@@ -240,10 +240,11 @@ __device__ __forceinline__ void adj_visit(int n, int k, int q, const Grid& G, co
                             rv[d] = min_image(G, xk[d], T.x[(size_t)d * n + j], d);
                             r2 += rv[d] * rv[d];
                         }
-                        const double r = sqrt(r2);
+                        if (!(r2 > 0.0)) continue;
                         const double hij = pair_h(K, T.h[k], T.h[j]);
-                        if (!(r < 2.0 * hij) || r == 0.0) continue;
-                        f(j, rv, (Real)r, Real(1) / (Real)r, 0.f, load(j));
+                        if (!(sqrt_pos(r2) < 2.0 * hij)) continue;
+                        const double inv_r = rsqrt_pos(r2);
+                        f(j, rv, r2 * inv_r, inv_r, 0.f, load(j));
                     }
                 }
             }

@@ -461,7 +461,7 @@ __device__ __forceinline__ void forces64_sums(int n, int i, const StateSet<doubl
                         const double hij = uni ? K.h_u : pair_h(K, hi, S.h[j]);
                         if (r2 > 4.0 * hij * hij * (1.0 + 1e-12)) continue;
                         if (!(r2 > 0.0)) continue;
-                        if (!(sqrt(r2) < 2.0 * hij)) continue;
+                        if (!(sqrt_pos(r2) < 2.0 * hij)) continue;     // as the density pass decides
                         body(j, rv, r2);
                     }
                 }
