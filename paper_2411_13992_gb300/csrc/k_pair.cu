@@ -47,7 +47,8 @@ namespace sphtv {
 // Measured, us a step (start of the comparison -> L = 1 / 4 / 8): 2-D 2,500
 // particles 116 -> 99 / 48 / 42, 8,100: 115 -> 100 / 55 / 55, 20,000: 120 ->
 // 103 / 102 / 113, 40,000: 250 -> 151 / 161 / 186; 3-D 4,096: 391 -> 358 /
-// 122 / 93, 17,576: 397 -> 363 / 259 / 276, 64,000: 889 (now 809) / 823.
+// 122 / 93, 17,576: 397 -> 363 / 259 / 276, 64,000: 889 (now 809) / 823; 3-D
+// with 8 / 16 lanes 343: 72.9 / 55.1, 1,331: 74.0 / 59.4, 2,197: 77.0 / 69.5.
 template <int L> struct Lanes {
     static constexpr int kThreads = L == 1 ? 256 : 512;    // most threads of a block
 };
@@ -676,7 +677,7 @@ static Lane64 lanes64(int dim, int n, int sms)
 }
 
 #define SPH_LANES64(kernel, DIM, L) \
-    ((L) == 1 ? kernel<DIM, 1> : (L) == 4 ? kernel<DIM, 4> : (L) == 8 ? kernel<DIM, 8> : kernel<DIM, 16>)
+    ((L) == 1 ? kernel<DIM, 1> : (L) == 4 ? kernel<DIM, 4> : (L) == 8 ? kernel<DIM, 8> : kernel<DIM, (DIM) == 3 ? 16 : 8>)
 
 int pair_blocks(int prec, int n, int sms) { return nblk(n, pair_threads(prec, n, sms)); }
 
