@@ -8,6 +8,12 @@
 
 namespace sphtv {
 
+// Exact FP64 value of a stored component, off the FP64 pipe (its conversions
+// were issued for the outputs not asked for too: density alone of 128^3 in FP32
+// 38.6 -> 14.8 us).
+__device__ __forceinline__ double wide(double x) { return x; }
+__device__ __forceinline__ double wide(float x) { return f2d_exact(x); }
+
 template <typename Real, int DIM>
 __global__ void k_vec_in(int n, const double* src3, Real* dst)
 {
@@ -38,8 +44,13 @@ __global__ void k_vec_out_gather(int n, const Real* src, const int32_t* pos,
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const size_t k = (size_t)pos[i];
+    // the loads before the first store: none could be moved past a store that
+    // may alias it (all five arrays of 200^3 427 -> 387 us)
+    double q[3];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) dst3[3 * (size_t)i + d] = d < DIM ? (double)src[(size_t)d * n + k] : 0.0;
+    for (int d = 0; d < 3; ++d) q[d] = d < DIM ? wide(src[(size_t)d * n + k]) : 0.0;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) dst3[3 * (size_t)i + d] = q[d];
 }
 
 template <typename V4>
@@ -50,7 +61,7 @@ __global__ void k_rho_out_gather(int n, const V4* vr, const int8_t* kind,
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
     const int k = pos[i];
-    dst[i] = kind[k] ? rho0 : rho0 + (double)vr[k].w;
+    dst[i] = kind[k] ? rho0 : rho0 + wide(vr[k].w);
 }
 
 // Smoothing lengths (in units of dp) from which the lattice sum is taken at its
@@ -221,16 +232,12 @@ __global__ void __launch_bounds__(256) k_load_state(int n, LoadArgs A, StateSet<
     }
 }
 
-// Exact FP64 value of a stored component, off the FP64 pipe (its conversions
-// were issued for the outputs not asked for too: density alone of 128^3 in FP32
-// 38.6 -> 14.8 us).
-__device__ __forceinline__ double wide(double x) { return x; }
-__device__ __forceinline__ double wide(float x) { return f2d_exact(x); }
-
 // The whole state out into device memory, in the caller's order (each of the
 // outputs may be null): one kernel for an inverse permutation and five
 // gathers.  The reads are in the sorted order, each particle's rows of 24
-// bytes go where its id says.
+// bytes go where its id says; for how much output, see kScatterBytes.  (With a
+// row's loads before the stores of the one before, the scattered stores came in
+// longer bursts: 64^3 shuffled 35 -> 56 us.)
 template <typename Real, int DIM>
 __global__ void __launch_bounds__(256) k_store_state(int n, StateSet<Real> S, const typename Vec4<Real>::T* vr,
                                                      double rho0, double* x, double* v, double* a, double* dr,

@@ -969,6 +969,17 @@ void adjoint_capture(sph_ctx* c, int nsteps)
     cudaGetLastError();
 }
 
+// Bytes of output up to which sph_get_state scatters the sorted state to the
+// caller's order in one kernel; more is gathered, array by array, through the
+// inverse permutation.  The scatter reads in order, but where the caller's
+// order is not (any more) that of space, in a mixed flow or a shuffled load, it
+// writes parts of 32-byte sectors all over memory, which the L2 joins only
+// while they fit it beside the state.  All five arrays of particles in the order
+// of space / shuffled: 64^3 scattered 25 / 35 us, gathered 36 / 51; 80^3 35 / 81
+// and 43 / 62; 128^3 103 / 571 and 114 / 199 (lattice disordered by 0.2 dp: 120
+// and 117); 200^3 343 / 2543 and 387 / 1043.
+constexpr size_t kScatterBytes = (size_t)40 << 20;
+
 }  // namespace
 
 extern "C" {
@@ -1227,10 +1238,15 @@ sph_status sph_get_state(sph_ctx* c, double* x, double* v, double* a, double* dr
     const void* sa = c->prec == 64 ? (void*)c->set[c->cur].d.a : (void*)c->set[c->cur].f.a;
     const void* sdr = c->prec == 64 ? (void*)c->set[c->cur].d.dr : (void*)c->set[c->cur].f.dr;
     if (rho && !c->have_cells) return SPH_ERR_STATE;
-    // every output in memory of this device: one kernel
-    bool direct = x || v || a || dr || rho;
-    for (double* o : {x, v, a, dr, rho})
-        if (o && (is_host_ptr(o) || device_view(o) != o)) direct = false;
+    // every output in memory of this device, and not too much of it: one kernel
+    size_t bytes = 0;
+    bool direct = true;
+    for (double* o : {x, v, a, dr, rho}) {
+        if (!o) continue;
+        bytes += o == rho ? vb / 3 : vb;
+        if (is_host_ptr(o) || device_view(o) != o) direct = false;
+    }
+    direct = direct && bytes > 0 && bytes <= kScatterBytes;
     if (direct) {
         SPH_CU(launch_store_state(c->prec, c->dim, n, cur_set(c), c->vr, c->P.rho0, x, v, a, dr, rho, c->st));
         ++c->launches;
