@@ -77,9 +77,10 @@ cudaError_t launch_kick_drift_key(int prec, int dim, int n, void* S, const doubl
 size_t scan_temp_elems(int n);
 cudaError_t launch_bin_scan(int32_t* count, int32_t* prefix, int n, int32_t* tile_off, unsigned* done,
                             cudaStream_t st);
+// old_of null: one kernel; else scratch of n for two (see k_order_permute).
 cudaError_t launch_order_permute(int prec, int dim, int n, int nbin, const SortBufs& B, void* src, void* dst,
                                  const Grid& G, float4* pos4, int32_t* cell, float* mf, int uniform_h, int carry_ad,
-                                 cudaStream_t st, const uint32_t* varies, float4* pos4c = nullptr);
+                                 cudaStream_t st, const uint32_t* varies, float4* pos4c, int32_t* old_of);
 cudaError_t launch_offsets(int dim, int n, const double* x, const double* h, const double* m, const int32_t* cell,
                            const Grid& G, int uniform_h, float4* pos4, cudaStream_t st);
 

@@ -55,6 +55,7 @@ struct sph_ctx {
     int cur;
     SortBufs sort;
     int32_t* start;      // the cells' starts (sort.cell_start)
+    int loaded_order;    // the state is in the order it was loaded in: no sort yet
     int count_zero;      // count[] is known to be all zero (a complete sort ran since it was cleared)
     void* vr;
     float4* pos4;
@@ -444,6 +445,12 @@ inline cudaError_t prof_mark(sph_ctx* c, int cls, int end)
         if (s_ != SPH_OK) return s_;     \
     } while (0)
 
+// Whether the next sort is the first of a loaded state too large for the L2 (80
+// bytes a particle of sorted arrays in FP32): see k_order_permute.
+constexpr int64_t kFirstSort = 1500000;
+
+bool first_sort(const sph_ctx* c) { return c->loaded_order && c->n >= kFirstSort; }
+
 // Kick-drift (optional), cell keys, counting sort with the arrays moved.
 sph_status run_sort(sph_ctx* c, int drift, int carry_ad)
 {
@@ -466,10 +473,12 @@ sph_status run_sort(sph_ctx* c, int drift, int carry_ad)
     c->count_zero = 1;
     SPH_MARK(SPH_K_SCAN, 1);
     SPH_MARK(SPH_K_PERMUTE, 0);
+    int32_t* old_of = first_sort(c) ? (int32_t*)c->stage : nullptr;
     SPH_CU(launch_order_permute(c->prec, c->dim, n, (int)sort_bins(c->G), B, cur_set(c), other_set(c), c->G, c->pos4,
-                                c->cell, c->mf, c->K32.uniform_h, carry_ad, c->st, c->err + 1, c->pos4c));
+                                c->cell, c->mf, c->K32.uniform_h, carry_ad, c->st, c->err + 1, c->pos4c, old_of));
     SPH_MARK(SPH_K_PERMUTE, 1);
-    c->launches += 3;
+    c->launches += old_of ? 4 : 3;
+    c->loaded_order = 0;
     c->cur = 1 - c->cur;
     return SPH_OK;
 }
@@ -784,6 +793,7 @@ sph_status load_state(sph_ctx* c, const double* x, const double* v, const double
                              &c->launches));
     c->have_state = 1;
     c->have_cells = 0;
+    c->loaded_order = 1;
     c->ad_given = a != nullptr;
     return SPH_OK;
 }
@@ -949,7 +959,7 @@ void adjoint_capture(sph_ctx* c, int nsteps)
     c->acur0 = c->cur;
     if (!graph_stream(c)) return;
     cudaStream_t user = c->st;
-    const int count_zero0 = c->count_zero;
+    const int count_zero0 = c->count_zero, loaded0 = c->loaded_order;
     const int64_t l0 = c->launches;
     cudaGraph_t g = nullptr;
     bool ok = cudaStreamBeginCapture(c->gst, cudaStreamCaptureModeThreadLocal) == cudaSuccess;
@@ -965,6 +975,7 @@ void adjoint_capture(sph_ctx* c, int nsteps)
     c->launches = l0;
     if (ok && cudaGraphInstantiate(&c->aexec, g, 0) == cudaSuccess) c->astate = 1;
     else c->count_zero = count_zero0;
+    c->loaded_order = loaded0;
     if (g) cudaGraphDestroy(g);
     cudaGetLastError();
 }
@@ -1142,6 +1153,13 @@ sph_status sph_step(sph_ctx* c, int32_t nsteps)
     if (!c || nsteps < 0) return SPH_ERR_ARG;
     const int32_t nsteps_in = nsteps;
     if (!c->have_cells) return SPH_ERR_STATE;
+    if (c->P.integrator == SPH_INT_KDK && nsteps > 0 && first_sort(c)) {
+        // built with a and dr given: the graphs hold the sorts of later steps
+        SPH_TRY(run_sort(c, 1, 0));
+        SPH_TRY(run_forces(c, 1, 1, 1));
+        if (c->prof_ev) ++c->prof_step;
+        --nsteps;
+    }
     if (c->P.integrator == SPH_INT_KDK && c->P.graphs && !c->prof_ev) {
         const int par = c->cur;      // an even number of steps brings the sets back to this parity
         auto replay = [&](int len, int steps) {
@@ -1450,6 +1468,7 @@ sph_status sph_step_adjoint(sph_ctx* c, const double* x0, const double* v0, cons
             SPH_TRY(graph_launch(c, c->aexec, 1));
             c->launches += c->alaunches;
             c->cur = c->acur1;
+            c->loaded_order = 0;       // a segment starts with the first sort of a loaded state, recorded as such
             replayed = true;
         }
     }
