@@ -112,7 +112,8 @@ struct Tape {
 // else h_j) and load(j) whatever else of j the caller gathers, which the FP32
 // list walk requests one neighbour ahead.
 // Lane q of a group of L takes the list's entries q, q + L, ...; a particle
-// with more neighbours than the list holds is walked over its cells by lane 0.
+// with more neighbours than the list holds is walked over its cells, in the
+// FP64 form cells q, q + L, ... by lane q.
 // FP32 form: 1/r from rsqrt and r = r^2/r, as the forward force pass takes
 // them; FP64 form: 1/r within one rounding, r = r^2 (1/r).
 template <typename Real, int DIM, int L, typename Load, typename F>
@@ -218,35 +219,28 @@ __device__ __forceinline__ void adj_visit(int n, int k, int q, const Grid& G, co
             }
             return;
         }
-        if (q) return;
-        // the exact test of the forward pass over the cells (minimum image,
-        // sqrt(r^2) < 2 h_kj by the same root)
-        const int SR = G.R, zr = DIM == 3 ? SR : 0;
-        for (int dz = -zr; dz <= zr; ++dz) {
-            int cz = DIM == 3 ? cell_step(G, c[2], dz, 2) : 0;
-            if (cz < 0) continue;
-            for (int dy = -SR; dy <= SR; ++dy) {
-                int cy = cell_step(G, c[1], dy, 1);
-                if (cy < 0) continue;
-                for (int dx = -SR; dx <= SR; ++dx) {
-                    int cx = cell_step(G, c[0], dx, 0);
-                    if (cx < 0) continue;
-                    const int cell = cx + G.nc[0] * (cy + G.nc[1] * cz);
-                    for (int j = T.start[cell]; j < T.start[cell + 1]; ++j) {
-                        if (j == k) continue;
-                        Real rv[3] = {0, 0, 0};
-                        double r2 = 0.0;
-                        for (int d = 0; d < DIM; ++d) {
-                            rv[d] = min_image(G, xk[d], T.x[(size_t)d * n + j], d);
-                            r2 += rv[d] * rv[d];
-                        }
-                        if (!(r2 > 0.0)) continue;
-                        const double hij = pair_h(K, T.h[k], T.h[j]);
-                        if (!(sqrt_pos(r2) < 2.0 * hij)) continue;
-                        const double inv_r = rsqrt_pos(r2);
-                        f(j, rv, r2 * inv_r, inv_r, 0.f, load(j));
-                    }
+        // the exact test of the forward pass over the cells q, q + L, ... of the
+        // stencil (minimum image, sqrt(r^2) < 2 h_kj by the same root)
+        constexpr int cells = DIM == 3 ? kSide * kSide * kSide : kSide * kSide;
+        for (int t = q; t < cells; t += L) {
+            const int cx = cell_step(G, c[0], t % kSide - kStencilR, 0);
+            const int cy = cell_step(G, c[1], t / kSide % kSide - kStencilR, 1);
+            const int cz = DIM == 3 ? cell_step(G, c[2], t / (kSide * kSide) - kStencilR, 2) : 0;
+            if (cx < 0 || cy < 0 || cz < 0) continue;
+            const int cell = cx + G.nc[0] * (cy + G.nc[1] * cz);
+            for (int j = T.start[cell]; j < T.start[cell + 1]; ++j) {
+                if (j == k) continue;
+                Real rv[3] = {0, 0, 0};
+                double r2 = 0.0;
+                for (int d = 0; d < DIM; ++d) {
+                    rv[d] = min_image(G, xk[d], T.x[(size_t)d * n + j], d);
+                    r2 += rv[d] * rv[d];
                 }
+                if (!(r2 > 0.0)) continue;
+                const double hij = pair_h(K, T.h[k], T.h[j]);
+                if (!(sqrt_pos(r2) < 2.0 * hij)) continue;
+                const double inv_r = rsqrt_pos(r2);
+                f(j, rv, r2 * inv_r, inv_r, 0.f, load(j));
             }
         }
     }

@@ -263,38 +263,45 @@ __device__ __forceinline__ double density64_group(int n, int i, bool active, Row
     }
     __syncwarp();
     const float ex = G.edgef[0], ey = G.edgef[1], ez = G.edgef[2];
-    int nf = 0;
-    for (int r = 0; r < NR; ++r) {
-        const RowRuns rr = rows[r];
-        const int len = rr.n0 + rr.n1;
-        const int most = __reduce_max_sync(kAll, len);
-        const int dy = r % kSide - R, dz = DIM == 3 ? r / kSide - R : 0;
-        for (int f0 = 0; f0 < most; f0 += L) {
-            const int f = f0 + q;
-            bool take = false;
-            uint32_t e = 0;
-            if (f < len) {
-                const int j = f < rr.n0 ? rr.j0 + f : rr.j1 + (f - rr.n0);
-                const float4 pj = pos4[j];
-                int dx = cell_of[j] - rr.row - D.ci[0];
-                if (dx > R) dx -= G.nc[0];                    // across the periodic x boundary
-                else if (dx < -R) dx += G.nc[0];
-                const float rx = (oi[0] - pj.x) - (float)dx * ex;
-                const float ry = (oi[1] - pj.y) - (float)dy * ey;
-                float r2 = rx * rx + ry * ry;
-                if (DIM == 3) {
-                    const float rz = (oi[2] - pj.z) - (float)dz * ez;
-                    r2 += rz * rz;
+    // the rows' candidates that pass the prefilter, L at a time, in the order of
+    // the walk: `keep` says which of them to count and to list
+    auto walk_rows = [&](bool walk, auto&& keep) {
+        int got = 0;
+        for (int r = 0; r < NR; ++r) {
+            const RowRuns rr = rows[r];
+            const int len = walk ? rr.n0 + rr.n1 : 0;
+            const int most = __reduce_max_sync(kAll, len);
+            const int dy = r % kSide - R, dz = DIM == 3 ? r / kSide - R : 0;
+            for (int f0 = 0; f0 < most; f0 += L) {
+                const int f = f0 + q;
+                bool take = false;
+                uint32_t e = 0;
+                if (f < len) {
+                    const int j = f < rr.n0 ? rr.j0 + f : rr.j1 + (f - rr.n0);
+                    const float4 pj = pos4[j];
+                    int dx = cell_of[j] - rr.row - D.ci[0];
+                    if (dx > R) dx -= G.nc[0];                    // across the periodic x boundary
+                    else if (dx < -R) dx += G.nc[0];
+                    const float rx = (oi[0] - pj.x) - (float)dx * ex;
+                    const float ry = (oi[1] - pj.y) - (float)dy * ey;
+                    float r2 = rx * rx + ry * ry;
+                    if (DIM == 3) {
+                        const float rz = (oi[2] - pj.z) - (float)dz * ez;
+                        r2 += rz * rz;
+                    }
+                    const uint32_t code = (uint32_t)((dx + R) + kSide * (dy + R) + kSide * kSide * (dz + R));
+                    e = ((uint32_t)j << kCodeBits) | code;
+                    take = r2 <= prefilter2(K, hi_f, pj.w) && keep(j, code);
                 }
-                take = r2 <= prefilter2(K, hi_f, pj.w);
-                e = ((uint32_t)j << kCodeBits) | (uint32_t)((dx + R) + kSide * (dy + R) + kSide * kSide * (dz + R));
+                const unsigned m = __ballot_sync(kAll, take) & group;
+                const int at = got + __popc(m & below);
+                if (take && at < cap) nbl[(size_t)at * n + i] = e;
+                got += __popc(m);
             }
-            const unsigned m = __ballot_sync(kAll, take) & group;
-            const int at = nf + __popc(m & below);
-            if (take && at < cap) nbl[(size_t)at * n + i] = e;
-            nf += __popc(m);
         }
-    }
+        return got;
+    };
+    const int nf = walk_rows(true, [](int, uint32_t) { return true; });
     __syncwarp();
     int cnt = 0;
     const bool fits = nf <= cap;
@@ -313,10 +320,13 @@ __device__ __forceinline__ double density64_group(int n, int i, bool active, Row
         if (keep && at != k) nbl[(size_t)at * n + i] = e;
         cnt += __popc(m);
     }
-    // more candidates than the list holds: one lane walks them in one pass
-    if (active && !fits) {
-        if (q == 0) return density64_thread<DIM>(n, i, S, start, G, K, pos4, cell_of, nbl, nbc, cap, false);
-        return 0.0;
+    // more candidates than the list holds: the lanes walk them again with the
+    // exact test inside the walk (as the force pass shares the cells; by one lane
+    // alone a step of 32^3 particles at h = 1.82 dp took 12.96 ms, shared 3.96,
+    // with one thread per particle 4.21)
+    if (__any_sync(kAll, active && !fits)) {
+        const int again = walk_rows(active && !fits, [&](int j, uint32_t code) { return D.exact(j, code); });
+        if (!fits) cnt = again;
     }
     if (active && q == 0) nbc[i] = cnt;
     return D.sigma;
@@ -363,8 +373,8 @@ __global__ void __launch_bounds__(Lanes<L>::kThreads, L == 1 ? 4 : 1) k_density_
 }
 
 // The pair sums of particle i over its neighbours k0, k0 + dk, ... of the
-// list, or over the cells when there is no list (or more neighbours than it
-// holds) and this thread is the one that scans them.
+// list, or over the stencil's cells k0, k0 + dk, ... when there is no list (or
+// more neighbours than it holds).
 template <int DIM>
 __device__ __forceinline__ void forces64_sums(int n, int i, const StateSet<double>& S,
                                               const int32_t* start, const Grid& G,
@@ -436,36 +446,30 @@ __device__ __forceinline__ void forces64_sums(int n, int i, const StateSet<doubl
             }
             body(j, rv, r2);
         }
-    } else if (k0 == 0) {
-        // no list (or more neighbours than it holds): scan the cells with
-        // the minimum image and the support test
-        const int SR = G.R, zr = DIM == 3 ? SR : 0;
-        for (int dz = -zr; dz <= zr; ++dz) {
-            int cz = DIM == 3 ? cell_step(G, ci[2], dz, 2) : 0;
-            if (cz < 0) continue;
-            for (int dy = -SR; dy <= SR; ++dy) {
-                int cy = cell_step(G, ci[1], dy, 1);
-                if (cy < 0) continue;
-                for (int dx = -SR; dx <= SR; ++dx) {
-                    int cx = cell_step(G, ci[0], dx, 0);
-                    if (cx < 0) continue;
-                    int cell = cx + G.nc[0] * (cy + G.nc[1] * cz);
-                    for (int j = start[cell]; j < start[cell + 1]; ++j) {
-                        if (j == i) continue;
-                        double rv[3] = {0, 0, 0};
-                        double r2 = 0.0;
+    } else {
+        // no list (or more neighbours than it holds): scan the cells k0, k0 + dk,
+        // ... of the stencil with the minimum image and the support test
+        constexpr int cells = DIM == 3 ? kSide * kSide * kSide : kSide * kSide;
+        for (int t = k0; t < cells; t += dk) {
+            const int cx = cell_step(G, ci[0], t % kSide - kStencilR, 0);
+            const int cy = cell_step(G, ci[1], t / kSide % kSide - kStencilR, 1);
+            const int cz = DIM == 3 ? cell_step(G, ci[2], t / (kSide * kSide) - kStencilR, 2) : 0;
+            if (cx < 0 || cy < 0 || cz < 0) continue;
+            const int cell = cx + G.nc[0] * (cy + G.nc[1] * cz);
+            for (int j = start[cell]; j < start[cell + 1]; ++j) {
+                if (j == i) continue;
+                double rv[3] = {0, 0, 0};
+                double r2 = 0.0;
 #pragma unroll
-                        for (int d = 0; d < DIM; ++d) {
-                            rv[d] = min_image(G, xi[d], S.x[(size_t)d * n + j], d);
-                            r2 += rv[d] * rv[d];
-                        }
-                        const double hij = uni ? K.h_u : pair_h(K, hi, S.h[j]);
-                        if (r2 > 4.0 * hij * hij * (1.0 + 1e-12)) continue;
-                        if (!(r2 > 0.0)) continue;
-                        if (!(sqrt_pos(r2) < 2.0 * hij)) continue;     // as the density pass decides
-                        body(j, rv, r2);
-                    }
+                for (int d = 0; d < DIM; ++d) {
+                    rv[d] = min_image(G, xi[d], S.x[(size_t)d * n + j], d);
+                    r2 += rv[d] * rv[d];
                 }
+                const double hij = uni ? K.h_u : pair_h(K, hi, S.h[j]);
+                if (r2 > 4.0 * hij * hij * (1.0 + 1e-12)) continue;
+                if (!(r2 > 0.0)) continue;
+                if (!(sqrt_pos(r2) < 2.0 * hij)) continue;     // as the density pass decides
+                body(j, rv, r2);
             }
         }
     }
