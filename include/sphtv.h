@@ -327,8 +327,9 @@ enum {
     SPH_K_ORDER = 2,       /* not timed: the order by id is part of SPH_K_PERMUTE */
     SPH_K_PERMUTE = 3,     /* order by id within the bins, permute the particle arrays */
     SPH_K_DENSITY = 4,     /* density summation (Eq. 8) */
-    SPH_K_FORCES = 5,      /* fused pair pass (Eq. 3, 5-7, 14-16) + closing kick */
-    SPH_K_FINALIZE = 6,    /* FP64 reductions and dt (Eq. 9-11) */
+    SPH_K_FORCES = 5,      /* fused pair pass (Eq. 3, 5-7, 14-16) + closing kick; up to 2,048
+                              blocks also the FP64 reductions and dt (Eq. 9-11) */
+    SPH_K_FINALIZE = 6,    /* FP64 reductions and dt of larger grids (else the two events alone) */
     SPH_K_ADVECT = 7,      /* SPH_INT_DUAL: viscous force + transport correction of an advection step */
     SPH_K_ACOUSTIC = 8,    /* SPH_INT_DUAL: all acoustic substeps of an advection step */
     SPH_K_NCLASS = 9

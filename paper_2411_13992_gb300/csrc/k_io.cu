@@ -1,8 +1,8 @@
 // k_io.cu -- state transfer kernels of libsphtv: the load of a state in the
 // caller's order ([n][3] rows into per-component arrays, wall velocities, the
 // input checks), the way back from the cell order, the adjoint's cotangents,
-// and the per-particle reference sums sigma0 of Eq. 8 (the perfect-lattice sum at the particle's own spacing
-// dp = (m/rho0)^(1/D) and smoothing length h).
+// and the per-particle reference sums sigma0 of Eq. 8 (the perfect-lattice sum
+// at the particle's own spacing dp = (m/rho0)^(1/D) and smoothing length h).
 #include "common.cuh"
 #include "launch.h"
 

@@ -1303,8 +1303,9 @@ __global__ void __launch_bounds__(kTPB32, forces_blocks(DIM, UNIFORM, U)) k_forc
         const int cnt = nbc[i];
         if (cnt <= cap) {
             // the neighbour list of the density pass: no candidate tests.
-            // Software pipeline: the list entries six ahead and the
-            // neighbour data three ahead are in flight while a pair is computed.
+            // Software pipeline: at uniform resolution 2 U list entries and U
+            // neighbours' data are in flight while U pairs are computed, else two
+            // entries and one neighbour's data beside a pair.
             const uint32_t* lp = nbl + i;
             auto one = [&](uint32_t ec, const float4& pj, const float4& oj) {
                 const float4 sh = tab[ec & ((1u << kCodeBits) - 1u)];
@@ -1402,7 +1403,6 @@ __global__ void __launch_bounds__(kTPB32, forces_blocks(DIM, UNIFORM, U)) k_forc
         const float lam = K.fr_on ? fringe_rate<float>(K, (float)S.x[i]) : 0.f;
 #pragma unroll
         for (int d = 0; d < DIM; ++d) {
-            // at uniform resolution the sums were taken without the factor C of W'/r
             const float pair_a = sums.a_value(d);
             // the fluid's momentum rate from its pair terms: minus the force on the walls
             if (K.body_force) part[9 + d] = m_i * (double)pair_a;
