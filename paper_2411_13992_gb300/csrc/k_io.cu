@@ -8,9 +8,12 @@
 
 namespace sphtv {
 
-// Exact FP64 value of a stored component, off the FP64 pipe (its conversions
-// were issued for the outputs not asked for too: density alone of 128^3 in FP32
-// 38.6 -> 14.8 us).
+// Exact FP64 value of a stored component, off the FP64 pipe: the read-back is
+// bound by its conversions otherwise, those of outputs not asked for among them
+// (density alone of 128^3 in FP32 38.6 -> 14.8 us).  Below kWideFrom particles a
+// thread's chain of operations counts for more than the pipe (2,916 particles:
+// 0.5 us), and the hardware converts.
+constexpr int kWideFrom = 20000;
 __device__ __forceinline__ double wide(double x) { return x; }
 __device__ __forceinline__ double wide(float x) { return f2d_exact(x); }
 
@@ -238,7 +241,7 @@ __global__ void __launch_bounds__(256) k_load_state(int n, LoadArgs A, StateSet<
 // bytes go where its id says; for how much output, see kScatterBytes.  (With a
 // row's loads before the stores of the one before, the scattered stores came in
 // longer bursts: 64^3 shuffled 35 -> 56 us.)
-template <typename Real, int DIM>
+template <typename Real, int DIM, bool WIDE>
 __global__ void __launch_bounds__(256) k_store_state(int n, StateSet<Real> S, const typename Vec4<Real>::T* vr,
                                                      double rho0, double* x, double* v, double* a, double* dr,
                                                      double* rho)
@@ -247,16 +250,17 @@ __global__ void __launch_bounds__(256) k_store_state(int n, StateSet<Real> S, co
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n) return;
     const size_t i = (size_t)S.id[k];
+    auto fp64 = [](auto q) { return WIDE ? wide(q) : (double)q; };
     auto row = [&](double* dst, const auto* src) {
         if (!dst) return;
 #pragma unroll
-        for (int d = 0; d < 3; ++d) dst[3 * i + d] = d < DIM ? wide(src[(size_t)d * n + k]) : 0.0;
+        for (int d = 0; d < 3; ++d) dst[3 * i + d] = d < DIM ? fp64(src[(size_t)d * n + k]) : 0.0;
     };
     row(x, S.x);
     row(v, S.v);
     row(a, S.a);
     row(dr, S.dr);
-    if (rho) rho[i] = S.kind[k] ? rho0 : rho0 + wide(vr[k].w);
+    if (rho) rho[i] = S.kind[k] ? rho0 : rho0 + fp64(vr[k].w);
 }
 
 // The adjoint's four cotangents between the caller's rows and [3][n]
@@ -358,12 +362,14 @@ cudaError_t launch_store_state(int prec, int dim, int n, const void* S, const vo
                                double* v, double* a, double* dr, double* rho, cudaStream_t st)
 {
     const int T = 256, nb = nblk(n, T);
-    if (prec == 64)
-        launch(dim == 2 ? k_store_state<double, 2> : k_store_state<double, 3>, nb, T, 0, st, n,
+    if (prec == 64) {
+        launch(dim == 2 ? k_store_state<double, 2, false> : k_store_state<double, 3, false>, nb, T, 0, st, n,
                *(const StateSet<double>*)S, (const double4_32a*)vr, rho0, x, v, a, dr, rho);
-    else
-        launch(dim == 2 ? k_store_state<float, 2> : k_store_state<float, 3>, nb, T, 0, st, n,
-               *(const StateSet<float>*)S, (const float4*)vr, rho0, x, v, a, dr, rho);
+        return cudaGetLastError();
+    }
+    auto kern = n < kWideFrom ? (dim == 2 ? k_store_state<float, 2, false> : k_store_state<float, 3, false>)
+                              : (dim == 2 ? k_store_state<float, 2, true> : k_store_state<float, 3, true>);
+    launch(kern, nb, T, 0, st, n, *(const StateSet<float>*)S, (const float4*)vr, rho0, x, v, a, dr, rho);
     return cudaGetLastError();
 }
 

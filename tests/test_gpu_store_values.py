@@ -11,9 +11,9 @@ from paper_2411_13992_gb300 import cases
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("dim", [2, 3])
-def test_single_outputs_of_extreme_values(dim):
-    c = (cases.tgv2d if dim == 2 else cases.tgv3d)(9, jitter_dp=0.1)
+@pytest.mark.parametrize("dim,side", [(2, 9), (3, 9), (2, 141), (2, 142), (3, 28)])     # the conversion changes at 20,000
+def test_single_outputs_of_extreme_values(dim, side):
+    c = (cases.tgv2d if dim == 2 else cases.tgv3d)(side, jitter_dp=0.1)
     n = c["n"]
     rng = np.random.default_rng(1)
     special = np.array([0.0, -0.0, 1e-45, -1e-45, 1.1754942e-38, -1.17549435e-38, 3.4028235e38, -3.4028235e38, 1.0])
