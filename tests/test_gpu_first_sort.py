@@ -27,8 +27,8 @@ def _case(share, n=SIDE * SIDE):
     return c
 
 
-def _same(s, t):
-    for k in KEYS:
+def _same(s, t, keys=KEYS):
+    for k in keys:
         assert np.array_equal(s[k], t[k]), k
 
 
@@ -102,3 +102,23 @@ def test_adjoint_segment_recorded_and_launched(share):
     for (_, b1, e1, s1), (_, b0, e0, s0) in zip(out[:2], out[2:]):
         assert e1 == e0 and all(np.array_equal(p, q) for p, q in zip(b1, b0))
         _same(s1, s0)
+
+
+@pytest.mark.parametrize("precision", [32, 64])
+def test_dual_integrator_carries_the_density_rate(precision):
+    c = _case(1.0)
+    rate = np.random.default_rng(9).standard_normal(c["n"])
+    if precision == 32:
+        rate = rate.astype(np.float32).astype(np.float64)
+    sim = sph.Simulation(c, precision=precision, integrator=sph.INT_DUAL)
+    try:
+        sim.set_state(drho=rate)
+        sim.build_cells()
+        first = sim.get_state()
+        assert np.array_equal(sim.density_rate(), rate)
+        sim.build_cells()
+        _same(first, sim.get_state(), ("x", "v", "rho"))     # (a and dr are the first step's)
+        assert np.array_equal(sim.density_rate(), rate)
+        sim.sync()
+    finally:
+        sim.close()
